@@ -22,7 +22,8 @@ namespace htd {
 namespace {
 thread_local std::string g_last_error;
 thread_local int64_t g_launches = 0;
-constexpr int kRoundsPerGraph = 16;
+constexpr int kRoundsPerGraph = 16;  // rebuild rounds
+constexpr int kSlotsPerGraph = 4;    // incremental slots
 }  // namespace
 
 void set_last_error(const std::string &msg) { g_last_error = msg; }
@@ -41,6 +42,7 @@ cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     return e;
 }
 GraphDev *graph_dev(htd_graph *g) { return &g->H.g; }
+void set_shared_device(htd_graph *g) { g->H.shared_device = true; }
 void add_launches(int64_t k) { g_launches += k; }
 
 }  // namespace htd
@@ -265,6 +267,7 @@ htd_status htd_h_support(htd_graph *g, int32_t h, int32_t *sup_dev, void *stream
     cudaStream_t user = static_cast<cudaStream_t>(stream);
     API_TRY(begin_call(H, user));
     API_TRY(prepare_work(H, h, h <= 2));
+    H->w.twin = false;
     H->w.dense_balls = false;  // h-support alone streams the smaller form of each ball
     H->w.inc3 = false;
     int64_t launches = 0;
@@ -290,7 +293,6 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     cudaStream_t user = static_cast<cudaStream_t>(stream);
     const bool timing = (flags & HTD_OPT_TIMING) != 0;
     const bool use_graph = (flags & HTD_OPT_NO_GRAPH) == 0;
-    const int R = htd::kRoundsPerGraph;
     htd_stats local;
     std::memset(&local, 0, sizeof(local));
     local.h = h;
@@ -319,6 +321,8 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         API_TRY(prepare_work(H, h, incremental, (flags & HTD_OPT_TINY_LOSS_TABLE) != 0));
         incremental = w.incremental;
         w.dense_balls = incremental && (h == 3 || ((flags & HTD_OPT_COMPACT_BALLS) == 0 && fits));
+        // a peel that shares the device keeps to a small part of what is free
+        API_TRY(htd::ensure_twin(H, (int64_t)(free_b / (H->shared_device ? 64 : 8))));
     }
     {
         htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, timing ? &local : nullptr);
@@ -332,7 +336,8 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     API_CHECK(cudaStreamSynchronize(H->pstream));
     API_TRY(check_status_err(w.status_host));
 
-    const int per_round = w.inc3 ? 5 : incremental ? 4 : h + 6;
+    // an incremental slot holds many rounds (the cluster round kernel)
+    const int R = incremental ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
     const bool persistent = incremental && h <= 2 && (flags & HTD_OPT_PERSISTENT_ROUNDS) != 0;
     if (persistent && w.status_host->alive > 0) {
         // one cooperative launch runs up to kPersistentSlots round slots; the host checks the
@@ -382,25 +387,27 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         const htd::DevStatus *sh = w.status_host;
         local.ms_select = sh->st_phase_ns[0] * 1e-6f;
         local.ms_find = sh->st_phase_ns[1] * 1e-6f;
-        local.ms_update = sh->st_phase_ns[2] * 1e-6f;
-        local.ms_minreduce = sh->st_phase_ns[3] * 1e-6f;
+        local.ms_update = sh->st_phase_ns[3] * 1e-6f;
+        local.ms_minreduce = sh->st_phase_ns[4] * 1e-6f;
         local.timed_slots = sh->st_slots;
     } else if (w.status_host->alive > 0) {
         // Graph path: R rounds per graph launch.  With HTD_OPT_TIMING a second graph with an
         // external event record at every phase boundary runs every kTimedEvery-th batch (the
         // events would otherwise slow every round); per-launch averages come from those.
         constexpr int kTimedEvery = 16;
-        if (timing && H->round_events.empty()) {
+        const bool by_events = timing && !incremental;  // incremental rounds time themselves
+        if (by_events && H->round_events.empty()) {
             H->round_events.resize(htd::kRoundEvents * R, nullptr);
             for (auto &e : H->round_events) API_CHECK(cudaEventCreate(&e));
         }
-        auto capture = [&](cudaGraphExec_t *exec, cudaEvent_t *ev) -> htd_status {
+        auto capture = [&](cudaGraphExec_t *exec, cudaEvent_t *ev, bool timed) -> htd_status {
             cudaGraph_t graph = nullptr;
             API_CHECK(cudaStreamBeginCapture(H->pstream, cudaStreamCaptureModeThreadLocal));
-            int64_t dummy = 0;
+            int64_t per_graph = 0;
             htd_status cs = HTD_OK;
             for (int r = 0; r < R && cs == HTD_OK; r++)
-                cs = htd::enqueue_round(H, H->pstream, &dummy, ev ? ev + htd::kRoundEvents * r : nullptr);
+                cs = htd::enqueue_round(H, H->pstream, &per_graph, ev ? ev + htd::kRoundEvents * r : nullptr,
+                                        timed);
             cudaError_t ce = cudaStreamEndCapture(H->pstream, &graph);
             if (cs != HTD_OK) {
                 if (graph) cudaGraphDestroy(graph);
@@ -417,20 +424,23 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
                 set_last_error(std::string("htd: graph instantiate: ") + cudaGetErrorString(ce));
                 return HTD_ECUDA;
             }
+            H->graph_launches = per_graph;
             return HTD_OK;
         };
         // the captured kernel arguments fix h, the round variant and the ball layout
         if (use_graph && (!H->graph_exec || H->graph_h != h || H->graph_incremental != incremental ||
-                          H->graph_dense != w.dense_balls)) {
+                          H->graph_dense != w.dense_balls || H->graph_shared != H->shared_device || H->graph_twin != w.twin)) {
             destroy_graph(H);
-            API_TRY(capture(&H->graph_exec, nullptr));
+            API_TRY(capture(&H->graph_exec, nullptr, false));
             H->graph_h = h;
             H->graph_rounds = R;
             H->graph_incremental = incremental;
             H->graph_dense = w.dense_balls;
+            H->graph_shared = H->shared_device;
+            H->graph_twin = w.twin;
         }
         if (use_graph && timing && !H->graph_exec_timed)
-            API_TRY(capture(&H->graph_exec_timed, H->round_events.data()));
+            API_TRY(capture(&H->graph_exec_timed, by_events ? H->round_events.data() : nullptr, true));
         // every active round removes at least one edge, so m/R + 2 batches always suffice
         const int64_t round_cap = H->g.m + 2 * R + 2;
         // continued incremental rounds handle at least one new lost pair per slot, and a
@@ -438,7 +448,7 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         const int64_t batch_cap =
             (H->g.m + (incremental ? w.status_host->st_ball_total / 2 + 1 : 0)) / R + 3;
         int64_t batches = 0;
-        bool timing_ok = timing;
+        bool timing_ok = by_events;
         while (w.status_host->alive > 0) {
             if (++batches > batch_cap) {
                 set_last_error("htd_truss_decompose: no progress within the batch cap");
@@ -447,12 +457,14 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
             const bool timed = timing_ok && (batches % kTimedEvery == 1);
             const int64_t slots_before = w.status_host->st_slots;
             if (use_graph) {
-                API_CHECK(cudaGraphLaunch(timed ? H->graph_exec_timed : H->graph_exec, H->pstream));
-                launches += (int64_t)R * per_round;
+                const bool second = timed || (timing && incremental);
+                API_CHECK(cudaGraphLaunch(second ? H->graph_exec_timed : H->graph_exec, H->pstream));
+                launches += H->graph_launches;
             } else {
                 for (int r = 0; r < R; r++) {
                     API_TRY(htd::enqueue_round(H, H->pstream, &launches,
-                                               timed ? &H->round_events[htd::kRoundEvents * r] : nullptr));
+                                               timed ? &H->round_events[htd::kRoundEvents * r] : nullptr,
+                                               timing));
                 }
             }
             count_launches();
@@ -488,16 +500,10 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
                     }
                     if (!timing_ok) break;
                     local.ms_select += t[0];
-                    if (incremental) {
-                        local.ms_remove += t[1];
-                        local.ms_find += t[2];
-                        local.ms_update += t[3] + t[4];
-                    } else {
-                        local.ms_find += t[1];
-                        local.ms_remove += t[2];
-                        local.ms_ball += t[3];
-                        local.ms_update += t[4];
-                    }
+                    local.ms_find += t[1];
+                    local.ms_remove += t[2];
+                    local.ms_ball += t[3];
+                    local.ms_update += t[4];
                     local.ms_minreduce += t[5];
                     local.timed_slots += 1;
                 }
@@ -507,6 +513,16 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
                 set_last_error("htd_truss_decompose: round cap exceeded");
                 return HTD_ETIMEOUT;
             }
+        }
+        if (timing && incremental) {
+            // as at the event-timed rounds: detection | radius-3 tests in the "remove" place
+            const unsigned long long *ns = w.status_host->st_phase_ns;
+            local.ms_select = ns[0] * 1e-6f;
+            local.ms_remove = (h == 3 ? ns[1] : 0) * 1e-6f;
+            local.ms_find = (h == 3 ? ns[2] : ns[1]) * 1e-6f;
+            local.ms_update = ns[3] * 1e-6f;
+            local.ms_minreduce = ns[4] * 1e-6f;
+            local.timed_slots = w.status_host->st_slots;
         }
     }
     const int64_t m = H->g.m;

@@ -11,13 +11,40 @@ namespace htd {
 constexpr int kMaxH = 8;
 constexpr int kWarp = 32;
 
+// Work counters of one removal round.  The launches of a round keep them in the status block;
+// the cluster round kernel keeps its own in the shared memory of one of its blocks.
+struct RoundCtr {
+    int32_t nF;                // frontier size of the current round
+    int32_t npitems;           // loss detection items of the current batch
+    int32_t nuitems;           // support update items of the current batch
+    int32_t nlost;             // lost-pair records of the current batch (duplicates nulled)
+    int32_t nlost2;            // radius-2 lost-pair records of the current round (h = 3)
+    int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
+    int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
+    int32_t pad;
+    long long touched;         // alive edges at endpoints of the batch's lost pairs (once per round)
+    long long upd_work;        // adjacency slots reserved for the batch's updates
+    long long nc3items;        // stored radius-3 candidate items of the current round (64-bit: the
+                               // reservations of a huge round may pass 2^31 before it halts)
+};
+
+// Lists of the cluster round kernel: its window, and the edges the last updates took to the
+// level.
+struct WindowCtr {
+    int32_t nwin, nnext;
+};
+
+// What the helpers of the cluster round kernel need of a phase they share.
+struct HelperJob {
+    int32_t phase, nitems, nF, round, win_hi, thr;
+};
+
 // Device-resident state of one peel.  Written only by kernels (and zero-initialised by
 // the host before the first pass); read by the host between CUDA-graph launches.
-struct DevStatus {
+struct DevStatus : RoundCtr {
     int32_t k;                 // current peeling level (Algorithm 1's k)
     int32_t round;             // removal rounds completed
     int64_t alive;             // edges not yet removed
-    int32_t nF;                // frontier size of the current round
     int32_t cand_cnt[kMaxH];   // candidate vertices found at BFS depth 0..h-1
     int32_t nchanged;          // vertices whose ball shrank this round
     int32_t nitems;            // h-support work items this round
@@ -40,19 +67,25 @@ struct DevStatus {
     unsigned long long st_bytes_hsup;  // algorithmic bytes, intersections
     unsigned long long st_bytes_hsup_init;  // the initial pass's share of st_bytes_hsup
     // incremental (h <= 2) rounds
-    int32_t nlost;             // lost-pair records of the current batch (duplicates nulled)
     int32_t cont;              // 1: the current round continues (its frontier is removed)
     int32_t unit_begin;        // first frontier edge side the next loss detection tests
-    int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
-    int32_t npitems;           // loss detection items of the current batch
-    int32_t nuitems;           // support update items of the current batch
-    int32_t pad1;
-    long long upd_work;        // adjacency slots reserved for the batch's updates
+    int32_t stage;             // graph path: first phase launch the cluster round kernel left to the
+                               // launches after it (RoundStage), kStageNone if none
+    // cluster round kernel with helpers (monotonic over the launches of one peel)
+    unsigned long long cl_tickets;  // clusters started
+    unsigned long long cl_exit;     // launches whose leader has finished
+    unsigned long long cl_reg;      // (launch << 32) | helper blocks started
+    unsigned long long cl_job;      // (launch << 40) | (job number << 16) | helper blocks taking part
+    unsigned long long cl_done;     // helper blocks that finished a job
+    HelperJob cl_work;
+    WindowCtr cl_wctr;
+    RoundCtr cl_ctr;
     unsigned bar_count;        // grid barrier of the persistent round kernel: groups arrived
     unsigned bar_gen;          // generation, advanced by the last arrival
     unsigned bar_group[64];    // blocks arrived, per group of 32 blocks
-    long long st_slots;        // round slots run by the persistent kernel
-    unsigned long long st_phase_ns[8];  // persistent kernel: time per phase (block 0's view)
+    long long st_slots;        // round slots run (rounds plus continued batches)
+    unsigned long long st_phase_ns[8];  // time per phase (one block's view)
+    unsigned long long st_phase_start;  // when the running phase launch began
     int64_t st_ball_total;     // sum of the initial ball sizes
     int64_t st_pairs;          // candidate pairs tested
     int64_t st_lost;           // lost pairs
@@ -60,15 +93,19 @@ struct DevStatus {
     unsigned long long st_bytes_detect;  // algorithmic bytes, loss detection
     unsigned long long st_bytes_update;  // algorithmic bytes, incremental support updates
     // incremental h = 3 rounds (radius-2 balls kept beside the radius-3 support balls)
-    int32_t nlost2;            // radius-2 lost-pair records of the current round
-    int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
-    long long nc3items;        // stored radius-3 candidate items of the current round (64-bit: the
-                               // reservations of a huge round may pass 2^31 before it halts)
     int64_t st_c3_pairs;       // radius-3 candidate pairs tested
     int64_t st_lost2;          // radius-2 lost pairs
     int64_t st_recovered;      // rounds finished by the rebuild recovery
 };
 
+// Phases of an incremental round, in order, as the graph path launches them.
+enum RoundStage : int32_t {
+    kStageNone = 0,
+    kStageSelect = 1,
+    kStageDetect = 2,
+    kStageTest3 = 3,
+    kStageDelta = 4,
+};
 
 enum : int32_t {
     kErrBallGrew = 1,        // a rebuilt ball was larger than before (cannot happen)

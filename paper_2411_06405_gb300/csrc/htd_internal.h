@@ -64,14 +64,23 @@ struct PeelWork {
     uint32_t *hub_bits = nullptr;  // nhub x Wpad words: alive neighbours as n-bit sets
     int32_t nhub = 0;
     int32_t hub_min_deg = 0;
-    int4 *pitems = nullptr;        // loss detection items (edge side, first slot, x, y), <= 32 pairs
+    int4 *pitems = nullptr;        // loss detection items, two int4 each, <= 32 pairs
     int64_t pitems_cap = 0;
     int4 *uitems = nullptr;        // support update items (first slot, v, w, row end), <= 32 slots
     int64_t uitems_cap = 0;
+    int32_t *win = nullptr;        // cluster round kernel: its window and its next frontier
+    int64_t win_cap = 0;           // edges each holds
+    int4 *erec = nullptr;          // 2m: per edge (u, v, slot_lo, slot_hi), (row u, end, row v, end)
+    int4 *srec = nullptr;          // 2m: per adjacency slot (neighbour, its row, its end, edge)
     int64_t upd_budget = 0;        // adjacency slots one batch of updates may visit
     // incremental h = 3: radius-2 balls (dense, x * Wpad) and their own metadata, used by
     // the loss tests and by the rebuild that finishes a round which ran out of room
     bool inc3 = false;
+    // Twin matrices of the dense balls (radius h, and radius 2 at h = 3): the stored balls minus
+    // the losses of the running batch.
+    bool twin = false;             // in use (set per call before the initial pass)
+    uint32_t *pool_new = nullptr;
+    uint32_t *pool2_new = nullptr;
     uint32_t *pool2 = nullptr;
     int32_t *ball_size2 = nullptr;
     int32_t *ball_nw2 = nullptr;
@@ -107,9 +116,13 @@ struct Handle {
     std::vector<cudaEvent_t> round_events;      // events of the timed graph
     int graph_h = 0;
     int graph_rounds = 0;
+    int64_t graph_launches = 0;    // kernels of one launch of it
     bool graph_incremental = false;
     bool graph_dense = false;      // ball layout the captured rounds address directly
     int num_sms = 0;
+    bool shared_device = false;    // peels of other streams run beside this one
+    bool graph_shared = false;     // the captured rounds' setting of it
+    bool graph_twin = false;       // the captured rounds use the twin matrices
 };
 
 void set_last_error(const std::string &msg);
@@ -129,11 +142,13 @@ void free_graph_dev(GraphDev *g);
 // Ball builder, h-support and peel rounds (htd_peel.cu).
 htd_status ensure_work(Handle *H, int32_t h, bool incremental, bool tiny_table = false);
 void free_work(PeelWork *w);
+htd_status ensure_twin(Handle *H, int64_t budget);
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
                         htd_stats *timing);
 // evs (nullable): kRoundEvents events marking the phase boundaries of the round.
 constexpr int kRoundEvents = 7;
-htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs);
+// timer (incremental rounds, instead of events): phase times go to the status block.
+htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer);
 
 // Persistent kernel running up to max_slots incremental round slots (htd_loss.cu).
 htd_status launch_persistent_rounds(Handle *H, cudaStream_t s, int max_slots, int64_t *launches);
@@ -147,6 +162,8 @@ htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches);
 
 // The normalised graph behind a public handle (htd_api.cu).
 GraphDev *graph_dev(htd_graph *g);
+// Tells a handle that its decompositions run beside others (they then take less of the device).
+void set_shared_device(htd_graph *g);
 
 // One small graph of a batch for the block-per-graph launch (htd_batch_block.cu): device
 // pointers into its union's CSR, its vertices [v0, v0 + L) and edges [e0, e0 + m) there,
@@ -165,8 +182,9 @@ htd_status batch_block_run(const std::vector<BlockGraphDescHost> &graphs, cudaSt
 htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_t max_iter, bool prune,
                       int32_t *truss_dev, int32_t *hval_dev, htd_hindex_stats *stats, cudaStream_t s);
 
-// One incremental round (h <= 3) as four (h = 3: five) launches, the graph path (htd_loss.cu).
-htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs,
-                                     unsigned record_flags);
+// One slot of incremental rounds (h <= 3), the graph path (htd_loss.cu): the cluster round
+// kernel, then four (h = 3: five) phase launches for the round it left to them.
+// timer: the phases' times are added to the status block.
+htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer);
 
 }  // namespace htd

@@ -8,7 +8,8 @@
 // for every (a,b) in F (for h = 1 only {a,b}).  Each such pair is tested in the new graph
 // (adjacent, or for h = 2 a common alive neighbour); a pair that fails is "lost": each
 // endpoint leaves the other's ball (distance is symmetric).  Lost pairs are deduplicated
-// in an open-addressing hash set.
+// in an open-addressing hash set, or, where memory allows a second copy of the ball matrix
+// (the "twin"), by clearing the pair's bits there: the twin is then the matrix of B_new.
 //
 // The h-support of an alive edge (x,y), x < y, then drops by exactly
 //     |L(x) ∩ B_old(y)| + |L(y) ∩ B_new(x)|,
@@ -23,6 +24,7 @@
 // batch of the same round, so it is skipped.  Detection records the first frontier edge
 // side it could not finish; the next round slot resumes there without selecting anew.
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 
 #include "htd_internal.h"
@@ -46,7 +48,7 @@ struct LossArgs {
     uint32_t *hub_bits_w;
     int32_t h;
     int32_t lost_max;
-    unsigned long long cap_mask;
+    unsigned cap_mask;
     const int32_t *row_ptr;
     const int32_t *col;
     const int32_t *col_live;
@@ -71,23 +73,33 @@ struct LossArgs {
     int32_t dense_all;  // every ball dense at pool + x * Wpad (no metadata lookup)
     int32_t hub_all;    // every vertex has its alive-adjacency set, at row x
     int32_t pitems_cap;
-    int4 *pitems;
+    int4 *pitems;       // two per item: (edge side, first slot, x, y), (row x, end, row y, end)
     int32_t uitems_cap;
     int4 *uitems;
     long long upd_budget;
     DevStatus *st;
     // h = 3: radius-2 balls and the round's radius-2 losses
     int32_t h3;         // incremental h = 3 round: overflows halt the round (host rebuild)
-    int32_t rec_r2;     // this launch records radius-2 losses (no support updates)
     uint32_t *pool2;    // dense radius-2 balls, row x at x * Wpad
     int32_t *ball_size2;
     unsigned long long *keys2;
-    unsigned long long cap2_mask;
+    unsigned cap2_mask;
     int4 *lost2;
     int32_t lost2_max;
     int32_t c3items_cap;
     int4 *c3items;
     int32_t *touch2;    // h = 3: round in which the vertex last lost a radius-2 member
+    // Twin ball matrices (null without): pool and pool2 hold the balls of before the batch,
+    // these the same minus the batch's losses so far.
+    uint32_t *pool_new;
+    uint32_t *pool2_new;
+    int32_t cluster;    // the slot starts with the cluster round kernel
+    int32_t timer;      // add the time of each phase to the status block
+    int32_t win_cap;    // cluster round kernel: edges its window and next-frontier lists hold
+    int32_t *win;
+    int32_t *next;
+    const int4 *erec;   // per edge: (u, v, slot in u's row, slot in v's row), (row u, row v)
+    const int4 *srec;   // per adjacency slot: (neighbour, its row, its row's end, edge)
 };
 
 __device__ __forceinline__ unsigned long long pair_key(int p, int q) {
@@ -95,14 +107,13 @@ __device__ __forceinline__ unsigned long long pair_key(int p, int q) {
     return ((unsigned long long)a << 32) | b;
 }
 
-// 64-bit finaliser of MurmurHash3 (public domain), used to spread pair keys.
-__device__ __forceinline__ unsigned long long mix64(unsigned long long k) {
-    k ^= k >> 33;
-    k *= 0xff51afd7ed558ccdull;
-    k ^= k >> 33;
-    k *= 0xc4ceb9fe1a85ec53ull;
-    k ^= k >> 33;
-    return k;
+// First slot of the pair {p,q} in a table of mask + 1 slots: multiplicative hashing (Knuth) of
+// both ids in 32 bits.  (With a 64-bit mix of the key, its two wide multiplications were a
+// third of the instructions of a support update that probes.)
+__device__ __forceinline__ unsigned pair_slot(int p, int q, unsigned mask) {
+    unsigned x = (unsigned)min(p, q) * 0x9e3779b1u + (unsigned)max(p, q) * 0x85ebca6bu;
+    x ^= x >> 15;
+    return x & mask;
 }
 
 // Status fields are written by other blocks between the phases of the persistent kernel:
@@ -114,14 +125,18 @@ __device__ __forceinline__ T vload(const T &x) {
 
 // A batch limit was reached at edge side u: h <= 2 resumes the round there in the next slot;
 // an h = 3 round halts and the host finishes it by rebuilds.
-__device__ __forceinline__ void overflow_at(const LossArgs &a, DevStatus *st, int u) {
-    if (a.h3) atomicOr(&st->halt, 1);
-    else atomicMin(&st->overflow_unit, u);
+__device__ __forceinline__ void overflow_at(const LossArgs &a, RoundCtr *c, int u) {
+    if (a.h3) atomicOr(&c->halt, 1);
+    else atomicMin(&c->overflow_unit, u);
 }
 
-// Round kernels do nothing once the peel is over or a round halted.
-__device__ __forceinline__ bool round_idle(const LossArgs &a) {
-    return vload(a.st->alive) == 0 || vload(a.st->halt) != 0;
+// Round kernels do nothing once the peel is over or a round halted, and a phase launch of a
+// slot with the cluster round kernel only runs from the phase that kernel left to it.
+__device__ __forceinline__ bool round_idle(const LossArgs &a, RoundStage phase) {
+    if (vload(a.st->alive) == 0 || vload(a.st->halt) != 0) return true;
+    if (!a.cluster) return false;
+    const int stage = vload(a.st->stage);
+    return stage == kStageNone || stage > phase;
 }
 
 // Alive-adjacency set of p if p has one (high degree), else null.
@@ -130,6 +145,10 @@ __device__ __forceinline__ const uint32_t *hub_set(const LossArgs &a, int p, uns
     reads++;
     const int hs = a.hub_slot[p];
     return hs >= 0 ? a.hub_bits + (int64_t)hs * a.Wpad : nullptr;
+}
+
+__device__ __forceinline__ bool bit_of(const uint32_t *m, int Wpad, int row, int col) {
+    return (m[(int64_t)row * Wpad + (col >> 5)] >> (col & 31)) & 1u;
 }
 
 // Is q an alive neighbour of p?  One bit of p's alive-adjacency set when p has one, else a
@@ -162,24 +181,14 @@ constexpr int kInlineScan = 8;
 
 enum PairState { kKept = 0, kLost = 1, kHard = 2 };
 
-// First test of the pair {p,q} (p != q) in the alive graph, by one lane: adjacency by
-// binary search in the shorter row, then (h = 2) a common alive neighbour when the shorter
-// row is at most kInlineScan long.  Longer scans are left to the warp (kHard).
-__device__ __forceinline__ int pair_quick(const LossArgs &a, int &p, int &q, unsigned &reads) {
-    const int dp = a.row_ptr[p + 1] - a.row_ptr[p];
-    const int dq = a.row_ptr[q + 1] - a.row_ptr[q];
-    reads += 4;
-    if (dp > dq) {  // p: the shorter row
-        const int t = p;
-        p = q;
-        q = t;
-    }
-    const uint32_t *qset = hub_set(a, q, reads);
-    if (alive_adjacent_set(a, qset, q, p, reads)) return kKept;
-    if (a.h < 2) return kLost;
+// Test of the non-adjacent pair {p,q} (h = 2) in the alive graph by one lane: p's row
+// [rb, re) is the shorter one; a common alive neighbour is looked for when it is at most
+// kInlineScan long, longer rows are left to the warp (kHard).
+template <bool kTwin>
+__device__ __forceinline__ int pair_quick(const LossArgs &a, int rb, int re, int q, unsigned &reads) {
     // with q's set every scanned neighbour costs one read; without it, a binary search
-    if (min(dp, dq) > kInlineScan) return kHard;
-    const int rb = a.row_ptr[p], re = a.row_ptr[p + 1];
+    if (re - rb > kInlineScan) return kHard;
+    const uint32_t *qset = kTwin ? a.hub_bits + (int64_t)q * a.Wpad : hub_set(a, q, reads);
     // four slots at a time: their loads (and their set lookups) are independent
     for (int s0 = rb; s0 < re; s0 += 4) {
         int y[4];
@@ -188,7 +197,10 @@ __device__ __forceinline__ int pair_quick(const LossArgs &a, int &p, int &q, uns
         bool hit = false;
 #pragma unroll
         for (int j = 0; j < 4; j++)
-            if (y[j] >= 0) hit |= alive_adjacent_set(a, qset, q, y[j], reads);
+            if (y[j] >= 0) {
+                if (kTwin) hit |= (qset[y[j] >> 5] >> (y[j] & 31)) & 1u;
+                else hit |= alive_adjacent_set(a, qset, q, y[j], reads);
+            }
         reads += (unsigned)min(4, re - s0);
         if (hit) return kKept;
     }
@@ -211,25 +223,20 @@ __device__ __forceinline__ T warp_incl_scan(T v) {
 // loads are independent, so a step costs two round trips whatever the count).
 constexpr int kWalkUnroll = 4;
 
-// Common alive neighbours for the warp's hard pairs (lanes with state == kHard; p the
-// shorter row), all at once: the pairs' rows of p are laid end to end and the warp walks
+// Common alive neighbours for the warp's hard pairs (lanes with state == kHard; p's row
+// [rb, re), the shorter one), all at once: the pairs' rows of p are laid end to end and the warp walks
 // the concatenation 32 x kWalkUnroll slots per step, each lane finding the pair its slot belongs to by a
 // binary search over the lanes' running row lengths.  A pair is kept at its first alive
 // neighbour that q also has; the walk skips kept pairs and stops once none is pending.
 // Called by whole warps.
-__device__ __forceinline__ void warp_hard_pairs(const LossArgs &a, int &state, int p, int q,
+template <bool kTwin>
+__device__ __forceinline__ void warp_hard_pairs(const LossArgs &a, int &state, int rb, int re, int q,
                                                 unsigned &reads) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool hard = state == kHard;
-    int rb = 0, len = 0;
-    const uint32_t *qset = nullptr;
-    if (hard) {
-        rb = a.row_ptr[p];
-        len = a.row_ptr[p + 1] - rb;
-        qset = hub_set(a, q, reads);
-        reads += 2;
-    }
+    const int len = hard ? re - rb : 0;
+    const uint32_t *qset = !hard ? nullptr : kTwin ? a.hub_bits + (int64_t)q * a.Wpad : hub_set(a, q, reads);
     const int incl = warp_incl_scan(len);
     const int excl = incl - len;
     const int total = __shfl_sync(full, incl, 31);
@@ -258,7 +265,8 @@ __device__ __forceinline__ void warp_hard_pairs(const LossArgs &a, int &state, i
                 __shfl_sync(full, reinterpret_cast<unsigned long long>(qset), own[j]));
             if (y[j] >= 0) {
                 reads++;
-                if (alive_adjacent_set(a, qs, qo, y[j], reads)) hits |= 1u << own[j];
+                if (kTwin ? (qs[y[j] >> 5] >> (y[j] & 31)) & 1u : alive_adjacent_set(a, qs, qo, y[j], reads))
+                    hits |= 1u << own[j];
             }
         }
         hits = __reduce_or_sync(full, hits);
@@ -302,54 +310,39 @@ __device__ __forceinline__ bool ball_contains(const LossArgs &a, int z, int w, u
     return ball_contains_meta(a, a.ball_meta[z], w, bytes);
 }
 
-// Records the lost pair {x,z} unless an earlier batch of this round handled it.  The
-// record and the pair's update work (both rows are visited by the support updates) are
-// reserved against the batch limits; a pair that does not fit marks its edge side u as
-// the point where the next slot of this round resumes.
-// Is the pair {p,q} among this batch's lost pairs?
-__device__ __forceinline__ bool lost_now(const LossArgs &a, int p, int q, unsigned &bytes) {
+// Is the pair {p,q} in the table of the batch's lost pairs?  `probes` counts its slots read.
+__device__ __forceinline__ bool in_pair_set(const unsigned long long *keys, unsigned mask, int p, int q,
+                                            unsigned &probes) {
     const unsigned long long key = pair_key(p, q);
-    unsigned long long slot = mix64(key) & a.cap_mask;
-    for (unsigned long long probe = 0; probe <= a.cap_mask; probe++) {
-        const unsigned long long k = a.keys[slot];
-        bytes += 8;
+    unsigned slot = pair_slot(p, q, mask);
+    for (unsigned probe = 0; probe <= mask; probe++) {
+        const unsigned long long k = keys[slot];
+        probes++;
         if (k == key) return true;
         if (k == kEmpty) return false;
-        slot = (slot + 1) & a.cap_mask;
+        slot = (slot + 1) & mask;
     }
     return false;
 }
 
-// Records the lost pairs {x, z} of a warp (lanes with lost == true; all lanes call it).
-// A pair whose stored bit is already clear was handled by an earlier batch of this round
-// and is skipped.  Each record and its update work (both rows are visited by the support
-// updates) are reserved against the batch limits with one atomic per warp and counter; a
-// pair that does not fit marks its edge side u as the point where the next slot of this
-// round resumes.  New pairs go into the lost-pair set, and their update items (runs of 32
-// slots of each endpoint's row) are written: by their own lane when few, else by the warp.
-__device__ __forceinline__ void record_lost_warp(const LossArgs &a, DevStatus *st, bool lost, int x,
-                                                 int z, int u, unsigned &reads) {
+// Records the lost pairs {x, z} of a warp (lanes with want == true; all lanes call it; the
+// stored bit of each is set: a pair whose bit is clear was handled by an earlier batch of
+// this round).  [rbx, rex) and [rbz, rez) are the endpoints' rows.  Each record and its
+// update work (both rows are visited by the support updates) are reserved against the batch
+// limits with one atomic per warp and counter; a pair that does not fit marks its edge side
+// u as the point where the next slot of this round resumes.  New pairs go into the lost-pair
+// set, and their update items (runs of 32 slots of each endpoint's row) are written: by
+// their own lane when few, else by the warp.  Also counts, once per round and vertex, the
+// alive edges whose support the round brings up to date (every alive edge at an endpoint of
+// a lost pair).
+// r2: radius-2 losses of an h = 3 round (recorded only: they change no support).
+// kTwin: the pair is new if its bit is still set in the twin matrix, which is cleared.
+template <bool r2, bool kTwin>
+__device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ctr, int round, bool want,
+                                                 int x, int z, int rbx, int rex, int rbz, int rez, int u) {
     constexpr int kOwnItems = 8;
     const int lane = threadIdx.x & 31;
-    const bool r2 = a.rec_r2 != 0;  // radius-2 losses of an h = 3 round: record only
-    bool want = false;
-    if (lost) {
-        if (r2) {
-            reads++;
-            want = (a.pool2[(int64_t)x * a.Wpad + (z >> 5)] >> (z & 31)) & 1u;
-        } else {
-            want = ball_contains(a, x, z, reads);
-        }
-    }
-    int rbx = 0, rex = 0, rbz = 0, rez = 0;
-    long long work = 0;
-    if (want && !r2) {
-        rbx = a.row_ptr[x];
-        rex = a.row_ptr[x + 1];
-        rbz = a.row_ptr[z];
-        rez = a.row_ptr[z + 1];
-        work = (long long)(rex - rbx) + (rez - rbz);
-    }
+    const long long work = (want && !r2) ? (long long)(rex - rbx) + (rez - rbz) : 0ll;
     const unsigned wantb = __ballot_sync(0xffffffffu, want);
     if (wantb == 0u) return;
     const long long wincl = warp_incl_scan(work);
@@ -359,39 +352,50 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, DevStatus *s
     int ibase = 0;
     if (lane == 0) {
         if (!r2)
-            wbase = (long long)atomicAdd((unsigned long long *)&st->upd_work, (unsigned long long)wtot);
-        ibase = atomicAdd(r2 ? &st->nlost2 : &st->nlost, __popc(wantb));
+            wbase = (long long)atomicAdd((unsigned long long *)&ctr->upd_work, (unsigned long long)wtot);
+        ibase = atomicAdd(r2 ? &ctr->nlost2 : &ctr->nlost, __popc(wantb));
     }
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
     ibase = __shfl_sync(0xffffffffu, ibase, 0);
     int4 *const lostv = r2 ? a.lost2 : a.lost;
     unsigned long long *const keys = r2 ? a.keys2 : a.keys;
-    const unsigned long long cmask = r2 ? a.cap2_mask : a.cap_mask;
+    const unsigned cmask = r2 ? a.cap2_mask : a.cap_mask;
     const int lmax = r2 ? a.lost2_max : a.lost_max;
     int rec_idx = -1;
     if (want) {
         const int idx = ibase + rank;
         if (idx >= lmax || (!r2 && wbase + wincl > a.upd_budget)) {
-            overflow_at(a, st, u);
+            overflow_at(a, ctr, u);
             if (idx < lmax) lostv[idx] = make_int4(-1, -1, -1, 0);
         } else {
-            const unsigned long long key = pair_key(x, z);
-            unsigned long long slot = mix64(key) & cmask;
             int4 rec = make_int4(-1, -1, -1, 0);  // null record: the pair is already held
-            for (unsigned long long probe = 0; probe <= cmask; probe++) {
-                const unsigned long long prev = atomicCAS(keys + slot, kEmpty, key);
-                if (prev == kEmpty) {
-                    rec = make_int4(min(x, z), max(x, z), (int)slot, 0);
-                    break;
+            if (kTwin) {
+                uint32_t *const twin = r2 ? a.pool2_new : a.pool_new;
+                // another warp may be recording the pair from its other end: the bit in the
+                // smaller id's row decides
+                const int lo = min(x, z), hi = max(x, z);
+                const uint32_t bit = 1u << (hi & 31);
+                if (atomicAnd(twin + (int64_t)lo * a.Wpad + (hi >> 5), ~bit) & bit) {
+                    atomicAnd(twin + (int64_t)hi * a.Wpad + (lo >> 5), ~(1u << (lo & 31)));
+                    rec = make_int4(lo, hi, 0, 0);
                 }
-                if (prev == key) break;
-                slot = (slot + 1) & cmask;
+            } else {
+                const unsigned long long key = pair_key(x, z);
+                unsigned slot = pair_slot(x, z, cmask);
+                for (unsigned probe = 0; probe <= cmask; probe++) {
+                    const unsigned long long prev = atomicCAS(keys + slot, kEmpty, key);
+                    if (prev == kEmpty) {
+                        rec = make_int4(min(x, z), max(x, z), (int)slot, 0);
+                        break;
+                    }
+                    if (prev == key) break;
+                    slot = (slot + 1) & cmask;
+                }
             }
             lostv[idx] = rec;
             if (rec.x >= 0) rec_idx = idx;
-            if (r2) {
+            if (r2 && !kTwin) {
                 // B2_new(v) differs from the stored B2(v) only at vertices marked here
-                const int round = vload(st->round);
                 a.touch2[x] = round;
                 a.touch2[z] = round;
             }
@@ -400,7 +404,11 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, DevStatus *s
     if (r2) return;  // radius-2 losses change no support directly
     // update items: direction 0 = v0 = min loses v1, direction 1 = v1 loses v0
     int v0 = 0, v1 = 0, rb0 = 0, re0 = 0, rb1 = 0, re1 = 0, n0 = 0, n1 = 0;
+    unsigned touched = 0u;
     if (rec_idx >= 0) {
+        const unsigned dx = (unsigned)a.deg_alive[x], dz = (unsigned)a.deg_alive[z];
+        if (atomicExch(a.vtouch + x, round) != round) touched += dx;
+        if (atomicExch(a.vtouch + z, round) != round) touched += dz;
         const bool xf = x < z;
         v0 = xf ? x : z;
         v1 = xf ? z : x;
@@ -413,7 +421,7 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, DevStatus *s
     }
     const int nincl = warp_incl_scan(n0 + n1);
     int nbase = 0;
-    if (lane == 31 && nincl) nbase = atomicAdd(&st->nuitems, nincl);
+    if (lane == 31 && nincl) nbase = atomicAdd(&ctr->nuitems, nincl);
     nbase = __shfl_sync(0xffffffffu, nbase, 31);
     const int base = nbase + nincl - (n0 + n1);
     if (rec_idx >= 0 && n0 + n1 <= kOwnItems) {
@@ -434,25 +442,35 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, DevStatus *s
             a.uitems[b + c] = (c < c0) ? make_int4(b0 + 32 * c, w0, w1, e0)
                                        : make_int4(b1 + 32 * (c - c0), w1, w0, e1);
     }
+    touched = __reduce_add_sync(0xffffffffu, touched);
+    if (lane == 0 && touched) atomicAdd((unsigned long long *)&ctr->touched, (unsigned long long)touched);
 }
 
 // Pair enumeration of edge side u = (edge F[u/2], side u%2): side 0 of (a,b) pairs a with
 // {b} and with N_old(b) \ {a} (slots start-1 .. re-1 of b's row, start-1 standing for b);
 // side 1 pairs b with N_old(a) \ {b}.  For h = 1 only {a,b}.
 struct UnitInfo {
-    int x, y, rb, start, stop;
+    int x, y, start, stop;
+    int4 rows;  // (row x, end, row y, end)
 };
 
 __device__ __forceinline__ UnitInfo unit_info(const LossArgs &a, int u) {
     UnitInfo r;
     const int e = a.frontier[u >> 1];
     const int side = u & 1;
-    r.x = side ? a.ev[e] : a.eu[e];
-    r.y = side ? a.eu[e] : a.ev[e];
-    r.rb = a.row_ptr[r.y];
-    r.start = (side == 0) ? r.rb - 1 : r.rb;
-    r.stop = (a.h < 2) ? ((side == 0) ? r.rb : r.rb) : a.row_ptr[r.y + 1];
+    const int4 ends = a.erec[2 * (int64_t)e], rows = a.erec[2 * (int64_t)e + 1];
+    r.x = side ? ends.y : ends.x;
+    r.y = side ? ends.x : ends.y;
+    r.rows = side ? make_int4(rows.z, rows.w, rows.x, rows.y) : rows;
+    r.start = (side == 0) ? r.rows.z - 1 : r.rows.z;
+    r.stop = (a.h < 2) ? r.rows.z : r.rows.w;
     return r;
+}
+
+// Detection item i: <= 32 pairs of edge side u from slot `first` on (u < 0: empty).
+__device__ __forceinline__ void write_pitem(const LossArgs &a, int i, int u, int first, int x, int y, int4 rows) {
+    a.pitems[2 * (int64_t)i] = make_int4(u, first, x, y);
+    a.pitems[2 * (int64_t)i + 1] = rows;
 }
 
 // Splits the frontier's edge sides into detection items of at most 32 pairs (one warp
@@ -466,11 +484,13 @@ __device__ void ph_pair_items(const LossArgs &a) {
     for (int b = u0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < units; b += stride) {
         const int u = b + lane;
         int nch = 0, start = 0, x = 0, y = 0;
+        int4 rows = make_int4(0, 0, 0, 0);
         if (u < units) {
             const UnitInfo r = unit_info(a, u);
             start = r.start;
             x = r.x;
             y = r.y;
+            rows = r.rows;
             nch = (r.stop - r.start + 31) >> 5;
         }
         int incl = nch;
@@ -494,16 +514,92 @@ __device__ void ph_pair_items(const LossArgs &a) {
             const int f = __shfl_sync(0xffffffffu, first, l), c_n = __shfl_sync(0xffffffffu, nch, l);
             const int ul = __shfl_sync(0xffffffffu, u, l), sl = __shfl_sync(0xffffffffu, start, l);
             const int xl = __shfl_sync(0xffffffffu, x, l), yl = __shfl_sync(0xffffffffu, y, l);
+            const int4 rl = make_int4(__shfl_sync(0xffffffffu, rows.x, l), __shfl_sync(0xffffffffu, rows.y, l),
+                                      __shfl_sync(0xffffffffu, rows.z, l), __shfl_sync(0xffffffffu, rows.w, l));
             const bool fl = __shfl_sync(0xffffffffu, fits, l);
             for (int c = lane; c < c_n && f + c < a.pitems_cap; c += 32)
-                a.pitems[f + c] = fl ? make_int4(ul, sl + 32 * c, xl, yl) : make_int4(-1, 0, 0, 0);
+                write_pitem(a, f + c, fl ? ul : -1, sl + 32 * c, xl, yl, rl);
         }
     }
+}
+
+// Warps that share one detection item: with few items, 2^split_log2 warps take the same
+// item and every 2^split_log2-th of its pairs, so that the walks of its hard pairs run side
+// by side instead of one after the other in one warp (the median round of R-MAT 16 at h = 2
+// has 79 items for 6,000 resident warps).
+// Where the counters a warp's records reserve from are in global memory, more than 2^2 warps
+// per item cost more in same-address atomics than their walks save.
+__device__ __forceinline__ int split_log2(int nitems, int nwarps, int most) {
+    int lg = 0;
+    while (lg < most && nitems <= (nwarps >> (lg + 1))) lg++;
+    return lg;
 }
 
 // Loss detection, one warp per item: lane i tests the pair of slot item.y + i.  A pair is
 // kept if its endpoints are adjacent or (h = 2) share an alive neighbour; the pairs whose
 // test needs a longer row scan are walked by the whole warp together.
+template <bool r2, bool kTwin>
+__device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps,
+                                             int nitems, int max_split, int round, unsigned &pairs,
+                                             unsigned &reads) {
+    const int lane = threadIdx.x & 31;
+    const int lg = a.h < 2 ? 0 : split_log2(nitems, nwarps, max_split), split = 1 << lg;
+    for (int w = gw; w < nitems << lg; w += nwarps) {
+        const int4 item = a.pitems[2 * (int64_t)(w >> lg)], rows = a.pitems[2 * (int64_t)(w >> lg) + 1];
+        const int u = item.x, x = item.z;
+        // sides past an overflow are redone by the next slot of the round: skip them now
+        if (u < 0 || u > vload(ctr->overflow_unit)) continue;
+        const int sl = item.y + lane;
+        int z = -1, rbz = 0, rez = 0;
+        if (sl < (a.h < 2 ? rows.z : rows.w) && (lane & (split - 1)) == (w & (split - 1))) {
+            if (sl < rows.z) {
+                z = item.w;
+                rbz = rows.z;
+                rez = rows.w;
+            } else {
+                // an old neighbour: alive, or removed in this round
+                const int4 s = a.srec[sl];
+                const int cl = a.col_live[sl];
+                reads += 5;
+                if (s.x != x && (cl >= 0 || cl == -(round + 1))) {
+                    z = s.x;
+                    rbz = s.y;
+                    rez = s.z;
+                }
+            }
+        }
+        // kept if adjacent, or if the stored bit is clear (an earlier batch, or in the twin
+        // matrix another warp, recorded the pair); both words are in x's rows, so their loads go out together
+        int state = kKept, p = rows.x, pe = rows.y, q = z;
+        if (z >= 0) {
+            pairs++;
+            const int64_t at = (int64_t)x * a.Wpad + (z >> 5);
+            bool adjacent, held;
+            if (kTwin) {
+                const uint32_t stored = r2 ? a.pool2_new[at] : a.pool_new[at];
+                adjacent = (a.hub_bits[at] >> (z & 31)) & 1u;
+                held = (stored >> (z & 31)) & 1u;
+                reads += 2;
+            } else {
+                const bool xs = rows.y - rows.x < rez - rbz;  // the longer row's set, if it has one
+                adjacent = alive_adjacent_set(a, hub_set(a, xs ? z : x, reads), xs ? z : x, xs ? x : z, reads);
+                held = r2 ? bit_of(a.pool2, a.Wpad, x, z) : ball_contains(a, x, z, reads);
+            }
+            if (held && !adjacent) {
+                if (rez - rbz < pe - p) {  // p: the shorter row
+                    p = rbz;
+                    pe = rez;
+                    q = x;
+                }
+                state = a.h < 2 ? kLost : pair_quick<kTwin>(a, p, pe, q, reads);
+            }
+        }
+        if (__any_sync(0xffffffffu, state == kHard)) warp_hard_pairs<kTwin>(a, state, p, pe, q, reads);
+        record_lost_warp<r2, kTwin>(a, ctr, round, state == kLost, x, z, rows.x, rows.y, rbz, rez, u);
+    }
+}
+
+template <bool r2>
 __device__ void ph_detect(const LossArgs &a) {
     __shared__ unsigned long long s_pairs, s_reads;
     DevStatus *st = a.st;
@@ -514,40 +610,11 @@ __device__ void ph_detect(const LossArgs &a) {
     __syncthreads();
     const int nitems = min(vload(st->npitems), a.pitems_cap), round = vload(st->round);
     const int lane = threadIdx.x & 31;
-    unsigned long long pairs = 0ull, reads_total = 0ull;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < nitems; it += nwarps) {
-        const int4 item = a.pitems[it];
-        const int u = item.x;
-        // sides past an overflow are redone by the next slot of the round: skip them now
-        if (u < 0 || u > *(volatile int *)&st->overflow_unit) continue;
-        UnitInfo r;
-        r.x = item.z;
-        r.y = item.w;
-        r.rb = a.row_ptr[r.y];
-        r.stop = (a.h < 2) ? r.rb : a.row_ptr[r.y + 1];
-        const int sl = item.y + lane;
-        int z = -1;
-        unsigned reads = 0;
-        if (sl < r.stop) {
-            if (sl < r.rb) {
-                z = r.y;
-            } else {
-                // an old neighbour: alive, or removed in this round
-                const int c = a.col[sl], cl = a.col_live[sl];
-                reads += 2;
-                if (c != r.x && (cl >= 0 || cl == -(round + 1))) z = c;
-            }
-        }
-        int state = kKept, p = r.x, q = z;
-        if (z >= 0) {
-            pairs++;
-            state = pair_quick(a, p, q, reads);
-        }
-        if (__any_sync(0xffffffffu, state == kHard)) warp_hard_pairs(a, state, p, q, reads);
-        record_lost_warp(a, st, state == kLost, r.x, z, u, reads);
-        reads_total += reads;
-    }
+    unsigned lane_pairs = 0u, lane_reads = 0u;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
+    if (a.pool_new) detect_items<r2, true>(a, st, gw, nwarps, nitems, 2, round, lane_pairs, lane_reads);
+    else detect_items<r2, false>(a, st, gw, nwarps, nitems, 2, round, lane_pairs, lane_reads);
+    unsigned long long pairs = lane_pairs, reads_total = lane_reads;
     for (int o = 16; o > 0; o >>= 1) {
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
         reads_total += __shfl_xor_sync(0xffffffffu, reads_total, o);
@@ -564,11 +631,102 @@ __device__ void ph_detect(const LossArgs &a) {
 }
 
 // Support updates, one warp per item (a directed loss v loses w, and <= 32 of v's slots),
-// both orientations in one pass against the stored balls of before this batch: an edge
-// (v,z) with v < z loses w from B(v) ∩ B(z) iff w in B_old(z); with v > z iff w in
-// B_new(z) = B_old(z) minus this batch's losses.  Distance is symmetric, so w in B(z) is
-// tested as z in B(w) (all lanes read one ball, at increasing z) and "w lost by z" as the
-// pair {w,z} in the lost-pair set.
+// both orientations in one pass: an edge (v,z) with v < z loses w from B(v) ∩ B(z) iff w in
+// B_old(z); with v > z iff w in B_new(z) = B_old(z) minus this batch's losses.  Distance is
+// symmetric, so w in B(z) is tested as z in B(w) (all lanes read one ball, at increasing z).
+// kWindow (the cluster round kernel): an edge whose support falls to win_hi joins the window,
+// one whose support falls to thr the next frontier.
+template <bool kWindow>
+__device__ __forceinline__ void lower_support(const LossArgs &a, WindowCtr *wctr, int eid, int win_hi, int thr) {
+    if (!kWindow) {
+        atomicSub(a.sup + eid, 1);
+        return;
+    }
+    // supports fall by one at a time: exactly one update takes the edge across
+    const int old = atomicSub(a.sup + eid, 1);
+    if (old == win_hi + 1) {
+        const int i = atomicAdd(&wctr->nwin, 1);
+        if (i < a.win_cap) a.win[i] = eid;
+    }
+    if (old == thr + 1) {
+        const int i = atomicAdd(&wctr->nnext, 1);
+        if (i < a.win_cap) a.next[i] = eid;
+    }
+}
+
+// What a warp counts over its update items (per lane), in place of running byte sums: the
+// updates are bound by the instructions they issue as much as by their loads.
+struct DeltaStats {
+    unsigned slots = 0u, tests = 0u, hits = 0u, probes = 0u, member_bytes = 0u;
+    // algorithmic bytes of the lane's share: 16 per item, the row slots, the words tested
+    __device__ unsigned bytes(unsigned items, bool twin) const {
+        return 16u * items + 4u * slots + (twin ? 4u * tests : member_bytes) + 8u * hits + 8u * probes;
+    }
+};
+
+// Block `blk` of `nblks` takes a contiguous share of the items (an item and the next often test
+// the same ball row), its warps every (blockDim / 32)-th of it.  A directed loss (v loses w)
+// tests z in B_old(w) or z in B_new(w), by the order of v and z: with the twin matrices that
+// is one bit of either, else a bit and, for B_new, a probe of the lost-pair set.
+template <bool kWindow, bool kTwin>
+__device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wctr, int blk, int nblks, int nitems,
+                                               int win_hi, int thr, DeltaStats &ds, unsigned &items) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const int share = (nitems + nblks - 1) / nblks;
+    const int first = min(nitems, blk * share), last = min(nitems, first + share);
+    // items in flight per warp: their loads are interleaved
+    constexpr int U = 2;
+    for (int it0 = first + wid; it0 < last; it0 += U * wpb) {
+        int4 item[U];  // (first slot, v, w, end of v's row)
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            const int it = it0 + j * wpb;
+            item[j] = (it < last) ? a.uitems[it] : make_int4(0, 0, 0, 0);
+            if (lane == 0) items += it < last;
+        }
+        int z[U], eid[U];
+        bool drop[U];
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            const int sl = item[j].x + lane;
+            const bool ok = sl < item[j].w;
+            z[j] = ok ? a.col_live[sl] : -1;
+            eid[j] = ok ? a.slot_eid[sl] : 0;
+            ds.slots += ok;
+        }
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            drop[j] = false;
+            if (z[j] >= 0) {
+                ds.tests++;
+                if (kTwin)
+                    drop[j] = bit_of(item[j].y < z[j] ? a.pool : a.pool_new, a.Wpad, item[j].z, z[j]);
+                else
+                    drop[j] = ball_contains(a, item[j].z, z[j], ds.member_bytes);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            if (!kTwin && drop[j] && item[j].y > z[j])
+                drop[j] = !in_pair_set(a.keys, a.cap_mask, item[j].z, z[j], ds.probes);
+            if (drop[j]) {
+                lower_support<kWindow>(a, wctr, eid[j], win_hi, thr);
+                ds.hits++;
+            }
+        }
+    }
+}
+
+template <bool kWindow, bool kTwin>
+__device__ __forceinline__ void delta_items(const LossArgs &a, WindowCtr *wctr, int blk, int nblks, int nitems,
+                                            int win_hi, int thr, unsigned &tests, unsigned &bytes) {
+    DeltaStats ds;
+    unsigned items = 0u;
+    delta_items_in<kWindow, kTwin>(a, wctr, blk, nblks, nitems, win_hi, thr, ds, items);
+    tests = ds.tests;
+    bytes = ds.bytes(items, kTwin);
+}
+
 __device__ void ph_delta(const LossArgs &a) {
     __shared__ unsigned long long s_tests, s_bytes;
     DevStatus *st = a.st;
@@ -579,53 +737,12 @@ __device__ void ph_delta(const LossArgs &a) {
     __syncthreads();
     const int nitems = min(vload(st->nuitems), a.uitems_cap);
     const int lane = threadIdx.x & 31;
-    unsigned long long tests = 0ull, bytes_total = 0ull;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    // four items per warp and step, their loads interleaved (one GB300, R-MAT 18 at h = 2:
-    // 4.80 s per decomposition against 4.86 s with two)
-    constexpr int U = 4;
-    for (int it0 = U * ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); it0 < nitems;
-         it0 += U * nwarps) {
-        int4 item[U];  // (first slot, v, w, end of v's row)
-#pragma unroll
-        for (int j = 0; j < U; j++)
-            item[j] = (it0 + j < nitems) ? a.uitems[it0 + j] : make_int4(0, 0, 0, 0);
-        int z[U], eid[U];
-        bool in_w[U];
-#pragma unroll
-        for (int j = 0; j < U; j++) {
-            const int sl = item[j].x + lane;
-            const bool ok = sl < item[j].w;
-            z[j] = ok ? a.col_live[sl] : -1;
-            eid[j] = ok ? a.slot_eid[sl] : 0;
-            if (lane == 0 && it0 + j < nitems) bytes_total += a.dense_all ? 16u : 24u;
-            if (ok) bytes_total += 4;
-        }
-#pragma unroll
-        for (int j = 0; j < U; j++) {
-            in_w[j] = false;
-            if (z[j] >= 0) {
-                tests++;
-                unsigned bytes = 0;
-                if (a.dense_all) {
-                    in_w[j] = (a.pool[(int64_t)item[j].z * a.Wpad + (z[j] >> 5)] >> (z[j] & 31)) & 1u;
-                    bytes += 4;
-                } else {
-                    in_w[j] = ball_contains(a, item[j].z, z[j], bytes);
-                }
-                bytes_total += bytes;
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < U; j++) {
-            unsigned bytes = 0;
-            if (in_w[j] && (item[j].y < z[j] || !lost_now(a, item[j].z, z[j], bytes))) {
-                atomicSub(a.sup + eid[j], 1);
-                bytes += 8;
-            }
-            bytes_total += bytes;
-        }
-    }
+    unsigned lane_tests = 0u, lane_bytes = 0u;
+    if (a.pool_new)
+        delta_items<false, true>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
+    else
+        delta_items<false, false>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
+    unsigned long long tests = lane_tests, bytes_total = lane_bytes;
     for (int o = 16; o > 0; o >>= 1) {
         tests += __shfl_xor_sync(0xffffffffu, tests, o);
         bytes_total += __shfl_xor_sync(0xffffffffu, bytes_total, o);
@@ -641,14 +758,11 @@ __device__ void ph_delta(const LossArgs &a) {
     }
 }
 
-// Clears every lost member from the stored balls and empties the hash slots.  Also counts,
-// once per round and vertex, the alive edges whose support the round brings up to date
-// (every alive edge at an endpoint of a lost pair).
-__device__ void ph_apply(const LossArgs &a) {
-    DevStatus *st = a.st;
-    const int nlost = min(vload(st->nlost), a.lost_max), round = vload(st->round);
-    unsigned long long touched = 0ull;
-    for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < 2 * nlost; d += gridDim.x * blockDim.x) {
+// Clears every lost member from the stored balls (each record's bits are set) and empties
+// the hash slots.
+// Thread t of nt; `real` counts the batch's lost pairs (its non-null records).
+__device__ __forceinline__ void apply_lost(const LossArgs &a, int t, int nt, int nlost, unsigned &real) {
+    for (int d = t; d < 2 * nlost; d += nt) {
         const int4 L = a.lost[d >> 1];
         if (L.x < 0) continue;
         const int v = (d & 1) ? L.y : L.x;
@@ -680,23 +794,23 @@ __device__ void ph_apply(const LossArgs &a) {
             }
         }
         if (word) {
-            const uint32_t old = atomicAnd(word, ~bit);
-            if (old & bit) atomicSub(a.ball_size + v, 1);
+            atomicAnd(word, ~bit);
+            atomicSub(a.ball_size + v, 1);
         }
-        if ((d & 1) == 0) a.keys[L.z] = kEmpty;
-        if (atomicExch(a.vtouch + v, round) != round) touched += (unsigned)a.deg_alive[v];
+        if ((d & 1) == 0) {
+            if (!a.pool_new) a.keys[L.z] = kEmpty;
+            real++;
+        }
     }
-    // lost pairs of this batch (non-null records), one atomic per warp
-    unsigned long long real = 0ull;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nlost; r += gridDim.x * blockDim.x)
-        real += (a.lost[r].x >= 0);
-    for (int o = 16; o > 0; o >>= 1) {
-        real += __shfl_xor_sync(0xffffffffu, real, o);
-        touched += __shfl_xor_sync(0xffffffffu, touched, o);
-    }
-    if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost, real);
-    if ((threadIdx.x & 31) == 0 && touched)
-        atomicAdd((unsigned long long *)&st->st_recomputed, touched);
+}
+
+__device__ void ph_apply(const LossArgs &a) {
+    DevStatus *st = a.st;
+    unsigned real = 0u;
+    apply_lost(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, min(vload(st->nlost), a.lost_max),
+               real);
+    real = __reduce_add_sync(0xffffffffu, real);  // one atomic per warp
+    if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost, (unsigned long long)real);
 }
 
 // ---- h = 3 -------------------------------------------------------------------------------
@@ -711,29 +825,20 @@ __device__ void ph_apply(const LossArgs &a) {
 // their own pair set) has listed first.  Radius-3 losses then take the support deltas of
 // the h = 2 rounds unchanged, on B3.
 
-// Is the pair {p,q} among this round's radius-2 losses?
-__device__ __forceinline__ bool lost2_now(const LossArgs &a, int p, int q, unsigned &bytes) {
-    const unsigned long long key = pair_key(p, q);
-    unsigned long long slot = mix64(key) & a.cap2_mask;
-    for (unsigned long long probe = 0; probe <= a.cap2_mask; probe++) {
-        const unsigned long long k = a.keys2[slot];
-        bytes += 8;
-        if (k == key) return true;
-        if (k == kEmpty) return false;
-        slot = (slot + 1) & a.cap2_mask;
-    }
-    return false;
-}
-
-// q in B2_new(z): the stored radius-2 bit, unless this round lost the pair (the pair set is
-// probed only for vertices that lost a radius-2 member this round).
+// q in B2_new(z): a bit of the twin matrix, or the stored radius-2 bit unless this round lost
+// the pair (the pair set is probed only for vertices that lost a radius-2 member this round).
+template <bool kTwin>
 __device__ __forceinline__ bool in_b2_new(const LossArgs &a, int z, int q, int round, unsigned &bytes) {
     bytes += 4;
-    if (!((a.pool2[(int64_t)z * a.Wpad + (q >> 5)] >> (q & 31)) & 1u)) return false;
+    if (kTwin) return bit_of(a.pool2_new, a.Wpad, z, q);
+    if (!bit_of(a.pool2, a.Wpad, z, q)) return false;
     if (z == q) return true;
     bytes += 4;
     if (a.touch2[z] != round) return true;
-    return !lost2_now(a, z, q, bytes);
+    unsigned probes = 0u;
+    const bool lost = in_pair_set(a.keys2, a.cap2_mask, z, q, probes);
+    bytes += 8 * probes;
+    return !lost;
 }
 
 // Position of the k-th (0-based) set bit of v (k < popc(v)).
@@ -770,17 +875,15 @@ __device__ __forceinline__ int4 c3_range_item(const LossArgs &a, int i, int nch)
     return side ? make_int4(eb, ea, w0, -1 - w1) : make_int4(ea, eb, w0, -1 - w1);
 }
 
-__device__ void ph_c3_items(const LossArgs &a) {
-    DevStatus *st = a.st;
-    const int nF = vload(st->nF), round = vload(st->round);
+__device__ __forceinline__ void c3_items(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps, int nF,
+                                         int round) {
     const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
     const long long nA = 2ll * c3_chunks(a) * nF;
     if (nA > a.c3items_cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->halt, 1);
+        if (gw == 0 && lane == 0) atomicOr(&ctr->halt, 1);
         return;
     }
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nF; i += nwarps) {
+    for (int i = gw; i < nF; i += nwarps) {
         const int e = a.frontier[i];
         const int ea = a.eu[e], eb = a.ev[e];
         const int rba = a.row_ptr[ea], rea = a.row_ptr[ea + 1];
@@ -798,10 +901,10 @@ __device__ void ph_c3_items(const LossArgs &a) {
             const int tot = __shfl_sync(0xffffffffu, incl, 31);
             long long b2 = 0;
             if (lane == 31 && tot)
-                b2 = (long long)atomicAdd((unsigned long long *)&st->nc3items, (unsigned long long)tot);
+                b2 = (long long)atomicAdd((unsigned long long *)&ctr->nc3items, (unsigned long long)tot);
             b2 = __shfl_sync(0xffffffffu, b2, 31);
             if (nA + b2 + tot > a.c3items_cap) {
-                if (lane == 0 && tot) atomicOr(&st->halt, 1);
+                if (lane == 0 && tot) atomicOr(&ctr->halt, 1);
                 continue;
             }
             const int first = (int)b2 + incl - cnt;
@@ -815,6 +918,7 @@ __device__ void ph_c3_items(const LossArgs &a) {
 // endpoint whose alive row is walked, t the other one; the pair is kept at the first alive
 // neighbour y of w with t in B2_new(y).  The rows are laid end to end and walked 128 slots
 // per step as in warp_hard_pairs.  Called by whole warps.
+template <bool kTwin>
 __device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int w, int t, int round,
                                            unsigned &reads) {
     const unsigned full = 0xffffffffu;
@@ -851,7 +955,7 @@ __device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int w,
             const int to = __shfl_sync(full, t, own[j]);
             if (y[j] >= 0) {
                 reads++;
-                if (in_b2_new(a, y[j], to, round, reads)) hits |= 1u << own[j];
+                if (in_b2_new<kTwin>(a, y[j], to, round, reads)) hits |= 1u << own[j];
             }
         }
         hits = __reduce_or_sync(full, hits);
@@ -863,12 +967,13 @@ __device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int w,
 
 // Tests the lanes' radius-3 candidate pairs {p,q} (q < 0: none; q is in B3_old(p)) in the
 // new graph and records the lost ones with their support-update items.  Whole warps.
-__device__ __forceinline__ void test_pairs3(const LossArgs &a, DevStatus *st, int p, int q, int round,
-                                            unsigned &reads, unsigned long long &pairs) {
+template <bool kTwin>
+__device__ __forceinline__ void test_pairs3(const LossArgs &a, RoundCtr *ctr, int p, int q, int round,
+                                            unsigned &reads, unsigned &pairs) {
     int state = kKept, w = p, t = q;
     if (q >= 0) {
         pairs++;
-        if (!in_b2_new(a, p, q, round, reads)) {
+        if (!in_b2_new<kTwin>(a, p, q, round, reads)) {
             state = kHard;
             reads += 2;
             if (a.deg_alive[q] < a.deg_alive[p]) {  // walk the shorter alive row
@@ -877,31 +982,25 @@ __device__ __forceinline__ void test_pairs3(const LossArgs &a, DevStatus *st, in
             }
         }
     }
-    if (__any_sync(0xffffffffu, state == kHard)) warp_walk3(a, state, w, t, round, reads);
-    record_lost_warp(a, st, state == kLost, p, q, 0, reads);
+    if (__any_sync(0xffffffffu, state == kHard)) warp_walk3<kTwin>(a, state, w, t, round, reads);
+    int rbp = 0, rep = 0, rbq = 0, req = 0;
+    if (state == kLost) {
+        rbp = a.row_ptr[p];
+        rep = a.row_ptr[p + 1];
+        rbq = a.row_ptr[q];
+        req = a.row_ptr[q + 1];
+    }
+    record_lost_warp<false, kTwin>(a, ctr, round, state == kLost, p, q, rbp, rep, rbq, req, 0);
 }
 
-// Radius-3 loss tests, one warp per candidate item.
-__device__ void ph_test3(const LossArgs &a) {
-    __shared__ unsigned long long s_pairs, s_reads;
-    DevStatus *st = a.st;
-    if (threadIdx.x == 0) {
-        s_pairs = 0ull;
-        s_reads = 0ull;
-    }
-    __syncthreads();
-    // a round whose items passed the capacity has halted (this kernel is then idle), so
-    // both counts fit the list here
-    const int nch = c3_chunks(a);
-    const long long nA64 = 2ll * nch * vload(st->nF);
-    if (nA64 > a.c3items_cap) return;
-    const int nA = (int)nA64;
-    const int nitems = nA + (int)min(vload(st->nc3items), (long long)a.c3items_cap - nA);
-    const int round = vload(st->round);
+// Radius-3 loss tests, one warp per candidate item: nA range items, then the stored ones.
+template <bool kTwin>
+__device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps, int nA,
+                                            int nitems, int round, unsigned &pairs, unsigned &reads) {
     const int lane = threadIdx.x & 31;
-    unsigned long long pairs = 0ull, reads_total = 0ull;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nch = c3_chunks(a);
+    // pairs another warp has recorded already are not candidates
+    const uint32_t *const b3 = kTwin ? a.pool_new : a.pool;
     // {x} x B2_old(y) restricted to B3_old(x), kC3Groups range items per warp and step: the
     // lanes of group g hold the words of item (step * kC3Groups + g) * nwarps + warp (items
     // of one warp step lie far apart, so their candidate counts average out), and the
@@ -910,13 +1009,12 @@ __device__ void ph_test3(const LossArgs &a) {
         const int it = (s0 * kC3Groups + lane / kC3Words) * nwarps + gw;
         int x = -1, wi = 0;
         uint32_t bits = 0u;
-        unsigned reads = 0;
         if (it < nA) {
             const int4 item = c3_range_item(a, it, nch);
             x = item.x;
             wi = item.z + lane % kC3Words;
             if (wi < -1 - item.w) {
-                bits = a.pool2[(int64_t)item.y * a.Wpad + wi] & a.pool[(int64_t)x * a.Wpad + wi];
+                bits = a.pool2[(int64_t)item.y * a.Wpad + wi] & b3[(int64_t)x * a.Wpad + wi];
                 reads += 2;
                 if (wi == (x >> 5)) bits &= ~(1u << (x & 31));
             }
@@ -937,15 +1035,13 @@ __device__ void ph_test3(const LossArgs &a) {
             const int ow = __shfl_sync(0xffffffffu, wi, o), ox = __shfl_sync(0xffffffffu, x, o);
             int q = -1;
             if (idx < total) q = (ow << 5) + nth_set_bit(ob, idx - ex);
-            test_pairs3(a, st, ox, q, round, reads, pairs);
+            test_pairs3<kTwin>(a, ctr, ox, q, round, reads, pairs);
         }
-        reads_total += reads;
     }
     // {x} x N_old(y) for the 32 slots of a stored item, restricted to B3_old(x): one per warp
     for (int it = nA + gw; it < nitems; it += nwarps) {
         const int4 item = a.c3items[it - nA];
         const int x = item.x;
-        unsigned reads = 0;
         const int sl = item.z + lane;
         int q = -1;
         if (sl < item.w) {
@@ -953,12 +1049,34 @@ __device__ void ph_test3(const LossArgs &a) {
             reads += 2;
             if (c != x && (cl >= 0 || cl == -(round + 1))) {
                 reads++;
-                if ((a.pool[(int64_t)x * a.Wpad + (c >> 5)] >> (c & 31)) & 1u) q = c;
+                if (bit_of(b3, a.Wpad, x, c)) q = c;
             }
         }
-        test_pairs3(a, st, x, q, round, reads, pairs);
-        reads_total += reads;
+        test_pairs3<kTwin>(a, ctr, x, q, round, reads, pairs);
     }
+}
+
+__device__ void ph_test3(const LossArgs &a) {
+    __shared__ unsigned long long s_pairs, s_reads;
+    DevStatus *st = a.st;
+    if (threadIdx.x == 0) {
+        s_pairs = 0ull;
+        s_reads = 0ull;
+    }
+    __syncthreads();
+    // a round whose items passed the capacity has halted (this kernel is then idle), so
+    // both counts fit the list here
+    const long long nA64 = 2ll * c3_chunks(a) * vload(st->nF);
+    if (nA64 > a.c3items_cap) return;
+    const int nA = (int)nA64;
+    const int nitems = nA + (int)min(vload(st->nc3items), (long long)a.c3items_cap - nA);
+    const int lane = threadIdx.x & 31;
+    unsigned lane_pairs = 0u, lane_reads = 0u;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
+    const int round = vload(st->round);
+    if (a.pool_new) test3_items<true>(a, st, gw, nwarps, nA, nitems, round, lane_pairs, lane_reads);
+    else test3_items<false>(a, st, gw, nwarps, nA, nitems, round, lane_pairs, lane_reads);
+    unsigned long long pairs = lane_pairs, reads_total = lane_reads;
     for (int o = 16; o > 0; o >>= 1) {
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
         reads_total += __shfl_xor_sync(0xffffffffu, reads_total, o);
@@ -975,23 +1093,28 @@ __device__ void ph_test3(const LossArgs &a) {
 }
 
 // Clears the round's radius-2 losses from the stored B2 (and their pair-set slots).
-__device__ void ph_apply2(const LossArgs &a) {
-    DevStatus *st = a.st;
-    const int nlost = min(vload(st->nlost2), a.lost2_max);
-    unsigned long long real = 0ull;
-    for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < 2 * nlost; d += gridDim.x * blockDim.x) {
+__device__ __forceinline__ void apply_lost2(const LossArgs &a, int t, int nt, int nlost, unsigned &real) {
+    for (int d = t; d < 2 * nlost; d += nt) {
         const int4 L = a.lost2[d >> 1];
         if (L.x < 0) continue;
         const int v = (d & 1) ? L.y : L.x;
         const int w = (d & 1) ? L.x : L.y;
         const uint32_t bit = 1u << (w & 31);
-        const uint32_t old = atomicAnd(a.pool2 + (int64_t)v * a.Wpad + (w >> 5), ~bit);
-        if (old & bit) atomicSub(a.ball_size2 + v, 1);
+        atomicAnd(a.pool2 + (int64_t)v * a.Wpad + (w >> 5), ~bit);
+        atomicSub(a.ball_size2 + v, 1);
         if ((d & 1) == 0) {
-            a.keys2[L.z] = kEmpty;
+            if (!a.pool_new) a.keys2[L.z] = kEmpty;
             real++;
         }
     }
+}
+
+__device__ void ph_apply2(const LossArgs &a) {
+    DevStatus *st = a.st;
+    unsigned lane_real = 0u;
+    apply_lost2(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x,
+                min(vload(st->nlost2), a.lost2_max), lane_real);
+    unsigned long long real = lane_real;
     for (int o = 16; o > 0; o >>= 1) real += __shfl_xor_sync(0xffffffffu, real, o);
     if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost2, real);
 }
@@ -999,61 +1122,59 @@ __device__ void ph_apply2(const LossArgs &a) {
 // One candidate edge per lane (p: it joins the frontier): warp-aggregated frontier slot,
 // removal (the removal step of Algorithm 1) and the detection items of its two edge sides.  Whole
 // warps call it.
-__device__ __forceinline__ void select_one(const LossArgs &a, DevStatus *st, bool p, int e, int k,
+__device__ __forceinline__ void select_one(const LossArgs &a, RoundCtr *ctr, bool p, int e, int k,
                                            int round) {
     const int lane = threadIdx.x & 31;
     const unsigned bal = __ballot_sync(0xffffffffu, p);
     if (bal == 0u) return;
+    int4 ends = make_int4(0, 0, 0, 0), rows = make_int4(0, 0, 0, 0);
+    if (p) {
+        ends = a.erec[2 * (int64_t)e];
+        rows = a.erec[2 * (int64_t)e + 1];
+    }
     int base = 0;
-    if (lane == 0) base = atomicAdd(&st->nF, __popc(bal));
+    if (lane == 0) base = atomicAdd(&ctr->nF, __popc(bal));
     base = __shfl_sync(0xffffffffu, base, 0);
     const int pos = base + __popc(bal & lanemask_lt());
-    int u_eu = 0, u_ev = 0, rb_u = 0, re_u = 0, rb_v = 0, re_v = 0, n0 = 0, n1 = 0;
+    int n0 = 0, n1 = 0;
     if (p) {
         a.frontier_w[pos] = e;
-        remove_edge(e, k, round, a.eu, a.ev, a.slot_lo, a.slot_hi, a.sup, a.truss,
-                    a.stamp_w, a.col_live_w, a.deg_alive_w, a.hub_slot, a.hub_bits_w, a.Wpad);
-        u_eu = a.eu[e];
-        u_ev = a.ev[e];
-        rb_u = a.row_ptr[u_eu];
-        re_u = a.row_ptr[u_eu + 1];
-        rb_v = a.row_ptr[u_ev];
-        re_v = a.row_ptr[u_ev + 1];
+        remove_edge(e, k, round, ends.x, ends.y, ends.z, ends.w, a.sup, a.truss, a.stamp_w, a.col_live_w,
+                    a.deg_alive_w, a.hub_all, a.hub_slot, a.hub_bits_w, a.Wpad);
         // side 0: eu with {ev} and N_old(ev); side 1: ev with N_old(eu); h = 1: {eu,ev}
-        n0 = (a.h < 2) ? 1 : (re_v - rb_v + 1 + 31) >> 5;
-        n1 = (a.h < 2) ? 0 : (re_u - rb_u + 31) >> 5;
+        n0 = (a.h < 2) ? 1 : (rows.w - rows.z + 1 + 31) >> 5;
+        n1 = (a.h < 2) ? 0 : (rows.y - rows.x + 31) >> 5;
     }
-    int incl = n0 + n1;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+    const int incl = warp_incl_scan(n0 + n1);
     int ibase = 0;
-    if (lane == 31 && tot) ibase = atomicAdd(&st->npitems, tot);
+    if (lane == 31) ibase = atomicAdd(&ctr->npitems, incl);
     ibase = __shfl_sync(0xffffffffu, ibase, 31);
     const int first = ibase + incl - (n0 + n1);
-    if (p && first + n0 > a.pitems_cap) overflow_at(a, st, 2 * pos);
-    if (p && n1 && first + n0 + n1 > a.pitems_cap) overflow_at(a, st, 2 * pos + 1);
-    unsigned todo = __ballot_sync(0xffffffffu, p);
+    const bool fits0 = first + n0 <= a.pitems_cap, fits1 = first + n0 + n1 <= a.pitems_cap;
+    if (p && !fits0) overflow_at(a, ctr, 2 * pos);
+    if (p && n1 && !fits1) overflow_at(a, ctr, 2 * pos + 1);
+    // few items are written by their own lane, a hub row's by the whole warp
+    constexpr int kOwnItems = 4;
+    auto write = [&](int c, int n0w, int f, int posw, int4 ew, int4 rw, bool f0, bool f1) {
+        if (c < n0w)
+            write_pitem(a, f + c, f0 ? 2 * posw : -1, rw.z - 1 + 32 * c, ew.x, ew.y, rw);
+        else
+            write_pitem(a, f + c, f1 ? 2 * posw + 1 : -1, rw.x + 32 * (c - n0w), ew.y, ew.x,
+                        make_int4(rw.z, rw.w, rw.x, rw.y));
+    };
+    if (p && n0 + n1 <= kOwnItems)
+        for (int c = 0; c < n0 + n1 && first + c < a.pitems_cap; c++) write(c, n0, first, pos, ends, rows, fits0, fits1);
+    unsigned todo = __ballot_sync(0xffffffffu, p && n0 + n1 > kOwnItems);
     while (todo) {
         const int l = __ffs(todo) - 1;
         todo &= todo - 1;
-        const int f = __shfl_sync(0xffffffffu, first, l);
+        const int f = __shfl_sync(0xffffffffu, first, l), pl = __shfl_sync(0xffffffffu, pos, l);
         const int c0 = __shfl_sync(0xffffffffu, n0, l), c1 = __shfl_sync(0xffffffffu, n1, l);
-        const int pl = __shfl_sync(0xffffffffu, pos, l);
-        const int xu = __shfl_sync(0xffffffffu, u_eu, l), xv = __shfl_sync(0xffffffffu, u_ev, l);
-        const int su = __shfl_sync(0xffffffffu, rb_u, l), sv0 = __shfl_sync(0xffffffffu, rb_v, l);
-        const bool fits0 = f + c0 <= a.pitems_cap, fits1 = f + c0 + c1 <= a.pitems_cap;
-        for (int c = lane; c < c0 + c1 && f + c < a.pitems_cap; c += 32) {
-            if (c < c0)
-                a.pitems[f + c] = fits0 ? make_int4(2 * pl, sv0 - 1 + 32 * c, xu, xv)
-                                        : make_int4(-1, 0, 0, 0);
-            else
-                a.pitems[f + c] = fits1 ? make_int4(2 * pl + 1, su + 32 * (c - c0), xv, xu)
-                                        : make_int4(-1, 0, 0, 0);
-        }
+        const int4 el = make_int4(__shfl_sync(0xffffffffu, ends.x, l), __shfl_sync(0xffffffffu, ends.y, l), 0, 0);
+        const int4 rl = make_int4(__shfl_sync(0xffffffffu, rows.x, l), __shfl_sync(0xffffffffu, rows.y, l),
+                                  __shfl_sync(0xffffffffu, rows.z, l), __shfl_sync(0xffffffffu, rows.w, l));
+        const bool l0 = __shfl_sync(0xffffffffu, fits0, l), l1 = __shfl_sync(0xffffffffu, fits1, l);
+        for (int c = lane; c < c0 + c1 && f + c < a.pitems_cap; c += 32) write(c, c0, f, pl, el, rl, l0, l1);
     }
 }
 
@@ -1092,55 +1213,75 @@ __device__ __forceinline__ void phase_entry() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// One launch per phase (the rounds of a CUDA graph).
-__global__ void __launch_bounds__(kBlock) k_inc_select(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_select_items(a);
-}
-__global__ void __launch_bounds__(kBlock) k_loss_detect(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_detect(a);
-}
-// h = 3: the radius-2 detection (a.rec_r2) and the round's radius-3 candidate items
-__global__ void __launch_bounds__(kBlock) k_loss_detect3(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_detect(a);
-    ph_c3_items(a);
-}
-__global__ void __launch_bounds__(kBlock) k_loss3_test(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_test3(a);
-}
-__global__ void __launch_bounds__(kBlock) k_loss_delta(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_delta(a);
-}
-__global__ void __launch_bounds__(kBlock) k_loss_apply_reduce(LossArgs a) {
-    phase_entry();
-    if (round_idle(a)) return;
-    ph_apply(a);
-    if (a.h3) ph_apply2(a);
-    minreduce_body<kBlock / 32>(a.sup, a.m, a.st, 0);
-}
-
-constexpr int kPBlock = 512;  // threads per block of the persistent kernel
-
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
 
+// Phases of a round whose time the status block adds up (st_phase_ns).
+enum TimedPhase { kTimeSelect = 0, kTimeDetect, kTimeTest3, kTimeDelta, kTimeReduce };
+
+// With a.timer: a phase launch starts, which ends the time of phase `done` (-1: the slot
+// begins).  One thread of the launch calls it; launches of a slot follow one another.
+__device__ __forceinline__ void phase_clock(const LossArgs &a, int done) {
+    if (!a.timer || blockIdx.x != 0 || threadIdx.x != 0) return;
+    const unsigned long long t = global_ns();
+    if (done >= 0) a.st->st_phase_ns[done] += t - a.st->st_phase_start;
+    a.st->st_phase_start = t;
+}
+
+// One launch per phase (the rounds of a CUDA graph).
+__global__ void __launch_bounds__(kBlock) k_inc_select(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageSelect)) return;
+    phase_clock(a, -1);
+    ph_select_items(a);
+}
+__global__ void __launch_bounds__(kBlock) k_loss_detect(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageDetect)) return;
+    phase_clock(a, kTimeSelect);
+    ph_detect<false>(a);
+}
+// h = 3: the radius-2 detection and the round's radius-3 candidate items
+__global__ void __launch_bounds__(kBlock) k_loss_detect3(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageDetect)) return;
+    phase_clock(a, kTimeSelect);
+    ph_detect<true>(a);
+    c3_items(a, a.st, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, gridDim.x * (blockDim.x >> 5),
+             vload(a.st->nF), vload(a.st->round));
+}
+__global__ void __launch_bounds__(kBlock) k_loss3_test(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageTest3)) return;
+    phase_clock(a, kTimeDetect);
+    ph_test3(a);
+}
+__global__ void __launch_bounds__(kBlock) k_loss_delta(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageDelta)) return;
+    phase_clock(a, a.h3 ? kTimeTest3 : kTimeDetect);
+    ph_delta(a);
+}
+__global__ void __launch_bounds__(kBlock) k_loss_apply_reduce(LossArgs a) {
+    phase_entry();
+    if (round_idle(a, kStageDelta)) return;
+    phase_clock(a, kTimeDelta);
+    ph_apply(a);
+    if (a.h3) ph_apply2(a);
+    if (minreduce_body<kBlock / 32>(a.sup, a.m, a.st, 0) && a.timer)
+        a.st->st_phase_ns[kTimeReduce] += global_ns() - a.st->st_phase_start;
+}
+
+constexpr int kPBlock = 512;  // threads per block of the persistent kernel
+
 // Persistent round kernel (cooperative launch, every block resident): runs up to
 // `max_slots` round slots, each the four phases of an incremental round separated by grid
 // barriers, and stops early once no edge is alive or an error is flagged.  Block 0 adds
 // the time of each phase to the status block.
-__global__ void __launch_bounds__(kPBlock, 3) k_rounds_persistent(LossArgs a, int max_slots) {
+__global__ void __launch_bounds__(kPBlock, 2) k_rounds_persistent(LossArgs a, int max_slots) {
     DevStatus *st = a.st;
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long t_prev = timer ? global_ns() : 0ull;
@@ -1156,16 +1297,524 @@ __global__ void __launch_bounds__(kPBlock, 3) k_rounds_persistent(LossArgs a, in
     for (int slot = 0; slot < max_slots; slot++) {
         if (vload(st->alive) == 0 || vload(st->err) != 0) break;
         ph_select_items(a);
-        if (!phase_done(0)) return;
-        ph_detect(a);
-        if (!phase_done(1)) return;
+        if (!phase_done(kTimeSelect)) return;
+        ph_detect<false>(a);
+        if (!phase_done(kTimeDetect)) return;
         ph_delta(a);
-        if (!phase_done(2)) return;
+        if (!phase_done(kTimeDelta)) return;
         // clearing the lost members touches balls and hash slots only; the reduction reads
         // supports only, and its last block closes the round after every block did both
         ph_apply(a);
         minreduce_body<kPBlock / 32>(a.sup, a.m, st, 0);
-        if (!phase_done(3)) return;
+        if (!phase_done(kTimeReduce)) return;
+    }
+}
+
+// ---- small rounds in one thread-block cluster --------------------------------------------
+//
+// Most rounds are small (R-MAT 16 at h = 2: 8 frontier edges and 12K update items in the
+// median), and a round of separate launches then costs its launches, two scans of every
+// support and a dozen dependent loads behind each launch.  This kernel runs such rounds in
+// ONE cluster of up to 16 blocks: the phases are split by hardware cluster barriers, the
+// round's counters sit in the shared memory of the cluster's first block, and the frontier
+// comes from a window instead of a scan.  It needs the twin ball matrices.
+//
+// Frontier: the edges the last round's updates took to the level (exactly one update sees
+// each crossing, since supports fall one at a time), else from the window.
+// Window: the list of edges whose support was at most win_hi when the list was built from a
+// full scan, plus every edge whose support has fallen to win_hi since.  While an alive edge is in it, the
+// smallest alive support is its smallest; when none is left it is rebuilt.
+//
+// A phase with more work than one cluster does quickly is shared with helpers: further
+// clusters of the same launch, which wait for jobs in global memory (bounded waits).  A
+// launch beside others on the device (batched and served decompositions) has no helpers.
+// A round that is too large even so is left, at the phase where it shows, to the phase
+// launches that follow in the slot (RoundStage); their state is the same.
+constexpr int kCBlock = 1024;        // threads per block
+constexpr int kCMaxBlocks = 16;      // blocks per cluster (the non-portable size)
+constexpr int kWinPerThread = 2;     // window edges each thread holds
+constexpr int kCRounds = 1024;       // rounds per launch
+// Work of a phase: the leader cluster runs up to kHelp... units alone and shares more with the
+// helpers; more than kMost... (kAlone... where the launch has no helpers) is left to the phase
+// launches.
+constexpr int kHelpDetect = 1024, kAloneDetect = 4096, kMostDetect = 1 << 16;     // detection items
+constexpr int kHelpTest3 = 1 << 12, kAloneTest3 = 1 << 17, kMostTest3 = 1 << 20;  // radius-3 items
+constexpr int kHelpDelta = 16384, kAloneDelta = 65536, kMostDelta = 1 << 21;       // update items
+constexpr unsigned long long kHelperWaitNs = 20000000000ull;  // a helper gives up waiting for a job
+constexpr unsigned long long kLeadWaitNs = 4000000000ull;     // the leader, for its helpers
+
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ unsigned cluster_blocks() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
+// The address of `p` (this block's shared memory) in the block of rank `rank`.
+template <typename T>
+__device__ __forceinline__ T *cluster_map(T *p, unsigned rank) {
+    unsigned long long r;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(reinterpret_cast<unsigned long long>(p)), "r"(rank));
+    return reinterpret_cast<T *>(r);
+}
+
+enum ClusterStat { kStatPairs = 0, kStatReads, kStatTests, kStatBytes, kStatLost, kStatTouched, kStatC3,
+                   kStatLost2, kNumStats };
+
+// Adds the warp's sum of v to the block's counter.
+__device__ __forceinline__ void stat_add(unsigned long long *s_stat, int which, unsigned v) {
+    const unsigned s = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && s) atomicAdd(s_stat + which, (unsigned long long)s);
+}
+
+__device__ __forceinline__ unsigned long long load_acquire(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void store_release(unsigned long long *p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// The phases helpers can share, as one call by block `blk` of `nblks`.  Consecutive detection
+// and candidate items go to different blocks.
+template <bool kH3>
+__device__ __forceinline__ void shared_phase(const LossArgs &a, RoundCtr *ctr, WindowCtr *wctr,
+                                             unsigned long long *s_stat, int phase, int blk, int nblks,
+                                             int max_split, const HelperJob &job) {
+    const int gw = (threadIdx.x >> 5) * nblks + blk, nwarps = nblks * (kCBlock / 32);
+    if (phase == kStageDetect) {
+        unsigned pairs = 0u, reads = 0u;
+        detect_items<kH3, true>(a, ctr, gw, nwarps, job.nitems, max_split, job.round, pairs, reads);
+        if (kH3) c3_items(a, ctr, gw, nwarps, job.nF, job.round);
+        stat_add(s_stat, kStatPairs, pairs);
+        stat_add(s_stat, kStatReads, reads);
+    } else if (kH3 && phase == kStageTest3) {
+        unsigned pairs = 0u, reads = 0u;
+        test3_items<true>(a, ctr, gw, nwarps, 2 * c3_chunks(a) * job.nF, job.nitems, job.round, pairs, reads);
+        stat_add(s_stat, kStatC3, pairs);
+        stat_add(s_stat, kStatReads, reads);
+    } else {
+        unsigned tests = 0u, bytes = 0u;
+        delta_items<true, true>(a, wctr, blk, nblks, job.nitems, job.win_hi, job.thr, tests, bytes);
+        stat_add(s_stat, kStatTests, tests);
+        stat_add(s_stat, kStatBytes, bytes);
+    }
+}
+
+__device__ __forceinline__ void flush_stats(DevStatus *st, unsigned long long *s_stat) {
+    const int tid = threadIdx.x;
+    if (tid < kNumStats && s_stat[tid]) {
+        unsigned long long *const out[kNumStats] = {
+            (unsigned long long *)&st->st_pairs, &st->st_bytes_detect, (unsigned long long *)&st->st_tests,
+            &st->st_bytes_update, (unsigned long long *)&st->st_lost, (unsigned long long *)&st->st_recomputed,
+            (unsigned long long *)&st->st_c3_pairs, (unsigned long long *)&st->st_lost2};
+        atomicAdd(out[tid], tid == kStatReads ? 4ull * s_stat[tid] : s_stat[tid]);
+    }
+}
+
+// A helper block: registers, then takes its share of every job whose helper count covers its
+// number, until the leader of launch `epoch` has finished.  A job word is (launch, job
+// number, helper blocks); a block that is not needed reads nothing else of the job.
+template <bool kH3>
+__device__ __forceinline__ void helper_blocks(const LossArgs &a, unsigned long long epoch, int nblk,
+                                           unsigned long long *s_stat) {
+    __shared__ unsigned long long s_word;
+    DevStatus *st = a.st;
+    unsigned long long seen = (epoch << 40);
+    int id = 0;
+    if (threadIdx.x == 0) {
+        atomicMax(&st->cl_reg, epoch << 32);
+        id = (int)(atomicAdd(&st->cl_reg, 1ull) & 0xffffffffull);
+    }
+    for (;;) {
+        if (threadIdx.x == 0) {
+            unsigned long long word = 0ull;  // 0: stop
+            const unsigned long long t0 = global_ns();
+            for (;;) {
+                const unsigned long long w = load_acquire(&st->cl_job);
+                if ((w >> 16) > (seen >> 16) && (w >> 40) == epoch) {
+                    seen = w;
+                    if (id < (int)(w & 0xffffull)) {
+                        word = w;
+                        break;
+                    }
+                }
+                if (load_acquire(&st->cl_exit) > epoch) break;
+                if (global_ns() - t0 > kHelperWaitNs) {
+                    atomicOr(&st->err, kErrBarrierTimeout);
+                    break;
+                }
+                __nanosleep(64);
+            }
+            __threadfence();
+            s_word = word ? (word & 0xffffull) | ((unsigned long long)id << 32) : 0ull;
+        }
+        __syncthreads();
+        const unsigned long long w = s_word;
+        if (w == 0ull) break;
+        const int blocks = nblk + (int)(w & 0xffffffffull), me = nblk + (int)(w >> 32);
+        HelperJob job;
+        job.phase = vload(st->cl_work.phase);
+        job.nitems = vload(st->cl_work.nitems);
+        job.nF = vload(st->cl_work.nF);
+        job.round = vload(st->cl_work.round);
+        job.win_hi = vload(st->cl_work.win_hi);
+        job.thr = vload(st->cl_work.thr);
+        shared_phase<kH3>(a, &st->cl_ctr, &st->cl_wctr, s_stat, job.phase, me, blocks, 2, job);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&st->cl_done, 1ull);
+        }
+    }
+    __syncthreads();
+    flush_stats(st, s_stat);
+}
+
+template <bool kH3>
+__global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_constant__ LossArgs a) {
+    __shared__ unsigned long long s_ticket;
+    __shared__ int s_helpers;
+    __shared__ RoundCtr s_ctr[2];
+    __shared__ WindowCtr s_wctr;
+    __shared__ int s_min[3];
+    __shared__ unsigned long long s_stat[kNumStats];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    DevStatus *st = a.st;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const unsigned rank = cluster_rank(), nblk = cluster_blocks();
+    const bool lead = rank == 0 && tid == 0;
+    const int nwarps = (int)nblk * (kCBlock / 32);
+    const int gw = wid * (int)nblk + (int)rank;  // consecutive items go to different blocks
+    const int nthreads = (int)nblk * kCBlock, gt = (int)rank * kCBlock + tid;
+    const int win_cap = a.win_cap;
+    // The first cluster of a launch to start leads; the others help.  Helpers that start late
+    // (or never, while the device is busy) are not waited for.
+    unsigned long long epoch = 0ull;
+    const int nclusters = (int)(gridDim.x / nblk);
+    if (nclusters > 1) {
+        if (lead) s_ticket = atomicAdd(&st->cl_tickets, 1ull);
+        cluster_sync();
+        const unsigned long long ticket = *(volatile unsigned long long *)cluster_map(&s_ticket, 0);
+        cluster_sync();
+        epoch = ticket / (unsigned)nclusters;
+        if (ticket % (unsigned)nclusters != 0ull) {
+            if (tid < kNumStats) s_stat[tid] = 0ull;
+            __syncthreads();
+            helper_blocks<kH3>(a, epoch, (int)nblk, s_stat);
+            return;
+        }
+    }
+    if (vload(st->alive) == 0 || vload(st->halt) != 0 || vload(st->err) != 0 || vload(st->cont)) {
+        cluster_sync();
+        if (lead) {
+            if (vload(st->cont)) st->stage = kStageSelect;  // a round of several batches: the launches'
+            store_release(&st->cl_exit, epoch + 1);
+        }
+        return;
+    }
+    unsigned long long job_seq = 0ull, done_base = 0ull;
+    if (lead) done_base = load_acquire(&st->cl_done);
+    // the counters of the round and of the one before it take turns
+    RoundCtr *const ctrs = cluster_map(&s_ctr[0], 0);
+    WindowCtr *const wctr = cluster_map(&s_wctr, 0);
+    auto reset_ctr = [&](RoundCtr *c) {
+        *c = RoundCtr{};
+        c->overflow_unit = INT_MAX;
+    };
+    if (tid == 0) {
+        reset_ctr(&s_ctr[0]);
+        reset_ctr(&s_ctr[1]);
+        s_wctr = WindowCtr{};
+        for (int j = 0; j < 3; j++) s_min[j] = INT_MAX;
+        for (int j = 0; j < kNumStats; j++) s_stat[j] = 0ull;
+    }
+    int k = vload(st->k), round = vload(st->round), levels = vload(st->levels);
+    int last_k = vload(st->last_k), max_k = vload(st->max_k);
+    long long alive = vload(st->alive);
+    const int first_round = round;
+    long long removed = 0;
+    int win_hi = 0, width = 8, buf = 0, stage = kStageNone;
+    bool applied = true, rebuild = true;
+    unsigned long long t_prev = a.timer && lead ? global_ns() : 0ull;
+    auto clock = [&](int phase) {
+        if (!a.timer || !lead) return;
+        const unsigned long long t = global_ns();
+        st->st_phase_ns[phase] += t - t_prev;
+        t_prev = t;
+    };
+    // smallest value the blocks put into s_min[buf] before the last barrier; the buffer used
+    // two reductions ago is reset (a barrier lies between its readers and this point, and
+    // another one before its next use)
+    auto cluster_min = [&]() -> int {
+        int v = lane < (int)nblk ? *(volatile int *)cluster_map(&s_min[buf], lane) : INT_MAX;
+        v = __reduce_min_sync(0xffffffffu, v);
+        if (tid == 0) s_min[(buf + 2) % 3] = INT_MAX;
+        buf = (buf + 1) % 3;
+        return v;
+    };
+    // One phase over `work` units, by the leader cluster alone or with the helpers that have
+    // started.  Counters of a shared phase are in global memory (a helper cannot reach the
+    // leader's shared memory): copied there before and back after.  Ends with a barrier; false
+    // if the helpers did not finish in time (an error is set: the peel ends).
+    auto run_phase = [&](int phase, RoundCtr *ctr, HelperJob job, long long work, int help) -> bool {
+        int helpers = 0;
+        if (nclusters > 1 && work > help) {
+            if (lead) {
+                const unsigned long long reg = load_acquire(&st->cl_reg);
+                s_helpers = (reg >> 32) == epoch ? (int)(reg & 0xffffull) : 0;
+                if (s_helpers > 0) {
+                    job.phase = phase;
+                    st->cl_work = job;
+                    st->cl_ctr = *ctr;
+                    st->cl_wctr = *wctr;
+                    job_seq++;
+                    store_release(&st->cl_job, (epoch << 40) | (job_seq << 16) | (unsigned)s_helpers);
+                }
+            }
+            cluster_sync();
+            helpers = *(volatile int *)cluster_map(&s_helpers, 0);
+        }
+        if (helpers == 0) {
+            shared_phase<kH3>(a, ctr, wctr, s_stat, phase, (int)rank, (int)nblk, 5, job);
+            cluster_sync();
+            return true;
+        }
+        const int blocks = (int)nblk + helpers;
+        shared_phase<kH3>(a, &st->cl_ctr, &st->cl_wctr, s_stat, phase, (int)rank, blocks, 2, job);
+        cluster_sync();
+        if (lead) {
+            done_base += (unsigned)helpers;
+            const unsigned long long t0 = global_ns();
+            while (load_acquire(&st->cl_done) < done_base) {
+                if (global_ns() - t0 > kLeadWaitNs) {
+                    atomicOr(&st->err, kErrBarrierTimeout);
+                    s_helpers = -1;
+                    break;
+                }
+            }
+            __threadfence();
+            RoundCtr c;
+            const int *from = reinterpret_cast<const int *>(&st->cl_ctr);
+            int *to = reinterpret_cast<int *>(&c);
+            for (int j = 0; j < (int)(sizeof(RoundCtr) / sizeof(int)); j++) to[j] = vload(from[j]);
+            *ctr = c;
+            wctr->nwin = vload(st->cl_wctr.nwin);
+            wctr->nnext = vload(st->cl_wctr.nnext);
+        }
+        cluster_sync();
+        return *(volatile int *)cluster_map(&s_helpers, 0) >= 0;
+    };
+    cluster_sync();
+    for (;;) {
+        RoundCtr *const ctr = ctrs + (round & 1), *const prev = ctrs + ((round & 1) ^ 1);
+        // the frontier: the edges the last updates took to the level, if any; else it comes
+        // from the window
+        const int nnext = rebuild || round - first_round >= kCRounds ? 0 : vload(wctr->nnext);
+        const bool direct = nnext > 0 && nnext <= win_cap;
+        int we[kWinPerThread];
+        bool take[kWinPerThread];
+        const int32_t *const list = direct ? a.next : a.win;
+        int nlist = direct ? nnext : min(vload(wctr->nwin), win_cap);
+        auto load_list = [&]() {
+#pragma unroll
+            for (int j = 0; j < kWinPerThread; j++) {
+                const int i = (lane + 32 * j) * nwarps + gw;
+                we[j] = i < nlist ? list[i] : -1;
+                take[j] = direct && we[j] >= 0;
+            }
+        };
+        load_list();
+        // the previous round's lost members leave the balls
+        if (!applied) {
+            unsigned real = 0u;
+            apply_lost(a, gt, nthreads, min(vload(prev->nlost), a.lost_max), real);
+            stat_add(s_stat, kStatLost, real);
+            if (kH3) {
+                real = 0u;
+                apply_lost2(a, gt, nthreads, min(vload(prev->nlost2), a.lost2_max), real);
+                stat_add(s_stat, kStatLost2, real);
+            }
+            applied = true;
+        }
+        if (!direct) {
+            int mn = INT_MAX;
+            const bool rebuilt = rebuild;
+            while (rebuild) {
+                cluster_sync();  // the old window is no longer read
+                if (lead) wctr->nwin = 0;
+                cluster_sync();
+                win_hi = k - 2 + width;
+                int lmin = INT_MAX;
+                const int64_t stride = 4 * (int64_t)nthreads;
+                for (int64_t e0 = 4 * ((int64_t)gt & ~31ll); e0 < a.m; e0 += stride) {
+                    int sv[4];
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int64_t e = e0 + 32 * j + lane;
+                        sv[j] = (e < a.m) ? a.sup[e] : INT_MAX;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        lmin = min(lmin, sv[j]);
+                        const unsigned bal = __ballot_sync(0xffffffffu, sv[j] <= win_hi);
+                        if (bal) {
+                            int base = 0;
+                            if (lane == 0) base = atomicAdd(&wctr->nwin, __popc(bal));
+                            base = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & lanemask_lt());
+                            if (sv[j] <= win_hi && base < win_cap) a.win[base] = (int)(e0 + 32 * j + lane);
+                        }
+                    }
+                }
+                lmin = __reduce_min_sync(0xffffffffu, lmin);
+                if (lane == 0 && lmin != INT_MAX) atomicMin(&s_min[buf], lmin);
+                cluster_sync();
+                mn = cluster_min();
+                nlist = vload(wctr->nwin);
+                if (mn == INT_MAX) {
+                    alive = 0;
+                    break;
+                }
+                k = max(k, mn + 2);
+                if (nlist > win_cap) {
+                    if (width == 0) {  // a frontier larger than the window
+                        stage = kStageSelect;
+                        break;
+                    }
+                    width >>= 2;
+                } else if (nlist > 0) {
+                    rebuild = false;
+                    if (nlist < win_cap / 16) width = min(2 * width + 1, 1 << 20);
+                }
+            }
+            if (rebuild) break;  // nothing alive, or left to the launches
+            if (rebuilt) load_list();
+            // the window's supports and their minimum
+            int ws[kWinPerThread];
+            int lmin = INT_MAX;
+#pragma unroll
+            for (int j = 0; j < kWinPerThread; j++) {
+                ws[j] = we[j] >= 0 ? a.sup[we[j]] : INT_MAX;
+                lmin = min(lmin, ws[j]);
+            }
+            lmin = __reduce_min_sync(0xffffffffu, lmin);
+            if (lane == 0 && lmin != INT_MAX) atomicMin(&s_min[buf], lmin);
+            const bool spilled = vload(wctr->nwin) > win_cap;
+            cluster_sync();
+            mn = cluster_min();
+            if (spilled) {  // crossings did not fit the list
+                width >>= 2;
+                rebuild = true;
+                continue;
+            }
+            if (mn == INT_MAX) {
+                if (alive == 0) break;
+                rebuild = true;
+                continue;
+            }
+            if (round - first_round >= kCRounds) break;
+            k = max(k, mn + 2);
+#pragma unroll
+            for (int j = 0; j < kWinPerThread; j++) take[j] = ws[j] <= k - 2;
+        }
+        // selection and removal, and the detection items of the frontier's edge sides
+#pragma unroll
+        for (int j = 0; j < kWinPerThread; j++) select_one(a, ctr, take[j], we[j], k, round);
+        cluster_sync();
+        clock(kTimeSelect);
+        // Every block takes the decisions of this loop alike: between two barriers they read
+        // only counters that nothing changes before the next one (overflow marks, which the
+        // phase now starting may set, are read where no phase sets them).
+        const int nF = vload(ctr->nF), npitems = vload(ctr->npitems);
+        if (lead) wctr->nnext = 0;  // read by all before the barrier, used again after the next
+        const int most_detect = nclusters > 1 ? kMostDetect : kAloneDetect;
+        const int most_test3 = nclusters > 1 ? kMostTest3 : kAloneTest3;
+        const int most_delta = nclusters > 1 ? kMostDelta : kAloneDelta;
+        const long long nA = kH3 ? 2ll * c3_chunks(a) * nF : 0ll;
+        if (npitems > min(most_detect, a.pitems_cap) || nA > most_test3) {
+            stage = kStageDetect;
+            break;
+        }
+        HelperJob job;
+        job.phase = 0;
+        job.nitems = npitems;
+        job.nF = nF;
+        job.round = round;
+        job.win_hi = win_hi;
+        job.thr = k - 2;
+        if (!run_phase(kStageDetect, ctr, job, npitems, kHelpDetect)) break;
+        clock(kTimeDetect);
+        if (kH3) {
+            // too many items, or no room for the items or the radius-2 losses (a halt)
+            const long long nc3 = vload(ctr->nc3items);
+            if (nA + nc3 > min(most_test3, a.c3items_cap) || vload(ctr->nlost2) > a.lost2_max) {
+                stage = kStageTest3;
+                break;
+            }
+            job.nitems = (int)(nA + nc3);
+            if (!run_phase(kStageTest3, ctr, job, nA + nc3, kHelpTest3)) break;
+            clock(kTimeTest3);
+        }
+        if (lead) {  // the round before is done with
+            s_stat[kStatTouched] += prev->touched;
+            reset_ctr(prev);
+        }
+        const int nuitems = vload(ctr->nuitems);
+        if (nuitems > most_delta || vload(ctr->overflow_unit) != INT_MAX || (kH3 && vload(ctr->halt) != 0)) {
+            stage = kStageDelta;
+            break;
+        }
+        job.nitems = nuitems;
+        if (!run_phase(kStageDelta, ctr, job, nuitems, kHelpDelta)) break;
+        clock(kTimeDelta);
+        // the round's bookkeeping (round_finalize's, kept by every thread alike)
+        if (k != last_k) {
+            levels++;
+            last_k = k;
+        }
+        max_k = max(max_k, k);
+        round++;
+        removed += nF;
+        alive -= nF;
+        applied = false;
+    }
+    cluster_sync();
+    if (lead) {
+        // a round left unfinished keeps its counters (`touched` among them: its closing
+        // launch adds them), the last finished one only adds its touched edges
+        RoundCtr *const ctr = ctrs + (round & 1), *const prev = ctrs + ((round & 1) ^ 1);
+        s_stat[kStatTouched] += prev->touched;
+        if (stage <= kStageSelect) reset_ctr(ctr);
+        *static_cast<RoundCtr *>(st) = *ctr;
+    }
+    __syncthreads();
+    flush_stats(st, s_stat);
+    if (lead) {
+        st->k = k;
+        st->round = round;
+        st->levels = levels;
+        st->last_k = last_k;
+        st->max_k = max_k;
+        st->alive = alive;
+        st->st_frontier += removed;
+        st->st_slots += round - first_round;
+        st->stage = stage;
+        st->unit_begin = 0;
+        if (a.timer) st->st_phase_start = global_ns();
+        store_release(&st->cl_exit, epoch + 1);
     }
 }
 
@@ -1175,7 +1824,7 @@ LossArgs loss_args(Handle *H) {
     LossArgs a;
     a.h = w.h;
     a.lost_max = (int32_t)w.lost_max;
-    a.cap_mask = (unsigned long long)(w.lost_cap - 1);
+    a.cap_mask = (unsigned)(w.lost_cap - 1);
     a.row_ptr = g.row_ptr;
     a.col = g.col;
     a.col_live = w.col_live;
@@ -1215,16 +1864,24 @@ LossArgs loss_args(Handle *H) {
     a.hub_bits_w = w.hub_bits;
     a.st = w.status;
     a.h3 = w.inc3 ? 1 : 0;
-    a.rec_r2 = 0;
     a.pool2 = w.pool2;
     a.ball_size2 = w.ball_size2;
     a.keys2 = w.lost2_keys;
-    a.cap2_mask = w.lost2_cap > 0 ? (unsigned long long)(w.lost2_cap - 1) : 0ull;
+    a.cap2_mask = w.lost2_cap > 0 ? (unsigned)(w.lost2_cap - 1) : 0u;
     a.lost2 = w.lost2;
     a.lost2_max = (int32_t)w.lost2_max;
     a.c3items_cap = (int32_t)w.c3items_cap;
     a.c3items = w.c3items;
     a.touch2 = w.touch2;
+    a.pool_new = w.twin ? w.pool_new : nullptr;
+    a.pool2_new = w.twin ? w.pool2_new : nullptr;
+    a.cluster = 0;
+    a.timer = 0;
+    a.win_cap = 0;
+    a.win = w.win;
+    a.next = w.win + w.win_cap;
+    a.erec = w.erec;
+    a.srec = w.srec;
     return a;
 }
 
@@ -1263,7 +1920,53 @@ namespace {
 struct PhaseGrids {
     int device = -1;
     int detect = 0, detect3 = 0, delta = 0, test3 = 0;
+    int cluster = 0;   // blocks of a cluster of the cluster round kernel (0: none fits the device)
+    int clusters = 0;  // clusters of a launch that has the device to itself
 };
+
+using PhaseKernel = void (*)(LossArgs);
+
+// Launch configuration of the cluster round kernel: `clusters` clusters of `blocks` blocks.
+struct ClusterLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    ClusterLaunch(int clusters, int blocks, cudaStream_t s, bool pdl) {
+        cfg.gridDim = dim3((unsigned)(clusters * blocks));
+        cfg.blockDim = dim3(kCBlock);
+        cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)blocks;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = pdl ? 2 : 1;
+    }
+};
+
+// The largest cluster both forms of the kernel can run as on this device: 16 blocks (which
+// needs the non-portable size), else 8, else none.
+// *resident: clusters of that size the whole device holds at once.
+int cluster_size(int *resident) {
+    for (int blocks = kCMaxBlocks; blocks >= 8; blocks /= 2) {
+        bool fits = true;
+        *resident = INT_MAX;
+        for (PhaseKernel kern : {PhaseKernel(k_rounds_cluster<false>), PhaseKernel(k_rounds_cluster<true>)}) {
+            if (blocks > 8)
+                fits = fits && cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                                    1) == cudaSuccess;
+            ClusterLaunch c(1, blocks, nullptr, false);
+            int n = 0;
+            fits = fits && cudaOccupancyMaxActiveClusters(&n, (const void *)kern, &c.cfg) == cudaSuccess && n > 0;
+            *resident = std::min(*resident, n);
+        }
+        if (fits) return blocks;
+        (void)cudaGetLastError();
+    }
+    *resident = 0;
+    return 0;
+}
 
 htd_status phase_grids(Handle *H, PhaseGrids &pg) {
     if (pg.device == H->g.device) return HTD_OK;
@@ -1280,6 +1983,10 @@ htd_status phase_grids(Handle *H, PhaseGrids &pg) {
     pg.detect3 = H->num_sms * od3;
     pg.delta = H->num_sms * ou;
     pg.test3 = H->num_sms * ot;
+    int resident = 0;
+    pg.cluster = cluster_size(&resident);
+    // one cluster's room stays free, so that another stream's leader can start beside it
+    pg.clusters = std::max(1, resident - 1);
     pg.device = H->g.device;
     return HTD_OK;
 }
@@ -1303,52 +2010,40 @@ cudaError_t launch_phase(void (*kernel)(LossArgs), int grid, cudaStream_t s, boo
 
 }  // namespace
 
-// Enqueues one incremental round as four launches (the graph path).  evs (nullable):
-// kRoundEvents events; phases are marked as select | - | detect | update | - | reduce.
-// Without events the launches are programmatic (each overlaps the previous one's tail).
-htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs,
-                                     unsigned record_flags) {
+// Enqueues one slot of incremental rounds (the graph path): the cluster round kernel, then
+// the launches of one round, which run from the phase that kernel left to them.  Every
+// launch is programmatic (it overlaps the previous one's tail).
+htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer) {
     LossArgs a = loss_args(H);
     static thread_local PhaseGrids pg;
     const htd_status gs = phase_grids(H, pg);
     if (gs != HTD_OK) return gs;
-    const bool pdl = evs == nullptr;
-    auto mark = [&](int i) {
-        if (evs) cudaEventRecordWithFlags(evs[i], s, record_flags);
-    };
+    const bool pdl = true;
+    a.cluster = (pg.cluster > 0 && H->w.twin) ? 1 : 0;
+    a.win_cap = (int32_t)std::min<int64_t>(H->w.win_cap, (int64_t)pg.cluster * kCBlock * kWinPerThread);
+    a.timer = timer ? 1 : 0;
     // the two scans over all edges use fewer blocks: the reduction's per-block atomics all
     // hit the same few counters
     const int grid_scan = H->num_sms * 2;
     cudaError_t e = cudaSuccess;
+    if (a.cluster) {
+        ClusterLaunch c(H->shared_device ? 1 : pg.clusters, pg.cluster, s, pdl);
+        e = cudaLaunchKernelEx(&c.cfg, a.h3 ? k_rounds_cluster<true> : k_rounds_cluster<false>, a);
+        *launches += 1;
+    }
     if (a.h3) {
         // select | radius-2 detection + radius-3 items | radius-3 tests | updates | - | reduce
-        LossArgs a2 = a;
-        a2.rec_r2 = 1;
-        mark(0);
         if (e == cudaSuccess) e = launch_phase(k_inc_select, grid_scan, s, pdl, a);
-        mark(1);
-        if (e == cudaSuccess) e = launch_phase(k_loss_detect3, pg.detect3, s, pdl, a2);
-        mark(2);
+        if (e == cudaSuccess) e = launch_phase(k_loss_detect3, pg.detect3, s, pdl, a);
         if (e == cudaSuccess) e = launch_phase(k_loss3_test, pg.test3, s, pdl, a);
-        mark(3);
         if (e == cudaSuccess) e = launch_phase(k_loss_delta, pg.delta, s, pdl, a);
-        mark(4);
-        mark(5);
         if (e == cudaSuccess) e = launch_phase(k_loss_apply_reduce, grid_scan, s, pdl, a);
-        mark(6);
         *launches += 5;
     } else {
-        mark(0);
         if (e == cudaSuccess) e = launch_phase(k_inc_select, grid_scan, s, pdl, a);
-        mark(1);
-        mark(2);
         if (e == cudaSuccess) e = launch_phase(k_loss_detect, pg.detect, s, pdl, a);
-        mark(3);
         if (e == cudaSuccess) e = launch_phase(k_loss_delta, pg.delta, s, pdl, a);
-        mark(4);
-        mark(5);
         if (e == cudaSuccess) e = launch_phase(k_loss_apply_reduce, grid_scan, s, pdl, a);
-        mark(6);
         *launches += 4;
     }
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -46,6 +46,7 @@ struct BallArgs {
     const int32_t *col_live;
     const int32_t *deg_alive;
     uint32_t *pool;
+    uint32_t *pool_new;   // nullable: a second copy of every dense ball stored
     const int64_t *ball_off;
     int32_t *ball_need;
     int32_t *ball_size;
@@ -235,6 +236,10 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
             } else if (dense) {
                 uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
                 for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) dst[i] = bits4[i];
+                if (a.pool_new) {
+                    uint4 *twin = reinterpret_cast<uint4 *>(a.pool_new + off);
+                    for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) twin[i] = bits4[i];
+                }
             } else {
                 uint2 *dst = reinterpret_cast<uint2 *>(a.pool + off);
                 int run = wbase;
@@ -495,8 +500,27 @@ __global__ void k_remove(const int32_t *__restrict__ frontier, DevStatus *st,
     if (st->alive == 0 || st->cont) return;  // a continued round removed its frontier already
     const int nF = st->nF, k = st->k, round = st->round;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nF; i += gridDim.x * blockDim.x)
-        remove_edge(frontier[i], k, round, eu, ev, slot_lo, slot_hi, sup, truss, stamp, col_live,
-                    deg_alive, hub_slot, hub_bits, Wpad);
+    {
+        const int e = frontier[i];
+        remove_edge(e, k, round, eu[e], ev[e], slot_lo[e], slot_hi[e], sup, truss, stamp, col_live,
+                    deg_alive, false, hub_slot, hub_bits, Wpad);
+    }
+}
+
+// The records the incremental rounds read instead of chasing pointers: per edge (u, v, its
+// two slots) and both rows' bounds, per adjacency slot (neighbour, its row's bounds, edge).
+__global__ void k_make_records(int64_t m, const int32_t *__restrict__ row_ptr,
+                               const int32_t *__restrict__ eu, const int32_t *__restrict__ ev,
+                               const int32_t *__restrict__ slot_lo, const int32_t *__restrict__ slot_hi,
+                               int4 *__restrict__ erec, int4 *__restrict__ srec) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+        const int u = eu[e], v = ev[e], lo = slot_lo[e], hi = slot_hi[e];
+        const int rbu = row_ptr[u], reu = row_ptr[u + 1], rbv = row_ptr[v], rev = row_ptr[v + 1];
+        erec[2 * e] = make_int4(u, v, lo, hi);
+        erec[2 * e + 1] = make_int4(rbu, reu, rbv, rev);
+        srec[lo] = make_int4(v, rbv, rev, (int)e);
+        srec[hi] = make_int4(u, rbu, reu, (int)e);
+    }
 }
 
 // Alive-adjacency n-bit sets of the high-degree vertices (all edges alive), block per hub.
@@ -558,6 +582,7 @@ BallArgs ball_args(Handle *H) {
     a.col_live = w.col_live;
     a.deg_alive = w.deg_alive;
     a.pool = w.pool;
+    a.pool_new = w.twin ? w.pool_new : nullptr;
     a.ball_off = w.ball_off;
     a.ball_need = w.ball_need;
     a.ball_size = w.ball_size;
@@ -624,8 +649,13 @@ void free_work(PeelWork *w) {
     cudaFree(w->hub_bits);
     cudaFree(w->pitems);
     cudaFree(w->uitems);
+    cudaFree(w->win);
+    cudaFree(w->erec);
+    cudaFree(w->srec);
     cudaFree(w->scan_tmp);
     cudaFree(w->pool2);
+    cudaFree(w->pool_new);
+    cudaFree(w->pool2_new);
     cudaFree(w->ball_size2);
     cudaFree(w->ball_nw2);
     cudaFree(w->ball_meta2);
@@ -745,8 +775,12 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
         // adjacency slots the updates of one batch may visit
         w.upd_budget = std::min<int64_t>((int64_t)1 << 30, std::max<int64_t>(1 << 16, 256 * m));
         w.uitems_cap = 2 * w.lost_max + w.upd_budget / 32 + 1024;
-        HTD_CHECK(alloc_n(&w.pitems, w.pitems_cap));
+        HTD_CHECK(alloc_n(&w.pitems, 2 * w.pitems_cap));
         HTD_CHECK(alloc_n(&w.uitems, w.uitems_cap));
+        w.win_cap = std::min<int64_t>(m, (int64_t)1 << 15);
+        HTD_CHECK(alloc_n(&w.win, 2 * w.win_cap));
+        HTD_CHECK(alloc_n(&w.erec, 2 * m));
+        HTD_CHECK(alloc_n(&w.srec, 2 * m));
         if (h == 3) {
             // radius-2 balls (dense) with their own metadata, the round's radius-2 losses and
             // the radius-3 candidate items
@@ -810,6 +844,30 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
 
 }  // namespace
 
+// Takes the twin ball matrices into use if they are there or can be had: every ball dense,
+// an alive-adjacency set at every vertex, and the copies no larger than `budget` bytes.
+// Without them the rounds keep the batch's losses in hash sets (same results).
+htd_status ensure_twin(Handle *H, int64_t budget) {
+    PeelWork &w = H->w;
+    const int64_t n = H->g.n, words = n * (int64_t)w.Wpad;
+    w.twin = false;
+    if (!w.incremental || !w.dense_balls || n == 0 || w.nhub != n || w.hub_min_deg != 1) return HTD_OK;
+    const int copies = w.inc3 ? 2 : 1;
+    if (!w.pool_new && copies * words * 4 > budget) return HTD_OK;
+    if (!w.pool_new) {
+        cudaError_t e = alloc_n(&w.pool_new, words);
+        if (e == cudaSuccess && copies == 2) e = alloc_n(&w.pool2_new, words);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            cudaFree(w.pool_new);
+            w.pool_new = nullptr;
+            return HTD_OK;
+        }
+    }
+    w.twin = true;
+    return HTD_OK;
+}
+
 // Initial pass: every vertex's ball (count, reserve, store) and every edge's h-support,
 // then the first min reduction.  Leaves the status ready for round 0.
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
@@ -831,11 +889,17 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
     HTD_CHECK(cudaMemsetAsync(w.stamp, 0xff, (m > 0 ? m : 1) * sizeof(int32_t), s));
     if (w.incremental) {
         HTD_CHECK(cudaMemsetAsync(w.edge_touch, 0xff, (n > 0 ? n : 1) * sizeof(int32_t), s));
-        HTD_CHECK(cudaMemsetAsync(w.lost_keys, 0xff, w.lost_cap * sizeof(unsigned long long), s));
+        if (!w.twin) HTD_CHECK(cudaMemsetAsync(w.lost_keys, 0xff, w.lost_cap * sizeof(unsigned long long), s));
         if (w.inc3) {
-            HTD_CHECK(cudaMemsetAsync(w.lost2_keys, 0xff, w.lost2_cap * sizeof(unsigned long long), s));
+            if (!w.twin)
+                HTD_CHECK(cudaMemsetAsync(w.lost2_keys, 0xff, w.lost2_cap * sizeof(unsigned long long), s));
             HTD_CHECK(cudaMemsetAsync(w.changed_stamp2, 0xff, (n > 0 ? n : 1) * sizeof(int32_t), s));
             HTD_CHECK(cudaMemsetAsync(w.touch2, 0xff, (n > 0 ? n : 1) * sizeof(int32_t), s));
+        }
+        if (m > 0) {
+            k_make_records<<<std::min<int64_t>((m + kBlock - 1) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
+                m, g.row_ptr, g.eu, g.ev, g.slot_lo, g.slot_hi, w.erec, w.srec);
+            (*launches)++;
         }
         if (w.nhub > 0) {
             k_hub_init<<<std::min(w.nhub, H->num_sms * 8), kBlock, 0, s>>>(w.hub_list, w.nhub, g.row_ptr,
@@ -922,12 +986,13 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
 
 // Enqueues one peel round.  evs (nullable) = kRoundEvents events at the phase boundaries:
 //   rebuild:     | select | candidates | remove | ball rebuild | items + h-support | reduce |
-//   incremental: | select | remove | loss detection | support updates | (empty) | reduce |
-htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs) {
+//   (incremental rounds add their phase times to the status block instead, with `timer`)
+htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer) {
     PeelWork &w = H->w;
     GraphDev &g = H->g;
     const int64_t m = g.m;
     const int gsmall = H->num_sms * 4;
+    if (w.incremental) return enqueue_incremental_round(H, s, launches, timer);
     // inside a stream capture an ordinary record only orders nodes; an external record
     // node really records the event each time the graph runs, so it can be timed
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -936,7 +1001,6 @@ htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent
     auto mark = [&](int i) {
         if (evs) cudaEventRecordWithFlags(evs[i], s, rec_flags);
     };
-    if (w.incremental) return enqueue_incremental_round(H, s, launches, evs, rec_flags);
     mark(0);
     k_select<<<w.grid_edges, kBlock, 0, s>>>(w.sup, m, w.status, w.frontier);
     mark(1);
@@ -977,6 +1041,7 @@ htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches) {
     b2.count_bytes = 0;
     b2.force_dense = 1;
     b2.pool = w.pool2;
+    b2.pool_new = w.twin ? w.pool2_new : nullptr;
     b2.ball_size = w.ball_size2;
     b2.ball_nw = w.ball_nw2;
     b2.ball_meta = w.ball_meta2;
@@ -1002,6 +1067,7 @@ __global__ void k_recover_reset(DevStatus *st) {
     st->nuitems = 0;
     st->nc3items = 0;
     st->upd_work = 0;
+    st->touched = 0;
     st->overflow_unit = INT_MAX;
     for (int j = 0; j < kMaxH; j++) st->cand_cnt[j] = 0;
     st->q_ball = 0;
@@ -1028,8 +1094,10 @@ htd_status recover_round_h3(Handle *H, cudaStream_t s, int64_t *launches) {
     PeelWork &w = H->w;
     GraphDev &g = H->g;
     const int gsmall = H->num_sms * 4;
-    HTD_CHECK(cudaMemsetAsync(w.lost_keys, 0xff, w.lost_cap * sizeof(unsigned long long), s));
-    HTD_CHECK(cudaMemsetAsync(w.lost2_keys, 0xff, w.lost2_cap * sizeof(unsigned long long), s));
+    if (!w.twin) {
+        HTD_CHECK(cudaMemsetAsync(w.lost_keys, 0xff, w.lost_cap * sizeof(unsigned long long), s));
+        HTD_CHECK(cudaMemsetAsync(w.lost2_keys, 0xff, w.lost2_cap * sizeof(unsigned long long), s));
+    }
     k_recover_reset<<<1, 1, 0, s>>>(w.status);
     k_cand_init<<<gsmall, kBlock, 0, s>>>(w.frontier, g.eu, g.ev, w.status, w.cand_stamp, w.cand_list);
     *launches += 2;
@@ -1044,6 +1112,7 @@ htd_status recover_round_h3(Handle *H, cudaStream_t s, int64_t *launches) {
     b2.count_bytes = 0;
     b2.force_dense = 1;
     b2.pool = w.pool2;
+    b2.pool_new = w.twin ? w.pool2_new : nullptr;
     b2.ball_size = w.ball_size2;
     b2.ball_nw = w.ball_nw2;
     b2.ball_meta = w.ball_meta2;

@@ -16,21 +16,21 @@ constexpr unsigned kBarrierSpinLimit = 1u << 24;
 // stamp, a support no selection matches, both adjacency slots marked dead with the round
 // (-(round + 1), so a slot tells by itself whether it died in the current round), alive
 // degrees and (when present) the endpoints' alive-adjacency sets updated.
-__device__ __forceinline__ void remove_edge(int e, int k, int round, const int32_t *eu,
-                                            const int32_t *ev, const int32_t *slot_lo,
-                                            const int32_t *slot_hi, int32_t *sup, int32_t *truss,
+// hub_all: every vertex has its set, at row x (hub_slot is not looked up).
+__device__ __forceinline__ void remove_edge(int e, int k, int round, int u, int v, int slot_lo,
+                                            int slot_hi, int32_t *sup, int32_t *truss,
                                             int32_t *stamp, int32_t *col_live, int32_t *deg_alive,
-                                            const int32_t *hub_slot, uint32_t *hub_bits, int Wpad) {
-    const int u = eu[e], v = ev[e];
+                                            bool hub_all, const int32_t *hub_slot, uint32_t *hub_bits,
+                                            int Wpad) {
     truss[e] = k;
     stamp[e] = round;
     sup[e] = INT_MAX;
-    col_live[slot_lo[e]] = -(round + 1);
-    col_live[slot_hi[e]] = -(round + 1);
+    col_live[slot_lo] = -(round + 1);
+    col_live[slot_hi] = -(round + 1);
     atomicSub(&deg_alive[u], 1);
     atomicSub(&deg_alive[v], 1);
     if (hub_slot) {
-        const int hu = hub_slot[u], hv = hub_slot[v];
+        const int hu = hub_all ? u : hub_slot[u], hv = hub_all ? v : hub_slot[v];
         if (hu >= 0) atomicAnd(hub_bits + (int64_t)hu * Wpad + (v >> 5), ~(1u << (v & 31)));
         if (hv >= 0) atomicAnd(hub_bits + (int64_t)hv * Wpad + (u >> 5), ~(1u << (u & 31)));
     }
@@ -69,6 +69,7 @@ __device__ __forceinline__ void round_finalize(DevStatus *st, int initial) {
     st->alive_acc = 0;
     st->done_blocks = 0u;
     if (!unfinished) st->nF = 0;
+    st->stage = kStageNone;
     for (int j = 0; j < kMaxH; j++) st->cand_cnt[j] = 0;
     st->nchanged = 0;
     st->nlost = 0;
@@ -77,6 +78,8 @@ __device__ __forceinline__ void round_finalize(DevStatus *st, int initial) {
     st->npitems = 0;
     st->nuitems = 0;
     st->upd_work = 0;
+    st->st_recomputed += st->touched;
+    st->touched = 0;
     st->nitems = 0;
     st->q_ball = 0;
     st->q_items = 0;
@@ -84,9 +87,10 @@ __device__ __forceinline__ void round_finalize(DevStatus *st, int initial) {
 }
 
 // Minimum alive support and alive count over all edges; the last block to finish closes the
-// round.  Every thread of every block calls it; `NW` = warps per block.
+// round.  Every thread of every block calls it; `NW` = warps per block.  Returns true in the
+// thread that closed the round.
 template <int NW>
-__device__ __forceinline__ void minreduce_body(const int32_t *__restrict__ sup, int64_t m,
+__device__ __forceinline__ bool minreduce_body(const int32_t *__restrict__ sup, int64_t m,
                                                DevStatus *st, int initial) {
     __shared__ int32_t s_min[NW];
     __shared__ long long s_cnt[NW];
@@ -132,8 +136,10 @@ __device__ __forceinline__ void minreduce_body(const int32_t *__restrict__ sup, 
         s_last = (ticket == gridDim.x - 1);
     }
     __syncthreads();
-    if (s_last && threadIdx.x == 0) round_finalize(st, initial);
+    const bool closes = s_last && threadIdx.x == 0;
+    if (closes) round_finalize(st, initial);
     __syncthreads();
+    return closes;
 }
 
 // Barrier across all blocks of a cooperative launch (all co-resident, at most 64 x 32

@@ -167,6 +167,7 @@ htd_status run_request(htd_server *S, Request &r, cudaStream_t s, WorkerBufs &b)
     int32_t n = 0;
     int64_t m = 0;
     htd_graph_info(g, &n, &m);
+    if (S->nworkers > 1) htd::set_shared_device(g);
     st = htd_truss_decompose_ex(g, r.h, S->flags, b.truss, nullptr, &r.stats, s);
     if (st == HTD_OK) st = htd_edges(g, b.eu, b.ev, s);
     if (st != HTD_OK) r.error = htd_last_error();
@@ -251,6 +252,10 @@ int64_t htd_footprint_estimate(int32_t n, int64_t m_in, int32_t h, int64_t free_
     const double fb = free_bytes > 0 ? (double)free_bytes : 0.0;
     if (h <= 3 && dense <= fb / 4.0) {
         bytes += dense * (h == 3 ? 2.0 : 1.0) + std::min(dense, std::min(fb / 4.0, 16.0 * (1 << 30)));
+        // twin matrices, which a request takes only while they are small
+        if (dense * (h == 3 ? 2.0 : 1.0) <= fb / 64.0) bytes += dense * (h == 3 ? 2.0 : 1.0);
+        // edge and slot records, detection items
+        bytes += 64.0 * M + 32.0 * std::min(std::max(2.0 * M, 4096.0), (double)(1 << 22));
         // lost-pair tables and support-update items
         bytes += (h == 3 ? 256.0 : 64.0) * (1 << 20) + 16.0 * std::min(256.0 * M, (double)(1 << 30)) / 32.0;
     } else {
