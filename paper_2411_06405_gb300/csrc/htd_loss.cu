@@ -219,61 +219,86 @@ __device__ __forceinline__ T warp_incl_scan(T v) {
     return v;
 }
 
-// Slots of the concatenated rows each lane loads per step of a warp's common walk (their
-// loads are independent, so a step costs two round trips whatever the count).
-constexpr int kWalkUnroll = 4;
+// Rows up to this long are walked by eight lanes, four rows side by side, longer ones by the
+// whole warp.
+constexpr int kShortRow = 64;
 
-// Common alive neighbours for the warp's hard pairs (lanes with state == kHard; p's row
-// [rb, re), the shorter one), all at once: the pairs' rows of p are laid end to end and the warp walks
-// the concatenation 32 x kWalkUnroll slots per step, each lane finding the pair its slot belongs to by a
-// binary search over the lanes' running row lengths.  A pair is kept at its first alive
-// neighbour that q also has; the walk skips kept pairs and stops once none is pending.
-// Called by whole warps.
+// Walks the rows [rb, re) of the warp's hard pairs (lanes with state == kHard; q the other
+// endpoint): a pair is kept at its first alive neighbour y with test(q, y).  Short rows: four
+// at a time, eight lanes each, 16 slots per row and step; long rows: one at a time, 128
+// slots per step.  Laying the rows end to end, as warp_walk3 does, keeps more lanes busy but
+// issues about 150 instructions per 128 slots against 25 per 64 here, and the walks of the
+// h = 2 rounds are bound by what they issue (R-MAT 16, h = 2: 601 ms against 640 ms).  Whole
+// warps call it.
+template <typename Test>
+__device__ __forceinline__ void warp_walk(const LossArgs &a, int &state, int rb, int re, int q, unsigned &reads,
+                                          Test test) {
+    __shared__ uint8_t s_lane[32][32];  // per warp: the lanes of its short rows
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool hard = state == kHard;
+    unsigned kept = 0u;
+    unsigned todo = __ballot_sync(full, hard && re - rb > kShortRow);
+    while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int b = __shfl_sync(full, rb, l), e = __shfl_sync(full, re, l), ql = __shfl_sync(full, q, l);
+        for (int s = b + lane; s - lane < e; s += 128) {
+            int y[4];
+            bool hit = false;
+#pragma unroll
+            for (int j = 0; j < 4; j++) y[j] = s + 32 * j < e ? a.col_live[s + 32 * j] : -1;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                if (y[j] >= 0) {
+                    reads++;
+                    hit |= test(ql, y[j]);
+                }
+            }
+            if (__any_sync(full, hit)) {
+                kept |= 1u << l;
+                break;
+            }
+        }
+    }
+    const bool mine = hard && re - rb <= kShortRow;
+    const unsigned shorts = __ballot_sync(full, mine);
+    const int count = __popc(shorts);
+    if (count) {
+        if (mine) s_lane[wid][__popc(shorts & lanemask_lt())] = (uint8_t)lane;
+        __syncwarp();
+        for (int r0 = 0; r0 < count; r0 += 4) {
+            const int r = r0 + (lane >> 3);
+            const int src = r < count ? s_lane[wid][r] : 0;
+            const int b = __shfl_sync(full, rb, src), e = __shfl_sync(full, re, src), ql = __shfl_sync(full, q, src);
+            int s = b + (lane & 7);
+            bool done = r >= count;
+            while (__any_sync(full, !done && s - (lane & 7) < e)) {
+                const int y0 = !done && s < e ? a.col_live[s] : -1;
+                const int y1 = !done && s + 8 < e ? a.col_live[s + 8] : -1;
+                bool hit = false;
+                if (y0 >= 0) hit = test(ql, y0);
+                if (y1 >= 0) hit |= test(ql, y1);
+                reads += (y0 >= 0) + (y1 >= 0);
+                const unsigned hits = __ballot_sync(full, hit);
+                done = done || ((hits >> (lane & 24)) & 0xffu) != 0u;
+                s += 16;
+            }
+            kept |= __reduce_or_sync(full, done && r < count ? 1u << src : 0u);
+        }
+        __syncwarp();
+    }
+    if (hard) state = ((kept >> lane) & 1u) ? kKept : kLost;
+}
+
+// Hard pairs at h = 2: a common alive neighbour ([rb, re): the endpoint with the shorter row).
 template <bool kTwin>
 __device__ __forceinline__ void warp_hard_pairs(const LossArgs &a, int &state, int rb, int re, int q,
                                                 unsigned &reads) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const bool hard = state == kHard;
-    const int len = hard ? re - rb : 0;
-    const uint32_t *qset = !hard ? nullptr : kTwin ? a.hub_bits + (int64_t)q * a.Wpad : hub_set(a, q, reads);
-    const int incl = warp_incl_scan(len);
-    const int excl = incl - len;
-    const int total = __shfl_sync(full, incl, 31);
-    unsigned pending = __ballot_sync(full, hard);
-    unsigned kept = 0u;
-    for (int base = 0; base < total && pending; base += 32 * kWalkUnroll) {
-        int y[kWalkUnroll], own[kWalkUnroll];
-#pragma unroll
-        for (int j = 0; j < kWalkUnroll; j++) {
-            const int idx = base + 32 * j + lane;
-            // owner lane: the number of lanes whose rows end at or before idx
-            int o = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (__shfl_sync(full, incl, o + step - 1) <= idx) o += step;
-            o = min(o, 31);
-            const int ex = __shfl_sync(full, excl, o), rbo = __shfl_sync(full, rb, o);
-            own[j] = o;
-            y[j] = (idx < total && ((pending >> o) & 1u)) ? a.col_live[rbo + idx - ex] : -1;
-        }
-        unsigned hits = 0u;
-#pragma unroll
-        for (int j = 0; j < kWalkUnroll; j++) {
-            const int qo = __shfl_sync(full, q, own[j]);
-            const uint32_t *qs = reinterpret_cast<const uint32_t *>(
-                __shfl_sync(full, reinterpret_cast<unsigned long long>(qset), own[j]));
-            if (y[j] >= 0) {
-                reads++;
-                if (kTwin ? (qs[y[j] >> 5] >> (y[j] & 31)) & 1u : alive_adjacent_set(a, qs, qo, y[j], reads))
-                    hits |= 1u << own[j];
-            }
-        }
-        hits = __reduce_or_sync(full, hits);
-        kept |= hits;
-        pending &= ~hits;
-    }
-    if (hard) state = ((kept >> lane) & 1u) ? kKept : kLost;
+    warp_walk(a, state, rb, re, q, reads, [&](int qo, int y) -> bool {
+        if (kTwin) return bit_of(a.hub_bits, a.Wpad, qo, y);
+        return alive_adjacent_set(a, hub_set(a, qo, reads), qo, y, reads);
+    });
 }
 
 // Is w in the stored ball of z (dense words, or sorted (word index, word) pairs)?
@@ -914,22 +939,20 @@ __device__ __forceinline__ void c3_items(const LossArgs &a, RoundCtr *ctr, int g
     }
 }
 
-// Common walk of the warp's hard radius-3 pairs (lanes with state == kHard): w is the
-// endpoint whose alive row is walked, t the other one; the pair is kept at the first alive
-// neighbour y of w with t in B2_new(y).  The rows are laid end to end and walked 128 slots
-// per step as in warp_hard_pairs.  Called by whole warps.
+// Common walk of the warp's hard radius-3 pairs (lanes with state == kHard): [rb, re) is the
+// row of one endpoint, t the other one; the pair is kept at the first alive neighbour y in
+// the row with t in B2_new(y).  The rows are laid end to end and walked 128 slots per step,
+// each lane finding the pair its slot belongs to by a binary search over the lanes' running
+// row lengths; the walk skips kept pairs.  (Eight lanes per row, as in warp_walk, makes the
+// many long rows wait for one another: R-MAT 4096 at h = 3 23 ms against 16 ms.)  Called by
+// whole warps.
 template <bool kTwin>
-__device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int w, int t, int round,
+__device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int rb, int re, int t, int round,
                                            unsigned &reads) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool hard = state == kHard;
-    int rb = 0, len = 0;
-    if (hard) {
-        rb = a.row_ptr[w];
-        len = a.row_ptr[w + 1] - rb;
-        reads += 2;
-    }
+    const int len = hard ? re - rb : 0;
     const int incl = warp_incl_scan(len);
     const int excl = incl - len;
     const int total = __shfl_sync(full, incl, 31);
@@ -965,31 +988,27 @@ __device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int w,
     if (hard) state = ((kept >> lane) & 1u) ? kKept : kLost;
 }
 
-// Tests the lanes' radius-3 candidate pairs {p,q} (q < 0: none; q is in B3_old(p)) in the
-// new graph and records the lost ones with their support-update items.  Whole warps.
+// Decides the lanes' radius-3 candidate pairs {p,q} (q < 0: none; q is in B3_old(p) and not in
+// B2_new(p)) in the new graph and records the lost ones with their support-update items.
+// Whole warps.
 template <bool kTwin>
-__device__ __forceinline__ void test_pairs3(const LossArgs &a, RoundCtr *ctr, int p, int q, int round,
-                                            unsigned &reads, unsigned &pairs) {
-    int state = kKept, w = p, t = q;
+__device__ __forceinline__ void decide_pairs3(const LossArgs &a, RoundCtr *ctr, int p, int q, int round,
+                                              unsigned &reads) {
+    int state = kKept, rb = 0, re = 0, t = q, rbp = 0, rep = 0, rbq = 0, req = 0;
     if (q >= 0) {
-        pairs++;
-        if (!in_b2_new<kTwin>(a, p, q, round, reads)) {
-            state = kHard;
-            reads += 2;
-            if (a.deg_alive[q] < a.deg_alive[p]) {  // walk the shorter alive row
-                w = q;
-                t = p;
-            }
-        }
-    }
-    if (__any_sync(0xffffffffu, state == kHard)) warp_walk3<kTwin>(a, state, w, t, round, reads);
-    int rbp = 0, rep = 0, rbq = 0, req = 0;
-    if (state == kLost) {
+        state = kHard;
         rbp = a.row_ptr[p];
         rep = a.row_ptr[p + 1];
         rbq = a.row_ptr[q];
         req = a.row_ptr[q + 1];
+        reads += 6;
+        const bool walk_q = a.deg_alive[q] < a.deg_alive[p];  // the shorter alive row
+        rb = walk_q ? rbq : rbp;
+        re = walk_q ? req : rep;
+        t = walk_q ? p : q;
     }
+    if (!__any_sync(0xffffffffu, q >= 0)) return;
+    warp_walk3<kTwin>(a, state, rb, re, t, round, reads);
     record_lost_warp<false, kTwin>(a, ctr, round, state == kLost, p, q, rbp, rep, rbq, req, 0);
 }
 
@@ -1014,9 +1033,13 @@ __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, in
             x = item.x;
             wi = item.z + lane % kC3Words;
             if (wi < -1 - item.w) {
-                bits = a.pool2[(int64_t)item.y * a.Wpad + wi] & b3[(int64_t)x * a.Wpad + wi];
+                const int64_t ax = (int64_t)x * a.Wpad + wi;
+                bits = a.pool2[(int64_t)item.y * a.Wpad + wi] & b3[ax];
                 reads += 2;
                 if (wi == (x >> 5)) bits &= ~(1u << (x & 31));
+                pairs += __popc(bits);
+                // pairs within distance 2 still are kept: one word decides 32 of them
+                if (kTwin) bits &= ~a.pool2_new[ax];
             }
         }
         const int cnt = __popc(bits);
@@ -1035,7 +1058,8 @@ __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, in
             const int ow = __shfl_sync(0xffffffffu, wi, o), ox = __shfl_sync(0xffffffffu, x, o);
             int q = -1;
             if (idx < total) q = (ow << 5) + nth_set_bit(ob, idx - ex);
-            test_pairs3<kTwin>(a, ctr, ox, q, round, reads, pairs);
+            if (!kTwin && q >= 0 && in_b2_new<kTwin>(a, ox, q, round, reads)) q = -1;
+            decide_pairs3<kTwin>(a, ctr, ox, q, round, reads);
         }
     }
     // {x} x N_old(y) for the 32 slots of a stored item, restricted to B3_old(x): one per warp
@@ -1049,10 +1073,12 @@ __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, in
             reads += 2;
             if (c != x && (cl >= 0 || cl == -(round + 1))) {
                 reads++;
-                if (bit_of(b3, a.Wpad, x, c)) q = c;
+                const bool in3 = bit_of(b3, a.Wpad, x, c), in2 = in_b2_new<kTwin>(a, x, c, round, reads);
+                pairs += in3;
+                if (in3 && !in2) q = c;
             }
         }
-        test_pairs3<kTwin>(a, ctr, x, q, round, reads, pairs);
+        decide_pairs3<kTwin>(a, ctr, x, q, round, reads);
     }
 }
 
@@ -1338,7 +1364,7 @@ constexpr int kCRounds = 1024;       // rounds per launch
 // helpers; more than kMost... (kAlone... where the launch has no helpers) is left to the phase
 // launches.
 constexpr int kHelpDetect = 1024, kAloneDetect = 4096, kMostDetect = 1 << 16;     // detection items
-constexpr int kHelpTest3 = 1 << 12, kAloneTest3 = 1 << 17, kMostTest3 = 1 << 20;  // radius-3 items
+constexpr int kHelpTest3 = 1 << 14, kAloneTest3 = 1 << 17, kMostTest3 = 1 << 20;  // radius-3 items
 constexpr int kHelpDelta = 16384, kAloneDelta = 65536, kMostDelta = 1 << 21;       // update items
 constexpr unsigned long long kHelperWaitNs = 20000000000ull;  // a helper gives up waiting for a job
 constexpr unsigned long long kLeadWaitNs = 4000000000ull;     // the leader, for its helpers
@@ -1398,7 +1424,7 @@ __device__ __forceinline__ void shared_phase(const LossArgs &a, RoundCtr *ctr, W
     if (phase == kStageDetect) {
         unsigned pairs = 0u, reads = 0u;
         detect_items<kH3, true>(a, ctr, gw, nwarps, job.nitems, max_split, job.round, pairs, reads);
-        if (kH3) c3_items(a, ctr, gw, nwarps, job.nF, job.round);
+        if (kH3) c3_items(a, ctr, nwarps - 1 - gw, nwarps, job.nF, job.round);  // the warps with fewest items first
         stat_add(s_stat, kStatPairs, pairs);
         stat_add(s_stat, kStatReads, reads);
     } else if (kH3 && phase == kStageTest3) {
