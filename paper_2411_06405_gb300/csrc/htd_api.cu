@@ -266,12 +266,12 @@ htd_status htd_h_support(htd_graph *g, int32_t h, int32_t *sup_dev, void *stream
     Handle *H = &g->H;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
     API_TRY(begin_call(H, user));
-    API_TRY(prepare_work(H, h, h <= 2));
+    API_TRY(prepare_work(H, h, false));
     H->w.twin = false;
     H->w.dense_balls = false;  // h-support alone streams the smaller form of each ball
     H->w.inc3 = false;
     int64_t launches = 0;
-    htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, nullptr);
+    htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, nullptr, true);
     htd::g_launches += launches;
     API_TRY(ip);
     if (H->g.m > 0)
@@ -325,7 +325,7 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         API_TRY(htd::ensure_twin(H, (int64_t)(free_b / (H->shared_device ? 64 : 8))));
     }
     {
-        htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, timing ? &local : nullptr);
+        htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, timing ? &local : nullptr, false);
         if (ip == HTD_OK) ip = htd::initial_pass_r2(H, H->pstream, &launches);
         htd::g_launches += launches;
         launches_counted = launches;

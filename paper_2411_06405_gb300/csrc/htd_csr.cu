@@ -199,9 +199,10 @@ __global__ void k_compact_rows(int32_t n, const int32_t *__restrict__ off,
                                const int32_t *__restrict__ colraw,
                                const int32_t *__restrict__ len_new,
                                const int32_t *__restrict__ row_ptr, int32_t *__restrict__ col,
-                               int32_t *__restrict__ fwd) {
+                               int32_t *__restrict__ fwd, unsigned long long *__restrict__ deg2) {
     const int lane = threadIdx.x & 31;
     const int nwarps = gridDim.x * (blockDim.x >> 5);
+    unsigned long long squares = 0ull;
     for (int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += nwarps) {
         const int b = off[x], len = len_new[x], d = row_ptr[x];
         int above = 0;
@@ -212,7 +213,9 @@ __global__ void k_compact_rows(int32_t n, const int32_t *__restrict__ off,
         }
         above = warp_sum(above);
         if (lane == 0) fwd[x] = above;
+        squares += (unsigned long long)len * (unsigned)len;
     }
+    if (lane == 0 && squares) atomicAdd(deg2, squares);
 }
 
 __global__ void k_assign_eids(int32_t n, const int32_t *__restrict__ row_ptr,
@@ -289,6 +292,7 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     int32_t *deg = nullptr, *off = nullptr, *fill = nullptr, *colraw = nullptr;
     int32_t *deg_new = nullptr, *lists = nullptr, *counters = nullptr, *fwd = nullptr;
     int32_t *fwd_off = nullptr;
+    unsigned long long *deg2 = nullptr;
     void *tmp = nullptr;
     int32_t host_ctr[4] = {0, 0, 0, 0};
     int64_t nn = n > 0 ? n : 1;
@@ -307,7 +311,8 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     HTD_TRY(cudaMallocAsync(&colraw, (raw_slots > 0 ? raw_slots : 1) * sizeof(int32_t), s));
     HTD_TRY(cudaMallocAsync(&deg_new, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMallocAsync(&lists, 2 * nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&counters, 4 * sizeof(int32_t), s));
+    HTD_TRY(cudaMallocAsync(&counters, 6 * sizeof(int32_t), s));
+    deg2 = reinterpret_cast<unsigned long long *>(counters + 4);
     HTD_TRY(cudaMallocAsync(&fwd, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMallocAsync(&fwd_off, (nn + 1) * sizeof(int32_t), s));
     HTD_TRY(cudaMallocAsync(&tmp, scan_temp_bytes(nn + raw_slots), s));
@@ -315,7 +320,7 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     HTD_TRY(cudaMemsetAsync(deg, 0, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMemsetAsync(fill, 0, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMemsetAsync(deg_new, 0, nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMemsetAsync(counters, 0, 4 * sizeof(int32_t), s));
+    HTD_TRY(cudaMemsetAsync(counters, 0, 6 * sizeof(int32_t), s));
 
     if (m_in > 0) {
         int gb = grid_for(m_in, kBlock, nsm * 8);
@@ -362,13 +367,14 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     }
     if (n > 0) {
         int gw = grid_for((int64_t)n * 32, kBlock, nsm * 16);
-        k_compact_rows<<<gw, kBlock, 0, s>>>(n, off, colraw, deg_new, g.row_ptr, g.col, fwd);
+        k_compact_rows<<<gw, kBlock, 0, s>>>(n, off, colraw, deg_new, g.row_ptr, g.col, fwd, deg2);
         (*launches)++;
         HTD_TRY(scan_exclusive<int32_t, int32_t>(fwd, fwd_off, n, tmp, s, launches));
         k_assign_eids<<<gw, kBlock, 0, s>>>(n, g.row_ptr, g.col, fwd, fwd_off, g.slot_eid, g.eu,
                                             g.ev, g.slot_lo, g.slot_hi);
         (*launches)++;
     }
+    HTD_TRY(cudaMemcpyAsync(&g.deg2, deg2, sizeof(g.deg2), cudaMemcpyDeviceToHost, s));
     HTD_TRY(cudaGetLastError());
     HTD_TRY(cudaStreamSynchronize(s));
 

@@ -24,6 +24,7 @@ struct GraphDev {
     int32_t *ev = nullptr;        // m
     int32_t *slot_lo = nullptr;   // m, slot of ev[e] in row eu[e]
     int32_t *slot_hi = nullptr;   // m, slot of eu[e] in row ev[e]
+    uint64_t deg2 = 0;            // sum of the squared degrees
 };
 
 // Device scratch of one h-support pass / peel, cached on the handle between calls.
@@ -63,6 +64,9 @@ struct PeelWork {
     int32_t *hub_list = nullptr;   // nhub vertices with such a set (degree >= hub_min_deg)
     uint32_t *hub_bits = nullptr;  // nhub x Wpad words: alive neighbours as n-bit sets
     int32_t nhub = 0;
+    uint32_t *or_rows = nullptr;   // h-support alone: adjacency sets of the high-degree vertices
+    int32_t *or_row_of = nullptr;  // n: row of the vertex among them, or -1
+    int32_t *or_list = nullptr;    // their vertices, then their number
     int32_t hub_min_deg = 0;
     int4 *pitems = nullptr;        // loss detection items, two int4 each, <= 32 pairs
     int64_t pitems_cap = 0;
@@ -82,6 +86,8 @@ struct PeelWork {
     uint32_t *pool_new = nullptr;
     uint32_t *pool2_new = nullptr;
     uint32_t *pool2 = nullptr;
+    bool inner_ready = false;      // pool2 was built before the radius-3 balls, which are ORs of it
+    int64_t *dense_off = nullptr;  // n+1 offsets x * Wpad
     int32_t *ball_size2 = nullptr;
     int32_t *ball_nw2 = nullptr;
     int2 *ball_meta2 = nullptr;
@@ -143,8 +149,9 @@ void free_graph_dev(GraphDev *g);
 htd_status ensure_work(Handle *H, int32_t h, bool incremental, bool tiny_table = false);
 void free_work(PeelWork *w);
 htd_status ensure_twin(Handle *H, int64_t budget);
+// support_only: h-support alone (no peel follows).
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
-                        htd_stats *timing);
+                        htd_stats *timing, bool support_only);
 // evs (nullable): kRoundEvents events marking the phase boundaries of the round.
 constexpr int kRoundEvents = 7;
 // timer (incremental rounds, instead of events): phase times go to the status block.

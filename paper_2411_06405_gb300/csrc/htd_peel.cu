@@ -47,7 +47,7 @@ struct BallArgs {
     const int32_t *deg_alive;
     uint32_t *pool;
     uint32_t *pool_new;   // nullable: a second copy of every dense ball stored
-    const int64_t *ball_off;
+    int64_t *ball_off;
     int32_t *ball_need;
     int32_t *ball_size;
     int32_t *ball_nw;
@@ -57,6 +57,13 @@ struct BallArgs {
     int32_t *changed_stamp;
     int32_t *bfs_lists;
     int64_t bfs_list_len;
+    // Adjacency rows as n-bit sets (nullable; h = 2, first build only): a neighbour of degree
+    // or_deg or more is expanded by ORing its row, row_of[y] (null: row y).
+    const uint32_t *rows;
+    const int32_t *row_of;
+    int32_t or_deg;
+    int32_t bump;           // storage is taken from the pool in the order of completion
+    const uint32_t *inner;  // k_ball_or: dense balls of radius h - 1, row x at x * Wpad
     DevStatus *st;
 };
 
@@ -101,10 +108,105 @@ __device__ __forceinline__ void expand_chunk(int32_t y, const int32_t *__restric
     __syncthreads();
 }
 
+// Stores B(x,h) from the block's n-bit set: its size and form, then dense or as (word index,
+// word) pairs (kModeCount: only the storage it needs; kModeRebuild: only if it shrank).
+template <int MODE>
+__device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *bits, int32_t *s_wsz,
+                                           int32_t *s_wnz, int64_t *s_off64) {
+    DevStatus *st = a.st;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int W = a.W;
+    const int seg = ((W + kNWarps - 1) / kNWarps + 31) & ~31;
+    uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
+    // ball size and non-zero words, per warp segment of words
+    const int w0 = wid * seg, w1 = min(W, w0 + seg);
+    int sz = 0, nz = 0;
+    for (int i = w0 + lane; i < w1; i += 32) {
+        const uint32_t w = bits[i];
+        sz += __popc(w);
+        nz += (w != 0u);
+    }
+    sz = warp_sum(sz);
+    nz = warp_sum(nz);
+    if (lane == 0) {
+        s_wsz[wid] = sz;
+        s_wnz[wid] = nz;
+    }
+    __syncthreads();
+    int size = 0, nzw = 0, wbase = 0;
+#pragma unroll
+    for (int j = 0; j < kNWarps; j++) {
+        size += s_wsz[j];
+        nzw += s_wnz[j];
+        if (j < wid) wbase += s_wnz[j];
+    }
+    const bool dense = a.force_dense || 2 * nzw > W;
+    const int stor = dense ? a.Wpad : ((2 * nzw + 3) & ~3);
+    bool store = true;
+    if (MODE == kModeCount) {
+        if (threadIdx.x == 0) a.ball_need[x] = stor;
+        store = false;
+    } else if (MODE == kModeRebuild) {
+        const int old = a.ball_size[x];
+        if (size == old) store = false;
+        else if (size > old) {
+            if (threadIdx.x == 0) atomicOr(&st->err, kErrBallGrew);
+            store = false;
+        }
+    }
+    if (store) {
+        int64_t off, cap = stor;
+        if (MODE == kModeStore && a.bump) {
+            if (threadIdx.x == 0) *s_off64 = (int64_t)atomicAdd((unsigned long long *)&st->pool_next,
+                                                                (unsigned long long)stor);
+            __syncthreads();
+            off = *s_off64;
+            if (threadIdx.x == 0) a.ball_off[x] = off;
+        } else {
+            off = a.ball_off[x];
+            cap = a.ball_off[x + 1] - off;
+        }
+        if (stor > cap) {
+            if (threadIdx.x == 0) atomicOr(&st->err, kErrBallCapacity);
+        } else if (dense) {
+            uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
+            for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) dst[i] = bits4[i];
+            if (a.pool_new) {
+                uint4 *twin = reinterpret_cast<uint4 *>(a.pool_new + off);
+                for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) twin[i] = bits4[i];
+            }
+        } else {
+            uint2 *dst = reinterpret_cast<uint2 *>(a.pool + off);
+            int run = wbase;
+            for (int i0 = w0; i0 < w1; i0 += 32) {
+                const int i = i0 + lane;
+                const uint32_t w = (i < w1) ? bits[i] : 0u;
+                const unsigned bal = __ballot_sync(0xffffffffu, w != 0u);
+                if (w != 0u) dst[run + __popc(bal & lanemask_lt())] = make_uint2((uint32_t)i, w);
+                run += __popc(bal);
+            }
+        }
+        if (threadIdx.x == 0 && stor <= cap) {
+            if (MODE == kModeStore) atomicAdd((unsigned long long *)&st->st_ball_total,
+                                              (unsigned long long)size);
+            a.ball_size[x] = size;
+            a.ball_nw[x] = dense ? -1 : nzw;
+            a.ball_meta[x] = make_int2((int)(off >> 2), dense ? -1 : nzw);
+            if (MODE == kModeRebuild) {
+                a.changed_stamp[x] = st->round;
+                a.changed_list[atomicAdd(&st->nchanged, 1)] = x;
+            }
+        }
+    }
+}
+
 // Builds B(x,h) for a list of vertices, one vertex per block at a time (work queue).
 //   kModeCount:   records the storage words the ball needs (first pass);
 //   kModeStore:   stores the ball at its reserved offset (second pass);
 //   kModeRebuild: rebuilds a peel candidate; stores it and marks x changed iff it shrank.
+// The builds are bound by the expansions (about 160 G adjacency slots/s).  On hub graphs most
+// of them expand the same few rows: with the rows of degree W/16 and more as n-bit sets
+// (L2-resident: 988 rows, 32 MB on R-MAT 18) their share becomes W/4 16-byte loads each.
 template <int MODE>
 __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
     extern __shared__ __align__(16) uint32_t bits[];
@@ -114,6 +216,9 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
     __shared__ int32_t s_cnt[2];
     __shared__ int32_t s_wsz[kNWarps], s_wnz[kNWarps];
     __shared__ unsigned long long s_bytes;
+    __shared__ int64_t s_off64;
+    __shared__ int32_t s_or[kBlock], s_nor;
+    const bool by_rows = MODE != kModeRebuild && a.rows != nullptr && a.h == 2;
 
     DevStatus *st = a.st;
     int count;
@@ -127,9 +232,7 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
         count = a.n;
         queue = (MODE == kModeCount) ? &st->q_count : &st->q_store;
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int W = a.W;
-    const int seg = ((W + kNWarps - 1) / kNWarps + 31) & ~31;
+    const int lane = threadIdx.x & 31;
     int32_t *lists[2] = {nullptr, nullptr};
     if (a.h >= 3) {
         lists[0] = a.bfs_lists + (int64_t)blockIdx.x * 2 * a.bfs_list_len;
@@ -170,8 +273,36 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
                 if (a.count_bytes && a.h >= 2) bytes += 8ull + 4ull * (unsigned)a.deg_alive[y];
             }
             if (a.h >= 2) {
+                if (by_rows) {
+                    // hubs among the neighbours are set aside: their rows are ORed in below
+                    if (threadIdx.x == 0) s_nor = 0;
+                    __syncthreads();
+                    if (y >= 0 && a.row_ptr[y + 1] - a.row_ptr[y] >= a.or_deg) {
+                        const int r = a.row_of ? a.row_of[y] : y;
+                        if (r >= 0) {
+                            s_or[atomicAdd(&s_nor, 1)] = r;
+                            y = -1;
+                        }
+                    }
+                }
                 expand_chunk(y, a.row_ptr, a.col_live, bits, s_off, s_beg, s_scan,
                              a.h >= 3 ? lists[0] : nullptr, &s_cnt[0]);
+                if (by_rows && s_nor > 0) {
+                    const int W4 = a.Wpad >> 2, nor = s_nor;
+                    const uint4 *rows4 = reinterpret_cast<const uint4 *>(a.rows);
+                    for (int i = threadIdx.x; i < W4; i += kBlock) {
+                        uint4 v = bits4[i];
+                        for (int k = 0; k < nor; k++) {
+                            const uint4 r = rows4[(int64_t)s_or[k] * W4 + i];
+                            v.x |= r.x;
+                            v.y |= r.y;
+                            v.z |= r.z;
+                            v.w |= r.w;
+                        }
+                        bits4[i] = v;
+                    }
+                    __syncthreads();
+                }
             }
         }
         // depth 3..h from the level lists
@@ -192,77 +323,7 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
         }
         __syncthreads();
 
-        // ball size and non-zero words, per warp segment of words
-        const int w0 = wid * seg, w1 = min(W, w0 + seg);
-        int sz = 0, nz = 0;
-        for (int i = w0 + lane; i < w1; i += 32) {
-            const uint32_t w = bits[i];
-            sz += __popc(w);
-            nz += (w != 0u);
-        }
-        sz = warp_sum(sz);
-        nz = warp_sum(nz);
-        if (lane == 0) {
-            s_wsz[wid] = sz;
-            s_wnz[wid] = nz;
-        }
-        __syncthreads();
-        int size = 0, nzw = 0, wbase = 0;
-#pragma unroll
-        for (int j = 0; j < kNWarps; j++) {
-            size += s_wsz[j];
-            nzw += s_wnz[j];
-            if (j < wid) wbase += s_wnz[j];
-        }
-        const bool dense = a.force_dense || 2 * nzw > W;
-        const int stor = dense ? a.Wpad : ((2 * nzw + 3) & ~3);
-        bool store = true;
-        if (MODE == kModeCount) {
-            if (threadIdx.x == 0) a.ball_need[x] = stor;
-            store = false;
-        } else if (MODE == kModeRebuild) {
-            const int old = a.ball_size[x];
-            if (size == old) store = false;
-            else if (size > old) {
-                if (threadIdx.x == 0) atomicOr(&st->err, kErrBallGrew);
-                store = false;
-            }
-        }
-        if (store) {
-            const int64_t off = a.ball_off[x];
-            const int64_t cap = a.ball_off[x + 1] - off;
-            if (stor > cap) {
-                if (threadIdx.x == 0) atomicOr(&st->err, kErrBallCapacity);
-            } else if (dense) {
-                uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
-                for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) dst[i] = bits4[i];
-                if (a.pool_new) {
-                    uint4 *twin = reinterpret_cast<uint4 *>(a.pool_new + off);
-                    for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) twin[i] = bits4[i];
-                }
-            } else {
-                uint2 *dst = reinterpret_cast<uint2 *>(a.pool + off);
-                int run = wbase;
-                for (int i0 = w0; i0 < w1; i0 += 32) {
-                    const int i = i0 + lane;
-                    const uint32_t w = (i < w1) ? bits[i] : 0u;
-                    const unsigned bal = __ballot_sync(0xffffffffu, w != 0u);
-                    if (w != 0u) dst[run + __popc(bal & lanemask_lt())] = make_uint2((uint32_t)i, w);
-                    run += __popc(bal);
-                }
-            }
-            if (threadIdx.x == 0 && stor <= cap) {
-                if (MODE == kModeStore) atomicAdd((unsigned long long *)&st->st_ball_total,
-                                                  (unsigned long long)size);
-                a.ball_size[x] = size;
-                a.ball_nw[x] = dense ? -1 : nzw;
-                a.ball_meta[x] = make_int2((int)(off >> 2), dense ? -1 : nzw);
-                if (MODE == kModeRebuild) {
-                    a.changed_stamp[x] = st->round;
-                    a.changed_list[atomicAdd(&st->nchanged, 1)] = x;
-                }
-            }
-        }
+        store_ball<MODE>(a, x, bits, s_wsz, s_wnz, &s_off64);
         __syncthreads();
     }
     if (a.count_bytes) {
@@ -272,6 +333,67 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
         if (lane == 0 && b) atomicAdd(&s_bytes, b);
         __syncthreads();
         if (threadIdx.x == 0 && s_bytes) atomicAdd(&st->st_bytes_ball, s_bytes);
+    }
+}
+
+// B(x,h) for every vertex as the OR of its own and its neighbours' dense balls of radius
+// h - 1, one vertex per block at a time: 2m rows of W words are read, coalesced, whatever the
+// radius, where the search by levels of k_ball visits every slot of every vertex within h - 1.
+__global__ void __launch_bounds__(kBlock) k_ball_or(BallArgs a) {
+    extern __shared__ __align__(16) uint32_t bits[];
+    __shared__ int32_t s_item, s_row[kBlock];
+    __shared__ int32_t s_wsz[kNWarps], s_wnz[kNWarps];
+    __shared__ int64_t s_off64;
+    DevStatus *st = a.st;
+    uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
+    const uint4 *in4 = reinterpret_cast<const uint4 *>(a.inner);
+    const int W4 = a.Wpad >> 2;
+    for (;;) {
+        if (threadIdx.x == 0) s_item = atomicAdd(&st->q_store, 1);
+        __syncthreads();
+        const int x = s_item;
+        if (x >= a.n) break;
+        const int rb = a.row_ptr[x], re = a.row_ptr[x + 1];
+        for (int c = rb; c == rb || c < re; c += kBlock) {
+            const int cnt = min(kBlock, re - c);
+            if (threadIdx.x < cnt) s_row[threadIdx.x] = a.col_live[c + threadIdx.x];
+            __syncthreads();
+            for (int i = threadIdx.x; i < W4; i += kBlock) {
+                uint4 v = c == rb ? in4[(int64_t)x * W4 + i] : bits4[i];
+#pragma unroll 4
+                for (int k = 0; k < cnt; k++) {
+                    const uint4 r = in4[(int64_t)s_row[k] * W4 + i];
+                    v.x |= r.x;
+                    v.y |= r.y;
+                    v.z |= r.z;
+                    v.w |= r.w;
+                }
+                bits4[i] = v;
+            }
+            __syncthreads();
+        }
+        store_ball<kModeStore>(a, x, bits, s_wsz, s_wnz, &s_off64);
+        __syncthreads();
+    }
+}
+
+// Offsets of dense balls: x * Wpad.
+__global__ void k_dense_offsets(int64_t n, int64_t Wpad, int64_t *__restrict__ off) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
+        off[x] = x * Wpad;
+}
+
+// Vertices of degree `deg` and more get a row (at most `cap` of them); the others none.
+__global__ void k_or_rows(int32_t n, const int32_t *__restrict__ row_ptr, int32_t deg, int32_t cap,
+                          int32_t *__restrict__ row_of, int32_t *__restrict__ list, int32_t *__restrict__ count) {
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
+        int r = -1;
+        if (row_ptr[x + 1] - row_ptr[x] >= deg) {
+            r = atomicAdd(count, 1);
+            if (r < cap) list[r] = x;
+            else r = -1;
+        }
+        row_of[x] = r;
     }
 }
 
@@ -524,11 +646,14 @@ __global__ void k_make_records(int64_t m, const int32_t *__restrict__ row_ptr,
 }
 
 // Alive-adjacency n-bit sets of the high-degree vertices (all edges alive), block per hub.
+// count (nullable): the number of hubs, at most nhub of them, as a device value.
 __global__ void __launch_bounds__(kBlock) k_hub_init(const int32_t *__restrict__ hub_list, int32_t nhub,
+                                                    const int32_t *__restrict__ count,
                                                     const int32_t *__restrict__ row_ptr,
                                                     const int32_t *__restrict__ col,
                                                     uint32_t *__restrict__ hub_bits, int32_t Wpad) {
-    for (int hb = blockIdx.x; hb < nhub; hb += gridDim.x) {
+    const int hubs = count ? min(nhub, *count) : nhub;
+    for (int hb = blockIdx.x; hb < hubs; hb += gridDim.x) {
         uint32_t *bits = hub_bits + (int64_t)hb * Wpad;
         for (int i = threadIdx.x; i < Wpad; i += kBlock) bits[i] = 0u;
         __syncthreads();
@@ -568,6 +693,11 @@ cudaError_t alloc_n(T **p, int64_t count) {
     return cudaMalloc(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T));
 }
 
+// Degree from which ORing a vertex's n-bit row beats expanding its slots: a row costs W/4
+// 16-byte loads, a slot about 60 cycles per 32 of them (R-MAT 18, W = 8,192: 512 gave 5.5 ms
+// by the model of 160 G slots/s and 12 TB/s, 256 6.3 ms, 1,024 7.4 ms).
+int32_t or_degree(const PeelWork &w) { return std::max(64, w.W / 16); }
+
 BallArgs ball_args(Handle *H) {
     PeelWork &w = H->w;
     GraphDev &g = H->g;
@@ -593,6 +723,11 @@ BallArgs ball_args(Handle *H) {
     a.changed_stamp = w.changed_stamp;
     a.bfs_lists = w.bfs_lists;
     a.bfs_list_len = w.bfs_list_len;
+    a.rows = nullptr;
+    a.row_of = nullptr;
+    a.or_deg = or_degree(w);
+    a.bump = 0;
+    a.inner = nullptr;
     a.st = w.status;
     return a;
 }
@@ -655,6 +790,10 @@ void free_work(PeelWork *w) {
     cudaFree(w->scan_tmp);
     cudaFree(w->pool2);
     cudaFree(w->pool_new);
+    cudaFree(w->or_rows);
+    cudaFree(w->dense_off);
+    cudaFree(w->or_row_of);
+    cudaFree(w->or_list);
     cudaFree(w->pool2_new);
     cudaFree(w->ball_size2);
     cudaFree(w->ball_nw2);
@@ -697,21 +836,10 @@ htd_status ensure_work(Handle *H, int32_t h, bool incremental, bool tiny_table) 
 }
 
 namespace {
-htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_table) {
+// Scratch every pass at this h needs.
+htd_status alloc_base(Handle *H, int32_t h) {
     PeelWork &w = H->w;
-    GraphDev &g = H->g;
-    incremental = incremental && h <= 3;
-    if (w.status && w.h == h && (!incremental || (w.lost_keys && w.lost_tiny == tiny_table))) {
-        w.incremental = incremental;
-        w.inc3 = incremental && h == 3;
-        return HTD_OK;
-    }
-    if (w.status) {
-        // the per-block BFS lists and the ball storage depend on h: rebuild everything
-        drop_graphs(H);
-        free_work(&w);
-    }
-    const int64_t n = g.n, m = g.m;
+    const int64_t n = H->g.n, m = H->g.m;
     w.h = h;
     w.W = (int32_t)((n + 31) / 32);
     if (w.W < 1) w.W = 1;
@@ -721,6 +849,7 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
     HTD_CHECK(raise_smem_limit((const void *)k_ball<kModeCount>, w.smem_ball));
     HTD_CHECK(raise_smem_limit((const void *)k_ball<kModeStore>, w.smem_ball));
     HTD_CHECK(raise_smem_limit((const void *)k_ball<kModeRebuild>, w.smem_ball));
+    HTD_CHECK(raise_smem_limit((const void *)k_ball_or, w.smem_ball));
     HTD_CHECK(raise_smem_limit((const void *)k_hsup, w.smem_hsup));
     int occ_ball = 0, occ_hsup = 0;
     HTD_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_ball, k_ball<kModeRebuild>,
@@ -755,6 +884,33 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
         w.bfs_list_len = n > 0 ? n : 1;
         HTD_CHECK(alloc_n(&w.bfs_lists, (int64_t)w.grid_ball * 2 * w.bfs_list_len));
     }
+    HTD_CHECK(cudaMalloc(&w.scan_tmp, scan_temp_bytes(n + 1)));
+    HTD_CHECK(alloc_n(&w.status, 1));
+    HTD_CHECK(cudaMallocHost(reinterpret_cast<void **>(&w.status_host), sizeof(DevStatus)));
+    return HTD_OK;
+}
+
+htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_table) {
+    PeelWork &w = H->w;
+    GraphDev &g = H->g;
+    incremental = incremental && h <= 3;
+    if (w.status && w.h == h && (!incremental || (w.lost_keys && w.lost_tiny == tiny_table))) {
+        w.incremental = incremental;
+        w.inc3 = incremental && h == 3;
+        return HTD_OK;
+    }
+    // scratch of an h-support pass at the same h only lacks the incremental rounds' part
+    const bool base_ready = w.status && w.h == h && !w.lost_keys;
+    if (w.status && !base_ready) {
+        // the per-block BFS lists and the ball storage depend on h: rebuild everything
+        drop_graphs(H);
+        free_work(&w);
+    }
+    const int64_t n = g.n, m = g.m;
+    if (!base_ready) {
+        const htd_status bs = alloc_base(H, h);
+        if (bs != HTD_OK) return bs;
+    }
     if (incremental) {
         // a round's lost pairs: half of a power-of-two table of 8 x (2m) slots (>= 2^12)
         // sized to stay L2-resident (at most 2^22 slots, 32 MiB); larger rounds run in batches
@@ -784,10 +940,10 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
         if (h == 3) {
             // radius-2 balls (dense) with their own metadata, the round's radius-2 losses and
             // the radius-3 candidate items
-            HTD_CHECK(alloc_n(&w.pool2, n * (int64_t)w.Wpad));
-            HTD_CHECK(alloc_n(&w.ball_size2, n));
-            HTD_CHECK(alloc_n(&w.ball_nw2, n));
-            HTD_CHECK(alloc_n(&w.ball_meta2, n));
+            if (!w.pool2) HTD_CHECK(alloc_n(&w.pool2, n * (int64_t)w.Wpad));
+            if (!w.ball_size2) HTD_CHECK(alloc_n(&w.ball_size2, n));
+            if (!w.ball_nw2) HTD_CHECK(alloc_n(&w.ball_nw2, n));
+            if (!w.ball_meta2) HTD_CHECK(alloc_n(&w.ball_meta2, n));
             HTD_CHECK(alloc_n(&w.changed_list2, n));
             HTD_CHECK(alloc_n(&w.changed_stamp2, n));
             HTD_CHECK(alloc_n(&w.touch2, n));
@@ -836,9 +992,6 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
     }
     w.incremental = incremental;
     w.inc3 = incremental && h == 3;
-    HTD_CHECK(cudaMalloc(&w.scan_tmp, scan_temp_bytes(n + 1)));
-    HTD_CHECK(alloc_n(&w.status, 1));
-    HTD_CHECK(cudaMallocHost(reinterpret_cast<void **>(&w.status_host), sizeof(DevStatus)));
     return HTD_OK;
 }
 
@@ -868,14 +1021,101 @@ htd_status ensure_twin(Handle *H, int64_t budget) {
     return HTD_OK;
 }
 
-// Initial pass: every vertex's ball (count, reserve, store) and every edge's h-support,
-// then the first min reduction.  Leaves the status ready for round 0.
+namespace {
+
+// Adjacency rows of the high-degree vertices as n-bit sets, built once per handle: at most
+// 512 MiB of them (more would not stay in L2, where the builds read them).
+htd_status ensure_or_rows(Handle *H, cudaStream_t s, int64_t *launches) {
+    PeelWork &w = H->w;
+    GraphDev &g = H->g;
+    if (w.or_rows) return HTD_OK;
+    const int64_t deg = or_degree(w);
+    const int32_t cap = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(2 * g.m / deg + 1, ((int64_t)512 << 20) / (4 * (int64_t)w.Wpad)));
+    HTD_CHECK(alloc_n(&w.or_rows, (int64_t)cap * w.Wpad));
+    HTD_CHECK(alloc_n(&w.or_row_of, g.n));
+    HTD_CHECK(alloc_n(&w.or_list, (int64_t)cap + 1));
+    int32_t *count = w.or_list + cap;
+    HTD_CHECK(cudaMemsetAsync(count, 0, sizeof(int32_t), s));
+    k_or_rows<<<std::min<int64_t>((g.n + kBlock - 1) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
+        g.n, g.row_ptr, (int32_t)deg, cap, w.or_row_of, w.or_list, count);
+    k_hub_init<<<std::min(cap, H->num_sms * 8), kBlock, 0, s>>>(w.or_list, cap, count, g.row_ptr, g.col, w.or_rows,
+                                                            w.Wpad);
+    *launches += 2;
+    HTD_CHECK(cudaGetLastError());
+    return HTD_OK;
+}
+
+// Radius-3 balls as ORs of the neighbours' radius-2 rows (2m rows of W words, about 6 TB/s)
+// against the search by levels (about the sum of squared degrees x the mean degree slots, 60
+// G/s): DC-SBM 200k 10 ms against 32 ms; ER of mean degree 8 at n = 200,000 6.7 ms against 2.
+bool or_beats_search(const Handle *H) {
+    const GraphDev &g = H->g;
+    const double rows = 8.0 * (double)g.m * (double)H->w.Wpad;
+    const double slots = std::min((double)g.deg2, (double)g.n * (double)g.n) * (2.0 * (double)g.m / (double)g.n);
+    return rows < 100.0 * slots;
+}
+
+// Radius-2 balls of every vertex, stored dense in pool2 with their own sizes.
+htd_status build_inner(Handle *H, cudaStream_t s, int64_t *launches) {
+    PeelWork &w = H->w;
+    BallArgs b2 = ball_args(H);
+    b2.h = 2;
+    b2.count_bytes = 0;
+    b2.force_dense = 1;
+    b2.pool = w.pool2;
+    b2.pool_new = w.twin ? w.pool2_new : nullptr;
+    if (w.dense_off) b2.ball_off = w.dense_off;
+    if (w.incremental && w.nhub == H->g.n && w.hub_min_deg == 1) b2.rows = w.hub_bits;
+    b2.ball_size = w.ball_size2;
+    b2.ball_nw = w.ball_nw2;
+    b2.ball_meta = w.ball_meta2;
+    b2.changed_list = w.changed_list2;
+    b2.changed_stamp = w.changed_stamp2;
+    b2.bfs_lists = nullptr;
+    HTD_CHECK(cudaMemsetAsync(&w.status->q_store, 0, sizeof(int32_t), s));
+    k_ball<kModeStore><<<w.grid_ball, kBlock, w.smem_ball, s>>>(b2);
+    (*launches)++;
+    HTD_CHECK(cudaGetLastError());
+    return HTD_OK;
+}
+
+// The dense radius-2 balls for it: those of the incremental peel, or (h-support) a pool of
+// their own where they fit an eighth of the free memory.
+htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t free_b) {
+    PeelWork &w = H->w;
+    const int64_t words = H->g.n * (int64_t)w.Wpad;
+    w.inner_ready = false;
+    if (!w.pool2) {
+        if ((double)words * 4 > (double)free_b / 8) return HTD_OK;
+        HTD_CHECK(alloc_n(&w.pool2, words));
+    }
+    if (!w.ball_size2) {
+        HTD_CHECK(alloc_n(&w.ball_size2, H->g.n));
+        HTD_CHECK(alloc_n(&w.ball_nw2, H->g.n));
+        HTD_CHECK(alloc_n(&w.ball_meta2, H->g.n));
+    }
+    if (!w.dense_off) {
+        HTD_CHECK(alloc_n(&w.dense_off, (int64_t)H->g.n + 1));
+        k_dense_offsets<<<std::min<int64_t>((H->g.n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
+            H->g.n, w.Wpad, w.dense_off);
+        (*launches)++;
+    }
+    const htd_status rs = build_inner(H, s, launches);
+    w.inner_ready = rs == HTD_OK;
+    return rs;
+}
+
+}  // namespace
+
+// Initial pass: every vertex's ball and every edge's h-support, then the first min reduction.
+// Leaves the status ready for round 0 (support_only: the supports are all that is wanted).
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
-                        htd_stats *timing) {
+                        htd_stats *timing, bool support_only) {
     PeelWork &w = H->w;
     GraphDev &g = H->g;
     const int64_t n = g.n, m = g.m;
-    (void)h;
+    w.inner_ready = false;
     std::memset(w.status_host, 0, sizeof(DevStatus));
     w.status_host->k = 2;
     w.status_host->min_acc = INT_MAX;
@@ -902,7 +1142,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             (*launches)++;
         }
         if (w.nhub > 0) {
-            k_hub_init<<<std::min(w.nhub, H->num_sms * 8), kBlock, 0, s>>>(w.hub_list, w.nhub, g.row_ptr,
+            k_hub_init<<<std::min(w.nhub, H->num_sms * 8), kBlock, 0, s>>>(w.hub_list, w.nhub, nullptr, g.row_ptr,
                                                                         g.col, w.hub_bits, w.Wpad);
             (*launches)++;
         }
@@ -921,13 +1161,35 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         HTD_CHECK(cudaEventCreate(&e3));
     }
     if (n > 0) {
-        k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
-        (*launches)++;
-        HTD_CHECK(cudaGetLastError());
-        HTD_CHECK(scan_exclusive<int32_t, int64_t>(w.ball_need, w.ball_off, n, w.scan_tmp, s, launches));
-        int64_t total = 0;
-        HTD_CHECK(cudaMemcpyAsync(&total, w.ball_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        HTD_CHECK(cudaStreamSynchronize(s));
+        if (support_only && h == 2) {
+            const htd_status rs = ensure_or_rows(H, s, launches);
+            if (rs != HTD_OK) return rs;
+            ba.rows = w.or_rows;
+            ba.row_of = w.or_row_of;
+        } else if (w.incremental && w.nhub == n && w.hub_min_deg == 1) {
+            ba.rows = w.hub_bits;  // alive-adjacency sets, every edge alive
+        }
+        // Storage: dense balls have fixed places; h-support alone takes places as the balls are
+        // done, from a pool with room for all of them dense where that is a quarter of the free
+        // memory; else a first pass counts.
+        int64_t total = n * (int64_t)w.Wpad;
+        size_t free_b = 0, total_b = 0;
+        HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
+        const bool room = total <= w.pool_words || (double)total * 4 <= (double)free_b / 4;
+        if (w.dense_balls) {
+            k_dense_offsets<<<std::min<int64_t>((n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(n, w.Wpad,
+                                                                                                    w.ball_off);
+            (*launches)++;
+        } else if (support_only && room && total < ((int64_t)1 << 33)) {
+            ba.bump = 1;
+        } else {
+            k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
+            (*launches)++;
+            HTD_CHECK(cudaGetLastError());
+            HTD_CHECK(scan_exclusive<int32_t, int64_t>(w.ball_need, w.ball_off, n, w.scan_tmp, s, launches));
+            HTD_CHECK(cudaMemcpyAsync(&total, w.ball_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+            HTD_CHECK(cudaStreamSynchronize(s));
+        }
         if (total >= ((int64_t)1 << 33)) {
             set_last_error("htd: h-hop balls need more than 32 GiB of storage");
             return HTD_EUNSUPPORTED;
@@ -949,8 +1211,21 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         }
         ba.pool = w.pool;
         w.pool_used = total;
+        // radius 3 from the dense radius-2 balls, where their rows cost less than the search
+        const uint32_t *inner = nullptr;
+        if (h == 3 && (ba.bump || w.inc3) && or_beats_search(H)) {
+            const htd_status rs = ensure_inner(H, s, launches, free_b);
+            if (rs != HTD_OK) return rs;
+            inner = w.inner_ready ? w.pool2 : nullptr;
+            HTD_CHECK(cudaMemsetAsync(&w.status->q_store, 0, sizeof(int32_t), s));
+        }
         if (timing) HTD_CHECK(cudaEventRecord(e0, s));
-        k_ball<kModeStore><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
+        if (inner) {
+            ba.inner = inner;
+            k_ball_or<<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
+        } else {
+            k_ball<kModeStore><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
+        }
         if (timing) HTD_CHECK(cudaEventRecord(e1, s));
         (*launches)++;
         HTD_CHECK(cudaGetLastError());
@@ -1031,28 +1306,10 @@ htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent
     return HTD_OK;
 }
 
-// Radius-2 balls of every vertex for the incremental h = 3 peel, stored dense in pool2
-// with their own sizes (the radius-3 balls and supports come from initial_pass).
+// Radius-2 balls of the incremental h = 3 peel, unless the radius-3 balls were made of them.
 htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches) {
-    PeelWork &w = H->w;
-    if (!w.inc3 || H->g.n == 0) return HTD_OK;
-    BallArgs b2 = ball_args(H);
-    b2.h = 2;
-    b2.count_bytes = 0;
-    b2.force_dense = 1;
-    b2.pool = w.pool2;
-    b2.pool_new = w.twin ? w.pool2_new : nullptr;
-    b2.ball_size = w.ball_size2;
-    b2.ball_nw = w.ball_nw2;
-    b2.ball_meta = w.ball_meta2;
-    b2.changed_list = w.changed_list2;
-    b2.changed_stamp = w.changed_stamp2;
-    b2.bfs_lists = nullptr;
-    HTD_CHECK(cudaMemsetAsync(&w.status->q_store, 0, sizeof(int32_t), s));
-    k_ball<kModeStore><<<w.grid_ball, kBlock, w.smem_ball, s>>>(b2);
-    (*launches)++;
-    HTD_CHECK(cudaGetLastError());
-    return HTD_OK;
+    if (!H->w.inc3 || H->g.n == 0 || H->w.inner_ready) return HTD_OK;
+    return build_inner(H, s, launches);
 }
 
 namespace {
