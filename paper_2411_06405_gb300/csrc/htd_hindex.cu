@@ -11,15 +11,19 @@
 // at most h edges and may use e itself; the common h-neighbourhood is that of the whole
 // graph G, which never changes.
 //
-// GPU form.  The graph is fixed, so every vertex's closed ball B(x,h) is built once, as a
-// sorted member list.  An order is two kernels:
-//   k_hx_pathkeys  one block per vertex x: P(x, .) over the members of B(x,h) by h rounds
-//                  of hop-limited relaxation (round r extends paths of at most r-1 edges by
-//                  one edge; a member is found in the sorted list by binary search);
-//   k_hx_edges     one warp per edge: the common members of the two sorted lists (u and v
-//                  excluded), their values min(P(u,w), P(v,w)) gathered in a per-warp
-//                  buffer, and H(.) by a binary search on y of the monotone test
-//                  "at least y values >= y".
+// GPU form.  The graph is fixed, so every vertex's closed ball B(x,h) is kept as a sorted
+// member list, taken from the balls the h-support pass (H^(0)) has just built.  An order is
+// two kernels, one block per vertex each, with that vertex's ball in shared memory as an
+// n-bit set and, per word, the rank of its first member: a member's place in the list is then
+// two shared-memory reads.  (Binary searches in the lists, about ten dependent loads for every
+// relaxation and every common member, made an order 12 ms on DC-SBM 50k at h = 2.)
+//   k_hx_pathkeys  P(x, .) over the members of B(x,h) by h rounds of hop-limited relaxation
+//                  (round r extends paths of at most r-1 edges by one edge);
+//   k_hx_edges     the edges the vertex owns (the endpoint with the larger ball), one warp
+//                  each: the other endpoint's members are streamed against the set, the values
+//                  min(P(u,w), P(v,w)) of the common ones gathered in a per-warp buffer, and
+//                  H(.) found by the monotone test "at least y values >= y", down from the
+//                  old key in growing steps (keys never increase), then by bisection.
 // Synchronous orders (Algorithm 2) write the new keys to a second array.  With pruning
 // (Lemma 4), from the second order on an edge keeps its key without being computed when no
 // edge near it fell across that key in the previous order: per vertex, the range of the
@@ -46,80 +50,39 @@ namespace {
 
 constexpr int kBlock = 256;
 
-// BFS of one block from x to depth h over all edges into the block's n-bit set; lists are
-// the block's two level lists (n entries each).
-__device__ void hx_bfs(int32_t x, int32_t h, const int32_t *__restrict__ row_ptr,
-                       const int32_t *__restrict__ col, uint32_t *bits, int32_t W, int32_t *l0,
-                       int32_t *l1, int32_t *s_cnt) {
-    for (int i = threadIdx.x; i < W; i += blockDim.x) bits[i] = 0u;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        bits[x >> 5] |= 1u << (x & 31);
-        l0[0] = x;
-        s_cnt[0] = 1;
-        s_cnt[1] = 0;
-    }
-    __syncthreads();
-    int32_t *cur = l0, *nxt = l1;
-    for (int d = 1; d <= h; d++) {
-        const int ncur = s_cnt[(d - 1) & 1];
-        if (ncur == 0) break;
-        for (int i = threadIdx.x; i < ncur; i += blockDim.x) {
-            const int y = cur[i];
-            for (int s = row_ptr[y]; s < row_ptr[y + 1]; s++) {
-                const int z = col[s];
-                const uint32_t m = 1u << (z & 31);
-                if (*(volatile uint32_t *)&bits[z >> 5] & m) continue;
-                if ((atomicOr(&bits[z >> 5], m) & m) == 0u && d < h) nxt[atomicAdd(&s_cnt[d & 1], 1)] = z;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_cnt[(d + 1) & 1] = 0;
-        __syncthreads();
-        int32_t *t = cur;
-        cur = nxt;
-        nxt = t;
-    }
-}
-
-// Ball sizes (MODE 0) or sorted member lists (MODE 1) of every vertex, block per vertex.
-template <int MODE>
-__global__ void __launch_bounds__(kBlock) k_hx_balls(int32_t n, int32_t h, const int32_t *__restrict__ row_ptr,
-                                                    const int32_t *__restrict__ col, int32_t W,
-                                                    int32_t *lists, int32_t *sizes,
-                                                    const int64_t *__restrict__ off,
-                                                    int32_t *__restrict__ members) {
-    extern __shared__ __align__(16) uint32_t bits[];
-    __shared__ int32_t s_cnt[2];
+// Sorted member lists of every vertex, block per vertex, from the stored balls (dense words,
+// or sorted (word index, word) pairs).
+__global__ void __launch_bounds__(kBlock) k_hx_members(int32_t n, int32_t W, const uint32_t *__restrict__ pool,
+                                                      const int64_t *__restrict__ ball_off,
+                                                      const int32_t *__restrict__ ball_nw,
+                                                      const int64_t *__restrict__ off,
+                                                      int32_t *__restrict__ members) {
     __shared__ int32_t s_scan[kBlock / 32];
-    int32_t *l0 = lists + (int64_t)blockIdx.x * 2 * n;
-    int32_t *l1 = l0 + n;
     for (int x = blockIdx.x; x < n; x += gridDim.x) {
-        hx_bfs(x, h, row_ptr, col, bits, W, l0, l1, s_cnt);
-        if (MODE == 0) {
-            int c = 0;
-            for (int i = threadIdx.x; i < W; i += blockDim.x) c += __popc(bits[i]);
-            const int tot = block_sum<kBlock, int>(c, s_scan);
-            if (threadIdx.x == 0) sizes[x] = tot;
-        } else {
-            // members in increasing order: words in chunks of one per thread
-            int64_t base = off[x];
-            for (int w0 = 0; w0 < W; w0 += kBlock) {
-                const int w = w0 + threadIdx.x;
-                uint32_t v = w < W ? bits[w] : 0u;
-                int tot;
-                const int ex = block_exclusive_scan<kBlock, int>(__popc(v), &tot, s_scan);
-                int k = 0;
-                while (v) {
-                    const int b = __ffs(v) - 1;
-                    v &= v - 1u;
-                    members[base + ex + k] = (w << 5) + b;
-                    k++;
+        const int nw = ball_nw[x], count = nw < 0 ? W : nw;
+        const uint32_t *words = pool + ball_off[x];
+        int64_t base = off[x];
+        for (int i0 = 0; i0 < count; i0 += kBlock) {
+            const int i = i0 + threadIdx.x;
+            int w = i;
+            uint32_t v = 0u;
+            if (i < count) {
+                if (nw < 0) {
+                    v = words[i];
+                } else {
+                    w = (int)words[2 * i];
+                    v = words[2 * i + 1];
                 }
-                base += tot;
             }
+            int tot;
+            int at = block_exclusive_scan<kBlock, int>(__popc(v), &tot, s_scan);
+            while (v) {
+                const int b = __ffs(v) - 1;
+                v &= v - 1u;
+                members[base + at++] = (w << 5) + b;
+            }
+            base += tot;
         }
-        __syncthreads();
     }
 }
 
@@ -136,106 +99,235 @@ __device__ __forceinline__ int find_member(const int32_t *__restrict__ m, int le
     return -1;
 }
 
-// P(x, .) for the vertices of `list` (all vertices if null), block per vertex.  `prev` is
-// the block's scratch of maxb entries (the values of the previous round).
+// A vertex's ball in shared memory: the n-bit set and, for every word that holds members,
+// the rank of its first one (the list is sorted, so that member knows its own rank).  Where
+// the two do not fit (words == 0), places are found by binary search in the list.
+struct BallIndex {
+    uint32_t *bits;
+    int32_t *rank;
+    const int32_t *m;  // member list
+    int32_t len;
+    int32_t words;
+
+    __device__ void clear_all() {
+        for (int i = threadIdx.x; i < words; i += blockDim.x) bits[i] = 0u;
+        __syncthreads();
+    }
+    __device__ void load(const int32_t *list, int n) {
+        m = list;
+        len = n;
+        if (words == 0) return;
+        for (int j = threadIdx.x; j < len; j += blockDim.x) {
+            const int z = m[j], w = z >> 5;
+            atomicOr(bits + w, 1u << (z & 31));
+            if (j == 0 || (m[j - 1] >> 5) != w) rank[w] = j;
+        }
+        __syncthreads();
+    }
+    // after a barrier; the next load needs one more
+    __device__ void unload() {
+        if (words == 0) return;
+        for (int j = threadIdx.x; j < len; j += blockDim.x) bits[m[j] >> 5] = 0u;
+    }
+    __device__ __forceinline__ int find(int z) const {
+        if (words == 0) return find_member(m, len, z);
+        const uint32_t v = bits[z >> 5], below = (1u << (z & 31)) - 1u;
+        return (v >> (z & 31)) & 1u ? rank[z >> 5] + __popc(v & below) : -1;
+    }
+};
+
+// P(x, .) for the vertices of `list` (all vertices if null; `count`, or *dcount of them), block
+// per vertex.  The values are kept in shared memory while they fit pcap entries, else in P;
+// `prev` is the block's scratch of maxb entries (the values of the previous round, h >= 3).
 __global__ void __launch_bounds__(kBlock) k_hx_pathkeys(const int32_t *__restrict__ list, int32_t count,
-                                                       int32_t h, const int32_t *__restrict__ row_ptr,
+                                                       const int32_t *__restrict__ dcount, int32_t h,
+                                                       const int32_t *__restrict__ row_ptr,
                                                        const int32_t *__restrict__ col,
                                                        const int32_t *__restrict__ slot_eid,
                                                        const int32_t *__restrict__ key,
                                                        const int64_t *__restrict__ off,
                                                        const int32_t *__restrict__ members,
                                                        int32_t *__restrict__ P, int32_t *prev_all,
-                                                       int64_t maxb) {
+                                                       int64_t maxb, int32_t words, int32_t pcap) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    BallIndex ball;
+    ball.bits = smem;
+    ball.rank = reinterpret_cast<int32_t *>(smem + words);
+    ball.words = words;
+    int32_t *const sp = reinterpret_cast<int32_t *>(smem + 2 * words);
     int32_t *prev = prev_all + (int64_t)blockIdx.x * maxb;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (dcount) count = *dcount;
+    ball.clear_all();
     for (int i = blockIdx.x; i < count; i += gridDim.x) {
         const int x = list ? list[i] : i;
         const int64_t o = off[x];
         const int len = (int)(off[x + 1] - o);
-        const int32_t *m = members + o;
-        int32_t *p = P + o;
-        for (int j = threadIdx.x; j < len; j += blockDim.x) p[j] = (m[j] == x) ? INT_MAX : -1;
+        int32_t *const p = len <= pcap ? sp : P + o;
+        for (int j = threadIdx.x; j < len; j += blockDim.x) p[j] = -1;
+        ball.load(members + o, len);
         __syncthreads();
-        for (int r = 1; r <= h; r++) {
-            for (int j = threadIdx.x; j < len; j += blockDim.x) prev[j] = p[j];
-            __syncthreads();
-            // one warp per member reached within r-1 edges; its lanes walk the row
-            for (int j = wid; j < len; j += nw) {
-                const int pv = prev[j];
+        const int rb = row_ptr[x], re = row_ptr[x + 1];
+        // round 1: the edges of x
+        if (threadIdx.x == 0) p[ball.find(x)] = INT_MAX;
+        for (int s = rb + threadIdx.x; s < re; s += blockDim.x) p[ball.find(col[s])] = key[slot_eid[s]];
+        __syncthreads();
+        // every neighbour of a vertex within r-1 <= h-1 edges of x is a member of the ball
+        for (int r = 2; r <= h; r++) {
+            if (r > 2) {
+                for (int j = threadIdx.x; j < len; j += blockDim.x) prev[j] = p[j];
+                __syncthreads();
+            }
+            // one warp per vertex reached within r-1 edges (r = 2: the row of x says which,
+            // and with what value); its lanes walk that vertex's row
+            const int sources = r == 2 ? re - rb : len;
+            for (int j = wid; j < sources; j += nw) {
+                const int pv = r == 2 ? key[slot_eid[rb + j]] : prev[j];
                 if (pv < 0) continue;
-                const int y = m[j];
-                for (int s = row_ptr[y] + lane; s < row_ptr[y + 1]; s += 32) {
-                    const int z = col[s];
-                    const int iz = find_member(m, len, z);
-                    if (iz < 0) continue;
+                const int y = r == 2 ? col[rb + j] : members[o + j];
+                const int ye = row_ptr[y + 1];
+                for (int s = row_ptr[y] + lane; s < ye; s += 32) {
+                    const int iz = ball.find(col[s]);
                     const int c = min(pv, key[slot_eid[s]]);
                     if (c > p[iz]) atomicMax(&p[iz], c);
                 }
             }
             __syncthreads();
         }
+        if (len <= pcap)
+            for (int j = threadIdx.x; j < len; j += blockDim.x) P[o + j] = p[j];
+        ball.unload();
+        __syncthreads();
     }
 }
 
-// New keys of the edges [e0, e1) (of elist[e0..e1) when elist is not null), one warp per
-// edge.  vals: the warp's buffer of maxd.
-__global__ void __launch_bounds__(kBlock) k_hx_edges(int64_t e0, int64_t e1, const int32_t *__restrict__ elist,
-                                                    const int32_t *__restrict__ eu,
-                                                    const int32_t *__restrict__ ev,
+// Work items of k_hx_edges: every kItemSlots adjacency slots of the vertices of `list` (all
+// vertices if null), so that a hub's edges are spread over many blocks.
+constexpr int kItemSlots = 64;
+
+__global__ void k_hx_items(const int32_t *__restrict__ list, int32_t count, const int32_t *__restrict__ dcount,
+                           const int32_t *__restrict__ row_ptr, int2 *__restrict__ items, int32_t *nitems) {
+    if (dcount) count = *dcount;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+        const int x = list ? list[i] : i;
+        const int rb = row_ptr[x], nch = (row_ptr[x + 1] - rb + kItemSlots - 1) / kItemSlots;
+        if (nch == 0) continue;
+        const int first = atomicAdd(nitems, nch);
+        for (int c = 0; c < nch; c++) items[first + c] = make_int2(x, rb + c * kItemSlots);
+    }
+}
+
+// New keys of the listed edges: those of [e0, e1), or with `emark` those with emark[e] ==
+// stamp.  A block takes an item (a vertex and a run of its slots) at a time from a queue, its
+// warps the listed edges that vertex owns.  vals: the warp's buffer of maxd.
+__global__ void __launch_bounds__(kBlock) k_hx_edges(const int2 *__restrict__ items, const int32_t *__restrict__ nitems,
+                                                    int32_t *queue, int64_t e0, int64_t e1,
+                                                    const int32_t *__restrict__ emark, int32_t stamp,
+                                                    const int32_t *__restrict__ row_ptr,
+                                                    const int32_t *__restrict__ col,
+                                                    const int32_t *__restrict__ slot_eid,
                                                     const int64_t *__restrict__ off,
                                                     const int32_t *__restrict__ members,
                                                     const int32_t *__restrict__ P,
                                                     const int32_t *key_in, int32_t *key_out,
                                                     int32_t *vals_all, int64_t maxd,
-                                                    unsigned long long *changed) {
+                                                    unsigned long long *changed, int32_t words, int32_t pcap) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ int32_t s_slot[kItemSlots], s_n, s_next, s_item;
+    BallIndex ball;
+    ball.bits = smem;
+    ball.rank = reinterpret_cast<int32_t *>(smem + words);
+    ball.words = words;
+    int32_t *const sp = reinterpret_cast<int32_t *>(smem + 2 * words);
     const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    int32_t *vals = vals_all + gw * maxd;
+    int32_t *vals = vals_all + ((int64_t)blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5)) * maxd;
     unsigned long long nchg = 0;
-    for (int64_t i = e0 + gw; i < e1; i += nwarps) {
-        const int64_t e = elist ? elist[i] : i;
-        int u = eu[e], v = ev[e];
-        int64_t ou = off[u], ov = off[v];
-        int lu = (int)(off[u + 1] - ou), lv = (int)(off[v + 1] - ov);
-        if (lu > lv) {  // walk the shorter list, search the longer one
-            const int t = u; u = v; v = t;
-            const int64_t to = ou; ou = ov; ov = to;
-            const int tl = lu; lu = lv; lv = tl;
+    const int count = *nitems;
+    ball.clear_all();
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_item = atomicAdd(queue, 1);
+            s_n = s_next = 0;
         }
-        const int32_t *mu = members + ou, *mv = members + ov;
-        int cnt = 0;
-        for (int j0 = 0; j0 < lu; j0 += 32) {
-            const int j = j0 + lane;
-            int val = -1;
-            if (j < lu) {
-                const int w = mu[j];
-                if (w != u && w != v) {
-                    const int iv = find_member(mv, lv, w);
-                    if (iv >= 0) val = min(P[ou + j], P[ov + iv]);
-                }
+        __syncthreads();
+        const int it = s_item;
+        if (it >= count) break;
+        const int2 item = items[it];
+        const int u = item.x;
+        const int64_t ou = off[u];
+        const int lu = (int)(off[u + 1] - ou);
+        const int sl = item.y + threadIdx.x;
+        if (threadIdx.x < kItemSlots && sl < row_ptr[u + 1]) {
+            const int v = col[sl], e = slot_eid[sl];
+            const bool listed = emark ? emark[e] == stamp : e >= e0 && e < e1;
+            const int lv = (int)(off[v + 1] - off[v]);
+            // the endpoint with the larger ball owns the edge: the smaller list is streamed
+            if (listed && (lu > lv || (lu == lv && u < v))) s_slot[atomicAdd(&s_n, 1)] = sl;
+        }
+        __syncthreads();
+        const int owned = s_n;
+        if (owned > 0) {
+            const int32_t *pu = P + ou;
+            if (lu <= pcap) {
+                for (int j = threadIdx.x; j < lu; j += blockDim.x) sp[j] = pu[j];
+                pu = sp;
             }
-            const unsigned b = __ballot_sync(0xffffffffu, val >= 0);
-            if (val >= 0) vals[cnt + __popc(b & ((1u << lane) - 1u))] = val;
-            cnt += __popc(b);
+            ball.load(members + ou, lu);
+            __syncthreads();
+            for (;;) {
+                int k = 0;
+                if (lane == 0) k = atomicAdd(&s_next, 1);
+                k = __shfl_sync(0xffffffffu, k, 0);
+                if (k >= owned) break;
+                const int s = s_slot[k], v = col[s], e = slot_eid[s];
+                const int64_t ov = off[v];
+                const int lv = (int)(off[v + 1] - ov);
+                const int32_t *mv = members + ov, *pv = P + ov;
+                int cnt = 0;
+                for (int j0 = 0; j0 < lv; j0 += 32) {
+                    const int j = j0 + lane;
+                    int val = -1;
+                    if (j < lv) {
+                        const int w = mv[j];
+                        const int iu = (w != u && w != v) ? ball.find(w) : -1;
+                        if (iu >= 0) val = min(pu[iu], pv[j]);
+                    }
+                    const unsigned b = __ballot_sync(0xffffffffu, val >= 0);
+                    if (val >= 0) vals[cnt + __popc(b & lanemask_lt())] = val;
+                    cnt += __popc(b);
+                }
+                __syncwarp();
+                // H = largest y in [0, cnt] with at least y values >= y; it is at most the old key
+                const int old = key_in[e];
+                int lo = 0, hi = cnt + 1, step = 1, mid = min(old, cnt);
+                while (hi - lo > 1) {
+                    int c = 0;
+                    for (int j = lane; j < cnt; j += 32) c += vals[j] >= mid;
+                    c = warp_sum(c);
+                    if (c >= mid) {
+                        lo = mid;
+                        if (mid == old) break;  // keys never increase
+                        step = 0;
+                    } else {
+                        hi = mid;
+                    }
+                    if (step > 0) {
+                        mid = max(hi - step, (lo + hi) >> 1);
+                        step *= 2;
+                    } else {
+                        mid = (lo + hi) >> 1;
+                    }
+                }
+                if (lane == 0) {
+                    if (lo != old) nchg++;
+                    key_out[e] = lo;
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+            ball.unload();
         }
-        __syncwarp();
-        // H = largest y in [0, cnt] with at least y values >= y (the test is monotone in y)
-        int lo = 0, hi = cnt + 1;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            int c = 0;
-            for (int j = lane; j < cnt; j += 32) c += vals[j] >= mid;
-            c = warp_sum(c);
-            if (c >= mid) lo = mid;
-            else hi = mid;
-        }
-        if (lane == 0) {
-            if (lo != key_in[e]) nchg++;
-            key_out[e] = lo;
-        }
-        __syncwarp();
+        __syncthreads();
     }
     if (lane == 0 && nchg) atomicAdd(changed, nchg);
 }
@@ -244,10 +336,12 @@ __global__ void __launch_bounds__(kBlock) k_hx_edges(int64_t e0, int64_t e1, con
 __global__ void k_hx_touch(int64_t e0, int64_t e1, const int32_t *__restrict__ eu,
                            const int32_t *__restrict__ ev, int32_t stamp, int32_t *mark,
                            int32_t *list, int32_t *count) {
-    for (int64_t i = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < e1 + 0; i += (int64_t)gridDim.x * blockDim.x) {
-        const int a = eu[i], b = ev[i];
-        if (atomicExch(&mark[a], stamp) != stamp) list[atomicAdd(count, 1)] = a;
-        if (atomicExch(&mark[b], stamp) != stamp) list[atomicAdd(count, 1)] = b;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = e0 + blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < e1; i0 += stride) {
+        const int64_t i = i0 + (threadIdx.x & 31);
+        const int a = i < e1 ? eu[i] : 0, b = i < e1 ? ev[i] : 0;
+        warp_append(i < e1 && atomicExch(&mark[a], stamp) != stamp, a, count, list);
+        warp_append(i < e1 && atomicExch(&mark[b], stamp) != stamp, b, count, list);
     }
 }
 
@@ -294,25 +388,35 @@ __global__ void __launch_bounds__(kBlock) k_hx_spread(int32_t n, const int32_t *
     }
 }
 
-// Pruning, step 3: an edge e = (u,v) with T = H^(n-1)(e) is listed for computation when
-// the hull [min(lo(u), lo(v)), max(hi(u), hi(v))] of the fallen values near it straddles
-// T (some value went from >= T to < T); otherwise H^(n)(e) = T (Lemma 4).  The endpoints of
-// listed edges are listed once each (mark holds the stamp of the order that listed them).
+// Pruning, step 3: an edge e = (u,v) with T = H^(n-1)(e) is listed for computation (emark =
+// stamp) when the hull [min(lo(u), lo(v)), max(hi(u), hi(v))] of the fallen values near it
+// straddles T (some value went from >= T to < T); otherwise H^(n)(e) = T (Lemma 4).  The
+// endpoints of listed edges are listed once each (mark holds the stamp of the order).
 __global__ void k_hx_select(int64_t m, const int32_t *__restrict__ eu, const int32_t *__restrict__ ev,
                             const int32_t *__restrict__ kcur, const int32_t *__restrict__ hi,
-                            const int32_t *__restrict__ lo, int32_t *knew, int32_t *elist,
+                            const int32_t *__restrict__ lo, int32_t *knew, int32_t *emark,
                             int32_t *ecount, int32_t stamp, int32_t *mark, int32_t *vlist,
                             int32_t *vcount) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const int u = eu[e], v = ev[e], T = kcur[e];
-        const int l = min(lo[u], lo[v]), hh = max(hi[u], hi[v]);
-        if (l < T && T <= hh) {
-            elist[atomicAdd(ecount, 1)] = (int32_t)e;
-            if (atomicExch(&mark[u], stamp) != stamp) vlist[atomicAdd(vcount, 1)] = u;
-            if (atomicExch(&mark[v], stamp) != stamp) vlist[atomicAdd(vcount, 1)] = v;
-        } else {
-            knew[e] = T;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); i0 < m; i0 += stride) {
+        const int64_t e = i0 + (threadIdx.x & 31);
+        int u = 0, v = 0;
+        bool listed = false;
+        if (e < m) {
+            u = eu[e];
+            v = ev[e];
+            const int T = kcur[e];
+            const int l = min(lo[u], lo[v]), hh = max(hi[u], hi[v]);
+            listed = l < T && T <= hh;
+            if (listed) emark[e] = stamp;
+            else knew[e] = T;
         }
+        const unsigned b = __ballot_sync(0xffffffffu, listed);
+        if ((threadIdx.x & 31) == 0 && b) atomicAdd(ecount, __popc(b));
+        const bool fu = listed && atomicExch(&mark[u], stamp) != stamp;
+        const bool fv = listed && atomicExch(&mark[v], stamp) != stamp;
+        warp_append(fu, u, vcount, vlist);
+        warp_append(fv, v, vcount, vlist);
     }
 }
 
@@ -340,14 +444,18 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
     GraphDev &g = H->g;
     const int64_t n = g.n, m = g.m;
     htd_status st = HTD_OK;
-    int32_t *sizes = nullptr, *members = nullptr, *P = nullptr, *prev = nullptr, *vals = nullptr;
-    int32_t *key = nullptr, *key2 = nullptr, *lists = nullptr, *mark = nullptr, *vlist = nullptr;
-    int32_t *dcount = nullptr, *kold = nullptr, *hi = nullptr, *lo = nullptr, *hi2 = nullptr, *lo2 = nullptr;
-    int32_t *elist = nullptr, *decount = nullptr, *hecount = nullptr;
+    int32_t *members = nullptr, *P = nullptr, *prev = nullptr, *vals = nullptr;
+    int32_t *key = nullptr, *key2 = nullptr, *mark = nullptr, *vlist = nullptr;
+    int32_t *kold = nullptr, *hi = nullptr, *lo = nullptr, *hi2 = nullptr, *lo2 = nullptr;
+    int32_t *emark = nullptr;
     int64_t *off = nullptr;
-    void *tmp = nullptr;
-    unsigned long long *dchanged = nullptr, *hchanged = nullptr;
-    int32_t *hcount = nullptr;
+    // edges changed in the order; vertices and edges listed
+    struct Counters {
+        unsigned long long changed;
+        int32_t vertices, edges;
+        int32_t items, queue;  // of the order's edge kernel
+    };
+    Counters *dctr = nullptr, *hctr = nullptr;
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     htd_hindex_stats loc;
     std::memset(&loc, 0, sizeof(loc));
@@ -355,46 +463,20 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
     loc.sweeps = sweeps;
     loc.pruned = prune ? 1 : 0;
     int64_t launches = 0;
+    PeelWork &w = H->w;
     const int W = (int)std::max<int64_t>(1, (n + 31) / 32);
-    const size_t smem = (size_t)W * 4;
-    int occ = 0, grid_v = 0;
-    int64_t total = 0, maxb = 0, maxd = 0;
+    int occ_p = 0, occ_e = 0, grid_p = 0, grid_e = 0;
+    int64_t total = 0, maxb = 0;
     std::vector<int32_t> hsizes;
+    // the ball index (set and ranks) where it leaves room for two blocks an SM, and path keys
+    // of up to kPathCap members beside it
+    constexpr int32_t kPathCap = 4096;
+    const int32_t words = 8 * (int64_t)W <= 90 * 1024 ? W : 0;
+    const size_t smem = 8 * (size_t)words + 4 * (size_t)kPathCap;
     if (m == 0) goto finish;
     HX_CHECK(cudaEventCreate(&t0));
     HX_CHECK(cudaEventCreate(&t1));
     HX_CHECK(cudaEventRecord(t0, s));
-    HX_CHECK(raise_smem_limit((const void *)k_hx_balls<0>, smem));
-    HX_CHECK(raise_smem_limit((const void *)k_hx_balls<1>, smem));
-    HX_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hx_balls<1>, kBlock, smem));
-    if (occ < 1) {
-        set_last_error("htd_hindex_decompose: an n-bit set does not fit in shared memory");
-        st = HTD_EUNSUPPORTED;
-        goto done;
-    }
-    grid_v = (int)std::min<int64_t>(n, (int64_t)H->num_sms * occ);
-    HX_CHECK(cudaMalloc(&sizes, n * 4));
-    HX_CHECK(cudaMalloc(&off, (n + 1) * 8));
-    HX_CHECK(cudaMalloc(&lists, (int64_t)grid_v * 2 * n * 4));
-    HX_CHECK(cudaMalloc(&tmp, scan_temp_bytes(n + 1)));
-    k_hx_balls<0><<<grid_v, kBlock, smem, s>>>((int32_t)n, h, g.row_ptr, g.col, W, lists, sizes, nullptr, nullptr);
-    launches++;
-    HX_CHECK(cudaGetLastError());
-    HX_CHECK(scan_exclusive<int32_t, int64_t>(sizes, off, n, tmp, s, &launches));
-    hsizes.resize(n);
-    HX_CHECK(cudaMemcpyAsync(&total, off + n, 8, cudaMemcpyDeviceToHost, s));
-    HX_CHECK(cudaMemcpyAsync(hsizes.data(), sizes, n * 4, cudaMemcpyDeviceToHost, s));
-    HX_CHECK(cudaStreamSynchronize(s));
-    for (int64_t x = 0; x < n; x++) maxb = std::max<int64_t>(maxb, hsizes[x]);
-    maxd = maxb;
-    loc.ball_entries = total;
-    HX_CHECK(cudaMalloc(&members, std::max<int64_t>(total, 1) * 4));
-    HX_CHECK(cudaMalloc(&P, std::max<int64_t>(total, 1) * 4));
-    k_hx_balls<1><<<grid_v, kBlock, smem, s>>>((int32_t)n, h, g.row_ptr, g.col, W, lists, sizes, off, members);
-    launches++;
-    HX_CHECK(cudaGetLastError());
-    cudaFree(lists);
-    lists = nullptr;
     {
         // H^(0) = sup(e,h), the h-support of every edge (the initial step of Algorithm 2)
         HX_CHECK(cudaMalloc(&key, m * 4));
@@ -405,17 +487,42 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
             goto done;
         }
     }
+    HX_CHECK(raise_smem_limit((const void *)k_hx_pathkeys, smem));
+    HX_CHECK(raise_smem_limit((const void *)k_hx_edges, smem));
+    HX_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_p, k_hx_pathkeys, kBlock, smem));
+    HX_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_e, k_hx_edges, kBlock, smem));
+    if (occ_p < 1 || occ_e < 1) {
+        set_last_error("htd_hindex_decompose: no resident block fits");
+        st = HTD_ECUDA;
+        goto done;
+    }
+    grid_p = H->num_sms * std::min(occ_p, 8);
+    grid_e = H->num_sms * std::min(occ_e, 8);
+    // member lists from the balls the h-support pass left in the handle's scratch
+    HX_CHECK(cudaMalloc(&off, (n + 1) * 8));
+    HX_CHECK(scan_exclusive<int32_t, int64_t>(w.ball_size, off, n, w.scan_tmp, s, &launches));
+    hsizes.resize(n);
+    HX_CHECK(cudaMemcpyAsync(&total, off + n, 8, cudaMemcpyDeviceToHost, s));
+    HX_CHECK(cudaMemcpyAsync(hsizes.data(), w.ball_size, n * 4, cudaMemcpyDeviceToHost, s));
+    HX_CHECK(cudaStreamSynchronize(s));
+    for (int64_t x = 0; x < n; x++) maxb = std::max<int64_t>(maxb, hsizes[x]);
+    loc.ball_entries = total;
+    HX_CHECK(cudaMalloc(&members, std::max<int64_t>(total, 1) * 4));
+    HX_CHECK(cudaMalloc(&P, std::max<int64_t>(total, 1) * 4));
+    k_hx_members<<<(unsigned)std::min<int64_t>(n, H->num_sms * 8), kBlock, 0, s>>>((int32_t)n, w.W, w.pool, w.ball_off,
+                                                                         w.ball_nw, off, members);
+    launches++;
+    HX_CHECK(cudaGetLastError());
     {
-        const int grid_p = H->num_sms * 4;
-        const int grid_e = H->num_sms * 8;
-        HX_CHECK(cudaMalloc(&prev, (int64_t)grid_p * std::max<int64_t>(maxb, 1) * 4));
-        HX_CHECK(cudaMalloc(&vals, (int64_t)grid_e * (kBlock / 32) * std::max<int64_t>(maxd, 1) * 4));
-        HX_CHECK(cudaMalloc(&dchanged, 8));
-        HX_CHECK(cudaMallocHost(&hchanged, 8));
+        // one block per vertex at most; prev is only read from the third round on
+        grid_p = (int)std::min<int64_t>(grid_p, n);
+        grid_e = (int)std::min<int64_t>(grid_e, n);
+        HX_CHECK(cudaMalloc(&prev, (h >= 3 ? (int64_t)grid_p : 1) * std::max<int64_t>(maxb, 1) * 4));
+        HX_CHECK(cudaMalloc(&vals, (int64_t)grid_e * (kBlock / 32) * std::max<int64_t>(maxb, 1) * 4));
+        HX_CHECK(cudaMalloc(&dctr, sizeof(Counters)));
+        HX_CHECK(cudaMallocHost(&hctr, sizeof(Counters)));
         HX_CHECK(cudaMalloc(&mark, n * 4));
         HX_CHECK(cudaMalloc(&vlist, n * 4));
-        HX_CHECK(cudaMalloc(&dcount, 4));
-        HX_CHECK(cudaMallocHost(&hcount, 4));
         HX_CHECK(cudaMemsetAsync(mark, 0xff, n * 4, s));
         if (prune) {
             HX_CHECK(cudaMalloc(&kold, m * 4));
@@ -423,10 +530,24 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
             HX_CHECK(cudaMalloc(&lo, n * 4));
             HX_CHECK(cudaMalloc(&hi2, n * 4));
             HX_CHECK(cudaMalloc(&lo2, n * 4));
-            HX_CHECK(cudaMalloc(&elist, m * 4));
-            HX_CHECK(cudaMalloc(&decount, 4));
-            HX_CHECK(cudaMallocHost(&hecount, 4));
+            HX_CHECK(cudaMalloc(&emark, m * 4));
+            HX_CHECK(cudaMemsetAsync(emark, 0xff, m * 4, s));
         }
+        const int64_t prev_stride = h >= 3 ? maxb : 0;
+        auto pathkeys = [&](const int32_t *list, int32_t count, const int32_t *dcount) {
+            k_hx_pathkeys<<<grid_p, kBlock, smem, s>>>(list, count, dcount, h, g.row_ptr, g.col, g.slot_eid, key, off,
+                                                       members, P, prev, prev_stride, words, kPathCap);
+            launches++;
+        };
+        // dctr->items and ->queue are zero
+        auto edges = [&](const int32_t *list, int32_t count, const int32_t *dcount, int64_t e0, int64_t e1,
+                         const int32_t *marks, int32_t stamp, int32_t *out) {
+            k_hx_items<<<H->num_sms * 2, kBlock, 0, s>>>(list, count, dcount, g.row_ptr, w.items, &dctr->items);
+            k_hx_edges<<<grid_e, kBlock, smem, s>>>(w.items, &dctr->items, &dctr->queue, e0, e1, marks, stamp,
+                                                    g.row_ptr, g.col, g.slot_eid, off, members, P, key, out, vals,
+                                                    maxb, &dctr->changed, words, kPathCap);
+            launches += 2;
+        };
         // every order before the fixed point lowers at least one key (Theorem 3): the sum
         // of H^(0) plus one orders always suffice
         std::vector<int32_t> k0(m);
@@ -439,13 +560,12 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
         int32_t it = 0;
         bool converged = false;
         while (!converged && (max_iter < 0 || it < max_iter) && it < cap) {
-            HX_CHECK(cudaMemsetAsync(dchanged, 0, 8, s));
-            if (S == 1 && prune && it > 0) {
+            HX_CHECK(cudaMemsetAsync(dctr, 0, sizeof(Counters), s));
+            const bool pruned = S == 1 && prune && it > 0;
+            if (pruned) {
                 // Lemma 4: list the edges that can still fall (key = H^(n-1), kold = H^(n-2))
                 HX_CHECK(cudaMemsetAsync(hi, 0xff, n * 4, s));
                 HX_CHECK(cudaMemsetAsync(lo, 0x7f, n * 4, s));
-                HX_CHECK(cudaMemsetAsync(dcount, 0, 4, s));
-                HX_CHECK(cudaMemsetAsync(decount, 0, 4, s));
                 k_hx_fall<<<H->num_sms * 4, kBlock, 0, s>>>(m, g.eu, g.ev, kold, key, hi, lo);
                 launches++;
                 for (int r = 1; r < h; r++) {
@@ -454,56 +574,46 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
                     std::swap(hi, hi2);
                     std::swap(lo, lo2);
                 }
-                k_hx_select<<<H->num_sms * 4, kBlock, 0, s>>>(m, g.eu, g.ev, key, hi, lo, key2, elist, decount,
-                                                             stamp++, mark, vlist, dcount);
+                k_hx_select<<<H->num_sms * 4, kBlock, 0, s>>>(m, g.eu, g.ev, key, hi, lo, key2, emark, &dctr->edges,
+                                                             stamp, mark, vlist, &dctr->vertices);
                 launches++;
-                HX_CHECK(cudaMemcpyAsync(hcount, dcount, 4, cudaMemcpyDeviceToHost, s));
-                HX_CHECK(cudaMemcpyAsync(hecount, decount, 4, cudaMemcpyDeviceToHost, s));
-                HX_CHECK(cudaStreamSynchronize(s));
-                if (*hecount > 0) {
-                    k_hx_pathkeys<<<grid_p, kBlock, 0, s>>>(vlist, *hcount, h, g.row_ptr, g.col, g.slot_eid, key,
-                                                            off, members, P, prev, maxb);
-                    k_hx_edges<<<grid_e, kBlock, 0, s>>>(0, *hecount, elist, g.eu, g.ev, off, members, P, key,
-                                                         key2, vals, maxd, dchanged);
-                    launches += 2;
-                }
-                loc.edge_evals += *hecount;
-                loc.vertex_evals += *hcount;
-                // H^(n-2) <- H^(n-1) <- H^(n)
-                std::swap(kold, key);
-                std::swap(key, key2);
+                pathkeys(vlist, 0, &dctr->vertices);
+                edges(vlist, 0, &dctr->vertices, 0, m, emark, stamp, key2);
+                stamp++;
             } else if (S == 1) {
-                k_hx_pathkeys<<<grid_p, kBlock, 0, s>>>(nullptr, (int32_t)n, h, g.row_ptr, g.col, g.slot_eid,
-                                                        key, off, members, P, prev, maxb);
-                k_hx_edges<<<grid_e, kBlock, 0, s>>>(0, m, nullptr, g.eu, g.ev, off, members, P, key, key2, vals,
-                                                     maxd, dchanged);
-                launches += 2;
+                pathkeys(nullptr, (int32_t)n, nullptr);
+                edges(nullptr, (int32_t)n, nullptr, 0, m, nullptr, 0, key2);
                 loc.edge_evals += m;
                 loc.vertex_evals += n;
-                if (prune) std::swap(kold, key);  // with pruning: H^(n-2) <- H^(n-1) <- H^(n)
-                std::swap(key, key2);
             } else {
                 for (int j = 0; j < S; j++) {
                     const int64_t e0 = m * j / S, e1 = m * (j + 1) / S;
                     if (e1 <= e0) continue;
-                    HX_CHECK(cudaMemsetAsync(dcount, 0, 4, s));
-                    k_hx_touch<<<H->num_sms * 2, kBlock, 0, s>>>(e0, e1, g.eu, g.ev, stamp++, mark, vlist, dcount);
-                    HX_CHECK(cudaMemcpyAsync(hcount, dcount, 4, cudaMemcpyDeviceToHost, s));
+                    HX_CHECK(cudaMemsetAsync(&dctr->vertices, 0, sizeof(Counters) - sizeof(dctr->changed), s));
+                    k_hx_touch<<<H->num_sms * 2, kBlock, 0, s>>>(e0, e1, g.eu, g.ev, stamp++, mark, vlist,
+                                                                &dctr->vertices);
+                    launches++;
+                    HX_CHECK(cudaMemcpyAsync(hctr, dctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
                     HX_CHECK(cudaStreamSynchronize(s));
-                    k_hx_pathkeys<<<grid_p, kBlock, 0, s>>>(vlist, *hcount, h, g.row_ptr, g.col, g.slot_eid, key,
-                                                            off, members, P, prev, maxb);
-                    k_hx_edges<<<grid_e, kBlock, 0, s>>>(e0, e1, nullptr, g.eu, g.ev, off, members, P, key, key,
-                                                         vals, maxd, dchanged);
-                    launches += 3;
+                    pathkeys(vlist, hctr->vertices, nullptr);
+                    edges(vlist, hctr->vertices, nullptr, e0, e1, nullptr, 0, key);
                     loc.edge_evals += e1 - e0;
-                    loc.vertex_evals += *hcount;
+                    loc.vertex_evals += hctr->vertices;
                 }
             }
             HX_CHECK(cudaGetLastError());
-            HX_CHECK(cudaMemcpyAsync(hchanged, dchanged, 8, cudaMemcpyDeviceToHost, s));
+            HX_CHECK(cudaMemcpyAsync(hctr, dctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
             HX_CHECK(cudaStreamSynchronize(s));
+            if (pruned) {
+                loc.edge_evals += hctr->edges;
+                loc.vertex_evals += hctr->vertices;
+            }
+            if (S == 1) {
+                if (prune) std::swap(kold, key);  // H^(n-2) <- H^(n-1) <- H^(n)
+                std::swap(key, key2);
+            }
             it++;
-            if (*hchanged == 0) converged = true;
+            if (hctr->changed == 0) converged = true;
         }
         loc.iterations = it;
         loc.converged = converged ? 1 : 0;
@@ -526,30 +636,23 @@ finish:
     if (stats) *stats = loc;
     add_launches(launches);
 done:
-    cudaFree(sizes);
     cudaFree(off);
-    cudaFree(lists);
-    cudaFree(tmp);
     cudaFree(members);
     cudaFree(P);
     cudaFree(prev);
     cudaFree(vals);
     cudaFree(key);
     cudaFree(key2);
-    cudaFree(dchanged);
     cudaFree(mark);
     cudaFree(vlist);
-    cudaFree(dcount);
     cudaFree(kold);
     cudaFree(hi);
     cudaFree(lo);
     cudaFree(hi2);
     cudaFree(lo2);
-    cudaFree(elist);
-    cudaFree(decount);
-    if (hecount) cudaFreeHost(hecount);
-    if (hchanged) cudaFreeHost(hchanged);
-    if (hcount) cudaFreeHost(hcount);
+    cudaFree(emark);
+    cudaFree(dctr);
+    if (hctr) cudaFreeHost(hctr);
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
     return st;
