@@ -304,7 +304,7 @@ extern "C" htd_status htd_truss_decompose_batched(
                 out_offsets[up.ids[j]] = out_pos + b[j];
                 out_m[up.ids[j]] = t[j] - b[j];
                 if (t[j] > b[j])
-                    descs.push_back(BlockGraphDescHost{gdv->row_ptr, gdv->col, gdv->slot_eid, gdv->eu, gdv->ev,
+                    descs.push_back(BlockGraphDescHost{gdv->row_ptr, gdv->col, gdv->eu, gdv->ev, gdv->slot_lo, gdv->slot_hi,
                                                        truss_dev + out_pos + b[j], b[j], t[j] - b[j],
                                                        up.mem[j].voff, up.mem[j].n, up.h});
             }

@@ -176,7 +176,7 @@ void set_shared_device(htd_graph *g);
 // pointers into its union's CSR, its vertices [v0, v0 + L) and edges [e0, e0 + m) there,
 // and where its t(e,h) go.
 struct BlockGraphDescHost {
-    const int32_t *row_ptr, *col, *slot_eid, *eu, *ev;
+    const int32_t *row_ptr, *col, *eu, *ev, *slot_lo, *slot_hi;
     int32_t *out;
     int64_t e0, m;
     int32_t v0, L, h;
