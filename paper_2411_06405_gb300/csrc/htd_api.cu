@@ -28,6 +28,66 @@ constexpr int kSlotsPerGraph = 4;    // incremental slots
 
 void set_last_error(const std::string &msg) { g_last_error = msg; }
 
+namespace {
+constexpr int kMaxDevices = 64;
+constexpr uint64_t kPoolKeeps = (uint64_t)2 << 30;
+constexpr size_t kStatusKeeps = 32;
+std::mutex g_mem_mutex;
+cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
+std::vector<DevStatus *> g_status;
+}  // namespace
+
+cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mutex);
+        if (!g_pool[dev]) {
+            cudaMemPoolProps props;
+            std::memset(&props, 0, sizeof(props));
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            e = cudaMemPoolCreate(&pool, &props);
+            uint64_t keeps = kPoolKeeps;
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keeps);
+            if (e != cudaSuccess) return e;
+            g_pool[dev] = pool;
+        }
+        pool = g_pool[dev];
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+DevStatus *take_status_host() {
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mutex);
+        if (!g_status.empty()) {
+            DevStatus *p = g_status.back();
+            g_status.pop_back();
+            return p;
+        }
+    }
+    DevStatus *p = nullptr;
+    if (cudaMallocHost(reinterpret_cast<void **>(&p), sizeof(DevStatus)) != cudaSuccess) return nullptr;
+    return p;
+}
+
+void give_status_host(DevStatus *p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mutex);
+        if (g_status.size() < kStatusKeeps) {
+            g_status.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
 cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     static std::mutex mu;
     static std::map<std::pair<int, const void *>, size_t> limit;
@@ -131,8 +191,10 @@ void htd_graph_free(htd_graph *g) {
     cudaSetDevice(H->g.device);
     if (H->pstream) cudaStreamSynchronize(H->pstream);
     destroy_graph(H);
-    htd::free_work(&H->w);
-    htd::free_graph_dev(&H->g);
+    htd::free_work(H);
+    htd::free_graph_dev(&H->g, H->pstream);
+    // what the pool does not keep goes back to the device now
+    if (H->pstream) cudaStreamSynchronize(H->pstream);
     for (cudaEvent_t e : H->round_events) cudaEventDestroy(e);
     H->round_events.clear();
     if (H->ev_in) cudaEventDestroy(H->ev_in);
@@ -167,8 +229,8 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
     int32_t *dsrc = nullptr, *ddst = nullptr;
     int64_t launches = 0;
     auto fail = [&](htd_status s) {
-        if (dsrc) cudaFree(dsrc);
-        if (ddst) cudaFree(ddst);
+        htd::dev_free(dsrc, H->pstream);
+        htd::dev_free(ddst, H->pstream);
         htd_graph_free(G);
         return s;
     };
@@ -188,8 +250,8 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
     if (st != HTD_OK) return fail(st);
     const int32_t *s_dev = src, *d_dev = dst;
     if (!inputs_on_device && m_in > 0) {
-        cudaError_t e = cudaMalloc(&dsrc, m_in * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&ddst, m_in * sizeof(int32_t));
+        cudaError_t e = htd::dev_alloc(&dsrc, m_in, H->pstream);
+        if (e == cudaSuccess) e = htd::dev_alloc(&ddst, m_in, H->pstream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dsrc, src, m_in * sizeof(int32_t), cudaMemcpyHostToDevice, H->pstream);
         if (e == cudaSuccess)
@@ -206,8 +268,8 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
     if (st != HTD_OK) return fail(st);
     st = end_call(H, user);
     if (st != HTD_OK) return fail(st);
-    if (dsrc) cudaFree(dsrc);
-    if (ddst) cudaFree(ddst);
+    htd::dev_free(dsrc, H->pstream);
+    htd::dev_free(ddst, H->pstream);
     *out = G;
     return HTD_OK;
 }
@@ -292,7 +354,7 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     htd::PeelWork &w = H->w;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
     const bool timing = (flags & HTD_OPT_TIMING) != 0;
-    const bool use_graph = (flags & HTD_OPT_NO_GRAPH) == 0;
+    const bool graphs_wanted = (flags & HTD_OPT_NO_GRAPH) == 0;
     htd_stats local;
     std::memset(&local, 0, sizeof(local));
     local.h = h;
@@ -395,6 +457,9 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         // external event record at every phase boundary runs every kTimedEvery-th batch (the
         // events would otherwise slow every round); per-launch averages come from those.
         constexpr int kTimedEvery = 16;
+        // slots that hold many rounds are launched directly: capturing and instantiating a graph
+        // costs more than the few slots of a peel save
+        const bool use_graph = graphs_wanted && !w.twin;
         const bool by_events = timing && !incremental;  // incremental rounds time themselves
         if (by_events && H->round_events.empty()) {
             H->round_events.resize(htd::kRoundEvents * R, nullptr);
@@ -446,7 +511,7 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         // continued incremental rounds handle at least one new lost pair per slot, and a
         // pair is lost at most once (sum of ball sizes / 2 pairs in all)
         const int64_t batch_cap =
-            (H->g.m + (incremental ? w.status_host->st_ball_total / 2 + 1 : 0)) / R + 3;
+            (H->g.m + (incremental ? w.status_host->st_ball_total / 2 + 1 : 0)) / (w.twin ? 1 : R) + 3;
         int64_t batches = 0;
         bool timing_ok = by_events;
         while (w.status_host->alive > 0) {
@@ -461,7 +526,9 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
                 API_CHECK(cudaGraphLaunch(second ? H->graph_exec_timed : H->graph_exec, H->pstream));
                 launches += H->graph_launches;
             } else {
-                for (int r = 0; r < R; r++) {
+                // the first slot often ends a small peel: one, then more at a time
+                const int slots = w.twin ? (int)std::min<int64_t>(R, batches) : R;
+                for (int r = 0; r < slots; r++) {
                     API_TRY(htd::enqueue_round(H, H->pstream, &launches,
                                                timed ? &H->round_events[htd::kRoundEvents * r] : nullptr,
                                                timing));
@@ -606,7 +673,7 @@ htd_status htd_truss_decompose_host(int32_t n, const int32_t *src_host, const in
     int32_t *truss_dev = nullptr;
     htd_status st = HTD_OK;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
-    if (cudaMalloc(&truss_dev, (m > 0 ? m : 1) * 4) != cudaSuccess) {
+    if (htd::dev_alloc(&truss_dev, m, user) != cudaSuccess) {
         set_last_error("htd_truss_decompose_host: output allocation failed");
         htd_graph_free(g);
         return HTD_ENOMEM;
@@ -623,7 +690,7 @@ htd_status htd_truss_decompose_host(int32_t n, const int32_t *src_host, const in
         }
     }
     if (st == HTD_OK) *m_out = m;
-    cudaFree(truss_dev);
+    htd::dev_free(truss_dev, user);
     htd_graph_free(g);
     return st;
 }

@@ -168,13 +168,21 @@ struct UnionScratch {
     Member *mem = nullptr;
     int32_t *usrc = nullptr, *udst = nullptr;
     int *bad = nullptr;
+    cudaStream_t s = nullptr;  // the stream its buffers are ordered on
     htd_graph *g = nullptr;
+    // the gathered pairs, which only the CSR builder reads
+    void drop_pairs() {
+        dev_free(mem, s);
+        dev_free(usrc, s);
+        dev_free(udst, s);
+        dev_free(bad, s);
+        mem = nullptr;
+        usrc = udst = nullptr;
+        bad = nullptr;
+    }
     ~UnionScratch() {
         if (g) htd_graph_free(g);
-        cudaFree(mem);
-        cudaFree(usrc);
-        cudaFree(udst);
-        cudaFree(bad);
+        drop_pairs();
     }
 };
 
@@ -194,10 +202,11 @@ htd_status build_union(const UnionPlan &up, const int32_t *src_dev, const int32_
     t->assign(mem.size(), 0);
     *mu_out = 0;
     if (pairs == 0) return HTD_OK;
-    cudaError_t e = cudaMalloc(&U->mem, mem.size() * sizeof(Member));
-    if (e == cudaSuccess) e = cudaMalloc(&U->usrc, pairs * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&U->udst, pairs * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&U->bad, sizeof(int));
+    U->s = s;
+    cudaError_t e = dev_alloc(&U->mem, (int64_t)mem.size(), s);
+    if (e == cudaSuccess) e = dev_alloc(&U->usrc, pairs, s);
+    if (e == cudaSuccess) e = dev_alloc(&U->udst, pairs, s);
+    if (e == cudaSuccess) e = dev_alloc(&U->bad, 1, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(U->mem, mem.data(), mem.size() * sizeof(Member), cudaMemcpyHostToDevice, s);
     const int none = INT32_MAX;
@@ -223,6 +232,7 @@ htd_status build_union(const UnionPlan &up, const int32_t *src_dev, const int32_
     }
     htd_status st = htd_build_csr((int32_t)nu, U->usrc, U->udst, pairs, 1, stream, &U->g);
     if (st != HTD_OK) return st;
+    U->drop_pairs();
     int32_t nn = 0;
     int64_t mu = 0;
     htd_graph_info(U->g, &nn, &mu);

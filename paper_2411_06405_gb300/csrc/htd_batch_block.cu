@@ -304,9 +304,9 @@ htd_status batch_block_run(const std::vector<BlockGraphDescHost> &graphs, cudaSt
     unsigned char *scratch = nullptr;
     unsigned long long *d_ctr = nullptr;  // rounds, then the queue head
     htd_status st = HTD_OK;
-    if (stride > 0) e = cudaMalloc(&scratch, grid * stride);
-    if (e == cudaSuccess) e = cudaMalloc(&d_gd, gd.size() * sizeof(BlockGraphDesc));
-    if (e == cudaSuccess) e = cudaMalloc(&d_ctr, 16);
+    if (stride > 0) e = dev_alloc(&scratch, grid * stride, s);
+    if (e == cudaSuccess) e = dev_alloc(&d_gd, (int64_t)gd.size(), s);
+    if (e == cudaSuccess) e = dev_alloc(&d_ctr, 2, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_gd, gd.data(), gd.size() * sizeof(BlockGraphDesc), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_ctr, 0, 16, s);
@@ -324,9 +324,9 @@ htd_status batch_block_run(const std::vector<BlockGraphDescHost> &graphs, cudaSt
         st = e == cudaErrorMemoryAllocation ? HTD_ENOMEM : HTD_ECUDA;
     }
     if (rounds_out) *rounds_out = (int64_t)hr;
-    cudaFree(scratch);
-    cudaFree(d_gd);
-    cudaFree(d_ctr);
+    dev_free(scratch, s);
+    dev_free(d_gd, s);
+    dev_free(d_ctr, s);
     return st;
 }
 

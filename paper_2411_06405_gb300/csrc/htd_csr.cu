@@ -262,14 +262,10 @@ int grid_for(int64_t work, int per_block, int cap) {
 
 }  // namespace
 
-void free_graph_dev(GraphDev *g) {
-    cudaFree(g->row_ptr);
-    cudaFree(g->col);
-    cudaFree(g->slot_eid);
-    cudaFree(g->eu);
-    cudaFree(g->ev);
-    cudaFree(g->slot_lo);
-    cudaFree(g->slot_hi);
+void free_graph_dev(GraphDev *g, cudaStream_t s) {
+    for (void *p : {(void *)g->row_ptr, (void *)g->col, (void *)g->slot_eid, (void *)g->eu, (void *)g->ev,
+                    (void *)g->slot_lo, (void *)g->slot_hi})
+        dev_free(p, s);
     *g = GraphDev{};
 }
 
@@ -305,18 +301,18 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     HTD_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     g.device = dev;
     g.n = n;
-    HTD_TRY(cudaMallocAsync(&deg, nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&off, (nn + 1) * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&fill, nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&colraw, (raw_slots > 0 ? raw_slots : 1) * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&deg_new, nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&lists, 2 * nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&counters, 6 * sizeof(int32_t), s));
+    HTD_TRY(dev_alloc(&deg, nn, s));
+    HTD_TRY(dev_alloc(&off, (nn + 1), s));
+    HTD_TRY(dev_alloc(&fill, nn, s));
+    HTD_TRY(dev_alloc(&colraw, raw_slots, s));
+    HTD_TRY(dev_alloc(&deg_new, nn, s));
+    HTD_TRY(dev_alloc(&lists, 2 * nn, s));
+    HTD_TRY(dev_alloc(&counters, 6, s));
     deg2 = reinterpret_cast<unsigned long long *>(counters + 4);
-    HTD_TRY(cudaMallocAsync(&fwd, nn * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&fwd_off, (nn + 1) * sizeof(int32_t), s));
-    HTD_TRY(cudaMallocAsync(&tmp, scan_temp_bytes(nn + raw_slots), s));
-    HTD_TRY(cudaMallocAsync(&g.row_ptr, (nn + 1) * sizeof(int32_t), s));
+    HTD_TRY(dev_alloc(&fwd, nn, s));
+    HTD_TRY(dev_alloc(&fwd_off, (nn + 1), s));
+    HTD_TRY(dev_alloc_bytes(&tmp, scan_temp_bytes(nn + raw_slots), s));
+    HTD_TRY(dev_alloc(&g.row_ptr, (nn + 1), s));
     HTD_TRY(cudaMemsetAsync(deg, 0, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMemsetAsync(fill, 0, nn * sizeof(int32_t), s));
     HTD_TRY(cudaMemsetAsync(deg_new, 0, nn * sizeof(int32_t), s));
@@ -358,12 +354,12 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     g.m = two_m / 2;
     {
         int64_t mm = g.m > 0 ? g.m : 1;
-        HTD_TRY(cudaMallocAsync(&g.col, 2 * mm * sizeof(int32_t), s));
-        HTD_TRY(cudaMallocAsync(&g.slot_eid, 2 * mm * sizeof(int32_t), s));
-        HTD_TRY(cudaMallocAsync(&g.eu, mm * sizeof(int32_t), s));
-        HTD_TRY(cudaMallocAsync(&g.ev, mm * sizeof(int32_t), s));
-        HTD_TRY(cudaMallocAsync(&g.slot_lo, mm * sizeof(int32_t), s));
-        HTD_TRY(cudaMallocAsync(&g.slot_hi, mm * sizeof(int32_t), s));
+        HTD_TRY(dev_alloc(&g.col, 2 * mm, s));
+        HTD_TRY(dev_alloc(&g.slot_eid, 2 * mm, s));
+        HTD_TRY(dev_alloc(&g.eu, mm, s));
+        HTD_TRY(dev_alloc(&g.ev, mm, s));
+        HTD_TRY(dev_alloc(&g.slot_lo, mm, s));
+        HTD_TRY(dev_alloc(&g.slot_hi, mm, s));
     }
     if (n > 0) {
         int gw = grid_for((int64_t)n * 32, kBlock, nsm * 16);
@@ -379,19 +375,19 @@ htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, i
     HTD_TRY(cudaStreamSynchronize(s));
 
 done:
-    cudaFreeAsync(deg, s);
-    cudaFreeAsync(off, s);
-    cudaFreeAsync(fill, s);
-    cudaFreeAsync(colraw, s);
-    cudaFreeAsync(deg_new, s);
-    cudaFreeAsync(lists, s);
-    cudaFreeAsync(counters, s);
-    cudaFreeAsync(fwd, s);
-    cudaFreeAsync(fwd_off, s);
-    cudaFreeAsync(tmp, s);
+    dev_free(deg, s);
+    dev_free(off, s);
+    dev_free(fill, s);
+    dev_free(colraw, s);
+    dev_free(deg_new, s);
+    dev_free(lists, s);
+    dev_free(counters, s);
+    dev_free(fwd, s);
+    dev_free(fwd_off, s);
+    dev_free(tmp, s);
     if (st != HTD_OK) {
         cudaStreamSynchronize(s);
-        free_graph_dev(&g);
+        free_graph_dev(&g, s);
         return st;
     }
     *out = g;

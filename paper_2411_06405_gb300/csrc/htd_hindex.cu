@@ -455,6 +455,7 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
         int32_t vertices, edges;
         int32_t items, queue;  // of the order's edge kernel
     };
+    static_assert(sizeof(Counters) <= sizeof(DevStatus), "read through the handle's pinned status block");
     Counters *dctr = nullptr, *hctr = nullptr;
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     htd_hindex_stats loc;
@@ -479,14 +480,15 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
     HX_CHECK(cudaEventRecord(t0, s));
     {
         // H^(0) = sup(e,h), the h-support of every edge (the initial step of Algorithm 2)
-        HX_CHECK(cudaMalloc(&key, m * 4));
-        HX_CHECK(cudaMalloc(&key2, m * 4));
+        HX_CHECK(dev_alloc(&key, m, s));
+        HX_CHECK(dev_alloc(&key2, m, s));
         htd_status hs = htd_h_support(G, h, key, s);
         if (hs != HTD_OK) {
             st = hs;
             goto done;
         }
     }
+    hctr = reinterpret_cast<Counters *>(w.status_host);  // the h-support pass is done with it
     HX_CHECK(raise_smem_limit((const void *)k_hx_pathkeys, smem));
     HX_CHECK(raise_smem_limit((const void *)k_hx_edges, smem));
     HX_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_p, k_hx_pathkeys, kBlock, smem));
@@ -499,7 +501,7 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
     grid_p = H->num_sms * std::min(occ_p, 8);
     grid_e = H->num_sms * std::min(occ_e, 8);
     // member lists from the balls the h-support pass left in the handle's scratch
-    HX_CHECK(cudaMalloc(&off, (n + 1) * 8));
+    HX_CHECK(dev_alloc(&off, n + 1, s));
     HX_CHECK(scan_exclusive<int32_t, int64_t>(w.ball_size, off, n, w.scan_tmp, s, &launches));
     hsizes.resize(n);
     HX_CHECK(cudaMemcpyAsync(&total, off + n, 8, cudaMemcpyDeviceToHost, s));
@@ -507,8 +509,8 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
     HX_CHECK(cudaStreamSynchronize(s));
     for (int64_t x = 0; x < n; x++) maxb = std::max<int64_t>(maxb, hsizes[x]);
     loc.ball_entries = total;
-    HX_CHECK(cudaMalloc(&members, std::max<int64_t>(total, 1) * 4));
-    HX_CHECK(cudaMalloc(&P, std::max<int64_t>(total, 1) * 4));
+    HX_CHECK(dev_alloc(&members, total, s));
+    HX_CHECK(dev_alloc(&P, total, s));
     k_hx_members<<<(unsigned)std::min<int64_t>(n, H->num_sms * 8), kBlock, 0, s>>>((int32_t)n, w.W, w.pool, w.ball_off,
                                                                          w.ball_nw, off, members);
     launches++;
@@ -517,20 +519,19 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
         // one block per vertex at most; prev is only read from the third round on
         grid_p = (int)std::min<int64_t>(grid_p, n);
         grid_e = (int)std::min<int64_t>(grid_e, n);
-        HX_CHECK(cudaMalloc(&prev, (h >= 3 ? (int64_t)grid_p : 1) * std::max<int64_t>(maxb, 1) * 4));
-        HX_CHECK(cudaMalloc(&vals, (int64_t)grid_e * (kBlock / 32) * std::max<int64_t>(maxb, 1) * 4));
-        HX_CHECK(cudaMalloc(&dctr, sizeof(Counters)));
-        HX_CHECK(cudaMallocHost(&hctr, sizeof(Counters)));
-        HX_CHECK(cudaMalloc(&mark, n * 4));
-        HX_CHECK(cudaMalloc(&vlist, n * 4));
+        HX_CHECK(dev_alloc(&prev, (h >= 3 ? (int64_t)grid_p : 1) * std::max<int64_t>(maxb, 1), s));
+        HX_CHECK(dev_alloc(&vals, (int64_t)grid_e * (kBlock / 32) * std::max<int64_t>(maxb, 1), s));
+        HX_CHECK(dev_alloc(&dctr, 1, s));
+        HX_CHECK(dev_alloc(&mark, n, s));
+        HX_CHECK(dev_alloc(&vlist, n, s));
         HX_CHECK(cudaMemsetAsync(mark, 0xff, n * 4, s));
         if (prune) {
-            HX_CHECK(cudaMalloc(&kold, m * 4));
-            HX_CHECK(cudaMalloc(&hi, n * 4));
-            HX_CHECK(cudaMalloc(&lo, n * 4));
-            HX_CHECK(cudaMalloc(&hi2, n * 4));
-            HX_CHECK(cudaMalloc(&lo2, n * 4));
-            HX_CHECK(cudaMalloc(&emark, m * 4));
+            HX_CHECK(dev_alloc(&kold, m, s));
+            HX_CHECK(dev_alloc(&hi, n, s));
+            HX_CHECK(dev_alloc(&lo, n, s));
+            HX_CHECK(dev_alloc(&hi2, n, s));
+            HX_CHECK(dev_alloc(&lo2, n, s));
+            HX_CHECK(dev_alloc(&emark, m, s));
             HX_CHECK(cudaMemsetAsync(emark, 0xff, m * 4, s));
         }
         const int64_t prev_stride = h >= 3 ? maxb : 0;
@@ -636,23 +637,22 @@ finish:
     if (stats) *stats = loc;
     add_launches(launches);
 done:
-    cudaFree(off);
-    cudaFree(members);
-    cudaFree(P);
-    cudaFree(prev);
-    cudaFree(vals);
-    cudaFree(key);
-    cudaFree(key2);
-    cudaFree(mark);
-    cudaFree(vlist);
-    cudaFree(kold);
-    cudaFree(hi);
-    cudaFree(lo);
-    cudaFree(hi2);
-    cudaFree(lo2);
-    cudaFree(emark);
-    cudaFree(dctr);
-    if (hctr) cudaFreeHost(hctr);
+    dev_free(off, s);
+    dev_free(members, s);
+    dev_free(P, s);
+    dev_free(prev, s);
+    dev_free(vals, s);
+    dev_free(key, s);
+    dev_free(key2, s);
+    dev_free(mark, s);
+    dev_free(vlist, s);
+    dev_free(kold, s);
+    dev_free(hi, s);
+    dev_free(lo, s);
+    dev_free(hi2, s);
+    dev_free(lo2, s);
+    dev_free(emark, s);
+    dev_free(dctr, s);
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
     return st;

@@ -60,8 +60,8 @@ struct PeelWork {
     bool lost_tiny = false;        // table forced to 128 slots (test option)
     int4 *lost = nullptr;          // (min, max, hash slot, 0) per lost pair
     int32_t *edge_touch = nullptr; // n: last round in which the vertex's ball lost a member
-    int32_t *hub_slot = nullptr;   // n: row of the vertex's alive-adjacency set, or -1
-    int32_t *hub_list = nullptr;   // nhub vertices with such a set (degree >= hub_min_deg)
+    int32_t *hub_slot = nullptr;   // n: row of the vertex's alive-adjacency set, or -1 (null: row x)
+    int32_t *hub_list = nullptr;   // nhub vertices with such a set (degree >= hub_min_deg; null: all)
     uint32_t *hub_bits = nullptr;  // nhub x Wpad words: alive neighbours as n-bit sets
     int32_t nhub = 0;
     uint32_t *or_rows = nullptr;   // h-support alone: adjacency sets of the high-degree vertices
@@ -132,6 +132,21 @@ struct Handle {
 };
 
 void set_last_error(const std::string &msg);
+// Device memory of graphs and scratch, ordered on `s`, from a pool of the library's own that
+// keeps at most 2 GiB of freed memory per device (a cudaMalloc and cudaFree for each of a
+// handle's fifty arrays took longer than a small decomposition, and every cudaFree waits for
+// the other streams' kernels).
+cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
+template <typename T>
+cudaError_t dev_alloc(T **p, int64_t count, cudaStream_t s) {
+    return dev_alloc_bytes(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T), s);
+}
+inline void dev_free(void *p, cudaStream_t s) {
+    if (p) cudaFreeAsync(p, s);
+}
+// Pinned status blocks, kept for the next handle (at most 32).
+DevStatus *take_status_host();
+void give_status_host(DevStatus *p);
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the current device.
 // The limit is a process-wide property of the function: it is only ever raised (under a
 // lock), so that a call for a small graph in one thread cannot lower it below what a
@@ -143,11 +158,11 @@ void add_launches(int64_t k);
 // CSR builder (htd_csr.cu).  src/dst are device pointers.
 htd_status build_csr_device(int32_t n, const int32_t *src, const int32_t *dst, int64_t m_in,
                             cudaStream_t s, GraphDev *out, int64_t *launches);
-void free_graph_dev(GraphDev *g);
+void free_graph_dev(GraphDev *g, cudaStream_t s);
 
 // Ball builder, h-support and peel rounds (htd_peel.cu).
 htd_status ensure_work(Handle *H, int32_t h, bool incremental, bool tiny_table = false);
-void free_work(PeelWork *w);
+void free_work(Handle *H);
 htd_status ensure_twin(Handle *H, int64_t budget);
 // support_only: h-support alone (no peel follows).
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,

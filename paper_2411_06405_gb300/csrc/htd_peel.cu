@@ -646,7 +646,7 @@ __global__ void k_make_records(int64_t m, const int32_t *__restrict__ row_ptr,
 }
 
 // Alive-adjacency n-bit sets of the high-degree vertices (all edges alive), block per hub.
-// count (nullable): the number of hubs, at most nhub of them, as a device value.
+// hub_list null: vertex x is hub x.  count (nullable): the number of hubs, at most nhub of them, as a device value.
 __global__ void __launch_bounds__(kBlock) k_hub_init(const int32_t *__restrict__ hub_list, int32_t nhub,
                                                     const int32_t *__restrict__ count,
                                                     const int32_t *__restrict__ row_ptr,
@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(kBlock) k_hub_init(const int32_t *__restrict__
         uint32_t *bits = hub_bits + (int64_t)hb * Wpad;
         for (int i = threadIdx.x; i < Wpad; i += kBlock) bits[i] = 0u;
         __syncthreads();
-        const int x = hub_list[hb];
+        const int x = hub_list ? hub_list[hb] : hb;
         for (int s = row_ptr[x] + threadIdx.x; s < row_ptr[x + 1]; s += kBlock) {
             const int y = col[s];
             atomicOr(bits + (y >> 5), 1u << (y & 31));
@@ -687,11 +687,6 @@ __global__ void k_init_deg(int32_t n, const int32_t *__restrict__ row_ptr,
             return (_e == cudaErrorMemoryAllocation) ? HTD_ENOMEM : HTD_ECUDA;       \
         }                                                                            \
     } while (0)
-
-template <typename T>
-cudaError_t alloc_n(T **p, int64_t count) {
-    return cudaMalloc(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T));
-}
 
 // Degree from which ORing a vertex's n-bit row beats expanding its slots: a row costs W/4
 // 16-byte loads, a slot about 60 cycles per 32 of them (R-MAT 18, W = 8,192: 512 gave 5.5 ms
@@ -757,56 +752,58 @@ HsupArgs hsup_args(Handle *H, int initial) {
 
 }  // namespace
 
-void free_work(PeelWork *w) {
-    cudaFree(w->pool);
-    cudaFree(w->ball_off);
-    cudaFree(w->ball_need);
-    cudaFree(w->ball_size);
-    cudaFree(w->ball_nw);
-    cudaFree(w->ball_meta);
-    cudaFree(w->col_live);
-    cudaFree(w->deg_alive);
-    cudaFree(w->sup);
-    cudaFree(w->truss);
-    cudaFree(w->stamp);
-    cudaFree(w->frontier);
-    cudaFree(w->cand_list);
-    cudaFree(w->cand_stamp);
-    cudaFree(w->changed_list);
-    cudaFree(w->changed_stamp);
-    cudaFree(w->items);
-    cudaFree(w->bfs_lists);
-    cudaFree(w->lost_keys);
-    cudaFree(w->lost);
-    cudaFree(w->edge_touch);
-    cudaFree(w->hub_slot);
-    cudaFree(w->hub_list);
-    cudaFree(w->hub_bits);
-    cudaFree(w->pitems);
-    cudaFree(w->uitems);
-    cudaFree(w->win);
-    cudaFree(w->erec);
-    cudaFree(w->srec);
-    cudaFree(w->scan_tmp);
-    cudaFree(w->pool2);
-    cudaFree(w->pool_new);
-    cudaFree(w->or_rows);
-    cudaFree(w->dense_off);
-    cudaFree(w->or_row_of);
-    cudaFree(w->or_list);
-    cudaFree(w->pool2_new);
-    cudaFree(w->ball_size2);
-    cudaFree(w->ball_nw2);
-    cudaFree(w->ball_meta2);
-    cudaFree(w->changed_list2);
-    cudaFree(w->changed_stamp2);
-    cudaFree(w->lost2_keys);
-    cudaFree(w->lost2);
-    cudaFree(w->c3items);
-    cudaFree(w->touch2);
-    cudaFree(w->status);
-    if (w->status_host) cudaFreeHost(w->status_host);
-    *w = PeelWork{};
+void free_work(Handle *H) {
+    PeelWork &w = H->w;
+    const cudaStream_t s = H->pstream;
+    dev_free(w.pool, s);
+    dev_free(w.ball_off, s);
+    dev_free(w.ball_need, s);
+    dev_free(w.ball_size, s);
+    dev_free(w.ball_nw, s);
+    dev_free(w.ball_meta, s);
+    dev_free(w.col_live, s);
+    dev_free(w.deg_alive, s);
+    dev_free(w.sup, s);
+    dev_free(w.truss, s);
+    dev_free(w.stamp, s);
+    dev_free(w.frontier, s);
+    dev_free(w.cand_list, s);
+    dev_free(w.cand_stamp, s);
+    dev_free(w.changed_list, s);
+    dev_free(w.changed_stamp, s);
+    dev_free(w.items, s);
+    dev_free(w.bfs_lists, s);
+    dev_free(w.lost_keys, s);
+    dev_free(w.lost, s);
+    dev_free(w.edge_touch, s);
+    dev_free(w.hub_slot, s);
+    dev_free(w.hub_list, s);
+    dev_free(w.hub_bits, s);
+    dev_free(w.pitems, s);
+    dev_free(w.uitems, s);
+    dev_free(w.win, s);
+    dev_free(w.erec, s);
+    dev_free(w.srec, s);
+    dev_free(w.scan_tmp, s);
+    dev_free(w.pool2, s);
+    dev_free(w.pool_new, s);
+    dev_free(w.or_rows, s);
+    dev_free(w.dense_off, s);
+    dev_free(w.or_row_of, s);
+    dev_free(w.or_list, s);
+    dev_free(w.pool2_new, s);
+    dev_free(w.ball_size2, s);
+    dev_free(w.ball_nw2, s);
+    dev_free(w.ball_meta2, s);
+    dev_free(w.changed_list2, s);
+    dev_free(w.changed_stamp2, s);
+    dev_free(w.lost2_keys, s);
+    dev_free(w.lost2, s);
+    dev_free(w.c3items, s);
+    dev_free(w.touch2, s);
+    dev_free(w.status, s);
+    give_status_host(w.status_host);
+    w = PeelWork{};
 }
 
 void drop_graphs(Handle *H);
@@ -830,7 +827,7 @@ htd_status ensure_work(Handle *H, int32_t h, bool incremental, bool tiny_table) 
     const htd_status st = ensure_work_impl(H, h, incremental, tiny_table);
     if (st != HTD_OK) {
         drop_graphs(H);
-        free_work(&H->w);
+        free_work(H);
     }
     return st;
 }
@@ -863,30 +860,34 @@ htd_status alloc_base(Handle *H, int32_t h) {
     w.grid_ball = H->num_sms * occ_ball;
     w.grid_hsup = H->num_sms * occ_hsup;
     w.grid_edges = H->num_sms * 4;
-    HTD_CHECK(alloc_n(&w.ball_off, n + 1));
-    HTD_CHECK(alloc_n(&w.ball_need, n));
-    HTD_CHECK(alloc_n(&w.ball_size, n));
-    HTD_CHECK(alloc_n(&w.ball_nw, n));
-    HTD_CHECK(alloc_n(&w.ball_meta, n));
-    HTD_CHECK(alloc_n(&w.col_live, 2 * m));
-    HTD_CHECK(alloc_n(&w.deg_alive, n));
-    HTD_CHECK(alloc_n(&w.sup, m));
-    HTD_CHECK(alloc_n(&w.truss, m));
-    HTD_CHECK(alloc_n(&w.stamp, m));
-    HTD_CHECK(alloc_n(&w.frontier, m));
-    HTD_CHECK(alloc_n(&w.cand_list, n));
-    HTD_CHECK(alloc_n(&w.cand_stamp, n));
-    HTD_CHECK(alloc_n(&w.changed_list, n));
-    HTD_CHECK(alloc_n(&w.changed_stamp, n));
+    HTD_CHECK(dev_alloc(&w.ball_off, n + 1, H->pstream));
+    HTD_CHECK(dev_alloc(&w.ball_need, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.ball_size, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.ball_nw, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.ball_meta, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.col_live, 2 * m, H->pstream));
+    HTD_CHECK(dev_alloc(&w.deg_alive, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.sup, m, H->pstream));
+    HTD_CHECK(dev_alloc(&w.truss, m, H->pstream));
+    HTD_CHECK(dev_alloc(&w.stamp, m, H->pstream));
+    HTD_CHECK(dev_alloc(&w.frontier, m, H->pstream));
+    HTD_CHECK(dev_alloc(&w.cand_list, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.cand_stamp, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.changed_list, n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.changed_stamp, n, H->pstream));
     w.items_cap = n + (2 * m + kItemChunk - 1) / kItemChunk + 1;
-    HTD_CHECK(alloc_n(&w.items, w.items_cap));
+    HTD_CHECK(dev_alloc(&w.items, w.items_cap, H->pstream));
     if (h >= 3) {
         w.bfs_list_len = n > 0 ? n : 1;
-        HTD_CHECK(alloc_n(&w.bfs_lists, (int64_t)w.grid_ball * 2 * w.bfs_list_len));
+        HTD_CHECK(dev_alloc(&w.bfs_lists, (int64_t)w.grid_ball * 2 * w.bfs_list_len, H->pstream));
     }
-    HTD_CHECK(cudaMalloc(&w.scan_tmp, scan_temp_bytes(n + 1)));
-    HTD_CHECK(alloc_n(&w.status, 1));
-    HTD_CHECK(cudaMallocHost(reinterpret_cast<void **>(&w.status_host), sizeof(DevStatus)));
+    HTD_CHECK(dev_alloc_bytes(&w.scan_tmp, scan_temp_bytes(n + 1), H->pstream));
+    HTD_CHECK(dev_alloc(&w.status, 1, H->pstream));
+    w.status_host = take_status_host();
+    if (!w.status_host) {
+        set_last_error("htd: pinned status block allocation failed");
+        return HTD_ENOMEM;
+    }
     return HTD_OK;
 }
 
@@ -904,7 +905,7 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
     if (w.status && !base_ready) {
         // the per-block BFS lists and the ball storage depend on h: rebuild everything
         drop_graphs(H);
-        free_work(&w);
+        free_work(H);
     }
     const int64_t n = g.n, m = g.m;
     if (!base_ready) {
@@ -922,72 +923,82 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
         w.lost_tiny = tiny_table;
         w.lost_cap = cap;
         w.lost_max = cap / 2;
-        HTD_CHECK(alloc_n(&w.lost_keys, cap));
-        HTD_CHECK(alloc_n(&w.lost, w.lost_max));
-        HTD_CHECK(alloc_n(&w.edge_touch, n));
+        HTD_CHECK(dev_alloc(&w.lost_keys, cap, H->pstream));
+        HTD_CHECK(dev_alloc(&w.lost, w.lost_max, H->pstream));
+        HTD_CHECK(dev_alloc(&w.edge_touch, n, H->pstream));
         // work items of the loss detection and of the support updates (per batch)
         // (sized with the graph: 2m adjacency slots)
         w.pitems_cap = std::min<int64_t>((int64_t)1 << 22, std::max<int64_t>(4096, 2 * m));
         // adjacency slots the updates of one batch may visit
         w.upd_budget = std::min<int64_t>((int64_t)1 << 30, std::max<int64_t>(1 << 16, 256 * m));
         w.uitems_cap = 2 * w.lost_max + w.upd_budget / 32 + 1024;
-        HTD_CHECK(alloc_n(&w.pitems, 2 * w.pitems_cap));
-        HTD_CHECK(alloc_n(&w.uitems, w.uitems_cap));
+        HTD_CHECK(dev_alloc(&w.pitems, 2 * w.pitems_cap, H->pstream));
+        HTD_CHECK(dev_alloc(&w.uitems, w.uitems_cap, H->pstream));
         w.win_cap = std::min<int64_t>(m, (int64_t)1 << 15);
-        HTD_CHECK(alloc_n(&w.win, 2 * w.win_cap));
-        HTD_CHECK(alloc_n(&w.erec, 2 * m));
-        HTD_CHECK(alloc_n(&w.srec, 2 * m));
+        HTD_CHECK(dev_alloc(&w.win, 2 * w.win_cap, H->pstream));
+        HTD_CHECK(dev_alloc(&w.erec, 2 * m, H->pstream));
+        HTD_CHECK(dev_alloc(&w.srec, 2 * m, H->pstream));
         if (h == 3) {
             // radius-2 balls (dense) with their own metadata, the round's radius-2 losses and
             // the radius-3 candidate items
-            if (!w.pool2) HTD_CHECK(alloc_n(&w.pool2, n * (int64_t)w.Wpad));
-            if (!w.ball_size2) HTD_CHECK(alloc_n(&w.ball_size2, n));
-            if (!w.ball_nw2) HTD_CHECK(alloc_n(&w.ball_nw2, n));
-            if (!w.ball_meta2) HTD_CHECK(alloc_n(&w.ball_meta2, n));
-            HTD_CHECK(alloc_n(&w.changed_list2, n));
-            HTD_CHECK(alloc_n(&w.changed_stamp2, n));
-            HTD_CHECK(alloc_n(&w.touch2, n));
+            if (!w.pool2) HTD_CHECK(dev_alloc(&w.pool2, n * (int64_t)w.Wpad, H->pstream));
+            if (!w.ball_size2) HTD_CHECK(dev_alloc(&w.ball_size2, n, H->pstream));
+            if (!w.ball_nw2) HTD_CHECK(dev_alloc(&w.ball_nw2, n, H->pstream));
+            if (!w.ball_meta2) HTD_CHECK(dev_alloc(&w.ball_meta2, n, H->pstream));
+            HTD_CHECK(dev_alloc(&w.changed_list2, n, H->pstream));
+            HTD_CHECK(dev_alloc(&w.changed_stamp2, n, H->pstream));
+            HTD_CHECK(dev_alloc(&w.touch2, n, H->pstream));
             int64_t cap2 = 4096;
             while (cap2 < 4 * m && cap2 < ((int64_t)1 << 22)) cap2 <<= 1;
             if (tiny_table) cap2 = 128;
             w.lost2_cap = cap2;
             w.lost2_max = cap2 / 2;
-            HTD_CHECK(alloc_n(&w.lost2_keys, cap2));
-            HTD_CHECK(alloc_n(&w.lost2, w.lost2_max));
+            HTD_CHECK(dev_alloc(&w.lost2_keys, cap2, H->pstream));
+            HTD_CHECK(dev_alloc(&w.lost2, w.lost2_max, H->pstream));
             w.c3items_cap = tiny_table ? 256
                                        : std::min<int64_t>((int64_t)1 << 25, std::max<int64_t>(1 << 16, 8 * m));
-            HTD_CHECK(alloc_n(&w.c3items, w.c3items_cap));
+            HTD_CHECK(dev_alloc(&w.c3items, w.c3items_cap, H->pstream));
         }
         // alive-adjacency n-bit sets: every vertex of degree >= T, the smallest power of two
         // for which they fit in min(16 GiB, a quarter of the free device memory)
-        std::vector<int32_t> rp(n + 1);
-        HTD_CHECK(cudaMemcpy(rp.data(), g.row_ptr, (n + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost));
         size_t free_b = 0, total_b = 0;
         HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
         const int64_t budget_words = std::min<int64_t>((int64_t)1 << 32, (int64_t)(free_b / 16));
-        int32_t T = 1;
-        int64_t cnt = 0;
-        for (;; T *= 2) {
-            cnt = 0;
-            for (int64_t x = 0; x < n; x++) cnt += (rp[x + 1] - rp[x] >= T);
-            if (cnt * w.Wpad <= budget_words || T > (1 << 24)) break;
-        }
-        std::vector<int32_t> slot(n > 0 ? n : 1, -1), list;
-        // T = 1: every vertex gets a set (isolated ones too), so set x sits at row x
-        for (int64_t x = 0; x < n; x++)
-            if (T == 1 || rp[x + 1] - rp[x] >= T) {
-                slot[x] = (int32_t)list.size();
-                list.push_back((int32_t)x);
+        if (n * w.Wpad <= budget_words) {
+            // T = 1: every vertex gets a set (isolated ones too), set x at row x, no lists needed
+            w.nhub = (int32_t)n;
+            w.hub_min_deg = 1;
+        } else {
+            std::vector<int32_t> rp(n + 1);
+            HTD_CHECK(cudaMemcpyAsync(rp.data(), g.row_ptr, (n + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                      H->pstream));
+            HTD_CHECK(cudaStreamSynchronize(H->pstream));
+            int32_t T = 2;
+            for (;; T *= 2) {
+                int64_t cnt = 0;
+                for (int64_t x = 0; x < n; x++) cnt += (rp[x + 1] - rp[x] >= T);
+                if (cnt * w.Wpad <= budget_words || T > (1 << 24)) break;
             }
-        w.nhub = (int32_t)list.size();
-        w.hub_min_deg = T;
-        HTD_CHECK(alloc_n(&w.hub_slot, n));
-        HTD_CHECK(cudaMemcpy(w.hub_slot, slot.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
+            std::vector<int32_t> slot(n, -1), list;
+            for (int64_t x = 0; x < n; x++)
+                if (rp[x + 1] - rp[x] >= T) {
+                    slot[x] = (int32_t)list.size();
+                    list.push_back((int32_t)x);
+                }
+            w.nhub = (int32_t)list.size();
+            w.hub_min_deg = T;
+            HTD_CHECK(dev_alloc(&w.hub_slot, n, H->pstream));
+            HTD_CHECK(cudaMemcpyAsync(w.hub_slot, slot.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice,
+                                      H->pstream));
+            if (w.nhub > 0) {
+                HTD_CHECK(dev_alloc(&w.hub_list, w.nhub, H->pstream));
+                HTD_CHECK(cudaMemcpyAsync(w.hub_list, list.data(), w.nhub * sizeof(int32_t),
+                                          cudaMemcpyHostToDevice, H->pstream));
+            }
+            HTD_CHECK(cudaStreamSynchronize(H->pstream));  // the lists are on this function's stack
+        }
         if (w.nhub > 0) {
-            HTD_CHECK(alloc_n(&w.hub_list, w.nhub));
-            HTD_CHECK(cudaMemcpy(w.hub_list, list.data(), w.nhub * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice));
-            HTD_CHECK(alloc_n(&w.hub_bits, (int64_t)w.nhub * w.Wpad));
+            HTD_CHECK(dev_alloc(&w.hub_bits, (int64_t)w.nhub * w.Wpad, H->pstream));
         }
     }
     w.incremental = incremental;
@@ -1008,11 +1019,11 @@ htd_status ensure_twin(Handle *H, int64_t budget) {
     const int copies = w.inc3 ? 2 : 1;
     if (!w.pool_new && copies * words * 4 > budget) return HTD_OK;
     if (!w.pool_new) {
-        cudaError_t e = alloc_n(&w.pool_new, words);
-        if (e == cudaSuccess && copies == 2) e = alloc_n(&w.pool2_new, words);
+        cudaError_t e = dev_alloc(&w.pool_new, words, H->pstream);
+        if (e == cudaSuccess && copies == 2) e = dev_alloc(&w.pool2_new, words, H->pstream);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
-            cudaFree(w.pool_new);
+            dev_free(w.pool_new, H->pstream);
             w.pool_new = nullptr;
             return HTD_OK;
         }
@@ -1032,9 +1043,9 @@ htd_status ensure_or_rows(Handle *H, cudaStream_t s, int64_t *launches) {
     const int64_t deg = or_degree(w);
     const int32_t cap = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(2 * g.m / deg + 1, ((int64_t)512 << 20) / (4 * (int64_t)w.Wpad)));
-    HTD_CHECK(alloc_n(&w.or_rows, (int64_t)cap * w.Wpad));
-    HTD_CHECK(alloc_n(&w.or_row_of, g.n));
-    HTD_CHECK(alloc_n(&w.or_list, (int64_t)cap + 1));
+    HTD_CHECK(dev_alloc(&w.or_rows, (int64_t)cap * w.Wpad, H->pstream));
+    HTD_CHECK(dev_alloc(&w.or_row_of, g.n, H->pstream));
+    HTD_CHECK(dev_alloc(&w.or_list, (int64_t)cap + 1, H->pstream));
     int32_t *count = w.or_list + cap;
     HTD_CHECK(cudaMemsetAsync(count, 0, sizeof(int32_t), s));
     k_or_rows<<<std::min<int64_t>((g.n + kBlock - 1) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
@@ -1088,15 +1099,15 @@ htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t fre
     w.inner_ready = false;
     if (!w.pool2) {
         if ((double)words * 4 > (double)free_b / 8) return HTD_OK;
-        HTD_CHECK(alloc_n(&w.pool2, words));
+        HTD_CHECK(dev_alloc(&w.pool2, words, H->pstream));
     }
     if (!w.ball_size2) {
-        HTD_CHECK(alloc_n(&w.ball_size2, H->g.n));
-        HTD_CHECK(alloc_n(&w.ball_nw2, H->g.n));
-        HTD_CHECK(alloc_n(&w.ball_meta2, H->g.n));
+        HTD_CHECK(dev_alloc(&w.ball_size2, H->g.n, H->pstream));
+        HTD_CHECK(dev_alloc(&w.ball_nw2, H->g.n, H->pstream));
+        HTD_CHECK(dev_alloc(&w.ball_meta2, H->g.n, H->pstream));
     }
     if (!w.dense_off) {
-        HTD_CHECK(alloc_n(&w.dense_off, (int64_t)H->g.n + 1));
+        HTD_CHECK(dev_alloc(&w.dense_off, (int64_t)H->g.n + 1, H->pstream));
         k_dense_offsets<<<std::min<int64_t>((H->g.n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
             H->g.n, w.Wpad, w.dense_off);
         (*launches)++;
@@ -1174,7 +1185,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         // memory; else a first pass counts.
         int64_t total = n * (int64_t)w.Wpad;
         size_t free_b = 0, total_b = 0;
-        HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
+        if (!w.dense_balls) HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
         const bool room = total <= w.pool_words || (double)total * 4 <= (double)free_b / 4;
         if (w.dense_balls) {
             k_dense_offsets<<<std::min<int64_t>((n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(n, w.Wpad,
@@ -1195,10 +1206,10 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             return HTD_EUNSUPPORTED;
         }
         if (total > w.pool_words) {
-            cudaFree(w.pool);
+            dev_free(w.pool, s);
             w.pool = nullptr;
             w.pool_words = 0;
-            HTD_CHECK(alloc_n(&w.pool, total));
+            HTD_CHECK(dev_alloc(&w.pool, total, H->pstream));
             w.pool_words = total;
             if (H->graph_exec) {  // the captured rounds hold the old pool pointer
                 cudaGraphExecDestroy(H->graph_exec);

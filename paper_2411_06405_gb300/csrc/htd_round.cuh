@@ -29,7 +29,7 @@ __device__ __forceinline__ void remove_edge(int e, int k, int round, int u, int 
     col_live[slot_hi] = -(round + 1);
     atomicSub(&deg_alive[u], 1);
     atomicSub(&deg_alive[v], 1);
-    if (hub_slot) {
+    if (hub_bits) {
         const int hu = hub_all ? u : hub_slot[u], hv = hub_all ? v : hub_slot[v];
         if (hu >= 0) atomicAnd(hub_bits + (int64_t)hu * Wpad + (v >> 5), ~(1u << (v & 31)));
         if (hv >= 0) atomicAnd(hub_bits + (int64_t)hv * Wpad + (u >> 5), ~(1u << (u & 31)));
