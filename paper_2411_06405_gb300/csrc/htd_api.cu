@@ -8,6 +8,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -30,14 +31,39 @@ void set_last_error(const std::string &msg) { g_last_error = msg; }
 
 namespace {
 constexpr int kMaxDevices = 64;
-constexpr uint64_t kPoolKeeps = (uint64_t)2 << 30;
+constexpr uint64_t kPoolKeeps = (uint64_t)512 << 20;
+// Larger blocks are cudaMalloc's: mapping 8.6 GB through the pool took 6 ms, through cudaMalloc
+// a fraction of one.
+constexpr size_t kLargeBytes = (size_t)64 << 20;
 constexpr size_t kStatusKeeps = 32;
 std::mutex g_mem_mutex;
 cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
 std::vector<DevStatus *> g_status;
+std::set<void *> g_large;
 }  // namespace
 
+void dev_free(void *p, cudaStream_t s) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mutex);
+        if (g_large.erase(p) == 0) {
+            cudaFreeAsync(p, s);
+            return;
+        }
+    }
+    cudaStreamSynchronize(s);
+    cudaFree(p);
+}
+
 cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    if (bytes >= kLargeBytes) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaSuccess) {
+            std::lock_guard<std::mutex> lk(g_mem_mutex);
+            g_large.insert(*p);
+        }
+        return e;
+    }
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;

@@ -11,6 +11,9 @@ namespace htd {
 constexpr int kMaxH = 8;
 constexpr int kWarp = 32;
 
+constexpr int kLostShift = 40;
+constexpr unsigned long long kTouchedMask = (1ull << kLostShift) - 1;
+
 // Work counters of one removal round.  The launches of a round keep them in the status block;
 // the cluster round kernel keeps its own in the shared memory of one of its blocks.
 struct RoundCtr {
@@ -22,7 +25,8 @@ struct RoundCtr {
     int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
     int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
     int32_t pad;
-    long long touched;         // alive edges at endpoints of the batch's lost pairs (once per round)
+    long long touched;         // the batch's lost pairs << kLostShift | alive edges at their endpoints
+                               // (each vertex once per round)
     long long upd_work;        // adjacency slots reserved for the batch's updates
     long long nc3items;        // stored radius-3 candidate items of the current round (64-bit: the
                                // reservations of a huge round may pass 2^31 before it halts)

@@ -15,7 +15,7 @@
 //   6. one thread per slot: compacted column, edge id, endpoints.
 // Steps 5 and 6 read sorted raw rows, so hub rows are spread over every block (a warp per row
 // left them to single warps: on R-MAT 18 compaction and edge ids took 745 us, one thread per
-// slot FINISH us).
+// slot 95 us).
 #include <cstdio>
 
 #include "htd_internal.h"

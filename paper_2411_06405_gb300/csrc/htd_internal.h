@@ -58,7 +58,7 @@ struct PeelWork {
     int64_t lost_cap = 0;          // hash slots (power of two)
     int64_t lost_max = 0;          // lost-pair records one batch may hold (half the slots)
     bool lost_tiny = false;        // table forced to 128 slots (test option)
-    int4 *lost = nullptr;          // (min, max, hash slot, 0) per lost pair
+    int4 *lost = nullptr;          // (min, max, hash slot, 0) per lost pair, two lists of lost_max
     int32_t *edge_touch = nullptr; // n: last round in which the vertex's ball lost a member
     int32_t *hub_slot = nullptr;   // n: row of the vertex's alive-adjacency set, or -1 (null: row x)
     int32_t *hub_list = nullptr;   // nhub vertices with such a set (degree >= hub_min_deg; null: all)
@@ -96,7 +96,7 @@ struct PeelWork {
     unsigned long long *lost2_keys = nullptr;  // hash set of the round's radius-2 lost pairs
     int64_t lost2_cap = 0;
     int64_t lost2_max = 0;
-    int4 *lost2 = nullptr;         // (min, max, hash slot, 0) per radius-2 lost pair
+    int4 *lost2 = nullptr;         // (min, max, hash slot, 0) per radius-2 lost pair, two lists
     int32_t *touch2 = nullptr;     // n: round in which the vertex last lost a radius-2 member
     int4 *c3items = nullptr;       // radius-3 candidate items of a round
     int64_t c3items_cap = 0;
@@ -132,18 +132,16 @@ struct Handle {
 };
 
 void set_last_error(const std::string &msg);
-// Device memory of graphs and scratch, ordered on `s`, from a pool of the library's own that
-// keeps at most 2 GiB of freed memory per device (a cudaMalloc and cudaFree for each of a
-// handle's fifty arrays took longer than a small decomposition, and every cudaFree waits for
-// the other streams' kernels).
+// Device memory of graphs and scratch, ordered on `s`: blocks under 64 MiB from a pool of the
+// library's own that keeps at most 512 MiB of freed memory per device (a cudaMalloc and
+// cudaFree for each of a handle's fifty arrays took longer than a small decomposition, and
+// every cudaFree waits for the other streams' kernels), larger ones from cudaMalloc.
 cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
 template <typename T>
 cudaError_t dev_alloc(T **p, int64_t count, cudaStream_t s) {
     return dev_alloc_bytes(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T), s);
 }
-inline void dev_free(void *p, cudaStream_t s) {
-    if (p) cudaFreeAsync(p, s);
-}
+void dev_free(void *p, cudaStream_t s);
 // Pinned status blocks, kept for the next handle (at most 32).
 DevStatus *take_status_host();
 void give_status_host(DevStatus *p);

@@ -335,6 +335,15 @@ __device__ __forceinline__ bool ball_contains(const LossArgs &a, int z, int w, u
     return ball_contains_meta(a, a.ball_meta[z], w, bytes);
 }
 
+// The lost-pair records of a round: two lists take turns, since the cluster round kernel clears
+// one round's from the balls while it records the next one's.
+__device__ __forceinline__ int4 *lost_list(const LossArgs &a, int round) {
+    return a.lost + (round & 1) * (int64_t)a.lost_max;
+}
+__device__ __forceinline__ int4 *lost2_list(const LossArgs &a, int round) {
+    return a.lost2 + (round & 1) * (int64_t)a.lost2_max;
+}
+
 // Is the pair {p,q} in the table of the batch's lost pairs?  `probes` counts its slots read.
 __device__ __forceinline__ bool in_pair_set(const unsigned long long *keys, unsigned mask, int p, int q,
                                             unsigned &probes) {
@@ -382,7 +391,7 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ct
     }
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
     ibase = __shfl_sync(0xffffffffu, ibase, 0);
-    int4 *const lostv = r2 ? a.lost2 : a.lost;
+    int4 *const lostv = r2 ? lost2_list(a, round) : lost_list(a, round);
     unsigned long long *const keys = r2 ? a.keys2 : a.keys;
     const unsigned cmask = r2 ? a.cap2_mask : a.cap_mask;
     const int lmax = r2 ? a.lost2_max : a.lost_max;
@@ -468,7 +477,8 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ct
                                        : make_int4(b1 + 32 * (c - c0), w1, w0, e1);
     }
     touched = __reduce_add_sync(0xffffffffu, touched);
-    if (lane == 0 && touched) atomicAdd((unsigned long long *)&ctr->touched, (unsigned long long)touched);
+    const unsigned long long recorded = __popc(__ballot_sync(0xffffffffu, rec_idx >= 0));
+    if (lane == 0 && recorded) atomicAdd((unsigned long long *)&ctr->touched, recorded << kLostShift | touched);
 }
 
 // Pair enumeration of edge side u = (edge F[u/2], side u%2): side 0 of (a,b) pairs a with
@@ -679,15 +689,17 @@ __device__ __forceinline__ void lower_support(const LossArgs &a, WindowCtr *wctr
     }
 }
 
-// What a warp counts over its update items (per lane), in place of running byte sums: the
-// updates are bound by the instructions they issue as much as by their loads.
+// What a lane counts over its update items: the updates are bound by the instructions they
+// issue, so bytes follow from the counts afterwards.
 struct DeltaStats {
-    unsigned slots = 0u, tests = 0u, hits = 0u, probes = 0u, member_bytes = 0u;
-    // algorithmic bytes of the lane's share: 16 per item, the row slots, the words tested
-    __device__ unsigned bytes(unsigned items, bool twin) const {
-        return 16u * items + 4u * slots + (twin ? 4u * tests : member_bytes) + 8u * hits + 8u * probes;
+    unsigned tests = 0u, hits = 0u, probes = 0u, member_bytes = 0u;
+    __device__ unsigned bytes(bool twin) const {
+        return (twin ? 4u * tests : member_bytes) + 8u * hits + 8u * probes;
     }
 };
+
+// Algorithmic bytes of an update item beside its lanes': itself and 32 row slots.
+constexpr unsigned kItemBytes = 16u + 4u * 32u;
 
 // Block `blk` of `nblks` takes a contiguous share of the items (an item and the next often test
 // the same ball row), its warps every (blockDim / 32)-th of it.  A directed loss (v loses w)
@@ -695,7 +707,7 @@ struct DeltaStats {
 // is one bit of either, else a bit and, for B_new, a probe of the lost-pair set.
 template <bool kWindow, bool kTwin>
 __device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wctr, int blk, int nblks, int nitems,
-                                               int win_hi, int thr, DeltaStats &ds, unsigned &items) {
+                                               int win_hi, int thr, DeltaStats &ds) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const int share = (nitems + nblks - 1) / nblks;
     const int first = min(nitems, blk * share), last = min(nitems, first + share);
@@ -707,7 +719,6 @@ __device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wct
         for (int j = 0; j < U; j++) {
             const int it = it0 + j * wpb;
             item[j] = (it < last) ? a.uitems[it] : make_int4(0, 0, 0, 0);
-            if (lane == 0) items += it < last;
         }
         int z[U], eid[U];
         bool drop[U];
@@ -717,7 +728,6 @@ __device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wct
             const bool ok = sl < item[j].w;
             z[j] = ok ? a.col_live[sl] : -1;
             eid[j] = ok ? a.slot_eid[sl] : 0;
-            ds.slots += ok;
         }
 #pragma unroll
         for (int j = 0; j < U; j++) {
@@ -746,10 +756,10 @@ template <bool kWindow, bool kTwin>
 __device__ __forceinline__ void delta_items(const LossArgs &a, WindowCtr *wctr, int blk, int nblks, int nitems,
                                             int win_hi, int thr, unsigned &tests, unsigned &bytes) {
     DeltaStats ds;
-    unsigned items = 0u;
-    delta_items_in<kWindow, kTwin>(a, wctr, blk, nblks, nitems, win_hi, thr, ds, items);
+    delta_items_in<kWindow, kTwin>(a, wctr, blk, nblks, nitems, win_hi, thr, ds);
     tests = ds.tests;
-    bytes = ds.bytes(items, kTwin);
+    bytes = ds.bytes(kTwin);
+    if (blk == 0 && threadIdx.x == 0) bytes += kItemBytes * (unsigned)nitems;
 }
 
 __device__ void ph_delta(const LossArgs &a) {
@@ -785,10 +795,11 @@ __device__ void ph_delta(const LossArgs &a) {
 
 // Clears every lost member from the stored balls (each record's bits are set) and empties
 // the hash slots.
-// Thread t of nt; `real` counts the batch's lost pairs (its non-null records).
-__device__ __forceinline__ void apply_lost(const LossArgs &a, int t, int nt, int nlost, unsigned &real) {
+// Thread t of nt.
+__device__ __forceinline__ void apply_lost(const LossArgs &a, int t, int nt, int nlost, int round) {
+    const int4 *const lost = lost_list(a, round);
     for (int d = t; d < 2 * nlost; d += nt) {
-        const int4 L = a.lost[d >> 1];
+        const int4 L = lost[d >> 1];
         if (L.x < 0) continue;
         const int v = (d & 1) ? L.y : L.x;
         const int w = (d & 1) ? L.x : L.y;
@@ -822,20 +833,13 @@ __device__ __forceinline__ void apply_lost(const LossArgs &a, int t, int nt, int
             atomicAnd(word, ~bit);
             atomicSub(a.ball_size + v, 1);
         }
-        if ((d & 1) == 0) {
-            if (!a.pool_new) a.keys[L.z] = kEmpty;
-            real++;
-        }
+        if ((d & 1) == 0 && !a.pool_new) a.keys[L.z] = kEmpty;
     }
 }
 
 __device__ void ph_apply(const LossArgs &a) {
-    DevStatus *st = a.st;
-    unsigned real = 0u;
-    apply_lost(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, min(vload(st->nlost), a.lost_max),
-               real);
-    real = __reduce_add_sync(0xffffffffu, real);  // one atomic per warp
-    if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost, (unsigned long long)real);
+    apply_lost(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, min(vload(a.st->nlost), a.lost_max),
+               vload(a.st->round));
 }
 
 // ---- h = 3 -------------------------------------------------------------------------------
@@ -1119,9 +1123,11 @@ __device__ void ph_test3(const LossArgs &a) {
 }
 
 // Clears the round's radius-2 losses from the stored B2 (and their pair-set slots).
-__device__ __forceinline__ void apply_lost2(const LossArgs &a, int t, int nt, int nlost, unsigned &real) {
+__device__ __forceinline__ void apply_lost2(const LossArgs &a, int t, int nt, int nlost, int round,
+                                            unsigned &real) {
+    const int4 *const lost = lost2_list(a, round);
     for (int d = t; d < 2 * nlost; d += nt) {
-        const int4 L = a.lost2[d >> 1];
+        const int4 L = lost[d >> 1];
         if (L.x < 0) continue;
         const int v = (d & 1) ? L.y : L.x;
         const int w = (d & 1) ? L.x : L.y;
@@ -1139,7 +1145,7 @@ __device__ void ph_apply2(const LossArgs &a) {
     DevStatus *st = a.st;
     unsigned lane_real = 0u;
     apply_lost2(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x,
-                min(vload(st->nlost2), a.lost2_max), lane_real);
+                min(vload(st->nlost2), a.lost2_max), vload(st->round), lane_real);
     unsigned long long real = lane_real;
     for (int o = 16; o > 0; o >>= 1) real += __shfl_xor_sync(0xffffffffu, real, o);
     if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost2, real);
@@ -1582,6 +1588,10 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         st->st_phase_ns[phase] += t - t_prev;
         t_prev = t;
     };
+    auto count_round = [&](const RoundCtr *c) {
+        s_stat[kStatTouched] += (unsigned long long)c->touched & kTouchedMask;
+        s_stat[kStatLost] += (unsigned long long)c->touched >> kLostShift;
+    };
     // smallest value the blocks put into s_min[buf] before the last barrier; the buffer used
     // two reductions ago is reset (a barrier lies between its readers and this point, and
     // another one before its next use)
@@ -1591,6 +1601,21 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         if (tid == 0) s_min[(buf + 2) % 3] = INT_MAX;
         buf = (buf + 1) % 3;
         return v;
+    };
+    // The previous round's lost members leave the balls.  Nothing before the next updates reads
+    // the old balls (h = 3: before the radius-3 tests), so this goes beside the detection, whose
+    // chain of loads hides it.
+    auto apply_previous = [&]() {
+        if (applied) return;
+        const RoundCtr *const prev = ctrs + ((round & 1) ^ 1);
+        const int t = nthreads - 1 - gt;  // the warps with fewest detection items first
+        apply_lost(a, t, nthreads, min(vload(prev->nlost), a.lost_max), round - 1);
+        if (kH3) {
+            unsigned real = 0u;
+            apply_lost2(a, t, nthreads, min(vload(prev->nlost2), a.lost2_max), round - 1, real);
+            stat_add(s_stat, kStatLost2, real);
+        }
+        applied = true;
     };
     // One phase over `work` units, by the leader cluster alone or with the helpers that have
     // started.  Counters of a shared phase are in global memory (a helper cannot reach the
@@ -1664,18 +1689,6 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             }
         };
         load_list();
-        // the previous round's lost members leave the balls
-        if (!applied) {
-            unsigned real = 0u;
-            apply_lost(a, gt, nthreads, min(vload(prev->nlost), a.lost_max), real);
-            stat_add(s_stat, kStatLost, real);
-            if (kH3) {
-                real = 0u;
-                apply_lost2(a, gt, nthreads, min(vload(prev->nlost2), a.lost2_max), real);
-                stat_add(s_stat, kStatLost2, real);
-            }
-            applied = true;
-        }
         if (!direct) {
             int mn = INT_MAX;
             const bool rebuilt = rebuild;
@@ -1781,6 +1794,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         job.round = round;
         job.win_hi = win_hi;
         job.thr = k - 2;
+        apply_previous();
         if (!run_phase(kStageDetect, ctr, job, npitems, kHelpDetect)) break;
         clock(kTimeDetect);
         if (kH3) {
@@ -1795,7 +1809,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             clock(kTimeTest3);
         }
         if (lead) {  // the round before is done with
-            s_stat[kStatTouched] += prev->touched;
+            count_round(prev);
             reset_ctr(prev);
         }
         const int nuitems = vload(ctr->nuitems);
@@ -1817,12 +1831,13 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         alive -= nF;
         applied = false;
     }
+    apply_previous();
     cluster_sync();
     if (lead) {
         // a round left unfinished keeps its counters (`touched` among them: its closing
         // launch adds them), the last finished one only adds its touched edges
         RoundCtr *const ctr = ctrs + (round & 1), *const prev = ctrs + ((round & 1) ^ 1);
-        s_stat[kStatTouched] += prev->touched;
+        count_round(prev);
         if (stage <= kStageSelect) reset_ctr(ctr);
         *static_cast<RoundCtr *>(st) = *ctr;
     }

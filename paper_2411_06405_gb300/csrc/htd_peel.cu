@@ -924,7 +924,7 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
         w.lost_cap = cap;
         w.lost_max = cap / 2;
         HTD_CHECK(dev_alloc(&w.lost_keys, cap, H->pstream));
-        HTD_CHECK(dev_alloc(&w.lost, w.lost_max, H->pstream));
+        HTD_CHECK(dev_alloc(&w.lost, 2 * w.lost_max, H->pstream));
         HTD_CHECK(dev_alloc(&w.edge_touch, n, H->pstream));
         // work items of the loss detection and of the support updates (per batch)
         // (sized with the graph: 2m adjacency slots)
@@ -954,7 +954,7 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
             w.lost2_cap = cap2;
             w.lost2_max = cap2 / 2;
             HTD_CHECK(dev_alloc(&w.lost2_keys, cap2, H->pstream));
-            HTD_CHECK(dev_alloc(&w.lost2, w.lost2_max, H->pstream));
+            HTD_CHECK(dev_alloc(&w.lost2, 2 * w.lost2_max, H->pstream));
             w.c3items_cap = tiny_table ? 256
                                        : std::min<int64_t>((int64_t)1 << 25, std::max<int64_t>(1 << 16, 8 * m));
             HTD_CHECK(dev_alloc(&w.c3items, w.c3items_cap, H->pstream));

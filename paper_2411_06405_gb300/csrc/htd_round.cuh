@@ -78,7 +78,8 @@ __device__ __forceinline__ void round_finalize(DevStatus *st, int initial) {
     st->npitems = 0;
     st->nuitems = 0;
     st->upd_work = 0;
-    st->st_recomputed += st->touched;
+    st->st_recomputed += (int64_t)((unsigned long long)st->touched & kTouchedMask);
+    st->st_lost += (int64_t)((unsigned long long)st->touched >> kLostShift);
     st->touched = 0;
     st->nitems = 0;
     st->q_ball = 0;

@@ -257,7 +257,7 @@ int64_t htd_footprint_estimate(int32_t n, int64_t m_in, int32_t h, int64_t free_
         // edge and slot records, detection items
         bytes += 64.0 * M + 32.0 * std::min(std::max(2.0 * M, 4096.0), (double)(1 << 22));
         // lost-pair tables and support-update items
-        bytes += (h == 3 ? 256.0 : 64.0) * (1 << 20) + 16.0 * std::min(256.0 * M, (double)(1 << 30)) / 32.0;
+        bytes += (h == 3 ? 384.0 : 96.0) * (1 << 20) + 16.0 * std::min(256.0 * M, (double)(1 << 30)) / 32.0;
     } else {
         bytes += 4.0 * N * std::min(W, 64.0);
     }
