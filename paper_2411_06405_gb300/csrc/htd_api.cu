@@ -23,8 +23,8 @@ namespace htd {
 namespace {
 thread_local std::string g_last_error;
 thread_local int64_t g_launches = 0;
-constexpr int kRoundsPerGraph = 16;  // rebuild rounds
-constexpr int kSlotsPerGraph = 4;    // incremental slots
+constexpr int kRoundsPerGraph = 16;  // rounds of one launch each phase
+constexpr int kSlotsPerGraph = 4;    // slots with the cluster round kernel
 }  // namespace
 
 void set_last_error(const std::string &msg) { g_last_error = msg; }
@@ -409,8 +409,9 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         API_TRY(prepare_work(H, h, incremental, (flags & HTD_OPT_TINY_LOSS_TABLE) != 0));
         incremental = w.incremental;
         w.dense_balls = incremental && (h == 3 || ((flags & HTD_OPT_COMPACT_BALLS) == 0 && fits));
-        // a peel that shares the device keeps to a small part of what is free
-        API_TRY(htd::ensure_twin(H, (int64_t)(free_b / (H->shared_device ? 64 : 8))));
+        // (beside other peels a quarter of what these have left: their admission counts twins.
+        // 4,096 graphs in 42 unions of up to 262,144 vertices 21.2 s without, 13.4 s with)
+        API_TRY(htd::ensure_twin(H, (int64_t)(free_b / (H->shared_device ? 4 : 8))));
     }
     {
         htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, timing ? &local : nullptr, false);
@@ -424,8 +425,8 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     API_CHECK(cudaStreamSynchronize(H->pstream));
     API_TRY(check_status_err(w.status_host));
 
-    // an incremental slot holds many rounds (the cluster round kernel)
-    const int R = incremental ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
+    // a slot with the cluster round kernel holds many rounds
+    const int R = incremental && w.twin ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
     const bool persistent = incremental && h <= 2 && (flags & HTD_OPT_PERSISTENT_ROUNDS) != 0;
     if (persistent && w.status_host->alive > 0) {
         // one cooperative launch runs up to kPersistentSlots round slots; the host checks the

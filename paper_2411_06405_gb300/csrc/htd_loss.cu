@@ -94,6 +94,7 @@ struct LossArgs {
     uint32_t *pool_new;
     uint32_t *pool2_new;
     int32_t cluster;    // the slot starts with the cluster round kernel
+    int32_t max_split;  // phase launches: log2 of the warps one detection item may take
     int32_t timer;      // add the time of each phase to the status block
     int32_t win_cap;    // cluster round kernel: edges its window and next-frontier lists hold
     int32_t *win;
@@ -647,8 +648,8 @@ __device__ void ph_detect(const LossArgs &a) {
     const int lane = threadIdx.x & 31;
     unsigned lane_pairs = 0u, lane_reads = 0u;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
-    if (a.pool_new) detect_items<r2, true>(a, st, gw, nwarps, nitems, 2, round, lane_pairs, lane_reads);
-    else detect_items<r2, false>(a, st, gw, nwarps, nitems, 2, round, lane_pairs, lane_reads);
+    if (a.pool_new) detect_items<r2, true>(a, st, gw, nwarps, nitems, a.max_split, round, lane_pairs, lane_reads);
+    else detect_items<r2, false>(a, st, gw, nwarps, nitems, a.max_split, round, lane_pairs, lane_reads);
     unsigned long long pairs = lane_pairs, reads_total = lane_reads;
     for (int o = 16; o > 0; o >>= 1) {
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
@@ -1917,6 +1918,7 @@ LossArgs loss_args(Handle *H) {
     a.pool_new = w.twin ? w.pool_new : nullptr;
     a.pool2_new = w.twin ? w.pool2_new : nullptr;
     a.cluster = 0;
+    a.max_split = H->shared_device ? 0 : 2;  // beside others, idle warps are theirs
     a.timer = 0;
     a.win_cap = 0;
     a.win = w.win;

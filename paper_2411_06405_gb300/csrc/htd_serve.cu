@@ -252,8 +252,8 @@ int64_t htd_footprint_estimate(int32_t n, int64_t m_in, int32_t h, int64_t free_
     const double fb = free_bytes > 0 ? (double)free_bytes : 0.0;
     if (h <= 3 && dense <= fb / 4.0) {
         bytes += dense * (h == 3 ? 2.0 : 1.0) + std::min(dense, std::min(fb / 4.0, 16.0 * (1 << 30)));
-        // twin matrices, which a request takes only while they are small
-        if (dense * (h == 3 ? 2.0 : 1.0) <= fb / 64.0) bytes += dense * (h == 3 ? 2.0 : 1.0);
+        // twin matrices (a peel takes them while they fit a quarter of what is free)
+        bytes += dense * (h == 3 ? 2.0 : 1.0);
         // edge and slot records, detection items
         bytes += 64.0 * M + 32.0 * std::min(std::max(2.0 * M, 4096.0), (double)(1 << 22));
         // lost-pair tables and support-update items
