@@ -372,9 +372,12 @@ __device__ __forceinline__ bool in_pair_set(const unsigned long long *keys, unsi
 // a lost pair).
 // r2: radius-2 losses of an h = 3 round (recorded only: they change no support).
 // kTwin: the pair is new if its bit is still set in the twin matrix, which is cleared.
+// counted: where the new pairs and the alive edges at them are added up (a phase launch keeps
+// them per block: every warp's atomic to one global word was a quarter of its same-address ones).
 template <bool r2, bool kTwin>
 __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ctr, int round, bool want,
-                                                 int x, int z, int rbx, int rex, int rbz, int rez, int u) {
+                                                 int x, int z, int rbx, int rex, int rbz, int rez, int u,
+                                                 unsigned long long *counted) {
     constexpr int kOwnItems = 8;
     const int lane = threadIdx.x & 31;
     const long long work = (want && !r2) ? (long long)(rex - rbx) + (rez - rbz) : 0ll;
@@ -479,7 +482,7 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ct
     }
     touched = __reduce_add_sync(0xffffffffu, touched);
     const unsigned long long recorded = __popc(__ballot_sync(0xffffffffu, rec_idx >= 0));
-    if (lane == 0 && recorded) atomicAdd((unsigned long long *)&ctr->touched, recorded << kLostShift | touched);
+    if (lane == 0 && recorded) atomicAdd(counted, recorded << kLostShift | touched);
 }
 
 // Pair enumeration of edge side u = (edge F[u/2], side u%2): side 0 of (a,b) pairs a with
@@ -542,8 +545,9 @@ __device__ void ph_pair_items(const LossArgs &a) {
         const int first = base + incl - nch;
         const bool fits = first + nch <= a.pitems_cap;
         if (!fits && nch) overflow_at(a, st, u);
-        // the whole warp writes each lane's items in turn (a hub row has hundreds)
-        unsigned todo = __ballot_sync(0xffffffffu, nch > 0);
+        // a lane writes its one item, the whole warp the others (a hub row has hundreds)
+        if (nch == 1 && first < a.pitems_cap) write_pitem(a, first, fits ? u : -1, start, x, y, rows);
+        unsigned todo = __ballot_sync(0xffffffffu, nch > 1);
         while (todo) {
             const int l = __ffs(todo) - 1;
             todo &= todo - 1;
@@ -571,15 +575,51 @@ __device__ __forceinline__ int split_log2(int nitems, int nwarps, int most) {
     return lg;
 }
 
+// Loss detection at h = 1: an item is one removed edge, whose endpoints are no longer adjacent.
+// 2^lg items per warp, one per lane: as few as keep every warp busy, as many as there are
+// for the atomics that reserve records, one set per warp (ER n = 400,000, 1.6 M edges in one
+// round: 9.6 ms with one item per warp).
+template <bool kTwin>
+__device__ __forceinline__ void detect_edges(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps, int nitems,
+                                             int round, unsigned &pairs, unsigned &reads,
+                                             unsigned long long *counted) {
+    const int lane = threadIdx.x & 31;
+    int lg = 0;
+    while (lg < 5 && (nitems >> lg) > nwarps) lg++;
+    for (int w = gw; w << lg < nitems; w += nwarps) {
+        const int i = (w << lg) + lane;
+        int4 item = make_int4(-1, 0, 0, 0), rows = make_int4(0, 0, 0, 0);
+        if (lane < 1 << lg && i < nitems) {
+            item = a.pitems[2 * (int64_t)i];
+            rows = a.pitems[2 * (int64_t)i + 1];
+        }
+        // edges past an overflow are redone by the next slot of the round
+        bool lost = item.x >= 0 && item.x <= vload(ctr->overflow_unit);
+        if (lost) {
+            pairs++;
+            // an earlier batch may have recorded the pair
+            if (kTwin) lost = bit_of(a.pool_new, a.Wpad, item.z, item.w);
+            else lost = ball_contains(a, item.z, item.w, reads);
+            reads += kTwin;
+        }
+        record_lost_warp<false, kTwin>(a, ctr, round, lost, item.z, item.w, rows.x, rows.y, rows.z, rows.w, item.x,
+                                       counted);
+    }
+}
+
 // Loss detection, one warp per item: lane i tests the pair of slot item.y + i.  A pair is
 // kept if its endpoints are adjacent or (h = 2) share an alive neighbour; the pairs whose
 // test needs a longer row scan are walked by the whole warp together.
 template <bool r2, bool kTwin>
 __device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps,
                                              int nitems, int max_split, int round, unsigned &pairs,
-                                             unsigned &reads) {
+                                             unsigned &reads, unsigned long long *counted) {
+    if (!r2 && a.h < 2) {
+        detect_edges<kTwin>(a, ctr, gw, nwarps, nitems, round, pairs, reads, counted);
+        return;
+    }
     const int lane = threadIdx.x & 31;
-    const int lg = a.h < 2 ? 0 : split_log2(nitems, nwarps, max_split), split = 1 << lg;
+    const int lg = split_log2(nitems, nwarps, max_split), split = 1 << lg;
     for (int w = gw; w < nitems << lg; w += nwarps) {
         const int4 item = a.pitems[2 * (int64_t)(w >> lg)], rows = a.pitems[2 * (int64_t)(w >> lg) + 1];
         const int u = item.x, x = item.z;
@@ -587,7 +627,7 @@ __device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, i
         if (u < 0 || u > vload(ctr->overflow_unit)) continue;
         const int sl = item.y + lane;
         int z = -1, rbz = 0, rez = 0;
-        if (sl < (a.h < 2 ? rows.z : rows.w) && (lane & (split - 1)) == (w & (split - 1))) {
+        if (sl < rows.w && (lane & (split - 1)) == (w & (split - 1))) {
             if (sl < rows.z) {
                 z = item.w;
                 rbz = rows.z;
@@ -605,12 +645,13 @@ __device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, i
             }
         }
         // kept if adjacent, or if the stored bit is clear (an earlier batch, or in the twin
-        // matrix another warp, recorded the pair); both words are in x's rows, so their loads go out together
+        // matrix another warp, recorded the pair): in the twin both words are in x's rows, so
+        // their loads go out together; else only a pair about to be recorded looks it up
         int state = kKept, p = rows.x, pe = rows.y, q = z;
         if (z >= 0) {
             pairs++;
             const int64_t at = (int64_t)x * a.Wpad + (z >> 5);
-            bool adjacent, held;
+            bool adjacent, held = true;
             if (kTwin) {
                 const uint32_t stored = r2 ? a.pool2_new[at] : a.pool_new[at];
                 adjacent = (a.hub_bits[at] >> (z & 31)) & 1u;
@@ -619,7 +660,6 @@ __device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, i
             } else {
                 const bool xs = rows.y - rows.x < rez - rbz;  // the longer row's set, if it has one
                 adjacent = alive_adjacent_set(a, hub_set(a, xs ? z : x, reads), xs ? z : x, xs ? x : z, reads);
-                held = r2 ? bit_of(a.pool2, a.Wpad, x, z) : ball_contains(a, x, z, reads);
             }
             if (held && !adjacent) {
                 if (rez - rbz < pe - p) {  // p: the shorter row
@@ -627,29 +667,31 @@ __device__ __forceinline__ void detect_items(const LossArgs &a, RoundCtr *ctr, i
                     pe = rez;
                     q = x;
                 }
-                state = a.h < 2 ? kLost : pair_quick<kTwin>(a, p, pe, q, reads);
+                state = pair_quick<kTwin>(a, p, pe, q, reads);
             }
         }
         if (__any_sync(0xffffffffu, state == kHard)) warp_hard_pairs<kTwin>(a, state, p, pe, q, reads);
-        record_lost_warp<r2, kTwin>(a, ctr, round, state == kLost, x, z, rows.x, rows.y, rbz, rez, u);
+        if (!kTwin && state == kLost && !(r2 ? bit_of(a.pool2, a.Wpad, x, z) : ball_contains(a, x, z, reads)))
+            state = kKept;
+        record_lost_warp<r2, kTwin>(a, ctr, round, state == kLost, x, z, rows.x, rows.y, rbz, rez, u, counted);
     }
 }
 
-template <bool r2>
-__device__ void ph_detect(const LossArgs &a) {
-    __shared__ unsigned long long s_pairs, s_reads;
+template <bool r2, bool kTwin>
+__device__ __forceinline__ void ph_detect(const LossArgs &a) {
+    __shared__ unsigned long long s_pairs, s_reads, s_counted;
     DevStatus *st = a.st;
     if (threadIdx.x == 0) {
         s_pairs = 0ull;
         s_reads = 0ull;
+        s_counted = 0ull;
     }
     __syncthreads();
     const int nitems = min(vload(st->npitems), a.pitems_cap), round = vload(st->round);
     const int lane = threadIdx.x & 31;
     unsigned lane_pairs = 0u, lane_reads = 0u;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
-    if (a.pool_new) detect_items<r2, true>(a, st, gw, nwarps, nitems, a.max_split, round, lane_pairs, lane_reads);
-    else detect_items<r2, false>(a, st, gw, nwarps, nitems, a.max_split, round, lane_pairs, lane_reads);
+    detect_items<r2, kTwin>(a, st, gw, nwarps, nitems, a.max_split, round, lane_pairs, lane_reads, &s_counted);
     unsigned long long pairs = lane_pairs, reads_total = lane_reads;
     for (int o = 16; o > 0; o >>= 1) {
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
@@ -664,6 +706,7 @@ __device__ void ph_detect(const LossArgs &a) {
         atomicAdd((unsigned long long *)&st->st_pairs, s_pairs);
         atomicAdd(&st->st_bytes_detect, 4ull * s_reads);
     }
+    if (threadIdx.x == 0 && s_counted) atomicAdd((unsigned long long *)&st->touched, s_counted);
 }
 
 // Support updates, one warp per item (a directed loss v loses w, and <= 32 of v's slots),
@@ -763,7 +806,8 @@ __device__ __forceinline__ void delta_items(const LossArgs &a, WindowCtr *wctr, 
     if (blk == 0 && threadIdx.x == 0) bytes += kItemBytes * (unsigned)nitems;
 }
 
-__device__ void ph_delta(const LossArgs &a) {
+template <bool kTwin>
+__device__ __forceinline__ void ph_delta(const LossArgs &a) {
     __shared__ unsigned long long s_tests, s_bytes;
     DevStatus *st = a.st;
     if (threadIdx.x == 0) {
@@ -774,10 +818,7 @@ __device__ void ph_delta(const LossArgs &a) {
     const int nitems = min(vload(st->nuitems), a.uitems_cap);
     const int lane = threadIdx.x & 31;
     unsigned lane_tests = 0u, lane_bytes = 0u;
-    if (a.pool_new)
-        delta_items<false, true>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
-    else
-        delta_items<false, false>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
+    delta_items<false, kTwin>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
     unsigned long long tests = lane_tests, bytes_total = lane_bytes;
     for (int o = 16; o > 0; o >>= 1) {
         tests += __shfl_xor_sync(0xffffffffu, tests, o);
@@ -998,7 +1039,7 @@ __device__ __forceinline__ void warp_walk3(const LossArgs &a, int &state, int rb
 // Whole warps.
 template <bool kTwin>
 __device__ __forceinline__ void decide_pairs3(const LossArgs &a, RoundCtr *ctr, int p, int q, int round,
-                                              unsigned &reads) {
+                                              unsigned &reads, unsigned long long *counted) {
     int state = kKept, rb = 0, re = 0, t = q, rbp = 0, rep = 0, rbq = 0, req = 0;
     if (q >= 0) {
         state = kHard;
@@ -1014,13 +1055,14 @@ __device__ __forceinline__ void decide_pairs3(const LossArgs &a, RoundCtr *ctr, 
     }
     if (!__any_sync(0xffffffffu, q >= 0)) return;
     warp_walk3<kTwin>(a, state, rb, re, t, round, reads);
-    record_lost_warp<false, kTwin>(a, ctr, round, state == kLost, p, q, rbp, rep, rbq, req, 0);
+    record_lost_warp<false, kTwin>(a, ctr, round, state == kLost, p, q, rbp, rep, rbq, req, 0, counted);
 }
 
 // Radius-3 loss tests, one warp per candidate item: nA range items, then the stored ones.
 template <bool kTwin>
 __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, int gw, int nwarps, int nA,
-                                            int nitems, int round, unsigned &pairs, unsigned &reads) {
+                                            int nitems, int round, unsigned &pairs, unsigned &reads,
+                                            unsigned long long *counted) {
     const int lane = threadIdx.x & 31;
     const int nch = c3_chunks(a);
     // pairs another warp has recorded already are not candidates
@@ -1064,7 +1106,7 @@ __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, in
             int q = -1;
             if (idx < total) q = (ow << 5) + nth_set_bit(ob, idx - ex);
             if (!kTwin && q >= 0 && in_b2_new<kTwin>(a, ox, q, round, reads)) q = -1;
-            decide_pairs3<kTwin>(a, ctr, ox, q, round, reads);
+            decide_pairs3<kTwin>(a, ctr, ox, q, round, reads, counted);
         }
     }
     // {x} x N_old(y) for the 32 slots of a stored item, restricted to B3_old(x): one per warp
@@ -1083,16 +1125,18 @@ __device__ __forceinline__ void test3_items(const LossArgs &a, RoundCtr *ctr, in
                 if (in3 && !in2) q = c;
             }
         }
-        decide_pairs3<kTwin>(a, ctr, x, q, round, reads);
+        decide_pairs3<kTwin>(a, ctr, x, q, round, reads, counted);
     }
 }
 
-__device__ void ph_test3(const LossArgs &a) {
-    __shared__ unsigned long long s_pairs, s_reads;
+template <bool kTwin>
+__device__ __forceinline__ void ph_test3(const LossArgs &a) {
+    __shared__ unsigned long long s_pairs, s_reads, s_counted;
     DevStatus *st = a.st;
     if (threadIdx.x == 0) {
         s_pairs = 0ull;
         s_reads = 0ull;
+        s_counted = 0ull;
     }
     __syncthreads();
     // a round whose items passed the capacity has halted (this kernel is then idle), so
@@ -1105,8 +1149,7 @@ __device__ void ph_test3(const LossArgs &a) {
     unsigned lane_pairs = 0u, lane_reads = 0u;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
     const int round = vload(st->round);
-    if (a.pool_new) test3_items<true>(a, st, gw, nwarps, nA, nitems, round, lane_pairs, lane_reads);
-    else test3_items<false>(a, st, gw, nwarps, nA, nitems, round, lane_pairs, lane_reads);
+    test3_items<kTwin>(a, st, gw, nwarps, nA, nitems, round, lane_pairs, lane_reads, &s_counted);
     unsigned long long pairs = lane_pairs, reads_total = lane_reads;
     for (int o = 16; o > 0; o >>= 1) {
         pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
@@ -1121,6 +1164,7 @@ __device__ void ph_test3(const LossArgs &a) {
         atomicAdd((unsigned long long *)&st->st_c3_pairs, s_pairs);
         atomicAdd(&st->st_bytes_detect, 4ull * s_reads);
     }
+    if (threadIdx.x == 0 && s_counted) atomicAdd((unsigned long long *)&st->touched, s_counted);
 }
 
 // Clears the round's radius-2 losses from the stored B2 (and their pair-set slots).
@@ -1264,6 +1308,10 @@ __device__ __forceinline__ void phase_clock(const LossArgs &a, int done) {
     a.st->st_phase_start = t;
 }
 
+// Resident blocks per SM a phase kernel is compiled for: left to itself the compiler gives up
+// loads in flight for more blocks, which the small rounds have no use for.
+constexpr int kPhaseBlocks = 4;
+
 // One launch per phase (the rounds of a CUDA graph).
 __global__ void __launch_bounds__(kBlock) k_inc_select(LossArgs a) {
     phase_entry();
@@ -1271,32 +1319,36 @@ __global__ void __launch_bounds__(kBlock) k_inc_select(LossArgs a) {
     phase_clock(a, -1);
     ph_select_items(a);
 }
-__global__ void __launch_bounds__(kBlock) k_loss_detect(LossArgs a) {
+template <bool kTwin>
+__global__ void __launch_bounds__(kBlock, kPhaseBlocks) k_loss_detect(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageDetect)) return;
     phase_clock(a, kTimeSelect);
-    ph_detect<false>(a);
+    ph_detect<false, kTwin>(a);
 }
 // h = 3: the radius-2 detection and the round's radius-3 candidate items
-__global__ void __launch_bounds__(kBlock) k_loss_detect3(LossArgs a) {
+template <bool kTwin>
+__global__ void __launch_bounds__(kBlock, kPhaseBlocks) k_loss_detect3(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageDetect)) return;
     phase_clock(a, kTimeSelect);
-    ph_detect<true>(a);
+    ph_detect<true, kTwin>(a);
     c3_items(a, a.st, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, gridDim.x * (blockDim.x >> 5),
              vload(a.st->nF), vload(a.st->round));
 }
-__global__ void __launch_bounds__(kBlock) k_loss3_test(LossArgs a) {
+template <bool kTwin>
+__global__ void __launch_bounds__(kBlock, kPhaseBlocks) k_loss3_test(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageTest3)) return;
     phase_clock(a, kTimeDetect);
-    ph_test3(a);
+    ph_test3<kTwin>(a);
 }
-__global__ void __launch_bounds__(kBlock) k_loss_delta(LossArgs a) {
+template <bool kTwin>
+__global__ void __launch_bounds__(kBlock, kPhaseBlocks) k_loss_delta(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageDelta)) return;
     phase_clock(a, a.h3 ? kTimeTest3 : kTimeDetect);
-    ph_delta(a);
+    ph_delta<kTwin>(a);
 }
 __global__ void __launch_bounds__(kBlock) k_loss_apply_reduce(LossArgs a) {
     phase_entry();
@@ -1331,9 +1383,11 @@ __global__ void __launch_bounds__(kPBlock, 2) k_rounds_persistent(LossArgs a, in
         if (vload(st->alive) == 0 || vload(st->err) != 0) break;
         ph_select_items(a);
         if (!phase_done(kTimeSelect)) return;
-        ph_detect<false>(a);
+        if (a.pool_new) ph_detect<false, true>(a);
+        else ph_detect<false, false>(a);
         if (!phase_done(kTimeDetect)) return;
-        ph_delta(a);
+        if (a.pool_new) ph_delta<true>(a);
+        else ph_delta<false>(a);
         if (!phase_done(kTimeDelta)) return;
         // clearing the lost members touches balls and hash slots only; the reduction reads
         // supports only, and its last block closes the round after every block did both
@@ -1430,13 +1484,15 @@ __device__ __forceinline__ void shared_phase(const LossArgs &a, RoundCtr *ctr, W
     const int gw = (threadIdx.x >> 5) * nblks + blk, nwarps = nblks * (kCBlock / 32);
     if (phase == kStageDetect) {
         unsigned pairs = 0u, reads = 0u;
-        detect_items<kH3, true>(a, ctr, gw, nwarps, job.nitems, max_split, job.round, pairs, reads);
+        detect_items<kH3, true>(a, ctr, gw, nwarps, job.nitems, max_split, job.round, pairs, reads,
+                                (unsigned long long *)&ctr->touched);
         if (kH3) c3_items(a, ctr, nwarps - 1 - gw, nwarps, job.nF, job.round);  // the warps with fewest items first
         stat_add(s_stat, kStatPairs, pairs);
         stat_add(s_stat, kStatReads, reads);
     } else if (kH3 && phase == kStageTest3) {
         unsigned pairs = 0u, reads = 0u;
-        test3_items<true>(a, ctr, gw, nwarps, 2 * c3_chunks(a) * job.nF, job.nitems, job.round, pairs, reads);
+        test3_items<true>(a, ctr, gw, nwarps, 2 * c3_chunks(a) * job.nF, job.nitems, job.round, pairs, reads,
+                          (unsigned long long *)&ctr->touched);
         stat_add(s_stat, kStatC3, pairs);
         stat_add(s_stat, kStatReads, reads);
     } else {
@@ -2011,13 +2067,14 @@ int cluster_size(int *resident) {
     return 0;
 }
 
+template <bool kTwin>
 htd_status phase_grids(Handle *H, PhaseGrids &pg) {
     if (pg.device == H->g.device) return HTD_OK;
     int od = 0, od3 = 0, ou = 0, ot = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od, k_loss_detect, kBlock, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od3, k_loss_detect3, kBlock, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ou, k_loss_delta, kBlock, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ot, k_loss3_test, kBlock, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od, k_loss_detect<kTwin>, kBlock, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od3, k_loss_detect3<kTwin>, kBlock, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ou, k_loss_delta<kTwin>, kBlock, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ot, k_loss3_test<kTwin>, kBlock, 0) != cudaSuccess ||
         od < 1 || od3 < 1 || ou < 1 || ot < 1) {
         set_last_error("incremental round: no resident block fits");
         return HTD_ECUDA;
@@ -2051,20 +2108,13 @@ cudaError_t launch_phase(void (*kernel)(LossArgs), int grid, cudaStream_t s, boo
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
-}  // namespace
-
-// Enqueues one slot of incremental rounds (the graph path): the cluster round kernel, then
-// the launches of one round, which run from the phase that kernel left to them.  Every
-// launch is programmatic (it overlaps the previous one's tail).
-htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer) {
-    LossArgs a = loss_args(H);
+template <bool kTwin>
+cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launches) {
     static thread_local PhaseGrids pg;
-    const htd_status gs = phase_grids(H, pg);
-    if (gs != HTD_OK) return gs;
+    if (phase_grids<kTwin>(H, pg) != HTD_OK) return cudaErrorInvalidConfiguration;
     const bool pdl = true;
-    a.cluster = (pg.cluster > 0 && H->w.twin) ? 1 : 0;
+    a.cluster = (pg.cluster > 0 && kTwin) ? 1 : 0;
     a.win_cap = (int32_t)std::min<int64_t>(H->w.win_cap, (int64_t)pg.cluster * kCBlock * kWinPerThread);
-    a.timer = timer ? 1 : 0;
     // the two scans over all edges use fewer blocks: the reduction's per-block atomics all
     // hit the same few counters
     const int grid_scan = H->num_sms * 2;
@@ -2074,21 +2124,29 @@ htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launche
         e = cudaLaunchKernelEx(&c.cfg, a.h3 ? k_rounds_cluster<true> : k_rounds_cluster<false>, a);
         *launches += 1;
     }
+    if (e == cudaSuccess) e = launch_phase(k_inc_select, grid_scan, s, pdl, a);
     if (a.h3) {
-        // select | radius-2 detection + radius-3 items | radius-3 tests | updates | - | reduce
-        if (e == cudaSuccess) e = launch_phase(k_inc_select, grid_scan, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_detect3, pg.detect3, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss3_test, pg.test3, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_delta, pg.delta, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_apply_reduce, grid_scan, s, pdl, a);
-        *launches += 5;
+        // select | radius-2 detection + radius-3 items | radius-3 tests | updates | reduce
+        if (e == cudaSuccess) e = launch_phase(k_loss_detect3<kTwin>, pg.detect3, s, pdl, a);
+        if (e == cudaSuccess) e = launch_phase(k_loss3_test<kTwin>, pg.test3, s, pdl, a);
     } else {
-        if (e == cudaSuccess) e = launch_phase(k_inc_select, grid_scan, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_detect, pg.detect, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_delta, pg.delta, s, pdl, a);
-        if (e == cudaSuccess) e = launch_phase(k_loss_apply_reduce, grid_scan, s, pdl, a);
-        *launches += 4;
+        if (e == cudaSuccess) e = launch_phase(k_loss_detect<kTwin>, pg.detect, s, pdl, a);
     }
+    if (e == cudaSuccess) e = launch_phase(k_loss_delta<kTwin>, pg.delta, s, pdl, a);
+    if (e == cudaSuccess) e = launch_phase(k_loss_apply_reduce, grid_scan, s, pdl, a);
+    *launches += a.h3 ? 5 : 4;
+    return e;
+}
+
+}  // namespace
+
+// Enqueues one slot of incremental rounds: with the twin matrices the cluster round kernel,
+// then the launches of one round, which run from the phase that kernel left to them.  Every
+// launch is programmatic (it overlaps the previous one's tail).
+htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer) {
+    LossArgs a = loss_args(H);
+    a.timer = timer ? 1 : 0;
+    cudaError_t e = H->w.twin ? launch_slot<true>(H, a, s, launches) : launch_slot<false>(H, a, s, launches);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_last_error(std::string("enqueue_incremental_round: ") + cudaGetErrorString(e));

@@ -121,6 +121,7 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
     // ball size and non-zero words, per warp segment of words
     const int w0 = wid * seg, w1 = min(W, w0 + seg);
     int sz = 0, nz = 0;
+#pragma unroll 4
     for (int i = w0 + lane; i < w1; i += 32) {
         const uint32_t w = bits[i];
         sz += __popc(w);
@@ -170,6 +171,7 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
             if (threadIdx.x == 0) atomicOr(&st->err, kErrBallCapacity);
         } else if (dense) {
             uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
+#pragma unroll 4
             for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) dst[i] = bits4[i];
             if (a.pool_new) {
                 uint4 *twin = reinterpret_cast<uint4 *>(a.pool_new + off);
@@ -178,6 +180,7 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
         } else {
             uint2 *dst = reinterpret_cast<uint2 *>(a.pool + off);
             int run = wbase;
+#pragma unroll 4
             for (int i0 = w0; i0 < w1; i0 += 32) {
                 const int i = i0 + lane;
                 const uint32_t w = (i < w1) ? bits[i] : 0u;
@@ -208,7 +211,7 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
 // of them expand the same few rows: with the rows of degree W/16 and more as n-bit sets
 // (L2-resident: 988 rows, 32 MB on R-MAT 18) their share becomes W/4 16-byte loads each.
 template <int MODE>
-__global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
+__global__ void __launch_bounds__(kBlock, 4) k_ball(BallArgs a) {
     extern __shared__ __align__(16) uint32_t bits[];
     __shared__ int32_t s_scan[kNWarps];
     __shared__ int32_t s_off[kBlock], s_beg[kBlock];
@@ -249,6 +252,7 @@ __global__ void __launch_bounds__(kBlock) k_ball(BallArgs a) {
         const int x = (MODE == kModeRebuild) ? a.cand_list[it] : it;
 
         uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
+#pragma unroll 4
         for (int i = threadIdx.x; i < (a.Wpad >> 2); i += kBlock) bits4[i] = make_uint4(0, 0, 0, 0);
         if (threadIdx.x == 0) {
             s_cnt[0] = 0;
