@@ -210,6 +210,8 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
 // The builds are bound by the expansions (about 160 G adjacency slots/s).  On hub graphs most
 // of them expand the same few rows: with the rows of degree W/16 and more as n-bit sets
 // (L2-resident: 988 rows, 32 MB on R-MAT 18) their share becomes W/4 16-byte loads each.
+// Four blocks per SM leave the compiler registers for loads in flight (R-MAT 8,192 by rebuilds
+// at h = 2 825 -> 790 ms; it takes 32 registers when left to itself).
 template <int MODE>
 __global__ void __launch_bounds__(kBlock, 4) k_ball(BallArgs a) {
     extern __shared__ __align__(16) uint32_t bits[];
@@ -343,7 +345,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball(BallArgs a) {
 // B(x,h) for every vertex as the OR of its own and its neighbours' dense balls of radius
 // h - 1, one vertex per block at a time: 2m rows of W words are read, coalesced, whatever the
 // radius, where the search by levels of k_ball visits every slot of every vertex within h - 1.
-__global__ void __launch_bounds__(kBlock) k_ball_or(BallArgs a) {
+// Four blocks per SM leave the compiler registers for the rows' loads: DC-SBM 200k at h = 3
+// 22.5 -> 19.6 ms, R-MAT 16 6.7 -> 5.8 ms for the whole h-support.
+__global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
     extern __shared__ __align__(16) uint32_t bits[];
     __shared__ int32_t s_item, s_row[kBlock];
     __shared__ int32_t s_wsz[kNWarps], s_wnz[kNWarps];
@@ -425,7 +429,10 @@ struct HsupArgs {
 // Ownership: x owns (x,y) if y's ball did not change this round, else the endpoint with
 // the larger stored ball owns it (ties: smaller id).  In the initial pass every ball
 // counts as changed, so each edge is computed exactly once.
-__global__ void __launch_bounds__(kBlock) k_hsup(HsupArgs a) {
+// Bound by the rows it streams.  Four loads in flight at six blocks per SM: R-MAT 18 at h = 2
+// 17.1 -> 16.9 ms for the whole h-support, DC-SBM 40k at h = 3 1.49 -> 1.41 ms; at five blocks R-MAT
+// 18 takes 14.7 ms, but graphs of short balls 5% more (ER n = 200,000 at h = 2 2.90 -> 3.04 ms).
+__global__ void __launch_bounds__(kBlock, 6) k_hsup(HsupArgs a) {
     extern __shared__ __align__(16) uint32_t bits[];
     __shared__ int32_t s_item;
     __shared__ unsigned long long s_bytes;
@@ -479,6 +486,7 @@ __global__ void __launch_bounds__(kBlock) k_hsup(HsupArgs a) {
             int cnt = 0;
             if (nwy < 0) {
                 const uint4 *p = pool4 + (offy >> 2);
+#pragma unroll 4
                 for (int i = lane; i < (a.Wpad >> 2); i += 32) {
                     const uint4 v = p[i];
                     const uint4 b = bits4[i];
@@ -487,6 +495,7 @@ __global__ void __launch_bounds__(kBlock) k_hsup(HsupArgs a) {
                 }
             } else {
                 const uint2 *p = pool2 + (offy >> 1);
+#pragma unroll 4
                 for (int j = lane; j < nwy; j += 32) {
                     const uint2 v = p[j];
                     cnt += __popc(bits[v.x] & v.y);
