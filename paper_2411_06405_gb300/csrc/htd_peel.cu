@@ -1058,9 +1058,18 @@ htd_status ensure_or_rows(Handle *H, cudaStream_t s, int64_t *launches) {
     const int64_t deg = or_degree(w);
     const int32_t cap = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(2 * g.m / deg + 1, ((int64_t)512 << 20) / (4 * (int64_t)w.Wpad)));
-    HTD_CHECK(dev_alloc(&w.or_rows, (int64_t)cap * w.Wpad, H->pstream));
-    HTD_CHECK(dev_alloc(&w.or_row_of, g.n, H->pstream));
-    HTD_CHECK(dev_alloc(&w.or_list, (int64_t)cap + 1, H->pstream));
+    cudaError_t e = dev_alloc(&w.or_row_of, g.n, H->pstream);
+    if (e == cudaSuccess) e = dev_alloc(&w.or_list, (int64_t)cap + 1, H->pstream);
+    if (e == cudaSuccess) e = dev_alloc(&w.or_rows, (int64_t)cap * w.Wpad, H->pstream);
+    if (e != cudaSuccess) {  // no room: every row is expanded
+        (void)cudaGetLastError();
+        dev_free(w.or_row_of, H->pstream);
+        dev_free(w.or_list, H->pstream);
+        w.or_row_of = nullptr;
+        w.or_list = nullptr;
+        w.or_rows = nullptr;
+        return HTD_OK;
+    }
     int32_t *count = w.or_list + cap;
     HTD_CHECK(cudaMemsetAsync(count, 0, sizeof(int32_t), s));
     k_or_rows<<<std::min<int64_t>((g.n + kBlock - 1) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
@@ -1080,6 +1089,13 @@ bool or_beats_search(const Handle *H) {
     const double rows = 8.0 * (double)g.m * (double)H->w.Wpad;
     const double slots = std::min((double)g.deg2, (double)g.n * (double)g.n) * (2.0 * (double)g.m / (double)g.n);
     return rows < 100.0 * slots;
+}
+
+void destroy_rounds(Handle *H) {
+    for (cudaGraphExec_t *e : {&H->graph_exec, &H->graph_exec_timed}) {
+        if (*e) cudaGraphExecDestroy(*e);
+        *e = nullptr;
+    }
 }
 
 // Radius-2 balls of every vertex, stored dense in pool2 with their own sizes.
@@ -1114,7 +1130,11 @@ htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t fre
     w.inner_ready = false;
     if (!w.pool2) {
         if ((double)words * 4 > (double)free_b / 8) return HTD_OK;
-        HTD_CHECK(dev_alloc(&w.pool2, words, H->pstream));
+        if (dev_alloc(&w.pool2, words, H->pstream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            w.pool2 = nullptr;
+            return HTD_OK;
+        }
     }
     if (!w.ball_size2) {
         HTD_CHECK(dev_alloc(&w.ball_size2, H->g.n, H->pstream));
@@ -1202,13 +1222,26 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         size_t free_b = 0, total_b = 0;
         if (!w.dense_balls) HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
         const bool room = total <= w.pool_words || (double)total * 4 <= (double)free_b / 4;
+        auto take_pool = [&]() -> cudaError_t {
+            if (total <= w.pool_words) return cudaSuccess;
+            dev_free(w.pool, s);
+            w.pool = nullptr;
+            w.pool_words = 0;
+            destroy_rounds(H);  // the captured rounds hold the old pool pointer
+            const cudaError_t e = dev_alloc(&w.pool, total, H->pstream);
+            if (e == cudaSuccess) w.pool_words = total;
+            else w.pool = nullptr;
+            return e;
+        };
         if (w.dense_balls) {
             k_dense_offsets<<<std::min<int64_t>((n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(n, w.Wpad,
                                                                                                     w.ball_off);
             (*launches)++;
         } else if (support_only && room && total < ((int64_t)1 << 33)) {
-            ba.bump = 1;
-        } else {
+            if (take_pool() == cudaSuccess) ba.bump = 1;
+            else (void)cudaGetLastError();
+        }
+        if (!w.dense_balls && !ba.bump) {
             k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
             (*launches)++;
             HTD_CHECK(cudaGetLastError());
@@ -1220,21 +1253,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             set_last_error("htd: h-hop balls need more than 32 GiB of storage");
             return HTD_EUNSUPPORTED;
         }
-        if (total > w.pool_words) {
-            dev_free(w.pool, s);
-            w.pool = nullptr;
-            w.pool_words = 0;
-            HTD_CHECK(dev_alloc(&w.pool, total, H->pstream));
-            w.pool_words = total;
-            if (H->graph_exec) {  // the captured rounds hold the old pool pointer
-                cudaGraphExecDestroy(H->graph_exec);
-                H->graph_exec = nullptr;
-            }
-            if (H->graph_exec_timed) {
-                cudaGraphExecDestroy(H->graph_exec_timed);
-                H->graph_exec_timed = nullptr;
-            }
-        }
+        HTD_CHECK(take_pool());
         ba.pool = w.pool;
         w.pool_used = total;
         // radius 3 from the dense radius-2 balls, where their rows cost less than the search
