@@ -128,6 +128,11 @@ cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     return e;
 }
 GraphDev *graph_dev(htd_graph *g) { return &g->H.g; }
+std::atomic<int32_t> &peels_in_flight(int device) {
+    static std::atomic<int32_t> counts[64];
+    return counts[device & 63];
+}
+
 void set_shared_device(htd_graph *g) { g->H.shared_device = true; }
 void add_launches(int64_t k) { g_launches += k; }
 
@@ -425,6 +430,8 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     API_CHECK(cudaStreamSynchronize(H->pstream));
     API_TRY(check_status_err(w.status_host));
 
+    const htd::PeelInFlight in_flight(H->g.device);
+    H->beside = std::max(1, (int)in_flight.count.load());
     // a slot with the cluster round kernel holds many rounds
     const int R = incremental && w.twin ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
     const bool persistent = incremental && h <= 2 && (flags & HTD_OPT_PERSISTENT_ROUNDS) != 0;

@@ -1,6 +1,7 @@
 // htd_internal.h -- host-side structures shared by the translation units of libhtruss.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -127,6 +128,7 @@ struct Handle {
     bool graph_dense = false;      // ball layout the captured rounds address directly
     int num_sms = 0;
     bool shared_device = false;    // peels of other streams run beside this one
+    int32_t beside = 1;            // peels in flight on the device when this one's rounds began
     bool graph_shared = false;     // the captured rounds' setting of it
     bool graph_twin = false;       // the captured rounds use the twin matrices
 };
@@ -184,6 +186,13 @@ htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches);
 GraphDev *graph_dev(htd_graph *g);
 // Tells a handle that its decompositions run beside others (they then take less of the device).
 void set_shared_device(htd_graph *g);
+// Peels in flight on a device, by whichever threads: they share its room for clusters.
+std::atomic<int32_t> &peels_in_flight(int device);
+struct PeelInFlight {
+    std::atomic<int32_t> &count;
+    explicit PeelInFlight(int device) : count(peels_in_flight(device)) { count++; }
+    ~PeelInFlight() { count--; }
+};
 
 // One small graph of a batch for the block-per-graph launch (htd_batch_block.cu): device
 // pointers into its union's CSR, its vertices [v0, v0 + L) and edges [e0, e0 + m) there,
