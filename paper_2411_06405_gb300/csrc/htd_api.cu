@@ -133,7 +133,10 @@ std::atomic<int32_t> &peels_in_flight(int device) {
     return counts[device & 63];
 }
 
-void set_shared_device(htd_graph *g) { g->H.shared_device = true; }
+void set_shared_device(htd_graph *g, int32_t peers) {
+    g->H.shared_device = true;
+    g->H.peers = peers;
+}
 void add_launches(int64_t k) { g_launches += k; }
 
 }  // namespace htd
@@ -431,7 +434,7 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     API_TRY(check_status_err(w.status_host));
 
     const htd::PeelInFlight in_flight(H->g.device);
-    H->beside = std::max(1, (int)in_flight.count.load());
+    H->beside = std::max(H->peers, (int32_t)in_flight.count.load());
     // a slot with the cluster round kernel holds many rounds
     const int R = incremental && w.twin ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
     const bool persistent = incremental && h <= 2 && (flags & HTD_OPT_PERSISTENT_ROUNDS) != 0;

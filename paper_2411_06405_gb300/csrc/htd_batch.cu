@@ -389,7 +389,7 @@ extern "C" htd_status htd_truss_decompose_batched(
     }
     const int nworkers = (int)std::min<size_t>(kBatchWorkers, std::max<size_t>(1, uplan.size()));
     for (Built &B : built)
-        if (nworkers > 1 && B.U->g) set_shared_device(B.U->g);
+        if (nworkers > 1 && B.U->g) set_shared_device(B.U->g, nworkers);
     std::mutex mu;
     std::condition_variable cv;
     int64_t used = 0;

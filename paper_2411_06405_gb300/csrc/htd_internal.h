@@ -128,6 +128,7 @@ struct Handle {
     bool graph_dense = false;      // ball layout the captured rounds address directly
     int num_sms = 0;
     bool shared_device = false;    // peels of other streams run beside this one
+    int32_t peers = 1;             // peels its batch or server runs at a time, this one included
     int32_t beside = 1;            // peels in flight on the device when this one's rounds began
     bool graph_shared = false;     // the captured rounds' setting of it
     bool graph_twin = false;       // the captured rounds use the twin matrices
@@ -185,7 +186,7 @@ htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches);
 // The normalised graph behind a public handle (htd_api.cu).
 GraphDev *graph_dev(htd_graph *g);
 // Tells a handle that its decompositions run beside others (they then take less of the device).
-void set_shared_device(htd_graph *g);
+void set_shared_device(htd_graph *g, int32_t peers);
 // Peels in flight on a device, by whichever threads: they share its room for clusters.
 std::atomic<int32_t> &peels_in_flight(int device);
 struct PeelInFlight {

@@ -1421,7 +1421,7 @@ __global__ void __launch_bounds__(kPBlock, 2) k_rounds_persistent(LossArgs a, in
 //
 // A phase with more work than one cluster does quickly is shared with helpers: further
 // clusters of the same launch, which wait for jobs in global memory (bounded waits).  A
-// launch beside others on the device (batched and served decompositions) has no helpers.
+// launch beside others on the device takes its share of the room, and may have no helpers.
 // A round that is too large even so is left, at the phase where it shows, to the phase
 // launches that follow in the slot (RoundStage); their state is the same.
 constexpr int kCBlock = 1024;        // threads per block
@@ -2133,7 +2133,7 @@ cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launche
         // another waiting until their launch ends (eight threads, DC-SBM 40k at h = 2: 52.6 ms a
         // peel with five helpers each, 28.5 ms with this; 49.2 ms with one launch per phase).  The share stays the same for a whole
         // peel: its launches number their clusters by a running count.
-        ClusterLaunch c(H->shared_device ? 1 : std::max(1, pg.clusters / H->beside), pg.cluster, s, pdl);
+        ClusterLaunch c(std::max(1, pg.clusters / H->beside), pg.cluster, s, pdl);
         e = cudaLaunchKernelEx(&c.cfg, a.h3 ? k_rounds_cluster<true> : k_rounds_cluster<false>, a);
         *launches += 1;
     }

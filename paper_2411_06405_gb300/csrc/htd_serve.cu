@@ -167,7 +167,7 @@ htd_status run_request(htd_server *S, Request &r, cudaStream_t s, WorkerBufs &b)
     int32_t n = 0;
     int64_t m = 0;
     htd_graph_info(g, &n, &m);
-    if (S->nworkers > 1) htd::set_shared_device(g);
+    if (S->nworkers > 1) htd::set_shared_device(g, S->nworkers);
     st = htd_truss_decompose_ex(g, r.h, S->flags, b.truss, nullptr, &r.stats, s);
     if (st == HTD_OK) st = htd_edges(g, b.eu, b.ev, s);
     if (st != HTD_OK) r.error = htd_last_error();
