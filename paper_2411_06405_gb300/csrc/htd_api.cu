@@ -40,6 +40,7 @@ std::mutex g_mem_mutex;
 cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
 std::vector<DevStatus *> g_status;
 std::set<void *> g_large;
+thread_local int64_t g_fail_alloc = 0;
 }  // namespace
 
 void dev_free(void *p, cudaStream_t s) {
@@ -56,6 +57,7 @@ void dev_free(void *p, cudaStream_t s) {
 }
 
 cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    if (g_fail_alloc > 0 && --g_fail_alloc == 0) return cudaErrorMemoryAllocation;
     if (bytes >= kLargeBytes) {
         const cudaError_t e = cudaMalloc(p, bytes);
         if (e == cudaSuccess) {
@@ -201,6 +203,15 @@ htd_status prepare_work(Handle *H, int32_t h, bool incremental, bool tiny = fals
 }  // namespace
 
 extern "C" {
+
+// For tests of what a call leaves behind when memory runs out: the calling thread's k-th
+// device allocation from now on fails (0: none).  Returns how many the previous setting still
+// lacked, 0 if it took effect.
+int64_t htd_test_fail_alloc(int64_t k) {
+    const int64_t left = htd::g_fail_alloc;
+    htd::g_fail_alloc = k;
+    return left;
+}
 
 const char *htd_status_string(htd_status s) {
     switch (s) {

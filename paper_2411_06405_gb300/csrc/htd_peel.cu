@@ -1123,28 +1123,26 @@ htd_status build_inner(Handle *H, cudaStream_t s, int64_t *launches) {
 }
 
 // The dense radius-2 balls for it: those of the incremental peel, or (h-support) a pool of
-// their own where they fit an eighth of the free memory.
+// their own where they fit an eighth of the free memory.  Where one of the arrays cannot be had
+// the search by levels, which needs none of them, does the work (inner_ready stays false).
 htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t free_b) {
     PeelWork &w = H->w;
-    const int64_t words = H->g.n * (int64_t)w.Wpad;
+    const int64_t n = H->g.n, words = n * (int64_t)w.Wpad;
     w.inner_ready = false;
-    if (!w.pool2) {
-        if ((double)words * 4 > (double)free_b / 8) return HTD_OK;
-        if (dev_alloc(&w.pool2, words, H->pstream) != cudaSuccess) {
-            (void)cudaGetLastError();
-            w.pool2 = nullptr;
-            return HTD_OK;
-        }
-    }
-    if (!w.ball_size2) {
-        HTD_CHECK(dev_alloc(&w.ball_size2, H->g.n, H->pstream));
-        HTD_CHECK(dev_alloc(&w.ball_nw2, H->g.n, H->pstream));
-        HTD_CHECK(dev_alloc(&w.ball_meta2, H->g.n, H->pstream));
-    }
+    if (!w.pool2 && (double)words * 4 > (double)free_b / 8) return HTD_OK;
+    auto have = [&](auto **p, int64_t count) {
+        if (*p) return true;
+        if (dev_alloc(p, count, H->pstream) == cudaSuccess) return true;
+        (void)cudaGetLastError();
+        *p = nullptr;
+        return false;
+    };
+    if (!have(&w.pool2, words) || !have(&w.ball_size2, n) || !have(&w.ball_nw2, n) || !have(&w.ball_meta2, n))
+        return HTD_OK;
     if (!w.dense_off) {
-        HTD_CHECK(dev_alloc(&w.dense_off, (int64_t)H->g.n + 1, H->pstream));
-        k_dense_offsets<<<std::min<int64_t>((H->g.n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(
-            H->g.n, w.Wpad, w.dense_off);
+        if (!have(&w.dense_off, n + 1)) return HTD_OK;
+        k_dense_offsets<<<std::min<int64_t>((n + kBlock) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(n, w.Wpad,
+                                                                                                w.dense_off);
         (*launches)++;
     }
     const htd_status rs = build_inner(H, s, launches);
