@@ -56,8 +56,9 @@ void dev_free(void *p, cudaStream_t s) {
     cudaFree(p);
 }
 
-cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
-    if (g_fail_alloc > 0 && --g_fail_alloc == 0) return cudaErrorMemoryAllocation;
+namespace {
+cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    if (g_fail_alloc > 0 && --g_fail_alloc == 0) bytes = (size_t)1 << 50;  // more than any device has
     if (bytes >= kLargeBytes) {
         const cudaError_t e = cudaMalloc(p, bytes);
         if (e == cudaSuccess) {
@@ -89,6 +90,14 @@ cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
+}  // namespace
+
+cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    const cudaError_t e = alloc_bytes(p, bytes, s);
+    // the caller gets it: left behind, the next launch's check would report it once more
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
 
 DevStatus *take_status_host() {
     {
@@ -100,8 +109,9 @@ DevStatus *take_status_host() {
         }
     }
     DevStatus *p = nullptr;
-    if (cudaMallocHost(reinterpret_cast<void **>(&p), sizeof(DevStatus)) != cudaSuccess) return nullptr;
-    return p;
+    if (cudaMallocHost(reinterpret_cast<void **>(&p), sizeof(DevStatus)) == cudaSuccess) return p;
+    (void)cudaGetLastError();
+    return nullptr;
 }
 
 void give_status_host(DevStatus *p) {

@@ -1037,7 +1037,6 @@ htd_status ensure_twin(Handle *H, int64_t budget) {
         cudaError_t e = dev_alloc(&w.pool_new, words, H->pstream);
         if (e == cudaSuccess && copies == 2) e = dev_alloc(&w.pool2_new, words, H->pstream);
         if (e != cudaSuccess) {
-            (void)cudaGetLastError();
             dev_free(w.pool_new, H->pstream);
             w.pool_new = nullptr;
             return HTD_OK;
@@ -1062,7 +1061,6 @@ htd_status ensure_or_rows(Handle *H, cudaStream_t s, int64_t *launches) {
     if (e == cudaSuccess) e = dev_alloc(&w.or_list, (int64_t)cap + 1, H->pstream);
     if (e == cudaSuccess) e = dev_alloc(&w.or_rows, (int64_t)cap * w.Wpad, H->pstream);
     if (e != cudaSuccess) {  // no room: every row is expanded
-        (void)cudaGetLastError();
         dev_free(w.or_row_of, H->pstream);
         dev_free(w.or_list, H->pstream);
         w.or_row_of = nullptr;
@@ -1133,7 +1131,6 @@ htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t fre
     auto have = [&](auto **p, int64_t count) {
         if (*p) return true;
         if (dev_alloc(p, count, H->pstream) == cudaSuccess) return true;
-        (void)cudaGetLastError();
         *p = nullptr;
         return false;
     };
@@ -1237,7 +1234,6 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             (*launches)++;
         } else if (support_only && room && total < ((int64_t)1 << 33)) {
             if (take_pool() == cudaSuccess) ba.bump = 1;
-            else (void)cudaGetLastError();
         }
         if (!w.dense_balls && !ba.bump) {
             k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);

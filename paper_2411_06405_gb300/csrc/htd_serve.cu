@@ -132,6 +132,7 @@ cudaError_t grow(WorkerBufs &b, int64_t m_in) {
         if (e == cudaSuccess) e = cudaMallocHost(&b.h_in, 2 * need * 4);
         if (e == cudaSuccess) e = cudaMallocHost(&b.h_out, 3 * need * 4);
         if (e != cudaSuccess) {
+            (void)cudaGetLastError();  // returned: the retried request's launches must not see it
             b.release();
             return e;
         }

@@ -111,3 +111,16 @@ def test_build(htd):
     for got, _ in failing_each(htd, lambda _: build(htd), lambda: None):
         for g in ([got] if got is not None else []) + [build(htd)]:
             assert all(torch.equal(x, y) for x, y in zip(htd.htd_csr(g), ref))
+
+
+def test_failure_is_reported_once(htd):
+    # the error of a failed allocation stays out of the next call's launch checks
+    lib = htd._lib.load()
+    g = build(htd)
+    for _ in range(3):
+        lib.htd_test_fail_alloc(1)
+        with pytest.raises(htd._lib.HtdError):
+            build(htd)
+        assert lib.htd_test_fail_alloc(0) == 0
+        htd.htd_h_support(g, 2)
+        build(htd)
