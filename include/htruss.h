@@ -23,7 +23,8 @@
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Work is ordered after
  *     prior work on `stream`; every call below except htd_h_support_static returns only
  *     after its results are complete and visible on `stream` (the calls synchronise
- *     internally).
+ *     internally).  A `stream` that is being captured into a graph is refused by all of
+ *     them (HTD_ECUDA), before anything joins the capture.
  *   - On error nothing is written to the outputs; the handle stays valid unless stated.
  *   - Errors: HTD_EINVAL (bad argument: NULL pointer, h outside [1, HTD_MAX_H], n < 0,
  *     vertex id outside [0,n)), HTD_ENOMEM (device allocation failed), HTD_ECUDA (a CUDA

@@ -99,6 +99,15 @@ cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
+htd_status refuse_capture(cudaStream_t user) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(user, &cap);
+    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) return HTD_OK;
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    set_last_error("htd: the caller's stream is being captured into a graph; these calls read results on the host");
+    return HTD_ECUDA;
+}
+
 DevStatus *take_status_host() {
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
@@ -175,6 +184,7 @@ namespace {
 
 htd_status begin_call(Handle *H, cudaStream_t user) {
     API_CHECK(cudaSetDevice(H->g.device));
+    API_TRY(htd::refuse_capture(user));
     API_CHECK(cudaEventRecord(H->ev_in, user));
     API_CHECK(cudaStreamWaitEvent(H->pstream, H->ev_in, 0));
     return HTD_OK;
@@ -278,6 +288,7 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
         return HTD_EOVERFLOW;
     }
     cudaStream_t user = static_cast<cudaStream_t>(stream);
+    API_TRY(htd::refuse_capture(user));
     htd_graph *G = new htd_graph();
     Handle *H = &G->H;
     htd_status st = HTD_OK;

@@ -288,6 +288,10 @@ extern "C" htd_status htd_truss_decompose_batched(
     acc.incremental = 1;
     int32_t unions = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (total_in > 0) {
+        const htd_status cs = refuse_capture(s);
+        if (cs != HTD_OK) return cs;
+    }
     int64_t out_pos = 0;
     // block mode: graphs of at most kBlockMaxN vertices and h <= 3 are peeled one per block
     const bool blocks = (flags & HTD_OPT_BATCH_BLOCKS) != 0;

@@ -145,6 +145,9 @@ cudaError_t dev_alloc(T **p, int64_t count, cudaStream_t s) {
     return dev_alloc_bytes(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T), s);
 }
 void dev_free(void *p, cudaStream_t s);
+// HTD_ECUDA while a graph is captured from the caller's stream.  Allocations made during a capture
+// are nodes of that graph: a handle would keep addresses that no memory stands behind.
+htd_status refuse_capture(cudaStream_t user);
 // Pinned status blocks, kept for the next handle (at most 32).
 DevStatus *take_status_host();
 void give_status_host(DevStatus *p);
