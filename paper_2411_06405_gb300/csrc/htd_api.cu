@@ -37,11 +37,34 @@ constexpr uint64_t kPoolKeeps = (uint64_t)512 << 20;
 constexpr size_t kLargeBytes = (size_t)64 << 20;
 constexpr size_t kStatusKeeps = 32;
 std::mutex g_mem_mutex;
-cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
-std::vector<DevStatus *> g_status;
+// Pools and pinned blocks end with their context (cudaDeviceReset): they are used only in it.
+struct ContextPool {
+    uint64_t context = 0;
+    cudaMemPool_t pool = nullptr;
+};
+struct PinnedStatus {
+    int device;
+    uint64_t context;
+    DevStatus *p;
+};
+ContextPool g_pool[kMaxDevices];
+std::vector<PinnedStatus> g_status;
 std::set<void *> g_large;
 thread_local int64_t g_fail_alloc = 0;
 }  // namespace
+
+uint64_t current_context() {
+    using GetId = int (*)(void *, unsigned long long *);
+    static const GetId get_id = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess)
+            fn = nullptr;
+        return found == cudaDriverEntryPointSuccess ? reinterpret_cast<GetId>(fn) : nullptr;
+    }();
+    unsigned long long id = 0;
+    return get_id && get_id(nullptr, &id) == 0 ? (uint64_t)id : 0;
+}
 
 void dev_free(void *p, cudaStream_t s) {
     if (!p) return;
@@ -71,10 +94,12 @@ cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
     if (e != cudaSuccess) return e;
+    const uint64_t context = current_context();
     cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
-        if (!g_pool[dev]) {
+        ContextPool &own = g_pool[dev];
+        if (!own.pool || own.context != context) {
             cudaMemPoolProps props;
             std::memset(&props, 0, sizeof(props));
             props.allocType = cudaMemAllocationTypePinned;
@@ -84,9 +109,10 @@ cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
             uint64_t keeps = kPoolKeeps;
             if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keeps);
             if (e != cudaSuccess) return e;
-            g_pool[dev] = pool;
+            own.context = context;
+            own.pool = pool;
         }
-        pool = g_pool[dev];
+        pool = own.pool;
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
@@ -109,11 +135,13 @@ htd_status refuse_capture(cudaStream_t user) {
 }
 
 DevStatus *take_status_host() {
+    const uint64_t context = current_context();
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
-        if (!g_status.empty()) {
-            DevStatus *p = g_status.back();
-            g_status.pop_back();
+        for (size_t i = g_status.size(); i-- > 0;) {
+            if (g_status[i].context != context) continue;
+            DevStatus *p = g_status[i].p;
+            g_status.erase(g_status.begin() + i);
             return p;
         }
     }
@@ -125,10 +153,15 @@ DevStatus *take_status_host() {
 
 void give_status_host(DevStatus *p) {
     if (!p) return;
+    int device = 0;
+    const uint64_t context = current_context();
+    cudaGetDevice(&device);
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
+        for (size_t i = g_status.size(); i-- > 0;)  // blocks of the device's earlier contexts went with them
+            if (g_status[i].device == device && g_status[i].context != context) g_status.erase(g_status.begin() + i);
         if (g_status.size() < kStatusKeeps) {
-            g_status.push_back(p);
+            g_status.push_back(PinnedStatus{device, context, p});
             return;
         }
     }
@@ -137,15 +170,16 @@ void give_status_host(DevStatus *p) {
 
 cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     static std::mutex mu;
-    static std::map<std::pair<int, const void *>, size_t> limit;
+    static std::map<std::pair<int, const void *>, std::pair<uint64_t, size_t>> limit;  // (context, bytes)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    const uint64_t context = current_context();
     std::lock_guard<std::mutex> lk(mu);
-    size_t &cur = limit[{dev, func}];
-    if (cur >= bytes) return cudaSuccess;
+    auto &cur = limit[{dev, func}];
+    if (cur.first == context && cur.second >= bytes) return cudaSuccess;
     e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) cur = bytes;
+    if (e == cudaSuccess) cur = {context, bytes};
     return e;
 }
 GraphDev *graph_dev(htd_graph *g) { return &g->H.g; }

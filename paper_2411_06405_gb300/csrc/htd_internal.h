@@ -151,6 +151,9 @@ htd_status refuse_capture(cudaStream_t user);
 // Pinned status blocks, kept for the next handle (at most 32).
 DevStatus *take_status_host();
 void give_status_host(DevStatus *p);
+// Id of the current context, unique over the process: what is kept beside handles (pools, pinned
+// blocks, limits raised on kernels, launch shapes) is valid in one context only.
+uint64_t current_context();
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the current device.
 // The limit is a process-wide property of the function: it is only ever raised (under a
 // lock), so that a call for a small graph in one thread cannot lower it below what a

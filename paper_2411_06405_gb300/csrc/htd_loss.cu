@@ -2027,6 +2027,7 @@ namespace {
 // Blocks of one full wave of a phase kernel (every block resident at once), per device.
 struct PhaseGrids {
     int device = -1;
+    uint64_t context = 0;
     int detect = 0, detect3 = 0, delta = 0, test3 = 0;
     int cluster = 0;   // blocks of a cluster of the cluster round kernel (0: none fits the device)
     int clusters = 0;  // clusters of a launch that has the device to itself
@@ -2078,7 +2079,8 @@ int cluster_size(int *resident) {
 
 template <bool kTwin>
 htd_status phase_grids(Handle *H, PhaseGrids &pg) {
-    if (pg.device == H->g.device) return HTD_OK;
+    const uint64_t context = current_context();
+    if (pg.device == H->g.device && pg.context == context) return HTD_OK;
     int od = 0, od3 = 0, ou = 0, ot = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od, k_loss_detect<kTwin>, kBlock, 0) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od3, k_loss_detect3<kTwin>, kBlock, 0) != cudaSuccess ||
@@ -2097,6 +2099,7 @@ htd_status phase_grids(Handle *H, PhaseGrids &pg) {
     // one cluster's room stays free, so that another stream's leader can start beside it
     pg.clusters = std::max(1, resident - 1);
     pg.device = H->g.device;
+    pg.context = context;
     return HTD_OK;
 }
 
