@@ -397,8 +397,14 @@ htd_status htd_server_info(htd_server *s, htd_server_stats *out);
  * workers and frees the server (uncollected results are lost).  NULL is ignored. */
 void htd_server_destroy(htd_server *s);
 
-/* Frees the handle and every device buffer it owns (NULL is ignored). */
+/* Frees the handle and every device buffer it owns (NULL is ignored).  Of the blocks under 64 MiB
+ * the library keeps at most 512 MiB per device for the handles to come, and up to 32 pinned host
+ * blocks of about 1 KiB; larger blocks go back to the device at once. */
 void htd_graph_free(htd_graph *g);
+
+/* Gives back the memory that no handle uses and that is kept for the next ones, of the current
+ * device.  Live handles stay as they are. */
+htd_status htd_trim_memory(void);
 
 /* Kernels this library has launched from the calling thread since it was loaded (a
  * diagnostic counter; graph launches count every kernel node they contain). */

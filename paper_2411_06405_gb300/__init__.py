@@ -29,6 +29,7 @@ __all__ = [
     "HtdStats",
     "Graph", "htd_build_csr", "htd_graph_info", "htd_edges", "htd_csr", "htd_h_support",
     "htd_truss_decompose", "htd_truss_decompose_host", "htd_h_support_static", "htd_graph_free",
+    "htd_trim_memory",
     "htd_truss_decompose_batched", "BatchInput", "Server", "htd_footprint_estimate", "htd_hindex_decompose",
     "library_path",
 ]
@@ -336,3 +337,9 @@ def htd_footprint_estimate(n: int, m_in: int, h: int, free_bytes: int) -> int:
 
 def htd_graph_free(g: Graph):
     g.free()
+
+
+def htd_trim_memory():
+    """Gives back device memory the library keeps for the next handles (at most 512 MiB per
+    device), on the current device."""
+    _lib.check(_lib.load().htd_trim_memory(), "htd_trim_memory")

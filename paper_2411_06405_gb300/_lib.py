@@ -35,7 +35,7 @@ EXPORTED = (
     "htd_graph_free", "htd_kernel_launch_count", "htd_status_string", "htd_last_error",
     "htd_h_support_static", "htd_truss_decompose_batched", "htd_batch_plan",
     "htd_hindex_decompose", "htd_hindex_decompose_ex", "htd_footprint_estimate", "htd_server_create", "htd_server_submit", "htd_server_poll",
-    "htd_server_wait", "htd_server_info", "htd_server_destroy",
+    "htd_server_wait", "htd_server_info", "htd_server_destroy", "htd_trim_memory",
 )
 
 
@@ -171,6 +171,7 @@ def load():
             "htd_truss_decompose_host": ([i32, p, p, i64, i32, p, p, p, ctypes.POINTER(i64), ps, p],
                                          ctypes.c_int),
             "htd_graph_free": ([p], None),
+            "htd_trim_memory": ([], ctypes.c_int),
             "htd_kernel_launch_count": ([], i64),
             "htd_h_support_static": ([i32, p, p, i64, p, p, i32, p, p], ctypes.c_int),
             "htd_truss_decompose_batched": ([i32, p, p, p, p, p, u32, i32, p, p, p,

@@ -168,6 +168,23 @@ void give_status_host(DevStatus *p) {
     cudaFreeHost(p);
 }
 
+htd_status trim_memory(int device) {
+    const uint64_t context = current_context();
+    std::lock_guard<std::mutex> lk(g_mem_mutex);
+    cudaError_t e = cudaSuccess;
+    if (device >= 0 && device < kMaxDevices && g_pool[device].pool && g_pool[device].context == context)
+        e = cudaMemPoolTrimTo(g_pool[device].pool, 0);
+    for (size_t i = g_status.size(); i-- > 0;) {
+        if (g_status[i].context != context) continue;
+        cudaFreeHost(g_status[i].p);
+        g_status.erase(g_status.begin() + i);
+    }
+    if (e == cudaSuccess) return HTD_OK;
+    (void)cudaGetLastError();
+    set_last_error(std::string("htd_trim_memory: ") + cudaGetErrorString(e));
+    return HTD_ECUDA;
+}
+
 cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     static std::mutex mu;
     static std::map<std::pair<int, const void *>, std::pair<uint64_t, size_t>> limit;  // (context, bytes)
@@ -300,6 +317,12 @@ void htd_graph_free(htd_graph *g) {
     if (H->ev_out) cudaEventDestroy(H->ev_out);
     if (H->pstream) cudaStreamDestroy(H->pstream);
     delete g;
+}
+
+htd_status htd_trim_memory(void) {
+    int dev = 0;
+    API_CHECK(cudaGetDevice(&dev));
+    return htd::trim_memory(dev);
 }
 
 htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int64_t m_in,

@@ -148,6 +148,8 @@ void dev_free(void *p, cudaStream_t s);
 // HTD_ECUDA while a graph is captured from the caller's stream.  Allocations made during a capture
 // are nodes of that graph: a handle would keep addresses that no memory stands behind.
 htd_status refuse_capture(cudaStream_t user);
+// Gives back what the pool and the list of pinned status blocks keep for the current context.
+htd_status trim_memory(int device);
 // Pinned status blocks, kept for the next handle (at most 32).
 DevStatus *take_status_host();
 void give_status_host(DevStatus *p);
