@@ -742,8 +742,9 @@ struct DeltaStats {
     }
 };
 
-// Algorithmic bytes of an update item beside its lanes': itself and 32 row slots.
-constexpr unsigned kItemBytes = 16u + 4u * 32u;
+// Algorithmic bytes of an update item beside its lanes': itself and 32 row slots.  (A batch may
+// have 50 M items: their bytes pass 2^32.)
+constexpr unsigned long long kItemBytes = 16ull + 4ull * 32ull;
 
 // Block `blk` of `nblks` takes a contiguous share of the items (an item and the next often test
 // the same ball row), its warps every (blockDim / 32)-th of it.  A directed loss (v loses w)
@@ -803,19 +804,18 @@ __device__ __forceinline__ void delta_items(const LossArgs &a, WindowCtr *wctr, 
     delta_items_in<kWindow, kTwin>(a, wctr, blk, nblks, nitems, win_hi, thr, ds);
     tests = ds.tests;
     bytes = ds.bytes(kTwin);
-    if (blk == 0 && threadIdx.x == 0) bytes += kItemBytes * (unsigned)nitems;
 }
 
 template <bool kTwin>
 __device__ __forceinline__ void ph_delta(const LossArgs &a) {
     __shared__ unsigned long long s_tests, s_bytes;
     DevStatus *st = a.st;
+    const int nitems = min(vload(st->nuitems), a.uitems_cap);
     if (threadIdx.x == 0) {
         s_tests = 0ull;
-        s_bytes = 0ull;
+        s_bytes = blockIdx.x == 0 ? kItemBytes * nitems : 0ull;
     }
     __syncthreads();
-    const int nitems = min(vload(st->nuitems), a.uitems_cap);
     const int lane = threadIdx.x & 31;
     unsigned lane_tests = 0u, lane_bytes = 0u;
     delta_items<false, kTwin>(a, nullptr, blockIdx.x, gridDim.x, nitems, 0, 0, lane_tests, lane_bytes);
@@ -1509,6 +1509,7 @@ __device__ __forceinline__ void shared_phase(const LossArgs &a, RoundCtr *ctr, W
         delta_items<true, true>(a, wctr, blk, nblks, job.nitems, job.win_hi, job.thr, tests, bytes);
         stat_add(s_stat, kStatTests, tests);
         stat_add(s_stat, kStatBytes, bytes);
+        if (blk == 0 && threadIdx.x == 0) atomicAdd(s_stat + kStatBytes, kItemBytes * job.nitems);
     }
 }
 

@@ -1,0 +1,38 @@
+"""The counters of htd_stats agree with what the calls did."""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def htd():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2411_06405_gb300 import build
+
+    build.build()
+    import paper_2411_06405_gb300 as mod
+
+    mod._lib.load()
+    torch.cuda.set_device(0)
+    return mod
+
+
+def test_update_bytes_of_batches_with_many_items(htd):
+    # 30 M edges at 200,000 vertices, h = 1: batches of up to 36 M update items.  Every removed
+    # edge brings an item per 32 slots of both its endpoints' rows; an item counts 144 bytes, a
+    # test 4 more and one that lowers a support 8 more
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    n, m = 200000, 30_000_000
+    src, dst = (torch.randint(0, n, (m,), generator=gen, device="cuda", dtype=torch.int32) for _ in range(2))
+    g = htd.htd_build_csr(n, src, dst)
+    deg = np.diff(htd.htd_csr(g)[0].cpu().numpy().astype(np.int64))
+    _, _, st = htd.htd_truss_decompose(g, 1)
+    g.free()
+    least = 144 * int((deg * ((deg + 31) // 32)).sum()) + 4 * st["member_tests"]
+    assert least <= st["alg_bytes_update"] <= least + 8 * st["member_tests"]
