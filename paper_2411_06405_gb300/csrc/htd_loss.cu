@@ -303,15 +303,15 @@ __device__ __forceinline__ void warp_hard_pairs(const LossArgs &a, int &state, i
 }
 
 // Is w in the stored ball of z (dense words, or sorted (word index, word) pairs)?
-// `bytes` counts the algorithmic bytes: 8 of metadata plus the words probed.
+// `reads` counts 4-byte words: two of metadata plus the words probed.
 __device__ __forceinline__ bool ball_contains_meta(const LossArgs &a, int2 meta, int w,
-                                                   unsigned &bytes) {
+                                                   unsigned &reads) {
     const int nw = meta.y;
     const int64_t off = (int64_t)(unsigned)meta.x << 2;
     const uint32_t bit = 1u << (w & 31);
     const uint32_t wi = (uint32_t)(w >> 5);
     if (nw < 0) {
-        bytes += 4;
+        reads++;
         return (a.pool[off + wi] & bit) != 0u;
     }
     const uint2 *p = reinterpret_cast<const uint2 *>(a.pool + off);
@@ -319,7 +319,7 @@ __device__ __forceinline__ bool ball_contains_meta(const LossArgs &a, int2 meta,
     while (lo <= hi) {
         const int mid = (lo + hi) >> 1;
         const uint2 v = p[mid];
-        bytes += 8;
+        reads += 2;
         if (v.x == wi) return (v.y & bit) != 0u;
         if (v.x < wi) lo = mid + 1;
         else hi = mid - 1;
@@ -327,13 +327,13 @@ __device__ __forceinline__ bool ball_contains_meta(const LossArgs &a, int2 meta,
     return false;
 }
 
-__device__ __forceinline__ bool ball_contains(const LossArgs &a, int z, int w, unsigned &bytes) {
+__device__ __forceinline__ bool ball_contains(const LossArgs &a, int z, int w, unsigned &reads) {
     if (a.dense_all) {
-        bytes += 4;
+        reads++;
         return (a.pool[(int64_t)z * a.Wpad + (w >> 5)] >> (w & 31)) & 1u;
     }
-    bytes += 8;
-    return ball_contains_meta(a, a.ball_meta[z], w, bytes);
+    reads += 2;
+    return ball_contains_meta(a, a.ball_meta[z], w, reads);
 }
 
 // The lost-pair records of a round: two lists take turns, since the cluster round kernel clears
@@ -736,9 +736,9 @@ __device__ __forceinline__ void lower_support(const LossArgs &a, WindowCtr *wctr
 // What a lane counts over its update items: the updates are bound by the instructions they
 // issue, so bytes follow from the counts afterwards.
 struct DeltaStats {
-    unsigned tests = 0u, hits = 0u, probes = 0u, member_bytes = 0u;
+    unsigned tests = 0u, hits = 0u, probes = 0u, member_reads = 0u;
     __device__ unsigned bytes(bool twin) const {
-        return (twin ? 4u * tests : member_bytes) + 8u * hits + 8u * probes;
+        return 4u * (twin ? tests : member_reads) + 8u * hits + 8u * probes;
     }
 };
 
@@ -782,7 +782,7 @@ __device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wct
                 if (kTwin)
                     drop[j] = bit_of(item[j].y < z[j] ? a.pool : a.pool_new, a.Wpad, item[j].z, z[j]);
                 else
-                    drop[j] = ball_contains(a, item[j].z, z[j], ds.member_bytes);
+                    drop[j] = ball_contains(a, item[j].z, z[j], ds.member_reads);
             }
         }
 #pragma unroll
@@ -899,16 +899,16 @@ __device__ void ph_apply(const LossArgs &a) {
 // q in B2_new(z): a bit of the twin matrix, or the stored radius-2 bit unless this round lost
 // the pair (the pair set is probed only for vertices that lost a radius-2 member this round).
 template <bool kTwin>
-__device__ __forceinline__ bool in_b2_new(const LossArgs &a, int z, int q, int round, unsigned &bytes) {
-    bytes += 4;
+__device__ __forceinline__ bool in_b2_new(const LossArgs &a, int z, int q, int round, unsigned &reads) {
+    reads++;
     if (kTwin) return bit_of(a.pool2_new, a.Wpad, z, q);
     if (!bit_of(a.pool2, a.Wpad, z, q)) return false;
     if (z == q) return true;
-    bytes += 4;
+    reads++;
     if (a.touch2[z] != round) return true;
     unsigned probes = 0u;
     const bool lost = in_pair_set(a.keys2, a.cap2_mask, z, q, probes);
-    bytes += 8 * probes;
+    reads += 2 * probes;
     return !lost;
 }
 

@@ -36,3 +36,14 @@ def test_update_bytes_of_batches_with_many_items(htd):
     g.free()
     least = 144 * int((deg * ((deg + 31) // 32)).sum()) + 4 * st["member_tests"]
     assert least <= st["alg_bytes_update"] <= least + 8 * st["member_tests"]
+
+
+def test_detection_bytes_of_a_clique(htd):
+    # h = 1, compact balls: a removed edge is one pair, and its one look-up reads two words of
+    # metadata and, in a clique's dense ball, one of the ball
+    n = 40
+    u, v = np.triu_indices(n, 1)
+    g = htd.htd_build_csr(n, u.astype(np.int32), v.astype(np.int32))
+    _, _, st = htd.htd_truss_decompose(g, 1, flags=htd.HTD_OPT_COMPACT_BALLS)
+    assert st["pairs_tested"] == g.m
+    assert st["alg_bytes_detect"] == 12 * g.m
