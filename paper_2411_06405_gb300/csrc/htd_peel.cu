@@ -356,12 +356,14 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
     uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
     const uint4 *in4 = reinterpret_cast<const uint4 *>(a.inner);
     const int W4 = a.Wpad >> 2;
+    unsigned long long bytes = 0ull;  // one thread's: the rows read
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(&st->q_store, 1);
         __syncthreads();
         const int x = s_item;
         if (x >= a.n) break;
         const int rb = a.row_ptr[x], re = a.row_ptr[x + 1];
+        bytes += 4ull * a.W * (unsigned)(re - rb + 1);
         for (int c = rb; c == rb || c < re; c += kBlock) {
             const int cnt = min(kBlock, re - c);
             if (threadIdx.x < cnt) s_row[threadIdx.x] = a.col_live[c + threadIdx.x];
@@ -383,6 +385,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
         store_ball<kModeStore>(a, x, bits, s_wsz, s_wnz, &s_off64);
         __syncthreads();
     }
+    if (a.count_bytes && threadIdx.x == 0 && bytes) atomicAdd(&st->st_bytes_ball, bytes);
 }
 
 // Offsets of dense balls: x * Wpad.

@@ -47,3 +47,16 @@ def test_detection_bytes_of_a_clique(htd):
     _, _, st = htd.htd_truss_decompose(g, 1, flags=htd.HTD_OPT_COMPACT_BALLS)
     assert st["pairs_tested"] == g.m
     assert st["alg_bytes_detect"] == 12 * g.m
+
+
+@pytest.mark.parametrize("n,ors", [(257, True), (20000, False)])
+def test_ball_bytes_at_radius_3(htd, n, ors):
+    # cycles: radius 3 by ORs of radius-2 rows on the short one (three rows of 9 words a
+    # vertex), by search on the long one (five vertices within two hops, 8 bytes and two slots
+    # each).  All edges go in one round; where that is finished by rebuilds, each ball is built
+    # once more, of a vertex without edges (8 bytes)
+    x = np.arange(n, dtype=np.int32)
+    g = htd.htd_build_csr(n, x, ((x + 1) % n).astype(np.int32))
+    _, _, st = htd.htd_truss_decompose(g, 3)
+    assert st["rounds"] == 1
+    assert st["alg_bytes_ball"] == n * ((3 * 4 * 9 if ors else 5 * 16) + 8 * st["rounds_rebuilt"])
