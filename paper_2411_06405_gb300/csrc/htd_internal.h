@@ -179,7 +179,9 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
 // evs (nullable): kRoundEvents events marking the phase boundaries of the round.
 constexpr int kRoundEvents = 7;
 // timer (incremental rounds, instead of events): phase times go to the status block.
-htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer);
+// by_cluster (twin matrices only): the slot starts with the cluster round kernel.
+htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer,
+                         bool by_cluster);
 
 // Persistent kernel running up to max_slots incremental round slots (htd_loss.cu).
 htd_status launch_persistent_rounds(Handle *H, cudaStream_t s, int max_slots, int64_t *launches);
@@ -220,9 +222,9 @@ htd_status batch_block_run(const std::vector<BlockGraphDescHost> &graphs, cudaSt
 htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_t max_iter, bool prune,
                       int32_t *truss_dev, int32_t *hval_dev, htd_hindex_stats *stats, cudaStream_t s);
 
-// One slot of incremental rounds (h <= 3), the graph path (htd_loss.cu): the cluster round
-// kernel, then four (h = 3: five) phase launches for the round it left to them.
+// One slot of incremental rounds (h <= 3), the graph path (htd_loss.cu): with by_cluster the
+// cluster round kernel, then four (h = 3: five) phase launches for the round it left to them.
 // timer: the phases' times are added to the status block.
-htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer);
+htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer, bool by_cluster);
 
 }  // namespace htd

@@ -2122,11 +2122,11 @@ cudaError_t launch_phase(void (*kernel)(LossArgs), int grid, cudaStream_t s, boo
 }
 
 template <bool kTwin>
-cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launches) {
+cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launches, bool by_cluster) {
     static thread_local PhaseGrids pg;
     if (phase_grids<kTwin>(H, pg) != HTD_OK) return cudaErrorInvalidConfiguration;
     const bool pdl = true;
-    a.cluster = (pg.cluster > 0 && kTwin) ? 1 : 0;
+    a.cluster = (pg.cluster > 0 && kTwin && by_cluster) ? 1 : 0;
     a.win_cap = (int32_t)std::min<int64_t>(H->w.win_cap, (int64_t)pg.cluster * kCBlock * kWinPerThread);
     // the two scans over all edges use fewer blocks: the reduction's per-block atomics all
     // hit the same few counters
@@ -2160,10 +2160,11 @@ cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launche
 // Enqueues one slot of incremental rounds: with the twin matrices the cluster round kernel,
 // then the launches of one round, which run from the phase that kernel left to them.  Every
 // launch is programmatic (it overlaps the previous one's tail).
-htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer) {
+htd_status enqueue_incremental_round(Handle *H, cudaStream_t s, int64_t *launches, bool timer, bool by_cluster) {
     LossArgs a = loss_args(H);
     a.timer = timer ? 1 : 0;
-    cudaError_t e = H->w.twin ? launch_slot<true>(H, a, s, launches) : launch_slot<false>(H, a, s, launches);
+    cudaError_t e = H->w.twin ? launch_slot<true>(H, a, s, launches, by_cluster)
+                              : launch_slot<false>(H, a, s, launches, false);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_last_error(std::string("enqueue_incremental_round: ") + cudaGetErrorString(e));

@@ -1304,12 +1304,13 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
 // Enqueues one peel round.  evs (nullable) = kRoundEvents events at the phase boundaries:
 //   rebuild:     | select | candidates | remove | ball rebuild | items + h-support | reduce |
 //   (incremental rounds add their phase times to the status block instead, with `timer`)
-htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer) {
+htd_status enqueue_round(Handle *H, cudaStream_t s, int64_t *launches, cudaEvent_t *evs, bool timer,
+                         bool by_cluster) {
     PeelWork &w = H->w;
     GraphDev &g = H->g;
     const int64_t m = g.m;
     const int gsmall = H->num_sms * 4;
-    if (w.incremental) return enqueue_incremental_round(H, s, launches, timer);
+    if (w.incremental) return enqueue_incremental_round(H, s, launches, timer, by_cluster);
     // inside a stream capture an ordinary record only orders nodes; an external record
     // node really records the event each time the graph runs, so it can be timed
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

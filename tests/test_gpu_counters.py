@@ -60,3 +60,18 @@ def test_ball_bytes_at_radius_3(htd, n, ors):
     _, _, st = htd.htd_truss_decompose(g, 3)
     assert st["rounds"] == 1
     assert st["alg_bytes_ball"] == n * ((3 * 4 * 9 if ors else 5 * 16) + 8 * st["rounds_rebuilt"])
+
+
+def test_rounds_of_many_batches_are_left_to_the_phase_launches(htd):
+    # 128-slot tables: nearly every round takes a dozen batches.  A batch is four launches; the
+    # cluster round kernel before each of them would be a fifth that has nothing to do
+    from synth import erdos_renyi_gnm
+
+    n = 2000
+    s, d = erdos_renyi_gnm(n, 8000, 3)
+    g = htd.htd_build_csr(n, s.astype(np.int32), d.astype(np.int32))
+    t, stamp, _ = htd.htd_truss_decompose(g, 2, stamps=True)
+    t2, stamp2, st = htd.htd_truss_decompose(g, 2, stamps=True, flags=htd.HTD_OPT_TINY_LOSS_TABLE)
+    assert torch.equal(t, t2) and torch.equal(stamp, stamp2)
+    assert st["slots"] > 5 * st["rounds"]
+    assert st["kernel_launches"] < 4.4 * st["slots"]
