@@ -746,23 +746,28 @@ struct DeltaStats {
 // have 50 M items: their bytes pass 2^32.)
 constexpr unsigned long long kItemBytes = 16ull + 4ull * 32ull;
 
-// Block `blk` of `nblks` takes a contiguous share of the items (an item and the next often test
-// the same ball row), its warps every (blockDim / 32)-th of it.  A directed loss (v loses w)
-// tests z in B_old(w) or z in B_new(w), by the order of v and z: with the twin matrices that
-// is one bit of either, else a bit and, for B_new, a probe of the lost-pair set.
+// A directed loss (v loses w) tests z in B_old(w) or z in B_new(w), by the order of v and z: with
+// the twin matrices that is one bit of either, else a bit and, for B_new, a probe of the lost-pair
+// set.  In the cluster round kernel block `blk` of `nblks` takes a contiguous share of the items
+// (an item and the next often test the same ball row), its warps every (blockDim / 32)-th of it,
+// two at a time.  The phase launches, whose rounds are larger, deal runs of four to the warps of
+// the whole grid: with the shares above, two at a time, R-MAT 18 with 16 M edges at h = 1 took
+// 182 us a round for them instead of 141, R-MAT 16 at h = 2 11.2 instead of 10.2.
 template <bool kWindow, bool kTwin>
 __device__ __forceinline__ void delta_items_in(const LossArgs &a, WindowCtr *wctr, int blk, int nblks, int nitems,
                                                int win_hi, int thr, DeltaStats &ds) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const int share = (nitems + nblks - 1) / nblks;
-    const int first = min(nitems, blk * share), last = min(nitems, first + share);
     // items in flight per warp: their loads are interleaved
-    constexpr int U = 2;
-    for (int it0 = first + wid; it0 < last; it0 += U * wpb) {
+    constexpr int U = kWindow ? 2 : 4;
+    const int share = (nitems + nblks - 1) / nblks;
+    const int first = kWindow ? min(nitems, blk * share) + wid : U * (blk * wpb + wid);
+    const int last = kWindow ? min(nitems, blk * share + share) : nitems;
+    const int step = kWindow ? U * wpb : U * wpb * nblks, next = kWindow ? wpb : 1;
+    for (int it0 = first; it0 < last; it0 += step) {
         int4 item[U];  // (first slot, v, w, end of v's row)
 #pragma unroll
         for (int j = 0; j < U; j++) {
-            const int it = it0 + j * wpb;
+            const int it = it0 + j * next;
             item[j] = (it < last) ? a.uitems[it] : make_int4(0, 0, 0, 0);
         }
         int z[U], eid[U];
@@ -1311,9 +1316,12 @@ __device__ __forceinline__ void phase_clock(const LossArgs &a, int done) {
 // Resident blocks per SM a phase kernel is compiled for: left to itself the compiler gives up
 // loads in flight for more blocks, which the small rounds have no use for.
 constexpr int kPhaseBlocks = 4;
+// The two scans over all edges use fewer blocks: the reduction's per-block atomics all hit the
+// same few counters.
+constexpr int kScanBlocks = 2;
 
 // One launch per phase (the rounds of a CUDA graph).
-__global__ void __launch_bounds__(kBlock) k_inc_select(LossArgs a) {
+__global__ void __launch_bounds__(kBlock, kScanBlocks) k_inc_select(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageSelect)) return;
     phase_clock(a, -1);
@@ -1350,7 +1358,9 @@ __global__ void __launch_bounds__(kBlock, kPhaseBlocks) k_loss_delta(LossArgs a)
     phase_clock(a, a.h3 ? kTimeTest3 : kTimeDetect);
     ph_delta<kTwin>(a);
 }
-__global__ void __launch_bounds__(kBlock) k_loss_apply_reduce(LossArgs a) {
+// Bound by the loads of its scan.  Two blocks per SM, which is what the scans are launched with,
+// leave registers for 16 of them a thread: 16 M supports 62 -> 29 us, 0.5 M 11.2 -> 9.9.
+__global__ void __launch_bounds__(kBlock, kScanBlocks) k_loss_apply_reduce(LossArgs a) {
     phase_entry();
     if (round_idle(a, kStageDelta)) return;
     phase_clock(a, kTimeDelta);
@@ -2128,9 +2138,7 @@ cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launche
     const bool pdl = true;
     a.cluster = (pg.cluster > 0 && kTwin && by_cluster) ? 1 : 0;
     a.win_cap = (int32_t)std::min<int64_t>(H->w.win_cap, (int64_t)pg.cluster * kCBlock * kWinPerThread);
-    // the two scans over all edges use fewer blocks: the reduction's per-block atomics all
-    // hit the same few counters
-    const int grid_scan = H->num_sms * 2;
+    const int grid_scan = H->num_sms * kScanBlocks;
     cudaError_t e = cudaSuccess;
     if (a.cluster) {
         // peels of several threads share the room for clusters: helpers of one keep the leader of
