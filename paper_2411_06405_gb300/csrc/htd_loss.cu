@@ -1776,7 +1776,11 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
                 win_hi = k - 2 + width;
                 int lmin = INT_MAX;
                 const int64_t stride = 4 * (int64_t)nthreads;
-                for (int64_t e0 = 4 * ((int64_t)gt & ~31ll); e0 < a.m; e0 += stride) {
+                // a full window ends the scan: where every round has a larger frontier than it
+                // holds, whole scans at each width by one cluster cost more than the round (R-MAT
+                // 18 with 16 M edges at h = 1: 912 -> 838 ms)
+                bool full = false;
+                for (int64_t e0 = 4 * ((int64_t)gt & ~31ll); e0 < a.m && !full; e0 += stride) {
                     int sv[4];
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
@@ -1792,6 +1796,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
                             if (lane == 0) base = atomicAdd(&wctr->nwin, __popc(bal));
                             base = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & lanemask_lt());
                             if (sv[j] <= win_hi && base < win_cap) a.win[base] = (int)(e0 + 32 * j + lane);
+                            full = __any_sync(0xffffffffu, base >= win_cap);
                         }
                     }
                 }
@@ -1800,18 +1805,21 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
                 cluster_sync();
                 mn = cluster_min();
                 nlist = vload(wctr->nwin);
-                if (mn == INT_MAX) {
-                    alive = 0;
-                    break;
-                }
-                k = max(k, mn + 2);
                 if (nlist > win_cap) {
+                    // the scan stopped there: its minimum is not that of all edges
                     if (width == 0) {  // a frontier larger than the window
                         stage = kStageSelect;
                         break;
                     }
                     width >>= 2;
-                } else if (nlist > 0) {
+                    continue;
+                }
+                if (mn == INT_MAX) {
+                    alive = 0;
+                    break;
+                }
+                k = max(k, mn + 2);
+                if (nlist > 0) {
                     rebuild = false;
                     if (nlist < win_cap / 16) width = min(2 * width + 1, 1 << 20);
                 }

@@ -179,3 +179,26 @@ def test_csr_rows_at_the_sort_edges(htd, oracle_mod):
         np.testing.assert_array_equal(eu_ref[slot_eid], np.minimum(xs, col))
         np.testing.assert_array_equal(ev_ref[slot_eid], np.maximum(xs, col))
         assert all((np.diff(col[row_ptr[x]:row_ptr[x + 1]]) > 0).all() for x in range(n))
+
+
+@pytest.mark.parametrize("h", [1, 2])
+def test_window_of_many_levels(htd, h):
+    # disjoint cliques of 4 to 12 vertices, 1,100 of each: a level has 6,600 to 72,600 edges, so
+    # that the window of the cluster rounds (32,768 edges) holds one level, several or not one
+    src, dst, ref, base = [], [], [], 0
+    for size in range(4, 13):
+        u, v = np.triu_indices(size, 1)
+        off = base + size * np.arange(1100)[:, None]
+        src.append((u + off).ravel())
+        dst.append((v + off).ravel())
+        ref.append(np.full(1100 * u.size, size))
+        base += 1100 * size
+    src, dst, ref = (np.concatenate(x) for x in (src, dst, ref))
+    # other vertex ids, so that the levels are mixed in the scan
+    perm = np.random.default_rng(9).permutation(base)
+    a, b = np.minimum(perm[src], perm[dst]), np.maximum(perm[src], perm[dst])
+    order = np.lexsort((b, a))
+    g = gpu_graph(htd, base, a, b)
+    t, _, st = htd.htd_truss_decompose(g, h)
+    np.testing.assert_array_equal(host(t), ref[order])
+    assert st["rounds"] == 9
