@@ -523,7 +523,6 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
     API_TRY(check_status_err(w.status_host));
 
     const htd::PeelInFlight in_flight(H->g.device);
-    H->beside = std::max(H->peers, (int32_t)in_flight.count.load());
     // a slot with the cluster round kernel holds many rounds
     const int R = incremental && w.twin ? htd::kSlotsPerGraph : htd::kRoundsPerGraph;
     const bool persistent = incremental && h <= 2 && (flags & HTD_OPT_PERSISTENT_ROUNDS) != 0;

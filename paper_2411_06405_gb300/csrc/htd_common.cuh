@@ -76,7 +76,7 @@ struct DevStatus : RoundCtr {
     int32_t stage;             // graph path: first phase launch the cluster round kernel left to the
                                // launches after it (RoundStage), kStageNone if none
     // cluster round kernel with helpers (monotonic over the launches of one peel)
-    unsigned long long cl_tickets;  // clusters started
+    unsigned long long cl_lead;     // last launch that has a leader
     unsigned long long cl_exit;     // launches whose leader has finished
     unsigned long long cl_reg;      // (launch << 32) | helper blocks started
     unsigned long long cl_job;      // (launch << 40) | (job number << 16) | helper blocks taking part

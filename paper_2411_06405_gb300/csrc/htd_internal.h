@@ -129,7 +129,7 @@ struct Handle {
     int num_sms = 0;
     bool shared_device = false;    // peels of other streams run beside this one
     int32_t peers = 1;             // peels its batch or server runs at a time, this one included
-    int32_t beside = 1;            // peels in flight on the device when this one's rounds began
+    int32_t cluster_launches = 0;  // launches of the cluster round kernel in this peel
     bool graph_shared = false;     // the captured rounds' setting of it
     bool graph_twin = false;       // the captured rounds use the twin matrices
 };

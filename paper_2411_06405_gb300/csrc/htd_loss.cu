@@ -94,6 +94,7 @@ struct LossArgs {
     uint32_t *pool_new;
     uint32_t *pool2_new;
     int32_t cluster;    // the slot starts with the cluster round kernel
+    int32_t launch;     // its number, from 1, among the launches of that kernel in this peel
     int32_t max_split;  // phase launches: log2 of the warps one detection item may take
     int32_t timer;      // add the time of each phase to the status block
     int32_t win_cap;    // cluster round kernel: edges its window and next-frontier lists hold
@@ -1595,8 +1596,7 @@ __device__ __forceinline__ void helper_blocks(const LossArgs &a, unsigned long l
 
 template <bool kH3>
 __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_constant__ LossArgs a) {
-    __shared__ unsigned long long s_ticket;
-    __shared__ int s_helpers;
+    __shared__ int s_leads, s_helpers;
     __shared__ RoundCtr s_ctr[2];
     __shared__ WindowCtr s_wctr;
     __shared__ int s_min[3];
@@ -1612,15 +1612,14 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
     const int win_cap = a.win_cap;
     // The first cluster of a launch to start leads; the others help.  Helpers that start late
     // (or never, while the device is busy) are not waited for.
-    unsigned long long epoch = 0ull;
+    const unsigned long long epoch = (unsigned long long)a.launch;
     const int nclusters = (int)(gridDim.x / nblk);
     if (nclusters > 1) {
-        if (lead) s_ticket = atomicAdd(&st->cl_tickets, 1ull);
+        if (lead) s_leads = atomicMax(&st->cl_lead, epoch) < epoch;
         cluster_sync();
-        const unsigned long long ticket = *(volatile unsigned long long *)cluster_map(&s_ticket, 0);
+        const bool leads = *(volatile int *)cluster_map(&s_leads, 0) != 0;
         cluster_sync();
-        epoch = ticket / (unsigned)nclusters;
-        if (ticket % (unsigned)nclusters != 0ull) {
+        if (!leads) {
             if (tid < kNumStats) s_stat[tid] = 0ull;
             __syncthreads();
             helper_blocks<kH3>(a, epoch, (int)nblk, s_stat);
@@ -2002,6 +2001,7 @@ LossArgs loss_args(Handle *H) {
     a.pool_new = w.twin ? w.pool_new : nullptr;
     a.pool2_new = w.twin ? w.pool2_new : nullptr;
     a.cluster = 0;
+    a.launch = 0;
     a.max_split = H->shared_device ? 0 : 2;  // beside others, idle warps are theirs
     a.timer = 0;
     a.win_cap = 0;
@@ -2149,11 +2149,17 @@ cudaError_t launch_slot(Handle *H, LossArgs &a, cudaStream_t s, int64_t *launche
     const int grid_scan = H->num_sms * kScanBlocks;
     cudaError_t e = cudaSuccess;
     if (a.cluster) {
-        // peels of several threads share the room for clusters: helpers of one keep the leader of
+        // Peels of several threads share the room for clusters: helpers of one keep the leader of
         // another waiting until their launch ends (eight threads, DC-SBM 40k at h = 2: 52.6 ms a
-        // peel with five helpers each, 28.5 ms with this; 49.2 ms with one launch per phase).  The share stays the same for a whole
-        // peel: its launches number their clusters by a running count.
-        ClusterLaunch c(std::max(1, pg.clusters / H->beside), pg.cluster, s, pdl);
+        // peel with five helpers each, 28.5 ms with this; 49.2 ms with one launch per phase).  The
+        // share follows the peels in flight from launch to launch, so that a peel which began
+        // alone makes room for the ones that join it (seven threads joining R-MAT 16 at h = 2: their
+        // slowest peel 290-342 ms with a share kept for the whole peel, 139-189 with this, 248 with
+        // one launch per phase).  (Job words hold 24 bits of the number.)
+        const int peels = std::max({H->peers, (int32_t)peels_in_flight(H->g.device).load(), 1});
+        a.launch = ++H->cluster_launches;
+        const int clusters = a.launch < (1 << 24) ? std::max(1, pg.clusters / peels) : 1;
+        ClusterLaunch c(clusters, pg.cluster, s, pdl);
         e = cudaLaunchKernelEx(&c.cfg, a.h3 ? k_rounds_cluster<true> : k_rounds_cluster<false>, a);
         *launches += 1;
     }

@@ -1160,6 +1160,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
     GraphDev &g = H->g;
     const int64_t n = g.n, m = g.m;
     w.inner_ready = false;
+    H->cluster_launches = 0;
     std::memset(w.status_host, 0, sizeof(DevStatus));
     w.status_host->k = 2;
     w.status_host->min_acc = INT_MAX;

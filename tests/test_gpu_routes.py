@@ -202,3 +202,42 @@ def test_window_of_many_levels(htd, h):
     t, _, st = htd.htd_truss_decompose(g, h)
     np.testing.assert_array_equal(host(t), ref[order])
     assert st["rounds"] == 9
+
+
+def test_peels_join_a_long_one(htd):
+    """A peel that begins alone has most of the room for clusters and makes room for the peels
+    that start beside it: its launches hold fewer and fewer clusters, then more again."""
+    long_case = (1 << 13, rmat(13, 8, 0.57, 0.19, 0.19, 6), 2)
+    short = [(2000 + 100 * i, erdos_renyi_gnm(2000 + 100 * i, 8000, 70 + i), 2 + i % 2) for i in range(6)]
+
+    def peel(case):
+        n, (s, d), h = case
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            t, stamp, _ = htd.htd_truss_decompose(gpu_graph(htd, n, s, d), h, stamps=True)
+            return host(t), host(stamp)
+
+    ref = [peel(c) for c in [long_case] + short]
+    out = {}
+    done = threading.Event()
+
+    def run_long():
+        for _ in range(3):
+            out[0] = peel(long_case)
+        done.set()
+
+    def run_short(i):
+        while True:
+            out[i] = peel(short[i - 1])
+            if done.wait(0.002 * i):
+                return
+
+    threads = [threading.Thread(target=run_long)]
+    threads += [threading.Thread(target=run_short, args=(i,)) for i in range(1, 7)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for i, (t, stamp) in enumerate(ref):
+        np.testing.assert_array_equal(out[i][0], t)
+        np.testing.assert_array_equal(out[i][1], stamp)
