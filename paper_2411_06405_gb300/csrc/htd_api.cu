@@ -51,6 +51,7 @@ ContextPool g_pool[kMaxDevices];
 std::vector<PinnedStatus> g_status;
 std::set<void *> g_large;
 thread_local int64_t g_fail_alloc = 0;
+thread_local bool g_no_helpers = false;
 }  // namespace
 
 uint64_t current_context() {
@@ -199,6 +200,7 @@ cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     if (e == cudaSuccess) cur = {context, bytes};
     return e;
 }
+bool test_no_helpers() { return g_no_helpers; }
 GraphDev *graph_dev(htd_graph *g) { return &g->H.g; }
 std::atomic<int32_t> &peels_in_flight(int device) {
     static std::atomic<int32_t> counts[64];
@@ -283,6 +285,10 @@ int64_t htd_test_fail_alloc(int64_t k) {
     htd::g_fail_alloc = k;
     return left;
 }
+
+// For tests: no helper cluster of the calling thread's peels takes part from now on, as on a device
+// with no room for them.
+void htd_test_no_helpers(int32_t on) { htd::g_no_helpers = on != 0; }
 
 const char *htd_status_string(htd_status s) {
     switch (s) {

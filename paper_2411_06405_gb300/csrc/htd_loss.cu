@@ -95,6 +95,7 @@ struct LossArgs {
     uint32_t *pool2_new;
     int32_t cluster;    // the slot starts with the cluster round kernel
     int32_t launch;     // its number, from 1, among the launches of that kernel in this peel
+    int32_t no_helpers; // cluster round kernel: helpers end at once (a test of a busy device)
     int32_t max_split;  // phase launches: log2 of the warps one detection item may take
     int32_t timer;      // add the time of each phase to the status block
     int32_t win_cap;    // cluster round kernel: edges its window and next-frontier lists hold
@@ -1440,8 +1441,10 @@ constexpr int kCMaxBlocks = 16;      // blocks per cluster (the non-portable siz
 constexpr int kWinPerThread = 2;     // window edges each thread holds
 constexpr int kCRounds = 1024;       // rounds per launch
 // Work of a phase: the leader cluster runs up to kHelp... units alone and shares more with the
-// helpers; more than kMost... (kAlone... where the launch has no helpers) is left to the phase
-// launches.  Sharing costs about 5 us of hand-over and turns the counters' shared-memory atomics
+// helpers that have started; more than kMost... with all of a launch's helpers, kAlone... with none
+// and in proportion between them, is left to the phase launches.  On a busy device helpers start
+// late or not at all (with none, R-MAT 16 with 4 M edges at h = 1 took 462 ms by the limits of a
+// launch with all of them, 200 by these; 167 with helpers).  Sharing costs about 5 us of hand-over and turns the counters' shared-memory atomics
 // into global ones: with helpers from 256 detection items on, ER n = 2,000 detects in 12 us a round
 // instead of 7; without helpers R-MAT 16 at h = 2 takes 800 ms instead of 640.
 constexpr int kHelpDetect = 1024, kAloneDetect = 4096, kMostDetect = 1 << 16;     // detection items
@@ -1596,7 +1599,7 @@ __device__ __forceinline__ void helper_blocks(const LossArgs &a, unsigned long l
 
 template <bool kH3>
 __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_constant__ LossArgs a) {
-    __shared__ int s_leads, s_helpers;
+    __shared__ int s_leads, s_helpers, s_failed;
     __shared__ RoundCtr s_ctr[2];
     __shared__ WindowCtr s_wctr;
     __shared__ int s_min[3];
@@ -1620,6 +1623,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         const bool leads = *(volatile int *)cluster_map(&s_leads, 0) != 0;
         cluster_sync();
         if (!leads) {
+            if (a.no_helpers) return;
             if (tid < kNumStats) s_stat[tid] = 0ull;
             __syncthreads();
             helper_blocks<kH3>(a, epoch, (int)nblk, s_stat);
@@ -1647,6 +1651,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         reset_ctr(&s_ctr[0]);
         reset_ctr(&s_ctr[1]);
         s_wctr = WindowCtr{};
+        s_failed = 0;
         for (int j = 0; j < 3; j++) s_min[j] = INT_MAX;
         for (int j = 0; j < kNumStats; j++) s_stat[j] = 0ull;
     }
@@ -1695,14 +1700,20 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
     };
     // One phase over `work` units, by the leader cluster alone or with the helpers that have
     // started.  Counters of a shared phase are in global memory (a helper cannot reach the
-    // leader's shared memory): copied there before and back after.  Ends with a barrier; false
-    // if the helpers did not finish in time (an error is set: the peel ends).
-    auto run_phase = [&](int phase, RoundCtr *ctr, HelperJob job, long long work, int help) -> bool {
+    // leader's shared memory): copied there before and back after.  Ends with a barrier, unless
+    // the work is too much (kLeft: nothing was done).
+    enum { kDone = 0, kLeft, kFailed };  // kFailed: the helpers did not finish in time (an error is set)
+    auto run_phase = [&](int phase, RoundCtr *ctr, HelperJob job, long long work, int help, int alone,
+                         int most) -> int {
         int helpers = 0;
-        if (nclusters > 1 && work > help) {
+        if (nclusters == 1) {
+            if (work > alone) return kLeft;
+        } else if (work > help) {
             if (lead) {
                 const unsigned long long reg = load_acquire(&st->cl_reg);
-                s_helpers = (reg >> 32) == epoch ? (int)(reg & 0xffffull) : 0;
+                const int started = (reg >> 32) == epoch ? (int)(reg & 0xffffull) : 0;
+                const long long room = alone + (long long)(most - alone) * started / ((nclusters - 1) * (int)nblk);
+                s_helpers = work > room ? -1 : started;
                 if (s_helpers > 0) {
                     job.phase = phase;
                     st->cl_work = job;
@@ -1714,11 +1725,12 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             }
             cluster_sync();
             helpers = *(volatile int *)cluster_map(&s_helpers, 0);
+            if (helpers < 0) return kLeft;
         }
         if (helpers == 0) {
             shared_phase<kH3>(a, ctr, wctr, s_stat, phase, (int)rank, (int)nblk, 5, job);
             cluster_sync();
-            return true;
+            return kDone;
         }
         const int blocks = (int)nblk + helpers;
         shared_phase<kH3>(a, &st->cl_ctr, &st->cl_wctr, s_stat, phase, (int)rank, blocks, 2, job);
@@ -1729,7 +1741,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             while (load_acquire(&st->cl_done) < done_base) {
                 if (global_ns() - t0 > kLeadWaitNs) {
                     atomicOr(&st->err, kErrBarrierTimeout);
-                    s_helpers = -1;
+                    s_failed = 1;
                     break;
                 }
             }
@@ -1743,7 +1755,8 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             wctr->nnext = vload(st->cl_wctr.nnext);
         }
         cluster_sync();
-        return *(volatile int *)cluster_map(&s_helpers, 0) >= 0;
+        // (not s_helpers: the leader may be in the next phase already and write it)
+        return *(volatile int *)cluster_map(&s_failed, 0) ? kFailed : kDone;
     };
     cluster_sync();
     for (;;) {
@@ -1863,11 +1876,8 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         // phase now starting may set, are read where no phase sets them).
         const int nF = vload(ctr->nF), npitems = vload(ctr->npitems);
         if (lead) wctr->nnext = 0;  // read by all before the barrier, used again after the next
-        const int most_detect = nclusters > 1 ? kMostDetect : kAloneDetect;
-        const int most_test3 = nclusters > 1 ? kMostTest3 : kAloneTest3;
-        const int most_delta = nclusters > 1 ? kMostDelta : kAloneDelta;
         const long long nA = kH3 ? 2ll * c3_chunks(a) * nF : 0ll;
-        if (npitems > min(most_detect, a.pitems_cap) || nA > most_test3) {
+        if (npitems > a.pitems_cap || nA > (nclusters > 1 ? kMostTest3 : kAloneTest3)) {
             stage = kStageDetect;
             break;
         }
@@ -1879,17 +1889,25 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         job.win_hi = win_hi;
         job.thr = k - 2;
         apply_previous();
-        if (!run_phase(kStageDetect, ctr, job, npitems, kHelpDetect)) break;
+        int got = run_phase(kStageDetect, ctr, job, npitems, kHelpDetect, kAloneDetect, kMostDetect);
+        if (got != kDone) {
+            if (got == kLeft) stage = kStageDetect;
+            break;
+        }
         clock(kTimeDetect);
         if (kH3) {
             // too many items, or no room for the items or the radius-2 losses (a halt)
             const long long nc3 = vload(ctr->nc3items);
-            if (nA + nc3 > min(most_test3, a.c3items_cap) || vload(ctr->nlost2) > a.lost2_max) {
+            if (nA + nc3 > a.c3items_cap || vload(ctr->nlost2) > a.lost2_max) {
                 stage = kStageTest3;
                 break;
             }
             job.nitems = (int)(nA + nc3);
-            if (!run_phase(kStageTest3, ctr, job, nA + nc3, kHelpTest3)) break;
+            got = run_phase(kStageTest3, ctr, job, nA + nc3, kHelpTest3, kAloneTest3, kMostTest3);
+            if (got != kDone) {
+                if (got == kLeft) stage = kStageTest3;
+                break;
+            }
             clock(kTimeTest3);
         }
         if (lead) {  // the round before is done with
@@ -1897,12 +1915,16 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
             reset_ctr(prev);
         }
         const int nuitems = vload(ctr->nuitems);
-        if (nuitems > most_delta || vload(ctr->overflow_unit) != INT_MAX || (kH3 && vload(ctr->halt) != 0)) {
+        if (vload(ctr->overflow_unit) != INT_MAX || (kH3 && vload(ctr->halt) != 0)) {
             stage = kStageDelta;
             break;
         }
         job.nitems = nuitems;
-        if (!run_phase(kStageDelta, ctr, job, nuitems, kHelpDelta)) break;
+        got = run_phase(kStageDelta, ctr, job, nuitems, kHelpDelta, kAloneDelta, kMostDelta);
+        if (got != kDone) {
+            if (got == kLeft) stage = kStageDelta;
+            break;
+        }
         clock(kTimeDelta);
         // the round's bookkeeping (round_finalize's, kept by every thread alike)
         if (k != last_k) {
@@ -2002,6 +2024,7 @@ LossArgs loss_args(Handle *H) {
     a.pool2_new = w.twin ? w.pool2_new : nullptr;
     a.cluster = 0;
     a.launch = 0;
+    a.no_helpers = test_no_helpers() ? 1 : 0;
     a.max_split = H->shared_device ? 0 : 2;  // beside others, idle warps are theirs
     a.timer = 0;
     a.win_cap = 0;

@@ -241,3 +241,22 @@ def test_peels_join_a_long_one(htd):
     for i, (t, stamp) in enumerate(ref):
         np.testing.assert_array_equal(out[i][0], t)
         np.testing.assert_array_equal(out[i][1], stamp)
+
+
+@pytest.mark.parametrize("scale,factor,h", [(14, 60, 1), (13, 8, 2), (11, 8, 3)])
+def test_rounds_that_no_helper_joins(htd, scale, factor, h):
+    """Where helper clusters do not start (a busy device), rounds too large for one cluster go to
+    the phase launches instead of running on its 16 SMs."""
+    s, d = rmat(scale, factor, 0.57, 0.19, 0.19, 8)
+    g = gpu_graph(htd, 1 << scale, s, d)
+    t, stamp, st = htd.htd_truss_decompose(g, h, stamps=True)
+    lib = htd._lib.load()
+    lib.htd_test_no_helpers(1)
+    try:
+        t2, stamp2, st2 = htd.htd_truss_decompose(g, h, stamps=True)
+    finally:
+        lib.htd_test_no_helpers(0)
+    assert torch.equal(t, t2) and torch.equal(stamp, stamp2)
+    assert st2["rounds"] == st["rounds"]
+    if h == 1:  # (rounds of up to a million update items)
+        assert st2["kernel_launches"] > st["kernel_launches"] + 40
