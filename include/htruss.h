@@ -29,7 +29,8 @@
  *   - Errors: HTD_EINVAL (bad argument: NULL pointer, h outside [1, HTD_MAX_H], n < 0,
  *     vertex id outside [0,n)), HTD_ENOMEM (device allocation failed), HTD_ECUDA (a CUDA
  *     call failed; htd_last_error() has the message), HTD_EOVERFLOW (2*m_in >= 2^31),
- *     HTD_EUNSUPPORTED (n > HTD_MAX_N), HTD_ETIMEOUT (the peel exceeded its round cap).
+ *     HTD_EUNSUPPORTED (n > HTD_MAX_N), HTD_ETIMEOUT (the peel exceeded its round cap, or a
+ *     wait between blocks of its kernels gave up after minutes without progress).
  *   - Functions are thread-safe for distinct handles; one handle must not be used by two
  *     threads at once.
  */

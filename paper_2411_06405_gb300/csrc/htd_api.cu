@@ -52,6 +52,7 @@ std::vector<PinnedStatus> g_status;
 std::set<void *> g_large;
 thread_local int64_t g_fail_alloc = 0;
 thread_local bool g_no_helpers = false;
+thread_local int32_t g_wait_polls = 0;
 }  // namespace
 
 uint64_t current_context() {
@@ -201,6 +202,7 @@ cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     return e;
 }
 bool test_no_helpers() { return g_no_helpers; }
+int32_t test_wait_polls() { return g_wait_polls; }
 GraphDev *graph_dev(htd_graph *g) { return &g->H.g; }
 std::atomic<int32_t> &peels_in_flight(int device) {
     static std::atomic<int32_t> counts[64];
@@ -260,6 +262,10 @@ void destroy_graph(Handle *H) {
 }
 
 htd_status check_status_err(const htd::DevStatus *st) {
+    if (st->err & htd::kErrBarrierTimeout) {
+        set_last_error("htd_truss_decompose: a wait between blocks of the round kernel gave up");
+        return HTD_ETIMEOUT;
+    }
     if (st->err) {
         set_last_error("htd: device-side consistency check failed (code " +
                        std::to_string(st->err) + ")");
@@ -290,13 +296,17 @@ int64_t htd_test_fail_alloc(int64_t k) {
 // with no room for them.
 void htd_test_no_helpers(int32_t on) { htd::g_no_helpers = on != 0; }
 
+// For tests: waits between the clusters of the calling thread's round kernels give up after so many
+// polls (0: the ordinary limit).
+void htd_test_wait_polls(int32_t polls) { htd::g_wait_polls = polls; }
+
 const char *htd_status_string(htd_status s) {
     switch (s) {
         case HTD_OK: return "ok";
         case HTD_EINVAL: return "invalid argument";
         case HTD_ENOMEM: return "device memory allocation failed";
         case HTD_ECUDA: return "CUDA error";
-        case HTD_ETIMEOUT: return "peel exceeded its round cap";
+        case HTD_ETIMEOUT: return "peel exceeded its round cap, or a wait in it gave up";
         case HTD_EOVERFLOW: return "graph too large for 32-bit adjacency offsets";
         case HTD_EUNSUPPORTED: return "graph too large for shared-memory balls";
     }
@@ -566,11 +576,6 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
             if (cudaEventElapsedTime(&ms, p0, p1) == cudaSuccess) {
                 local.ms_round_kernel += ms;
                 local.round_kernel_launches += 1;
-            }
-            if (w.status_host->err & htd::kErrBarrierTimeout) {
-                set_last_error("htd_truss_decompose: a grid barrier of the round kernel timed out");
-                ps = HTD_ETIMEOUT;
-                break;
             }
             ps = check_status_err(w.status_host);
         }

@@ -81,6 +81,7 @@ struct DevStatus : RoundCtr {
     unsigned long long cl_reg;      // (launch << 32) | helper blocks started
     unsigned long long cl_job;      // (launch << 40) | (job number << 16) | helper blocks taking part
     unsigned long long cl_done;     // helper blocks that finished a job
+    int32_t cl_beat;                // changes from round to round
     HelperJob cl_work;
     WindowCtr cl_wctr;
     RoundCtr cl_ctr;
@@ -116,7 +117,7 @@ enum : int32_t {
     kErrBallGrew = 1,        // a rebuilt ball was larger than before (cannot happen)
     kErrBallCapacity = 2,    // a ball did not fit its storage (cannot happen)
     kErrListOverflow = 4,    // a per-block BFS list overflowed (cannot happen)
-    kErrBarrierTimeout = 16, // a grid barrier gave up waiting
+    kErrBarrierTimeout = 16, // a wait between blocks (grid barrier, helper clusters) gave up
 };
 
 __device__ __forceinline__ unsigned lanemask_lt() {

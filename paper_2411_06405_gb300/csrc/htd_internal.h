@@ -195,8 +195,9 @@ htd_status initial_pass_r2(Handle *H, cudaStream_t s, int64_t *launches);
 
 // The normalised graph behind a public handle (htd_api.cu).
 GraphDev *graph_dev(htd_graph *g);
-// Set by htd_test_no_helpers for the calling thread.
+// Set by htd_test_no_helpers and htd_test_wait_polls for the calling thread.
 bool test_no_helpers();
+int32_t test_wait_polls();
 // Tells a handle that its decompositions run beside others (they then take less of the device).
 void set_shared_device(htd_graph *g, int32_t peers);
 // Peels in flight on a device, by whichever threads: they share its room for clusters.

@@ -95,6 +95,7 @@ struct LossArgs {
     uint32_t *pool2_new;
     int32_t cluster;    // the slot starts with the cluster round kernel
     int32_t launch;     // its number, from 1, among the launches of that kernel in this peel
+    int32_t wait_polls; // cluster round kernel: polls without progress after which a wait gives up
     int32_t no_helpers; // cluster round kernel: helpers end at once (a test of a busy device)
     int32_t max_split;  // phase launches: log2 of the warps one detection item may take
     int32_t timer;      // add the time of each phase to the status block
@@ -1450,8 +1451,10 @@ constexpr int kCRounds = 1024;       // rounds per launch
 constexpr int kHelpDetect = 1024, kAloneDetect = 4096, kMostDetect = 1 << 16;     // detection items
 constexpr int kHelpTest3 = 1 << 14, kAloneTest3 = 1 << 17, kMostTest3 = 1 << 20;  // radius-3 items
 constexpr int kHelpDelta = 16384, kAloneDelta = 65536, kMostDelta = 1 << 21;       // update items
-constexpr unsigned long long kHelperWaitNs = 20000000000ull;  // a helper gives up waiting for a job
-constexpr unsigned long long kLeadWaitNs = 4000000000ull;     // the leader, for its helpers
+// Polls (of about a microsecond) without any progress on the other side after which a helper gives
+// up waiting for a job, or the leader for its helpers: some minutes, which no phase within the limits
+// above takes.  Counted in polls, so that time in which the device runs others does not count.
+constexpr int kWaitPolls = 1 << 27;
 
 __device__ __forceinline__ void cluster_sync() {
     __syncwarp();
@@ -1555,8 +1558,7 @@ __device__ __forceinline__ void helper_blocks(const LossArgs &a, unsigned long l
     for (;;) {
         if (threadIdx.x == 0) {
             unsigned long long word = 0ull;  // 0: stop
-            const unsigned long long t0 = global_ns();
-            for (;;) {
+            for (int polls = 0, beat = vload(st->cl_beat);; polls++) {
                 const unsigned long long w = load_acquire(&st->cl_job);
                 if ((w >> 16) > (seen >> 16) && (w >> 40) == epoch) {
                     seen = w;
@@ -1566,9 +1568,14 @@ __device__ __forceinline__ void helper_blocks(const LossArgs &a, unsigned long l
                     }
                 }
                 if (load_acquire(&st->cl_exit) > epoch) break;
-                if (global_ns() - t0 > kHelperWaitNs) {
-                    atomicOr(&st->err, kErrBarrierTimeout);
-                    break;
+                if (polls >= a.wait_polls) {
+                    const int now = vload(st->cl_beat);
+                    if (now == beat) {
+                        atomicOr(&st->err, kErrBarrierTimeout);
+                        break;
+                    }
+                    beat = now;
+                    polls = 0;
                 }
                 __nanosleep(64);
             }
@@ -1737,9 +1744,15 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         cluster_sync();
         if (lead) {
             done_base += (unsigned)helpers;
-            const unsigned long long t0 = global_ns();
-            while (load_acquire(&st->cl_done) < done_base) {
-                if (global_ns() - t0 > kLeadWaitNs) {
+            unsigned long long last = 0ull;
+            for (int polls = 0;; polls++) {
+                const unsigned long long done = load_acquire(&st->cl_done);
+                if (done >= done_base) break;
+                if (done != last) {
+                    last = done;
+                    polls = 0;
+                }
+                if (polls >= a.wait_polls || vload(st->err) != 0) {
                     atomicOr(&st->err, kErrBarrierTimeout);
                     s_failed = 1;
                     break;
@@ -1875,6 +1888,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         // only counters that nothing changes before the next one (overflow marks, which the
         // phase now starting may set, are read where no phase sets them).
         const int nF = vload(ctr->nF), npitems = vload(ctr->npitems);
+        if (lead) *(volatile int *)&st->cl_beat = round + 1;  // for the helpers: rounds go on
         if (lead) wctr->nnext = 0;  // read by all before the barrier, used again after the next
         const long long nA = kH3 ? 2ll * c3_chunks(a) * nF : 0ll;
         if (npitems > a.pitems_cap || nA > (nclusters > 1 ? kMostTest3 : kAloneTest3)) {
@@ -2024,6 +2038,7 @@ LossArgs loss_args(Handle *H) {
     a.pool2_new = w.twin ? w.pool2_new : nullptr;
     a.cluster = 0;
     a.launch = 0;
+    a.wait_polls = test_wait_polls() > 0 ? test_wait_polls() : kWaitPolls;
     a.no_helpers = test_no_helpers() ? 1 : 0;
     a.max_split = H->shared_device ? 0 : 2;  // beside others, idle warps are theirs
     a.timer = 0;
