@@ -166,7 +166,11 @@ htd_status htd_csr(const htd_graph *g, int32_t *row_ptr_dev, int32_t *col_dev,
 
 /* h-support of every edge (Def. 2, Def. 3; the initial h-support loop of Algorithm 2):
  * sup_dev[e] = |N(u,h) ∩ N(v,h)| in the whole graph, u and v excluded.
- * sup_dev: device buffer of m int32.  1 <= h <= HTD_MAX_H. */
+ * sup_dev: device buffer of m int32.  1 <= h <= HTD_MAX_H.
+ * The balls stay in the handle's scratch until it is freed: per vertex an n-bit set, or 8 bytes for
+ * each of its 32-vertex groups with members where that is less.  Room for them is taken by an upper
+ * bound from the degrees, and at h = 3 n bits more per vertex may be held; what is held beyond the
+ * balls is given back at the end of the call where it is more than a 32nd of the device's memory. */
 htd_status htd_h_support(htd_graph *g, int32_t h, int32_t *sup_dev, void *stream);
 
 /* (k,h)-truss decomposition (Def. 4; Sec. 3 peeling): truss_dev[e] = t(e,h) for every

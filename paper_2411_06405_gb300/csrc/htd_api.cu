@@ -281,6 +281,27 @@ htd_status prepare_work(Handle *H, int32_t h, bool incremental, bool tiny = fals
 
 }  // namespace
 
+namespace htd {
+htd_status h_support_run(Handle *H, int32_t h, int32_t *sup_dev, cudaStream_t user) {
+    API_TRY(begin_call(H, user));
+    API_TRY(prepare_work(H, h, false));
+    H->w.twin = false;
+    H->w.dense_balls = false;  // h-support alone streams the smaller form of each ball
+    H->w.inc3 = false;
+    int64_t launches = 0;
+    const htd_status ip = initial_pass(H, h, H->pstream, &launches, nullptr, true);
+    g_launches += launches;
+    API_TRY(ip);
+    if (H->g.m > 0)
+        API_CHECK(cudaMemcpyAsync(sup_dev, H->w.sup, H->g.m * 4, cudaMemcpyDeviceToDevice, H->pstream));
+    API_CHECK(cudaMemcpyAsync(H->w.status_host, H->w.status, sizeof(DevStatus), cudaMemcpyDeviceToHost,
+                              H->pstream));
+    API_TRY(end_call(H, user));
+    if (H->w.status_host->pool_next > 0) H->w.support_words = H->w.status_host->pool_next;
+    return check_status_err(H->w.status_host);
+}
+}  // namespace htd
+
 extern "C" {
 
 // For tests of what a call leaves behind when memory runs out: the calling thread's k-th
@@ -464,23 +485,9 @@ htd_status htd_h_support(htd_graph *g, int32_t h, int32_t *sup_dev, void *stream
         set_last_error("htd_h_support: NULL argument or h outside [1, HTD_MAX_H]");
         return HTD_EINVAL;
     }
-    Handle *H = &g->H;
-    cudaStream_t user = static_cast<cudaStream_t>(stream);
-    API_TRY(begin_call(H, user));
-    API_TRY(prepare_work(H, h, false));
-    H->w.twin = false;
-    H->w.dense_balls = false;  // h-support alone streams the smaller form of each ball
-    H->w.inc3 = false;
-    int64_t launches = 0;
-    htd_status ip = htd::initial_pass(H, h, H->pstream, &launches, nullptr, true);
-    htd::g_launches += launches;
-    API_TRY(ip);
-    if (H->g.m > 0)
-        API_CHECK(cudaMemcpyAsync(sup_dev, H->w.sup, H->g.m * 4, cudaMemcpyDeviceToDevice, H->pstream));
-    API_CHECK(cudaMemcpyAsync(H->w.status_host, H->w.status, sizeof(htd::DevStatus),
-                              cudaMemcpyDeviceToHost, H->pstream));
-    API_TRY(end_call(H, user));
-    return check_status_err(H->w.status_host);
+    const htd_status st = htd::h_support_run(&g->H, h, sup_dev, static_cast<cudaStream_t>(stream));
+    htd::trim_support(&g->H);
+    return st;
 }
 
 htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32_t *truss_dev,
@@ -781,8 +788,10 @@ htd_status htd_hindex_decompose_ex(htd_graph *g, int32_t h, int32_t sweeps, int3
     Handle *H = &g->H;
     cudaStream_t user = static_cast<cudaStream_t>(stream);
     API_TRY(begin_call(H, user));
-    API_TRY(htd::hindex_run(g, H, h, sweeps, max_iter, (flags & HTD_HX_PRUNE) != 0u, truss_dev, hval_dev,
-                            stats, H->pstream));
+    const htd_status hs = htd::hindex_run(g, H, h, sweeps, max_iter, (flags & HTD_HX_PRUNE) != 0u, truss_dev,
+                                          hval_dev, stats, H->pstream);
+    htd::trim_support(H);
+    API_TRY(hs);
     return end_call(H, user);
 }
 

@@ -92,6 +92,7 @@ struct DevStatus : RoundCtr {
     unsigned long long st_phase_ns[8];  // time per phase (one block's view)
     unsigned long long st_phase_start;  // when the running phase launch began
     int64_t pool_next;         // words of ball storage taken (places handed out as balls are done)
+    int64_t ball_bound;        // words that storage takes at most
     int64_t st_ball_total;     // sum of the initial ball sizes
     int64_t st_pairs;          // candidate pairs tested
     int64_t st_lost;           // lost pairs

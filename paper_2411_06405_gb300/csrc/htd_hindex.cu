@@ -482,7 +482,7 @@ htd_status hindex_run(htd_graph *G, Handle *H, int32_t h, int32_t sweeps, int32_
         // H^(0) = sup(e,h), the h-support of every edge (the initial step of Algorithm 2)
         HX_CHECK(dev_alloc(&key, m, s));
         HX_CHECK(dev_alloc(&key2, m, s));
-        htd_status hs = htd_h_support(G, h, key, s);
+        htd_status hs = h_support_run(H, h, key, s);
         if (hs != HTD_OK) {
             st = hs;
             goto done;

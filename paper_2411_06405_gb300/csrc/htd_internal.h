@@ -86,6 +86,8 @@ struct PeelWork {
     bool twin = false;             // in use (set per call before the initial pass)
     uint32_t *pool_new = nullptr;
     uint32_t *pool2_new = nullptr;
+    int64_t support_words = 0;     // words the compact balls of this h take (0: not known yet)
+    int64_t keep_bytes = 0;        // what an h-support pass may hold beyond its balls
     uint32_t *pool2 = nullptr;
     bool inner_ready = false;      // pool2 was built before the radius-3 balls, which are ORs of it
     int64_t *dense_off = nullptr;  // n+1 offsets x * Wpad
@@ -176,6 +178,10 @@ htd_status ensure_twin(Handle *H, int64_t budget);
 // support_only: h-support alone (no peel follows).
 htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
                         htd_stats *timing, bool support_only);
+// Gives back what an h-support pass held beyond its balls, if that is much.
+void trim_support(Handle *H);
+// htd_h_support without that: the balls stay in the handle's scratch.
+htd_status h_support_run(Handle *H, int32_t h, int32_t *sup_dev, cudaStream_t user);
 // evs (nullable): kRoundEvents events marking the phase boundaries of the round.
 constexpr int kRoundEvents = 7;
 // timer (incremental rounds, instead of events): phase times go to the status block.

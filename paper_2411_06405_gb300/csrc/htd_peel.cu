@@ -62,7 +62,8 @@ struct BallArgs {
     const uint32_t *rows;
     const int32_t *row_of;
     int32_t or_deg;
-    int32_t bump;           // storage is taken from the pool in the order of completion
+    int64_t bump;           // words of the pool, from which storage is taken in the order of
+                            // completion (0: every ball has its place)
     const uint32_t *inner;  // k_ball_or: dense balls of radius h - 1, row x at x * Wpad
     DevStatus *st;
 };
@@ -162,13 +163,22 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
                                                                 (unsigned long long)stor);
             __syncthreads();
             off = *s_off64;
+            cap = a.bump - off;
+            if (stor > cap) off = 0;  // an error: the ball is left empty
             if (threadIdx.x == 0) a.ball_off[x] = off;
         } else {
             off = a.ball_off[x];
             cap = a.ball_off[x + 1] - off;
         }
         if (stor > cap) {
-            if (threadIdx.x == 0) atomicOr(&st->err, kErrBallCapacity);
+            if (threadIdx.x == 0) {
+                atomicOr(&st->err, kErrBallCapacity);
+                if (MODE == kModeStore) {
+                    a.ball_size[x] = 0;
+                    a.ball_nw[x] = 0;
+                    a.ball_meta[x] = make_int2(0, 0);
+                }
+            }
         } else if (dense) {
             uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
 #pragma unroll 4
@@ -392,6 +402,46 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
 __global__ void k_dense_offsets(int64_t n, int64_t Wpad, int64_t *__restrict__ off) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x)
         off[x] = x * Wpad;
+}
+
+// Upper bounds of the ball sizes, for storage without a counting pass: |B(x,1)| = degree + 1, and
+// |B(x,r)| is at most the sum of |B(y,r-1)| over the neighbours y of x (1 without any).  Sums stop
+// at `cap`, from which on a ball may be dense.  One warp per vertex.
+__global__ void __launch_bounds__(kBlock) k_ball_bound(int32_t n, int32_t cap, const int32_t *__restrict__ row_ptr,
+                                                      const int32_t *__restrict__ col,
+                                                      const int32_t *__restrict__ inner,
+                                                      int32_t *__restrict__ bound) {
+    const int lane = threadIdx.x & 31, nwarps = gridDim.x * (blockDim.x >> 5);
+    for (int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += nwarps) {
+        const int rb = row_ptr[x], re = row_ptr[x + 1];
+        int sum = 0;
+        if (!inner) {
+            sum = re - rb + 1;
+        } else {
+            for (int s0 = rb; s0 < re && sum < cap; s0 += 128) {
+                int v = 0;  // 128 values of at most `cap`, about n / 32
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int s = s0 + 32 * j + lane;
+                    if (s < re) v += inner[col[s]];
+                }
+                sum += __reduce_add_sync(0xffffffffu, v);
+            }
+            sum = max(sum, 1);
+        }
+        if (lane == 0) bound[x] = min(sum, cap);
+    }
+}
+
+// Storage of balls of at most the given sizes: dense, or a (word index, word) pair per member.
+__global__ void __launch_bounds__(kBlock) k_bound_words(int32_t n, int32_t Wpad, const int32_t *__restrict__ bound,
+                                                       DevStatus *st) {
+    unsigned long long words = 0ull;
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x)
+        words += (unsigned)min(Wpad, (2 * bound[x] + 3) & ~3);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) words += __shfl_xor_sync(0xffffffffu, words, o);
+    if ((threadIdx.x & 31) == 0 && words) atomicAdd((unsigned long long *)&st->ball_bound, words);
 }
 
 // Vertices of degree `deg` and more get a row (at most `cap` of them); the others none.
@@ -1150,7 +1200,50 @@ htd_status ensure_inner(Handle *H, cudaStream_t s, int64_t *launches, size_t fre
     return rs;
 }
 
+// Words that the balls of an h-support pass take at most.
+htd_status bound_storage(Handle *H, int32_t h, cudaStream_t s, int64_t *launches, int64_t *words) {
+    PeelWork &w = H->w;
+    GraphDev &g = H->g;
+    const int grid = (int)std::min<int64_t>(((int64_t)g.n * 32 + kBlock - 1) / kBlock, H->num_sms * 8);
+    int32_t *bound = w.ball_need, *inner = w.cand_list;  // neither is in use yet
+    for (int r = 1; r <= h; r++) {
+        std::swap(bound, inner);
+        k_ball_bound<<<grid, kBlock, 0, s>>>(g.n, w.Wpad, g.row_ptr, g.col, r > 1 ? inner : nullptr, bound);
+    }
+    k_bound_words<<<std::min<int64_t>((g.n + kBlock - 1) / kBlock, H->num_sms * 8), kBlock, 0, s>>>(g.n, w.Wpad, bound,
+                                                                                            w.status);
+    *launches += h + 1;
+    HTD_CHECK(cudaGetLastError());
+    HTD_CHECK(cudaMemcpyAsync(words, &w.status->ball_bound, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    HTD_CHECK(cudaStreamSynchronize(s));
+    return HTD_OK;
+}
+
 }  // namespace
+
+// What an h-support pass held beyond its balls goes back where it is more than a 32nd of the
+// device's memory (room that later peels, of this handle and others, look for): the radius-2 rows
+// that radius-3 balls were made of, and a pool taken by the bound that came out much too large.
+// Up to there a repeated call saves taking them again (DC-SBM 200k at h = 3, 5 GB of rows: 4 ms of
+// 23).  Scratch of a peel on the handle stays.
+void trim_support(Handle *H) {
+    PeelWork &w = H->w;
+    if (w.lost_keys || w.keep_bytes <= 0) return;
+    const int64_t rows = w.pool2 ? 4 * H->g.n * (int64_t)w.Wpad : 0;
+    const int64_t spare = w.pool ? 4 * (w.pool_words - w.support_words) : 0;
+    if (rows + spare <= w.keep_bytes) return;
+    if (w.pool2) {
+        dev_free(w.pool2, H->pstream);
+        w.pool2 = nullptr;
+        w.inner_ready = false;
+    }
+    if (spare > w.keep_bytes) {
+        destroy_rounds(H);
+        dev_free(w.pool, H->pstream);
+        w.pool = nullptr;
+        w.pool_words = 0;
+    }
+}
 
 // Initial pass: every vertex's ball and every edge's h-support, then the first min reduction.
 // Leaves the status ready for round 0 (support_only: the supports are all that is wanted).
@@ -1215,11 +1308,25 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             ba.rows = w.hub_bits;  // alive-adjacency sets, every edge alive
         }
         // Storage: dense balls have fixed places; h-support alone takes places as the balls are
-        // done, from a pool with room for all of them dense where that is a quarter of the free
-        // memory; else a first pass counts.
+        // done, from a pool with room for them: all dense where that is 64 MiB at most, else by an
+        // upper bound, from the second call on what they took.  Where that is more than a quarter
+        // of the free memory a first pass counts.
         int64_t total = n * (int64_t)w.Wpad;
         size_t free_b = 0, total_b = 0;
-        if (!w.dense_balls) HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
+        if (!w.dense_balls) {
+            HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
+            w.keep_bytes = (int64_t)(total_b / 32);
+        }
+        if (support_only) {
+            if (w.support_words > 0) {
+                total = w.support_words;
+            } else if (total > ((int64_t)1 << 24)) {
+                int64_t words = 0;
+                const htd_status bs = bound_storage(H, h, s, launches, &words);
+                if (bs != HTD_OK) return bs;
+                total = std::min(total, words);
+            }
+        }
         const bool room = total <= w.pool_words || (double)total * 4 <= (double)free_b / 4;
         auto take_pool = [&]() -> cudaError_t {
             if (total <= w.pool_words) return cudaSuccess;
@@ -1237,7 +1344,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
                                                                                                     w.ball_off);
             (*launches)++;
         } else if (support_only && room && total < ((int64_t)1 << 33)) {
-            if (take_pool() == cudaSuccess) ba.bump = 1;
+            if (take_pool() == cudaSuccess) ba.bump = w.pool_words;
         }
         if (!w.dense_balls && !ba.bump) {
             k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
@@ -1246,6 +1353,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
             HTD_CHECK(scan_exclusive<int32_t, int64_t>(w.ball_need, w.ball_off, n, w.scan_tmp, s, launches));
             HTD_CHECK(cudaMemcpyAsync(&total, w.ball_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
             HTD_CHECK(cudaStreamSynchronize(s));
+            w.support_words = total;
         }
         if (total >= ((int64_t)1 << 33)) {
             set_last_error("htd: h-hop balls need more than 32 GiB of storage");
@@ -1256,7 +1364,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         w.pool_used = total;
         // radius 3 from the dense radius-2 balls, where their rows cost less than the search
         const uint32_t *inner = nullptr;
-        if (h == 3 && (ba.bump || w.inc3) && or_beats_search(H)) {
+        if (h == 3 && (ba.bump > 0 || w.inc3) && or_beats_search(H)) {
             const htd_status rs = ensure_inner(H, s, launches, free_b);
             if (rs != HTD_OK) return rs;
             inner = w.inner_ready ? w.pool2 : nullptr;
