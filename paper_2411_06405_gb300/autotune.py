@@ -39,7 +39,10 @@ CANDIDATES = [
     {"max_union_vertices": 1 << 16, "flags": _lib.HTD_OPT_REBUILD},
 ]
 DEFAULT = {"max_union_vertices": 1 << 18, "flags": 0}
-BLOCK_MAX_NCLASS = 9  # log2 class of n above which one block per graph is not tried
+# log2 class of n above which one block per graph is not tried: it won in 28 of 29 groups up to
+# class 9 and in 3 of 8 of class 10 (43 graphs of n about 1,500 at h = 2: 10.3 ms against 12.0 as
+# unions), in none of class 11 and 12, where it took up to eleven times as long
+BLOCK_MAX_NCLASS = 10
 
 
 def group_key(n: int, src, dst, h: int) -> str:
@@ -87,8 +90,7 @@ def tune(graphs, sample: int = 64, candidates=None, seed: int = 0):
         nclass = int(key.split("_")[1][1:])
         times = {}
         for ci, c in enumerate(cands):
-            # one block per graph only pays for graphs of up to about a thousand vertices
-            # (a block's rounds grow with n^2 / 32 words); larger groups skip that candidate
+            # a block's rounds grow with n^2 / 32 words: larger groups skip that candidate
             if c["flags"] & _lib.HTD_OPT_BATCH_BLOCKS and nclass > BLOCK_MAX_NCLASS:
                 continue
             times[ci] = _time_batch(htd, torch, pick, c)

@@ -98,3 +98,17 @@ def test_autotune_partition_sends_block_groups_to_one_call():
     assert autotune._partition(graphs, None) == [([0, 1, 2, 3], autotune.DEFAULT["max_union_vertices"],
                                                   autotune.DEFAULT["flags"])]
     assert autotune._partition([], table) == []
+
+
+def test_committed_table_is_of_the_present_candidates():
+    # every group's setting is the fastest of the candidates that tune() times now
+    from paper_2411_06405_gb300 import _lib, autotune
+
+    for key, ent in autotune.load(autotune.TABLE_PATH).items():
+        ms = {int(i): t for i, t in ent["ms"].items()}
+        blocks_tried = int(key.split("_")[1][1:]) <= autotune.BLOCK_MAX_NCLASS
+        tried = {i for i, c in enumerate(autotune.CANDIDATES)
+                 if blocks_tried or not c["flags"] & _lib.HTD_OPT_BATCH_BLOCKS}
+        assert set(ms) == tried, key
+        best = autotune.CANDIDATES[min(ms, key=ms.get)]
+        assert {k: ent[k] for k in best} == best, key
