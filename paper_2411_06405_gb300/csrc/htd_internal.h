@@ -89,6 +89,7 @@ struct PeelWork {
     int64_t support_words = 0;     // words the compact balls of this h take (0: not known yet)
     int64_t keep_bytes = 0;        // what an h-support pass may hold beyond its balls
     uint32_t *pool2 = nullptr;
+    int64_t or_bytes = 0;          // algorithmic bytes of the balls made by ORs in the last pass
     bool inner_ready = false;      // pool2 was built before the radius-3 balls, which are ORs of it
     int64_t *dense_off = nullptr;  // n+1 offsets x * Wpad
     int32_t *ball_size2 = nullptr;

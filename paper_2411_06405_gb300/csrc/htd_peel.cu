@@ -366,14 +366,12 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
     uint4 *bits4 = reinterpret_cast<uint4 *>(bits);
     const uint4 *in4 = reinterpret_cast<const uint4 *>(a.inner);
     const int W4 = a.Wpad >> 2;
-    unsigned long long bytes = 0ull;  // one thread's: the rows read
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(&st->q_store, 1);
         __syncthreads();
         const int x = s_item;
         if (x >= a.n) break;
         const int rb = a.row_ptr[x], re = a.row_ptr[x + 1];
-        bytes += 4ull * a.W * (unsigned)(re - rb + 1);
         for (int c = rb; c == rb || c < re; c += kBlock) {
             const int cnt = min(kBlock, re - c);
             if (threadIdx.x < cnt) s_row[threadIdx.x] = a.col_live[c + threadIdx.x];
@@ -395,7 +393,6 @@ __global__ void __launch_bounds__(kBlock, 4) k_ball_or(BallArgs a) {
         store_ball<kModeStore>(a, x, bits, s_wsz, s_wnz, &s_off64);
         __syncthreads();
     }
-    if (a.count_bytes && threadIdx.x == 0 && bytes) atomicAdd(&st->st_bytes_ball, bytes);
 }
 
 // Offsets of dense balls: x * Wpad.
@@ -1253,6 +1250,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
     GraphDev &g = H->g;
     const int64_t n = g.n, m = g.m;
     w.inner_ready = false;
+    w.or_bytes = 0;
     H->cluster_launches = 0;
     std::memset(w.status_host, 0, sizeof(DevStatus));
     w.status_host->k = 2;
@@ -1373,6 +1371,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         if (timing) HTD_CHECK(cudaEventRecord(e0, s));
         if (inner) {
             ba.inner = inner;
+            w.or_bytes = 4 * (int64_t)w.W * (n + 2 * m);  // every row once, and once per adjacency slot
             k_ball_or<<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
         } else {
             k_ball<kModeStore><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
