@@ -1,4 +1,4 @@
-// htd_loss.cu -- exact incremental h-support updates for h <= 2.
+// htd_loss.cu -- exact incremental h-support updates for h <= 3 and the kernels that run the rounds.
 //
 // For h <= 2 the members a removal can take out of a ball are few and can be listed: an
 // old path of length <= h that used a removed edge (a,b) is a-b itself, x-a-b with x in
