@@ -30,7 +30,6 @@ constexpr int kSlotsPerGraph = 4;    // slots with the cluster round kernel
 void set_last_error(const std::string &msg) { g_last_error = msg; }
 
 namespace {
-constexpr int kMaxDevices = 64;
 constexpr uint64_t kPoolKeeps = (uint64_t)512 << 20;
 // Larger blocks are cudaMalloc's: mapping 8.6 GB through the pool took 6 ms, through cudaMalloc
 // a fraction of one.
@@ -38,16 +37,12 @@ constexpr size_t kLargeBytes = (size_t)64 << 20;
 constexpr size_t kStatusKeeps = 32;
 std::mutex g_mem_mutex;
 // Pools and pinned blocks end with their context (cudaDeviceReset): they are used only in it.
-struct ContextPool {
-    uint64_t context = 0;
-    cudaMemPool_t pool = nullptr;
-};
 struct PinnedStatus {
     int device;
     uint64_t context;
     DevStatus *p;
 };
-ContextPool g_pool[kMaxDevices];
+std::map<std::pair<int, uint64_t>, cudaMemPool_t> g_pool;  // by device and context
 std::vector<PinnedStatus> g_status;
 std::set<void *> g_large;
 thread_local int64_t g_fail_alloc = 0;
@@ -94,14 +89,13 @@ cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     }
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
     if (e != cudaSuccess) return e;
     const uint64_t context = current_context();
     cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
-        ContextPool &own = g_pool[dev];
-        if (!own.pool || own.context != context) {
+        const auto own = g_pool.find({dev, context});
+        if (own == g_pool.end()) {
             cudaMemPoolProps props;
             std::memset(&props, 0, sizeof(props));
             props.allocType = cudaMemAllocationTypePinned;
@@ -111,10 +105,10 @@ cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
             uint64_t keeps = kPoolKeeps;
             if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keeps);
             if (e != cudaSuccess) return e;
-            own.context = context;
-            own.pool = pool;
+            g_pool[{dev, context}] = pool;
+        } else {
+            pool = own->second;
         }
-        pool = own.pool;
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
@@ -160,8 +154,11 @@ void give_status_host(DevStatus *p) {
     cudaGetDevice(&device);
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
-        for (size_t i = g_status.size(); i-- > 0;)  // blocks of the device's earlier contexts went with them
-            if (g_status[i].device == device && g_status[i].context != context) g_status.erase(g_status.begin() + i);
+        // full of blocks of the device's other contexts: most likely ended, and the blocks with them
+        if (g_status.size() >= kStatusKeeps)
+            for (size_t i = g_status.size(); i-- > 0;)
+                if (g_status[i].device == device && g_status[i].context != context)
+                    g_status.erase(g_status.begin() + i);
         if (g_status.size() < kStatusKeeps) {
             g_status.push_back(PinnedStatus{device, context, p});
             return;
@@ -174,8 +171,8 @@ htd_status trim_memory(int device) {
     const uint64_t context = current_context();
     std::lock_guard<std::mutex> lk(g_mem_mutex);
     cudaError_t e = cudaSuccess;
-    if (device >= 0 && device < kMaxDevices && g_pool[device].pool && g_pool[device].context == context)
-        e = cudaMemPoolTrimTo(g_pool[device].pool, 0);
+    const auto own = g_pool.find({device, context});
+    if (own != g_pool.end()) e = cudaMemPoolTrimTo(own->second, 0);
     for (size_t i = g_status.size(); i-- > 0;) {
         if (g_status[i].context != context) continue;
         cudaFreeHost(g_status[i].p);
