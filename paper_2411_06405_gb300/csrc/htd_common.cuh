@@ -18,13 +18,13 @@ constexpr unsigned long long kTouchedMask = (1ull << kLostShift) - 1;
 // the cluster round kernel keeps its own in the shared memory of one of its blocks.
 struct RoundCtr {
     int32_t nF;                // frontier size of the current round
-    int32_t npitems;           // loss detection items of the current batch
     int32_t nuitems;           // support update items of the current batch
     int32_t nlost;             // lost-pair records of the current batch (duplicates nulled)
     int32_t nlost2;            // radius-2 lost-pair records of the current round (h = 3)
     int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
     int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
-    int32_t pad;
+    long long npitems;         // loss detection items of the current batch (64-bit: a round may want
+                               // more than 2^31, of which the list's capacity is taken)
     long long touched;         // the batch's lost pairs << kLostShift | alive edges at their endpoints
                                // (each vertex once per round)
     long long upd_work;        // adjacency slots reserved for the batch's updates

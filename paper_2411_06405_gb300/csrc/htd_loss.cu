@@ -515,6 +515,14 @@ __device__ __forceinline__ void write_pitem(const LossArgs &a, int i, int u, int
     a.pitems[2 * (int64_t)i + 1] = rows;
 }
 
+// Place of the first of a warp's `tot` detection items (the value of lane 31 counts; all lanes call it).
+__device__ __forceinline__ long long reserve_pitems(RoundCtr *ctr, int tot) {
+    long long base = 0;
+    if ((threadIdx.x & 31) == 31 && tot)
+        base = (long long)atomicAdd((unsigned long long *)&ctr->npitems, (unsigned long long)tot);
+    return __shfl_sync(0xffffffffu, base, 31);
+}
+
 // Splits the frontier's edge sides into detection items of at most 32 pairs (one warp
 // each), so a hub row is spread over many warps.  Sides that do not fit the item list are
 // left to the next slot of the round (resume point).
@@ -522,9 +530,9 @@ __device__ void ph_pair_items(const LossArgs &a) {
     DevStatus *st = a.st;
     const int units = 2 * vload(st->nF), u0 = vload(st->unit_begin);
     const int lane = threadIdx.x & 31;
-    const int stride = gridDim.x * blockDim.x;
-    for (int b = u0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < units; b += stride) {
-        const int u = b + lane;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t b = u0 + blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); b < units; b += stride) {
+        const int u = (int)min(b + lane, (int64_t)units);
         int nch = 0, start = 0, x = 0, y = 0;
         int4 rows = make_int4(0, 0, 0, 0);
         if (u < units) {
@@ -542,11 +550,9 @@ __device__ void ph_pair_items(const LossArgs &a) {
             if (lane >= o) incl += t;
         }
         const int tot = __shfl_sync(0xffffffffu, incl, 31);
-        int base = 0;
-        if (lane == 31 && tot) base = atomicAdd(&st->npitems, tot);
-        base = __shfl_sync(0xffffffffu, base, 31);
-        const int first = base + incl - nch;
-        const bool fits = first + nch <= a.pitems_cap;
+        const long long at = reserve_pitems(st, tot) + incl - nch;
+        const int first = (int)min(at, (long long)a.pitems_cap);
+        const bool fits = at + nch <= a.pitems_cap;
         if (!fits && nch) overflow_at(a, st, u);
         // a lane writes its one item, the whole warp the others (a hub row has hundreds)
         if (nch == 1 && first < a.pitems_cap) write_pitem(a, first, fits ? u : -1, start, x, y, rows);
@@ -690,7 +696,7 @@ __device__ __forceinline__ void ph_detect(const LossArgs &a) {
         s_counted = 0ull;
     }
     __syncthreads();
-    const int nitems = min(vload(st->npitems), a.pitems_cap), round = vload(st->round);
+    const int nitems = (int)min(vload(st->npitems), (long long)a.pitems_cap), round = vload(st->round);
     const int lane = threadIdx.x & 31;
     unsigned lane_pairs = 0u, lane_reads = 0u;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = gridDim.x * (blockDim.x >> 5);
@@ -1231,11 +1237,9 @@ __device__ __forceinline__ void select_one(const LossArgs &a, RoundCtr *ctr, boo
         n1 = (a.h < 2) ? 0 : (rows.y - rows.x + 31) >> 5;
     }
     const int incl = warp_incl_scan(n0 + n1);
-    int ibase = 0;
-    if (lane == 31) ibase = atomicAdd(&ctr->npitems, incl);
-    ibase = __shfl_sync(0xffffffffu, ibase, 31);
-    const int first = ibase + incl - (n0 + n1);
-    const bool fits0 = first + n0 <= a.pitems_cap, fits1 = first + n0 + n1 <= a.pitems_cap;
+    const long long at = reserve_pitems(ctr, incl) + incl - (n0 + n1);
+    const int first = (int)min(at, (long long)a.pitems_cap);
+    const bool fits0 = at + n0 <= a.pitems_cap, fits1 = at + n0 + n1 <= a.pitems_cap;
     if (p && !fits0) overflow_at(a, ctr, 2 * pos);
     if (p && n1 && !fits1) overflow_at(a, ctr, 2 * pos + 1);
     // few items are written by their own lane, a hub row's by the whole warp
@@ -1887,7 +1891,8 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         // Every block takes the decisions of this loop alike: between two barriers they read
         // only counters that nothing changes before the next one (overflow marks, which the
         // phase now starting may set, are read where no phase sets them).
-        const int nF = vload(ctr->nF), npitems = vload(ctr->npitems);
+        const int nF = vload(ctr->nF);
+        const long long npitems = vload(ctr->npitems);
         if (lead) *(volatile int *)&st->cl_beat = round + 1;  // for the helpers: rounds go on
         if (lead) wctr->nnext = 0;  // read by all before the barrier, used again after the next
         const long long nA = kH3 ? 2ll * c3_chunks(a) * nF : 0ll;
@@ -1897,7 +1902,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         }
         HelperJob job;
         job.phase = 0;
-        job.nitems = npitems;
+        job.nitems = (int)npitems;
         job.nF = nF;
         job.round = round;
         job.win_hi = win_hi;

@@ -260,3 +260,17 @@ def test_rounds_that_no_helper_joins(htd, scale, factor, h):
     assert st2["rounds"] == st["rounds"]
     if h == 1:  # (rounds of up to a million update items)
         assert st2["kernel_launches"] > st["kernel_launches"] + 40
+
+
+def test_clique_of_more_items_than_an_int_holds(htd):
+    # all 12.5 M edges of a clique go in one round: 25 M edge sides of 157 detection items each are
+    # 3.9e9 items, of which the list takes its 2^22
+    n = 5000
+    u, v = (torch.from_numpy(x.astype(np.int32)).cuda() for x in np.triu_indices(n, 1))
+    g = htd.htd_build_csr(n, u, v)
+    for flags in (0, htd.HTD_OPT_PERSISTENT_ROUNDS, htd.HTD_OPT_COMPACT_BALLS):
+        t, _, st = htd.htd_truss_decompose(g, 2, flags=flags)
+        assert bool((t == n).all()) and st["rounds"] == 1
+    t, _, _ = htd.htd_truss_decompose(g, 3)
+    assert bool((t == n).all())
+    g.free()
