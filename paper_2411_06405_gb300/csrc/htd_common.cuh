@@ -19,8 +19,9 @@ constexpr unsigned long long kTouchedMask = (1ull << kLostShift) - 1;
 struct RoundCtr {
     int32_t nF;                // frontier size of the current round
     int32_t nuitems;           // support update items of the current batch
-    int32_t nlost;             // lost-pair records of the current batch (duplicates nulled)
-    int32_t nlost2;            // radius-2 lost-pair records of the current round (h = 3)
+    // lost-pair records wanted in the current batch (duplicates nulled), and radius-2 ones (h = 3):
+    // unsigned, since 2^25 radius-3 items of up to 128 pairs may want more than 2^31
+    uint32_t nlost, nlost2;
     int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
     int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
     long long npitems;         // loss detection items of the current batch (64-bit: a round may want

@@ -390,21 +390,21 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ct
     const int rank = __popc(wantb & lanemask_lt());
     const long long wtot = __shfl_sync(0xffffffffu, wincl, 31);
     long long wbase = 0;
-    int ibase = 0;
+    unsigned ibase = 0u;
     if (lane == 0) {
         if (!r2)
             wbase = (long long)atomicAdd((unsigned long long *)&ctr->upd_work, (unsigned long long)wtot);
-        ibase = atomicAdd(r2 ? &ctr->nlost2 : &ctr->nlost, __popc(wantb));
+        ibase = atomicAdd(r2 ? &ctr->nlost2 : &ctr->nlost, (unsigned)__popc(wantb));
     }
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
     ibase = __shfl_sync(0xffffffffu, ibase, 0);
     int4 *const lostv = r2 ? lost2_list(a, round) : lost_list(a, round);
     unsigned long long *const keys = r2 ? a.keys2 : a.keys;
     const unsigned cmask = r2 ? a.cap2_mask : a.cap_mask;
-    const int lmax = r2 ? a.lost2_max : a.lost_max;
+    const unsigned lmax = (unsigned)(r2 ? a.lost2_max : a.lost_max);
     int rec_idx = -1;
     if (want) {
-        const int idx = ibase + rank;
+        const unsigned idx = ibase + (unsigned)rank;
         if (idx >= lmax || (!r2 && wbase + wincl > a.upd_budget)) {
             overflow_at(a, ctr, u);
             if (idx < lmax) lostv[idx] = make_int4(-1, -1, -1, 0);
@@ -434,7 +434,7 @@ __device__ __forceinline__ void record_lost_warp(const LossArgs &a, RoundCtr *ct
                 }
             }
             lostv[idx] = rec;
-            if (rec.x >= 0) rec_idx = idx;
+            if (rec.x >= 0) rec_idx = (int)idx;
             if (r2 && !kTwin) {
                 // B2_new(v) differs from the stored B2(v) only at vertices marked here
                 a.touch2[x] = round;
@@ -894,7 +894,7 @@ __device__ __forceinline__ void apply_lost(const LossArgs &a, int t, int nt, int
 }
 
 __device__ void ph_apply(const LossArgs &a) {
-    apply_lost(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, min(vload(a.st->nlost), a.lost_max),
+    apply_lost(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, (int)min(vload(a.st->nlost), (unsigned)a.lost_max),
                vload(a.st->round));
 }
 
@@ -1204,7 +1204,7 @@ __device__ void ph_apply2(const LossArgs &a) {
     DevStatus *st = a.st;
     unsigned lane_real = 0u;
     apply_lost2(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x,
-                min(vload(st->nlost2), a.lost2_max), vload(st->round), lane_real);
+                (int)min(vload(st->nlost2), (unsigned)a.lost2_max), vload(st->round), lane_real);
     unsigned long long real = lane_real;
     for (int o = 16; o > 0; o >>= 1) real += __shfl_xor_sync(0xffffffffu, real, o);
     if ((threadIdx.x & 31) == 0 && real) atomicAdd((unsigned long long *)&st->st_lost2, real);
@@ -1701,10 +1701,10 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         if (applied) return;
         const RoundCtr *const prev = ctrs + ((round & 1) ^ 1);
         const int t = nthreads - 1 - gt;  // the warps with fewest detection items first
-        apply_lost(a, t, nthreads, min(vload(prev->nlost), a.lost_max), round - 1);
+        apply_lost(a, t, nthreads, (int)min(vload(prev->nlost), (unsigned)a.lost_max), round - 1);
         if (kH3) {
             unsigned real = 0u;
-            apply_lost2(a, t, nthreads, min(vload(prev->nlost2), a.lost2_max), round - 1, real);
+            apply_lost2(a, t, nthreads, (int)min(vload(prev->nlost2), (unsigned)a.lost2_max), round - 1, real);
             stat_add(s_stat, kStatLost2, real);
         }
         applied = true;
@@ -1917,7 +1917,7 @@ __global__ void __launch_bounds__(kCBlock, 1) k_rounds_cluster(const __grid_cons
         if (kH3) {
             // too many items, or no room for the items or the radius-2 losses (a halt)
             const long long nc3 = vload(ctr->nc3items);
-            if (nA + nc3 > a.c3items_cap || vload(ctr->nlost2) > a.lost2_max) {
+            if (nA + nc3 > a.c3items_cap || vload(ctr->nlost2) > (unsigned)a.lost2_max) {
                 stage = kStageTest3;
                 break;
             }
