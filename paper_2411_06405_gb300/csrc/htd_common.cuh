@@ -74,6 +74,8 @@ struct DevStatus : RoundCtr {
     // incremental (h <= 2) rounds
     int32_t cont;              // 1: the current round continues (its frontier is removed)
     int32_t unit_begin;        // first frontier edge side the next loss detection tests
+    int32_t unit_span;         // edge sides it takes items of (a continued round; else all)
+    int32_t pitems_cap;        // detection items one batch holds
     int32_t stage;             // graph path: first phase launch the cluster round kernel left to the
                                // launches after it (RoundStage), kStageNone if none
     // cluster round kernel with helpers (monotonic over the launches of one peel)

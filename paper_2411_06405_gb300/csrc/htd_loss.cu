@@ -523,13 +523,17 @@ __device__ __forceinline__ long long reserve_pitems(RoundCtr *ctr, int tot) {
     return __shfl_sync(0xffffffffu, base, 31);
 }
 
-// Splits the frontier's edge sides into detection items of at most 32 pairs (one warp
-// each), so a hub row is spread over many warps.  Sides that do not fit the item list are
-// left to the next slot of the round (resume point).
+// Items of the frontier's remaining edge sides, of at most 32 pairs (one warp each), so a hub
+// row is spread over many warps.  Sides beyond unit_span, or that do not fit the item list, are
+// left to the next slot of the round (resume point).  (Dense graphs: without the span the sides
+// that fitted were spread over all of them, the resume point moved by a few sides a slot or not
+// at all, and a round could take every slot a peel is given.)
 __device__ void ph_pair_items(const LossArgs &a) {
     DevStatus *st = a.st;
-    const int units = 2 * vload(st->nF), u0 = vload(st->unit_begin);
+    const int all = 2 * vload(st->nF), u0 = vload(st->unit_begin);
+    const int units = (int)min((int64_t)all, (int64_t)u0 + vload(st->unit_span));
     const int lane = threadIdx.x & 31;
+    if (units < all && blockIdx.x == 0 && threadIdx.x == 0) overflow_at(a, st, units);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t b = u0 + blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); b < units; b += stride) {
         const int u = (int)min(b + lane, (int64_t)units);

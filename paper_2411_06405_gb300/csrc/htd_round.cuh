@@ -47,6 +47,15 @@ __device__ __forceinline__ void round_finalize(DevStatus *st, int initial) {
     const int nF = st->nF;
     const bool unfinished = !initial && st->overflow_unit != INT_MAX && al > 0;
     st->cont = unfinished ? 1 : 0;
+    // Edge sides reserve their items in no order, so where they do not all fit any side may be left
+    // over, the first one among them: the next batch takes as many sides as should fit (less, if
+    // that is wrong again, until it is right)
+    if (!unfinished) {
+        st->unit_span = INT_MAX;
+    } else if (st->npitems > st->pitems_cap) {
+        const long long sides = min(st->unit_span, 2 * nF - st->unit_begin);
+        st->unit_span = (int)max(1ll, sides * st->pitems_cap / st->npitems * 7 / 8);
+    }
     st->unit_begin = unfinished ? st->overflow_unit : 0;
     st->overflow_unit = INT_MAX;
     if (!initial && nF > 0 && !unfinished) {

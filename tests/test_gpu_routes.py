@@ -274,3 +274,17 @@ def test_clique_of_more_items_than_an_int_holds(htd):
     t, _, _ = htd.htd_truss_decompose(g, 3)
     assert bool((t == n).all())
     g.free()
+
+
+def test_batches_of_a_round_move_on(htd):
+    # a dense graph: one round has three times the detection items that a batch holds.  The sides
+    # that fit a batch are its first ones, so that a handful of batches finish the round
+    n = 3000
+    s, d = erdos_renyi_gnm(n, 200000, 30)
+    g = gpu_graph(htd, n, s, d)
+    ref = None
+    for flags in (0, htd.HTD_OPT_PERSISTENT_ROUNDS, htd.HTD_OPT_COMPACT_BALLS) * 4:
+        t, stamp, st = htd.htd_truss_decompose(g, 2, stamps=True, flags=flags)
+        assert st["slots"] < st["rounds"] + 20, flags
+        ref = ref or (t, stamp)
+        assert torch.equal(t, ref[0]) and torch.equal(stamp, ref[1])
