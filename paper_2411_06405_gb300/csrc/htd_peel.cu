@@ -1313,11 +1313,9 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         // of the free memory a first pass counts.
         int64_t total = n * (int64_t)w.Wpad;
         size_t free_b = 0, total_b = 0;
-        if (!w.dense_balls) {
+        if (support_only) {
             HTD_CHECK(cudaMemGetInfo(&free_b, &total_b));
             w.keep_bytes = (int64_t)(total_b / 32);
-        }
-        if (support_only) {
             if (w.support_words > 0) {
                 total = w.support_words;
             } else if (total > ((int64_t)1 << 24)) {
