@@ -17,13 +17,6 @@ constexpr unsigned long long kTouchedMask = (1ull << kLostShift) - 1;
 // Work counters of one removal round.  The launches of a round keep them in the status block;
 // the cluster round kernel keeps its own in the shared memory of one of its blocks.
 struct RoundCtr {
-    int32_t nF;                // frontier size of the current round
-    int32_t nuitems;           // support update items of the current batch
-    // lost-pair records wanted in the current batch (duplicates nulled), and radius-2 ones (h = 3):
-    // unsigned, since 2^25 radius-3 items of up to 128 pairs may want more than 2^31
-    uint32_t nlost, nlost2;
-    int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
-    int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
     long long npitems;         // loss detection items of the current batch (64-bit: a round may want
                                // more than 2^31, of which the list's capacity is taken)
     long long touched;         // the batch's lost pairs << kLostShift | alive edges at their endpoints
@@ -31,6 +24,14 @@ struct RoundCtr {
     long long upd_work;        // adjacency slots reserved for the batch's updates
     long long nc3items;        // stored radius-3 candidate items of the current round (64-bit: the
                                // reservations of a huge round may pass 2^31 before it halts)
+    // lost-pair records wanted in the current batch (duplicates nulled), and radius-2 ones (h = 3):
+    // unsigned, since 2^25 radius-3 items of up to 128 pairs may want more than 2^31
+    uint32_t nlost, nlost2;
+    int32_t nuitems;           // support update items of the current batch
+    int32_t overflow_unit;     // smallest edge side whose lost pairs did not fit (INT_MAX)
+    int32_t unused[4];         // (what follows shares a sector with the fields after it)
+    int32_t halt;              // 1: a round ran out of room; the host finishes it by rebuilds
+    int32_t nF;                // frontier size of the current round
 };
 
 // Lists of the cluster round kernel: its window, and the edges the last updates took to the
@@ -46,10 +47,16 @@ struct HelperJob {
 
 // Device-resident state of one peel.  Written only by kernels (and zero-initialised by
 // the host before the first pass); read by the host between CUDA-graph launches.
+// Every kernel of a round begins with `alive` and goes on with the frontier, the round and the level:
+// they lie in one 32-byte sector with nF, so that the kernel waits for L2 once (in three sectors a
+// rebuild round's launches took 0.2 to 0.6 us longer each).
 struct DevStatus : RoundCtr {
+    int64_t alive;             // edges not yet removed
     int32_t k;                 // current peeling level (Algorithm 1's k)
     int32_t round;             // removal rounds completed
-    int64_t alive;             // edges not yet removed
+    int32_t cont;              // 1: the current round continues (its frontier is removed)
+    int32_t stage;             // graph path: first phase launch the cluster round kernel left to the
+                               // launches after it (RoundStage), kStageNone if none
     int32_t cand_cnt[kMaxH];   // candidate vertices found at BFS depth 0..h-1
     int32_t nchanged;          // vertices whose ball shrank this round
     int32_t nitems;            // h-support work items this round
@@ -72,12 +79,9 @@ struct DevStatus : RoundCtr {
     unsigned long long st_bytes_hsup;  // algorithmic bytes, intersections
     unsigned long long st_bytes_hsup_init;  // the initial pass's share of st_bytes_hsup
     // incremental (h <= 2) rounds
-    int32_t cont;              // 1: the current round continues (its frontier is removed)
     int32_t unit_begin;        // first frontier edge side the next loss detection tests
     int32_t unit_span;         // edge sides it takes items of (a continued round; else all)
     int32_t pitems_cap;        // detection items one batch holds
-    int32_t stage;             // graph path: first phase launch the cluster round kernel left to the
-                               // launches after it (RoundStage), kStageNone if none
     // cluster round kernel with helpers (monotonic over the launches of one peel)
     unsigned long long cl_lead;     // last launch that has a leader
     unsigned long long cl_exit;     // launches whose leader has finished
@@ -107,6 +111,8 @@ struct DevStatus : RoundCtr {
     int64_t st_lost2;          // radius-2 lost pairs
     int64_t st_recovered;      // rounds finished by the rebuild recovery
 };
+
+static_assert(sizeof(RoundCtr) == 72, "halt and nF lie in the third sector, before DevStatus::alive");
 
 // Phases of an incremental round, in order, as the graph path launches them.
 enum RoundStage : int32_t {
