@@ -653,6 +653,8 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
         const int64_t batch_cap =
             (H->g.m + (incremental ? w.status_host->st_ball_total / 2 + 1 : 0)) / (w.twin ? 1 : R) + 3;
         int64_t batches = 0;
+        int cluster_reads = 0;  // reads of the status before slots with the cluster round kernel
+        int continued = 0;      // reads in a row that found a round of several batches
         bool timing_ok = by_events;
         while (w.status_host->alive > 0) {
             if (++batches > batch_cap) {
@@ -671,11 +673,17 @@ htd_status htd_truss_decompose_ex(htd_graph *g, int32_t h, uint32_t flags, int32
                 // slot the cluster round kernel would return at once (128-slot tables, ER
                 // n = 2,000 at h = 2: 49 ms with it, 35 without)
                 const bool by_cluster = w.twin && w.status_host->cont == 0;
-                const int slots = by_cluster ? (int)std::min<int64_t>(R, batches) : htd::kRoundsPerGraph;
+                // (such a round often needs one batch more: two slots, then more at a time, and one
+                // with the cluster kernel for what comes after it)
+                const bool in_batches = w.twin && !by_cluster;
+                const int slots = by_cluster   ? std::min(R, ++cluster_reads)
+                                  : in_batches ? std::min(htd::kRoundsPerGraph, 2 << std::min(continued, 3)) + 1
+                                               : htd::kRoundsPerGraph;
+                continued = in_batches ? continued + 1 : 0;
                 for (int r = 0; r < slots; r++) {
                     API_TRY(htd::enqueue_round(H, H->pstream, &launches,
                                                timed ? &H->round_events[htd::kRoundEvents * r] : nullptr,
-                                               timing, by_cluster));
+                                               timing, by_cluster || (in_batches && r == slots - 1)));
                 }
             }
             count_launches();
