@@ -295,6 +295,7 @@ htd_status h_support_run(Handle *H, int32_t h, int32_t *sup_dev, cudaStream_t us
                               H->pstream));
     API_TRY(end_call(H, user));
     if (H->w.status_host->pool_next > 0) H->w.support_words = H->w.status_host->pool_next;
+    if (H->w.status_host->pool_next > H->w.pool_words) H->w.status_host->err |= kErrBallCapacity;
     return check_status_err(H->w.status_host);
 }
 }  // namespace htd

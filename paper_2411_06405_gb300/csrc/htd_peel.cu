@@ -62,8 +62,8 @@ struct BallArgs {
     const uint32_t *rows;
     const int32_t *row_of;
     int32_t or_deg;
-    int64_t bump;           // words of the pool, from which storage is taken in the order of
-                            // completion (0: every ball has its place)
+    int32_t bump;           // storage is taken from the pool in the order of completion; the pool
+                            // has room for all of it (bound_storage, or an earlier pass)
     const uint32_t *inner;  // k_ball_or: dense balls of radius h - 1, row x at x * Wpad
     DevStatus *st;
 };
@@ -163,22 +163,13 @@ __device__ __forceinline__ void store_ball(const BallArgs &a, int x, uint32_t *b
                                                                 (unsigned long long)stor);
             __syncthreads();
             off = *s_off64;
-            cap = a.bump - off;
-            if (stor > cap) off = 0;  // an error: the ball is left empty
             if (threadIdx.x == 0) a.ball_off[x] = off;
         } else {
             off = a.ball_off[x];
             cap = a.ball_off[x + 1] - off;
         }
         if (stor > cap) {
-            if (threadIdx.x == 0) {
-                atomicOr(&st->err, kErrBallCapacity);
-                if (MODE == kModeStore) {
-                    a.ball_size[x] = 0;
-                    a.ball_nw[x] = 0;
-                    a.ball_meta[x] = make_int2(0, 0);
-                }
-            }
+            if (threadIdx.x == 0) atomicOr(&st->err, kErrBallCapacity);
         } else if (dense) {
             uint4 *dst = reinterpret_cast<uint4 *>(a.pool + off);
 #pragma unroll 4
@@ -430,7 +421,9 @@ __global__ void __launch_bounds__(kBlock) k_ball_bound(int32_t n, int32_t cap, c
     }
 }
 
-// Storage of balls of at most the given sizes: dense, or a (word index, word) pair per member.
+// Storage of balls of at most the given sizes: dense, or a (word index, word) pair per member.  A
+// ball is stored as pairs when these take at most its W words, and a word holds a member at least,
+// so that store_ball never takes more (tests/test_ball_bound.py).
 __global__ void __launch_bounds__(kBlock) k_bound_words(int32_t n, int32_t Wpad, const int32_t *__restrict__ bound,
                                                        DevStatus *st) {
     unsigned long long words = 0ull;
@@ -1342,7 +1335,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
                                                                                                     w.ball_off);
             (*launches)++;
         } else if (support_only && room && total < ((int64_t)1 << 33)) {
-            if (take_pool() == cudaSuccess) ba.bump = w.pool_words;
+            if (take_pool() == cudaSuccess) ba.bump = 1;
         }
         if (!w.dense_balls && !ba.bump) {
             k_ball<kModeCount><<<w.grid_ball, kBlock, w.smem_ball, s>>>(ba);
@@ -1362,7 +1355,7 @@ htd_status initial_pass(Handle *H, int32_t h, cudaStream_t s, int64_t *launches,
         w.pool_used = total;
         // radius 3 from the dense radius-2 balls, where their rows cost less than the search
         const uint32_t *inner = nullptr;
-        if (h == 3 && (ba.bump > 0 || w.inc3) && or_beats_search(H)) {
+        if (h == 3 && (ba.bump || w.inc3) && or_beats_search(H)) {
             const htd_status rs = ensure_inner(H, s, launches, free_b);
             if (rs != HTD_OK) return rs;
             inner = w.inner_ready ? w.pool2 : nullptr;
