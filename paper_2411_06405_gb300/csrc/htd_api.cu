@@ -48,6 +48,7 @@ std::set<void *> g_large;
 thread_local int64_t g_fail_alloc = 0;
 thread_local bool g_no_helpers = false;
 thread_local int32_t g_wait_polls = 0;
+thread_local uint64_t g_context = 0;  // of the thread's present call
 }  // namespace
 
 uint64_t current_context() {
@@ -90,7 +91,7 @@ cudaError_t alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const uint64_t context = current_context();
+    const uint64_t context = g_context;
     cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
@@ -121,7 +122,14 @@ cudaError_t dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
-htd_status refuse_capture(cudaStream_t user) {
+uint64_t call_context() { return g_context; }
+
+htd_status enter_call(cudaStream_t user) {
+    g_context = current_context();
+    if (g_context == 0) {  // a thread's first call: the runtime has not bound its context yet
+        (void)cudaFree(nullptr);
+        g_context = current_context();
+    }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const cudaError_t e = cudaStreamIsCapturing(user, &cap);
     if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) return HTD_OK;
@@ -131,7 +139,7 @@ htd_status refuse_capture(cudaStream_t user) {
 }
 
 DevStatus *take_status_host() {
-    const uint64_t context = current_context();
+    const uint64_t context = g_context;
     {
         std::lock_guard<std::mutex> lk(g_mem_mutex);
         for (size_t i = g_status.size(); i-- > 0;) {
@@ -190,7 +198,7 @@ cudaError_t raise_smem_limit(const void *func, size_t bytes) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const uint64_t context = current_context();
+    const uint64_t context = g_context;
     std::lock_guard<std::mutex> lk(mu);
     auto &cur = limit[{dev, func}];
     if (cur.first == context && cur.second >= bytes) return cudaSuccess;
@@ -234,12 +242,17 @@ using htd::set_last_error;
 
 namespace {
 
-htd_status begin_call(Handle *H, cudaStream_t user) {
-    API_CHECK(cudaSetDevice(H->g.device));
-    API_TRY(htd::refuse_capture(user));
+// The handle's stream goes on after what is on the caller's.
+htd_status follow_caller(Handle *H, cudaStream_t user) {
     API_CHECK(cudaEventRecord(H->ev_in, user));
     API_CHECK(cudaStreamWaitEvent(H->pstream, H->ev_in, 0));
     return HTD_OK;
+}
+
+htd_status begin_call(Handle *H, cudaStream_t user) {
+    API_CHECK(cudaSetDevice(H->g.device));
+    API_TRY(htd::enter_call(user));
+    return follow_caller(H, user);
 }
 
 htd_status end_call(Handle *H, cudaStream_t user) {
@@ -380,7 +393,7 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
         return HTD_EOVERFLOW;
     }
     cudaStream_t user = static_cast<cudaStream_t>(stream);
-    API_TRY(htd::refuse_capture(user));
+    API_TRY(htd::enter_call(user));
     htd_graph *G = new htd_graph();
     Handle *H = &G->H;
     htd_status st = HTD_OK;
@@ -404,7 +417,7 @@ htd_status htd_build_csr(int32_t n, const int32_t *src, const int32_t *dst, int6
             return fail(HTD_ECUDA);
         }
     }
-    st = begin_call(H, user);
+    st = follow_caller(H, user);
     if (st != HTD_OK) return fail(st);
     const int32_t *s_dev = src, *d_dev = dst;
     if (!inputs_on_device && m_in > 0) {

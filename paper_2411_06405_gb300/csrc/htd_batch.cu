@@ -289,7 +289,7 @@ extern "C" htd_status htd_truss_decompose_batched(
     int32_t unions = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (total_in > 0) {
-        const htd_status cs = refuse_capture(s);
+        const htd_status cs = enter_call(s);
         if (cs != HTD_OK) return cs;
     }
     int64_t out_pos = 0;

@@ -148,9 +148,10 @@ cudaError_t dev_alloc(T **p, int64_t count, cudaStream_t s) {
     return dev_alloc_bytes(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T), s);
 }
 void dev_free(void *p, cudaStream_t s);
-// HTD_ECUDA while a graph is captured from the caller's stream.  Allocations made during a capture
-// are nodes of that graph: a handle would keep addresses that no memory stands behind.
-htd_status refuse_capture(cudaStream_t user);
+// Begins a call, before its first allocation: HTD_ECUDA while a graph is captured from the caller's
+// stream (allocations made during a capture are nodes of that graph: a handle would keep addresses
+// that no memory stands behind), else notes the context that the call's allocations belong to.
+htd_status enter_call(cudaStream_t user);
 // Gives back what the pool and the list of pinned status blocks keep for the current context.
 htd_status trim_memory(int device);
 // Pinned status blocks, kept for the next handle (at most 32).
@@ -159,6 +160,8 @@ void give_status_host(DevStatus *p);
 // Id of the current context, unique over the process: what is kept beside handles (pools, pinned
 // blocks, limits raised on kernels, launch shapes) is valid in one context only.
 uint64_t current_context();
+// The same for the thread's present call, found once by enter_call: a call allocates a dozen times.
+uint64_t call_context();
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the current device.
 // The limit is a process-wide property of the function: it is only ever raised (under a
 // lock), so that a call for a small graph in one thread cannot lower it below what a

@@ -2145,7 +2145,7 @@ int cluster_size(int *resident) {
 
 template <bool kTwin>
 htd_status phase_grids(Handle *H, PhaseGrids &pg) {
-    const uint64_t context = current_context();
+    const uint64_t context = call_context();
     if (pg.device == H->g.device && pg.context == context) return HTD_OK;
     int od = 0, od3 = 0, ou = 0, ot = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&od, k_loss_detect<kTwin>, kBlock, 0) != cudaSuccess ||

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 CHILD = r"""
-import ctypes, glob, sys
+import ctypes, glob, sys, threading
 import numpy as np
 from paper_2411_06405_gb300 import _lib
 from synth import erdos_renyi_gnm
@@ -43,6 +43,12 @@ for _ in range(2):
     assert rt.cudaSetDevice(0) == 0 and rt.cudaDeviceReset() == 0
     for h in (3, 2, 1, 4, 2):
         assert all(np.array_equal(a, b) for a, b in zip(run(h), ref[h])), h
+    # a thread that has made no CUDA call before
+    got = []
+    th = threading.Thread(target=lambda: got.append(run(2)))
+    th.start()
+    th.join()
+    assert all(np.array_equal(a, b) for a, b in zip(got[0], ref[2]))
 print("same after reset")
 """
 
